@@ -29,6 +29,49 @@ __device__ __forceinline__ void mma_bf16_16816(float (&c)[4], const uint32_t (&a
         : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
+// The shot boundaries off[B][S+1] as kernels get them, a row of `stride` entries per prompt.  For the
+// scoring pass three entries of kNoBound follow the S + 1 boundaries of every row, so that it can
+// walk along a row one boundary ahead without comparing indices (and a row without boundaries is
+// these three alone).  A table of up to kTableArgs entries (three kilobytes: 8 prompts of 92 shots, or
+// one of 764) travels in the launch's own parameters; a larger one is copied to the workspace and `ptr` is
+// its address.  A copy of a small table costs a host-to-device transfer of 1.5 us and a gap of 2 to
+// 5 us on either side of it.
+constexpr int kTableArgs = 768;
+constexpr int kNoBound = 0x7fffffff;
+constexpr int kTableEnd = 3;
+struct ShotTable {
+    const int* ptr;            // device table, or NULL: the entries are in `data`
+    int stride;
+    int data[kTableArgs];
+};
+// Boundaries of prompt b.
+__device__ __forceinline__ const int* table_row(const ShotTable& t, int b) {
+    return (t.ptr ? t.ptr : t.data) + (size_t)b * t.stride;
+}
+// Number of the n ascending entries o[0..n) that are <= x.
+__device__ __forceinline__ int count_le(const int* o, int n, int x) {
+    int lo = 0;
+    while (lo < n) {
+        const int mid = (lo + n) >> 1;
+        if (o[mid] <= x) lo = mid + 1; else n = mid;
+    }
+    return lo;
+}
+// The same by a whole warp, 32 probes a round: at most three rounds for 8,193 entries.
+__device__ __forceinline__ int count_le_warp(const int* o, int n, int x) {
+    const int lane = threadIdx.x & 31;
+    int lo = 0;
+    while (n > 0) {
+        const int step = (n + 31) >> 5;
+        const int first = lane * step;
+        const bool le = first < n && o[lo + min(first + step, n) - 1] <= x;
+        const int skip = min(__popc(__ballot_sync(0xffffffffu, le)) * step, n);   // whole blocks that are <= x
+        lo += skip;
+        n = min(step, n - skip) - 1;                                                // the next block's last entry is > x
+    }
+    return lo;
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

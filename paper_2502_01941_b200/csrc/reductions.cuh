@@ -8,7 +8,9 @@
 //                              fix one reference per item (score_fast.cuh, score_stream.cuh)
 //   part_m [U][P][Rpad]       per (piece, row) reference -- written only by the exact kernel
 //                              (score_tc.cuh), whose running maximum moves inside an item
-//   redo   [U*nchunk]         1 for the items the exact kernel recomputed after the fast one
+//   redo   [U*nchunk]         not 0 for the items the exact kernel recomputed after the fast one
+// The piece of segment s (0 = before the first shot, i + 1 = shot i, S + 1 = the question) in item j
+// of a unit has index s + j.
 // An item is "exact" when every item is (`all_exact`: the exact kernel did all the work) or when
 // its redo flag is set; its rows' statistics are then rebuilt from its pieces.
 // row_stats_kernel, shot_mass_kernel, shot_score_from_mass_kernel, shot_score_from_tokens_kernel:
@@ -23,13 +25,20 @@ struct PartialView {
     const float* part_z;      // [U][P][Rpad]
     const float* item_m;      // [U * nchunk][Rpad]
     const float* item_z;      // [U * nchunk][Rpad]
-    const int* redo;          // [U * nchunk], or NULL
-    const int* chunk_first;   // [B][cf_stride]: first piece of every item of a prompt; entry nchunk = number of pieces
-    int cf_stride, nchunk, P, Rpad, all_exact;
+    const unsigned long long* redo;   // [U * nchunk], or NULL
+    int nchunk, chunk_keys;   // items of a unit, keys of an item
+    int N, S, P, Rpad, all_exact;     // S = -1: the pieces are the items
 };
 
 __device__ __forceinline__ bool item_is_exact(const PartialView& v, int item) {
     return v.all_exact || (v.redo && v.redo[item]);
+}
+// First and last piece of item j of a unit whose prompt has the boundaries o.
+__device__ __forceinline__ int first_piece(const PartialView& v, const int* o, int j) {
+    return count_le(o, v.S + 1, j * v.chunk_keys) + j;
+}
+__device__ __forceinline__ int last_piece(const PartialView& v, const int* o, int j) {
+    return count_le(o, v.S + 1, min(v.N, (j + 1) * v.chunk_keys) - 1) + j;
 }
 // (m, z) of two partial sums merged: z relative to the larger reference
 __device__ __forceinline__ void merge_mz(float& m, float& z, float mq, float zq) {
@@ -40,16 +49,15 @@ __device__ __forceinline__ void merge_mz(float& m, float& z, float mq, float zq)
 }
 // Row r of unit u over all of its keys: m = max reference, z = sum exp2(x - m).  Items in index
 // order, an exact item's pieces in index order: the result does not depend on scheduling.
-__device__ __forceinline__ void row_stats_of(const PartialView& v, int u, int b, int r, float& m, float& z) {
+__device__ __forceinline__ void row_stats_of(const PartialView& v, const int* o, int u, int r, float& m, float& z) {
     m = SHOTKV_NEG_INF;
     z = 0.f;
-    const int* cf = v.chunk_first + (size_t)b * v.cf_stride;
     for (int j = 0; j < v.nchunk; ++j) {
         const int item = u * v.nchunk + j;
         if (item_is_exact(v, item)) {
             const float* pm = v.part_m + (size_t)u * v.P * v.Rpad + r;
             const float* pz = v.part_z + (size_t)u * v.P * v.Rpad + r;
-            for (int q = cf[j]; q < cf[j + 1]; ++q) merge_mz(m, z, pm[(size_t)q * v.Rpad], pz[(size_t)q * v.Rpad]);
+            for (int q = first_piece(v, o, j), last = last_piece(v, o, j); q <= last; ++q) merge_mz(m, z, pm[(size_t)q * v.Rpad], pz[(size_t)q * v.Rpad]);
         } else {
             merge_mz(m, z, v.item_m[(size_t)item * v.Rpad + r], v.item_z[(size_t)item * v.Rpad + r]);
         }
@@ -58,12 +66,11 @@ __device__ __forceinline__ void row_stats_of(const PartialView& v, int u, int b,
 
 // Per (unit, row): m = max over the unit's keys, Z = sum exp2(x - m); stores m and 1/Z (0 for
 // padding rows and rows without weight).
-__global__ void row_stats_kernel(const PartialView v, int units_per_prompt, int R, float* __restrict__ row_m,
-                                 float* __restrict__ row_invz) {
+__global__ void row_stats_kernel(const PartialView v, int R, float* __restrict__ row_m, float* __restrict__ row_invz) {
     const int u = blockIdx.x;
     for (int r = threadIdx.x; r < v.Rpad; r += blockDim.x) {
         float m = 0.f, z = 0.f;
-        if (r < R) row_stats_of(v, u, u / units_per_prompt, r, m, z);   // padding rows carry no weight; their partials may be anything
+        if (r < R) row_stats_of(v, nullptr, u, r, m, z);   // (plain items: S = -1)  padding rows carry no weight; their partials may be anything
         row_m[(size_t)u * v.Rpad + r] = (r < R && m != SHOTKV_NEG_INF) ? m : 0.f;
         row_invz[(size_t)u * v.Rpad + r] = (r < R && z > 0.f) ? 1.f / z : 0.f;
     }
@@ -77,10 +84,9 @@ __global__ void row_stats_kernel(const PartialView v, int units_per_prompt, int 
 // exp2(m_item[r] - m[r]) / Z[r] is the same for all pieces of an item and is formed once per
 // item, so an ordinary piece costs one read of its z and eight multiply-adds per lane (an exact
 // item's pieces carry their own references and pay one exp2 per row).  Phase 3 adds the pieces of
-// each shot in index order.  piece_seg is ascending: 0 = tokens before the first shot, 1..S =
-// shots, S+1 = the question, larger = list padding.  Shared memory: P + 2 * THREADS floats.
+// each shot in index order.  Shared memory: P + 2 * THREADS floats.
 template <int THREADS>
-__global__ void __launch_bounds__(THREADS) shot_mass_kernel(const PartialView v, const int* __restrict__ piece_seg, int R,
+__global__ void __launch_bounds__(THREADS) shot_mass_kernel(const PartialView v, const __grid_constant__ ShotTable tab, int R,
                                                            int L, int Hkv, int S, float* __restrict__ unit_shot) {
     constexpr int NW = THREADS / 32, NH = THREADS / 128;
     static_assert(THREADS == 128 || THREADS == 256, "one thread per padded window row");
@@ -91,12 +97,12 @@ __global__ void __launch_bounds__(THREADS) shot_mass_kernel(const PartialView v,
     const int u = blockIdx.x;
     const int b = u / (L * Hkv);
     const int r = threadIdx.x, warp = r >> 5, lane = r & 31;
-    const int* seg = piece_seg + (size_t)b * v.P;
-    const int* cf = v.chunk_first + (size_t)b * v.cf_stride;
-    const int nreal = cf[v.nchunk];              // pieces that are not list padding (they come first)
+    const int* o = table_row(tab, b);
+    __shared__ int2 range[64];                   // first and last piece of every item
+    for (int j = r; j < v.nchunk; j += THREADS) range[j] = make_int2(first_piece(v, o, j), last_piece(v, o, j));
     {
         float m = SHOTKV_NEG_INF, z = 0.f;
-        if (r < R) row_stats_of(v, u, b, r, m, z);
+        if (r < R) row_stats_of(v, o, u, r, m, z);
         row_m[r] = m == SHOTKV_NEG_INF ? 0.f : m;
         row_w[r] = (r < R && z > 0.f) ? 1.f / z : 0.f;
     }
@@ -125,7 +131,7 @@ __global__ void __launch_bounds__(THREADS) shot_mass_kernel(const PartialView v,
                 f[h].w = rw[h].w > 0.f ? ex2f(mi.w - rm[h].w) * rw[h].w : 0.f;
             }
         }
-        for (int q = cf[j] + warp; q < cf[j + 1]; q += NW) {
+        for (int q = range[j].x + warp; q <= range[j].y; q += NW) {
             float a = 0.f;
 #pragma unroll
             for (int h = 0; h < NH; ++h) {
@@ -148,29 +154,22 @@ __global__ void __launch_bounds__(THREADS) shot_mass_kernel(const PartialView v,
         }
     }
     __syncthreads();
-    // shot i owns the consecutive pieces with seg == i + 1; find them by binary search
     for (int i = threadIdx.x; i < S; i += THREADS) {
-        int lo = 0, hi = nreal;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (seg[mid] < i + 1) lo = mid + 1; else hi = mid;
-        }
         float s = 0.f;
-        for (int q = lo; q < nreal && seg[q] == i + 1; ++q) s += piece_mass[q];
+        for (int j = o[i] / v.chunk_keys, last = (o[i + 1] - 1) / v.chunk_keys; j <= last; ++j) s += piece_mass[i + 1 + j];
         unit_shot[(size_t)u * S + i] = s;
     }
 }
 
 // Score(s_i) = (1/k_i) * sum over the kv heads of the unit masses (prefill score equation).
-__global__ void shot_score_from_mass_kernel(const float* __restrict__ unit_shot, const int* __restrict__ off, int L,
+__global__ void shot_score_from_mass_kernel(const float* __restrict__ unit_shot, const __grid_constant__ ShotTable tab, int L,
                                             int Hkv, int S, float* __restrict__ shot_scores) {
     const int bl = blockIdx.x;
-    const int b = bl / L;
+    const int* o = table_row(tab, bl / L);
     for (int i = threadIdx.x; i < S; i += blockDim.x) {
         float s = 0.f;
         for (int h = 0; h < Hkv; ++h) s += unit_shot[((size_t)bl * Hkv + h) * S + i];
-        const int k = off[(size_t)b * (S + 1) + i + 1] - off[(size_t)b * (S + 1) + i];
-        shot_scores[(size_t)bl * S + i] = s / (float)k;
+        shot_scores[(size_t)bl * S + i] = s / (float)(o[i + 1] - o[i]);
     }
 }
 
@@ -180,13 +179,13 @@ __global__ void shot_score_from_mass_kernel(const float* __restrict__ unit_shot,
 // the units are sentence-sized and number in the thousands.)
 constexpr int kShotsPerCta = 8;
 __global__ void __launch_bounds__(32 * kShotsPerCta) shot_score_from_tokens_kernel(const float* __restrict__ imp,
-                                                                                   const int* __restrict__ off, int L,
+                                                                                   const __grid_constant__ ShotTable tab, int L,
                                                                                    int Hkv, int N, int S,
                                                                                    float* __restrict__ shot_scores) {
     const int i = blockIdx.x * kShotsPerCta + (threadIdx.x >> 5), bl = blockIdx.y, lane = threadIdx.x & 31;
     if (i >= S) return;
-    const int b = bl / L;
-    const int lo = off[(size_t)b * (S + 1) + i], hi = off[(size_t)b * (S + 1) + i + 1];
+    const int* o = table_row(tab, bl / L);
+    const int lo = o[i], hi = o[i + 1];
     float a = 0.f;
     for (int h = 0; h < Hkv; ++h) {
         const float* row = imp + ((size_t)bl * Hkv + h) * N;

@@ -171,7 +171,7 @@ __device__ __forceinline__ void peel_chunk(uint32_t (&r)[32], float scale, float
 template <int D, int PE>
 __global__ void __launch_bounds__(ScoreFastCfg<D>::kThreads, 1)
     score_fast_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const int q_box_rows,
-                      const int k_box_rows, const ScoreTcParams p) {
+                      const int k_box_rows, const ScoreTcParams p, const __grid_constant__ ShotTable tab) {
     using Cfg = ScoreFastCfg<D>;
     constexpr int TN = tc::kTileKeys, MB = 1;
     constexpr int NSL = Cfg::kSlices, SLW = TN / NSL, NCH = SLW / 32, RD = Cfg::kRingDepth;
@@ -212,20 +212,22 @@ __global__ void __launch_bounds__(ScoreFastCfg<D>::kThreads, 1)
             const int u = it / p.nchunk, j = it - u * p.nchunk;
             const int lo = j * p.chunk_keys, hi = min(p.N, lo + p.chunk_keys);
             const int nt = (hi - lo + TN - 1) / TN;
-            const int bprompt = u / units_per_prompt;
-            const int2* pcs = p.pieces + (size_t)bprompt * p.P;
-            int pi = p.chunk_first[(size_t)bprompt * p.cf_stride + j];
-            const int pi_last = p.chunk_first[(size_t)bprompt * p.cf_stride + j + 1];
+            const int* o = table_row(tab, u / units_per_prompt);
+            int sg = count_le_warp(o, p.S + 1, lo);        // segment of the current piece
             // end of the current piece, and of the one after it: fetched one piece ahead so that the
             // load's latency never sits between a piece end and the next comparison
-            int pend = pi < pi_last ? pcs[pi].y : 0x7fffffff;
-            int pend_n = pi + 1 < pi_last ? pcs[pi + 1].y : 0x7fffffff;
+            const int* next = o + sg + 1;
+            int pend = next[-1], pend_n = next[0];
+            // this warp's flag of the item: set when a sum leaves the range (the exact kernel redoes the item)
+            unsigned char* flag = reinterpret_cast<unsigned char*>(p.redo + it) + (warp - 4);
+            if (lane == 0) *flag = 0;
+            __syncwarp();
             float m_ref = SHOTKV_NEG_INF, neg = 0.f;       // reference exponent of this (row, slice, item); neg = -m_ref
             float item_mm = SHOTKV_NEG_INF, item_zz = 0.f; // leader: the row's statistics over the item's pieces so far
             uint64_t z[2] = {0ull, 0ull};                  // four running sums of the current piece, as two packed pairs
             const int plain_end = min(hi, p.N - p.W + 1);  // keys below this count for every window row
 
-            // piece `pi` is complete for this thread's columns.  A follower (slice > 0) posts its (m, z)
+            // the current piece is complete for this thread's columns.  A follower (slice > 0) posts its (m, z)
             // in the next slot of its ring; the leader (slice 0) collects one slot from every follower
             // of its rows, merges, and writes the piece's partials.
             auto flush = [&]() {
@@ -240,10 +242,7 @@ __global__ void __launch_bounds__(ScoreFastCfg<D>::kThreads, 1)
                 const uint32_t par = (uint32_t)(nflush / RD) & 1u;
                 // out of range (or not a number): the exact kernel redoes the item.  Tested on this
                 // slice's own sum, before any rescaling by another slice's reference could hide it.
-                if (live && !(zz < tc::kRedoAbove)) {
-                    p.redo[it] = 1;
-                    *p.redo_any = 1;
-                }
+                if (live && !(zz < tc::kRedoAbove)) *flag = 1;
                 if (slice != 0) {
                     const int ring = (blk * 4 + quad) * (NSL - 1) + (slice - 1);
                     const int rs = ring * RD + slot;
@@ -279,7 +278,7 @@ __global__ void __launch_bounds__(ScoreFastCfg<D>::kThreads, 1)
                     for (int s = 1; s < NSL; ++s) zz += zs[s - 1] * ex2f(ms[s - 1] - mu);
                     // the merged reference is the larger of the slices' references, both fixed on the item's
                     // first tile: the same for every piece of the item, so only z goes out per piece
-                    const size_t o = ((size_t)u * p.P + pi) * p.Rpad + row;
+                    const size_t o = ((size_t)u * p.P + sg + j) * p.Rpad + row;
                     p.part_z[o] = live ? zz : 0.f;
                     {
                         const float mn = fmaxf(item_mm, mm);
@@ -290,9 +289,9 @@ __global__ void __launch_bounds__(ScoreFastCfg<D>::kThreads, 1)
                 }
                 z[0] = z[1] = 0ull;
                 ++nflush;
-                ++pi;
+                ++sg;
                 pend = pend_n;
-                pend_n = pi + 1 < pi_last ? pcs[pi + 1].y : 0x7fffffff;
+                pend_n = *++next;
             };
 
             // 32 columns starting at key kc0 that hold the end of the keys, the causal window, or a piece end
@@ -371,7 +370,8 @@ __global__ void __launch_bounds__(ScoreFastCfg<D>::kThreads, 1)
                 acc ^= 1;
             }
             if (!ok) break;
-            while (pi < pi_last) flush();
+            while (pend < hi) flush();                     // boundaries behind this slice's last column
+            flush();                                       // the piece that the item's end cuts
             if (slice == 0) {
                 p.item_m[(size_t)it * p.Rpad + row] = live ? item_mm : 0.f;
                 p.item_z[(size_t)it * p.Rpad + row] = live ? item_zz : 0.f;

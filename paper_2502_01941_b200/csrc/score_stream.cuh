@@ -73,7 +73,7 @@ __device__ __forceinline__ void tmem_ld_wait(uint32_t (&v)[32]) {
 template <int D, int PE>
 __global__ void __launch_bounds__(ScoreStreamCfg<D>::kThreads, 1)
     score_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const int q_box_rows,
-                        const int k_box_rows, const ScoreTcParams p) {
+                        const int k_box_rows, const ScoreTcParams p, const __grid_constant__ ShotTable tab) {
     using Cfg = ScoreStreamCfg<D>;
     constexpr int TN = tc::kTileKeys, MB = 2;
     extern __shared__ unsigned char smem_raw[];
@@ -104,44 +104,40 @@ __global__ void __launch_bounds__(ScoreStreamCfg<D>::kThreads, 1)
         const int units_per_prompt = p.L * p.Hkv;
         const uint32_t tlane = pp.tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(blk * TN);
         int tiles_before = 0;                              // tiles of earlier items (fixes the accumulator buffer of every tile)
-        uint32_t tfphase0 = 0, tfphase1 = 0;
+        uint32_t tfphase = 0;                              // bit a: the phase of buffer a's barrier
         bool ok = true;
         uint32_t ra[32], rb[32];                           // even and odd chunks of a tile
         for (int it = item_begin; it < item_end && ok; ++it) {
             const int u = it / p.nchunk, j = it - u * p.nchunk;
             const int lo = j * p.chunk_keys, hi = min(p.N, lo + p.chunk_keys);
             const int nt = max(0, (hi - lo + TN - 1) / TN);
-            const int bprompt = u / units_per_prompt;
-            const int2* pcs = p.pieces + (size_t)bprompt * p.P;
-            int pi = p.chunk_first[(size_t)bprompt * p.cf_stride + j];
-            const int pi_last = p.chunk_first[(size_t)bprompt * p.cf_stride + j + 1];
+            const int* o = table_row(tab, u / units_per_prompt);
+            const int sg = count_le_warp(o, p.S + 1, lo);  // segment of the first piece
             // end of the current piece, and of the one after it (fetched one piece ahead)
-            int pend = pi < pi_last ? pcs[pi].y : 0x7fffffff;
-            int pend_n = pi + 1 < pi_last ? pcs[pi + 1].y : 0x7fffffff;
+            const int* next = o + sg + 1;
+            int pend = next[-1], pend_n = next[0];
+            // this warp's flag of the item: set when a sum leaves the range (the exact kernel redoes the item)
+            if (lane == 0) reinterpret_cast<unsigned char*>(p.redo + it)[warp - 4] = 0;
+            __syncwarp();
             float m_ref = SHOTKV_NEG_INF, neg = 0.f;       // reference exponent of this (row, item); neg = -m_ref
             uint64_t z[2] = {0ull, 0ull};                  // four running sums of the current piece, as two packed pairs
             const int plain_end = min(hi, p.N - p.W + 1);  // keys below this count for every window row
-            float* out_z = p.part_z + ((size_t)u * p.P + pi) * p.Rpad + row;
+            float* out_z = p.part_z + ((size_t)u * p.P + sg + j) * p.Rpad + row;
             float zsum = 0.f;                              // sum of the item's pieces so far (they share m_ref)
 
-            // piece `pi` is complete: write its partials and move on to the next piece
+            // the current piece is complete: write its partials and move on to the next piece
             auto flush = [&]() {
                 float s0, s1, s2, s3;
                 tc::unpack2(z[0], s0, s1);
                 tc::unpack2(z[1], s2, s3);
                 const float zz = (s0 + s1) + (s2 + s3);
-                // out of range (or not a number): the exact kernel redoes the item
-                if (live && !(zz < tc::kRedoAbove)) {
-                    p.redo[it] = 1;
-                    *p.redo_any = 1;
-                }
+                if (live && !(zz < tc::kRedoAbove)) reinterpret_cast<unsigned char*>(p.redo + it)[warp - 4] = 1;   // out of range, or not a number
                 *out_z = live ? zz : 0.f;
                 out_z += p.Rpad;
                 zsum += zz;
                 z[0] = z[1] = 0ull;
-                ++pi;
                 pend = pend_n;
-                pend_n = pi + 1 < pi_last ? pcs[pi + 1].y : 0x7fffffff;
+                pend_n = *++next;
             };
 
             // 32 columns starting at key kc that hold the end of the keys, the causal window, or a piece end
@@ -169,14 +165,14 @@ __global__ void __launch_bounds__(ScoreStreamCfg<D>::kThreads, 1)
             };
             // waits (bounded) until the accumulators of the tile in buffer `a` are complete
             auto wait_tile = [&](int a) {
-                const uint32_t tph = a ? tfphase1 : tfphase0;
+                const uint32_t tph = (tfphase >> a) & 1u;
                 // usually ready: one test by the whole warp, made uniform before anything depends on it
                 if (!__all_sync(0xffffffffu, tc::mbar_try(pp.tfull(a, blk), tph))) {
                     bool w = lane == 0 ? tc::mbar_wait(pp.tfull(a, blk), tph, pp.abort_flag, p.err, p.wait_cycles) : true;   // one poller per warp
                     w = __shfl_sync(0xffffffffu, w, 0);
                     if (!w) ok = false;
                 }
-                if (a) tfphase1 ^= 1; else tfphase0 ^= 1;
+                tfphase ^= 1u << a;
                 tc::fence_after_sync();
             };
 
@@ -230,9 +226,9 @@ __global__ void __launch_bounds__(ScoreStreamCfg<D>::kThreads, 1)
                 have_a = false;
                 if (t + 1 < nt) {
                     const int an = a ^ 1;
-                    const uint32_t tph = an ? tfphase1 : tfphase0;
+                    const uint32_t tph = (tfphase >> an) & 1u;
                     if (__all_sync(0xffffffffu, tc::mbar_try(pp.tfull(an, blk), tph))) {
-                        if (an) tfphase1 ^= 1; else tfphase0 ^= 1;
+                        tfphase ^= 1u << an;
                         tc::fence_after_sync();
                         tc::tmem_ld32_issue(ra, tlane + (uint32_t)(an * MB * TN));
                         have_a = true;
@@ -241,7 +237,7 @@ __global__ void __launch_bounds__(ScoreStreamCfg<D>::kThreads, 1)
                 chunk(rb, kc0 + 96);
             }
             if (!ok) break;
-            while (pi < pi_last) flush();
+            flush();                                       // the piece that the item's end cuts
             // the row's statistics over the whole item: its reference and the sum of its pieces
             p.item_m[(size_t)it * p.Rpad + row] = live ? m_ref : 0.f;
             p.item_z[(size_t)it * p.Rpad + row] = live ? zsum : 0.f;

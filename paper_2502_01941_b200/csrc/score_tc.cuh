@@ -8,7 +8,11 @@
 // Persistent CTAs, one per SM, each owning a contiguous range of work items.  An item is one
 // (unit, chunk): unit = prompt x layer x kv head, chunk = a run of whole 128-key tiles of that
 // unit's keys.  Chunk ends and shot boundaries cut the keys into "pieces"; per (piece, window
-// row) the kernel emits a reference maximum m and z = sum exp2(x - m) over the piece's keys.
+// row) the kernel emits a reference maximum m and z = sum exp2(x - m) over the piece's keys.  With
+// segment 0 = the tokens before the first shot, i + 1 = shot i and S + 1 = the question, the piece
+// of segment s in chunk j has index s + j: along the keys every piece end raises s or j or both, so
+// no two pieces share an index and no table of pieces is needed (an index is left unused where a
+// boundary falls on a chunk end).
 // Warp roles:
 //   warp 0      tensor-memory allocation; TMA producer: the unit's window queries Q (once per unit) and K tiles of 128 keys
 //               into a ring of 128-byte-swizzled shared-memory stages
@@ -33,10 +37,8 @@
 namespace shotkv {
 
 struct ScoreTcParams {
-    const int2* pieces;       // [B][P] key ranges [lo, hi), ascending, covering [0, N)
-    const int* chunk_first;   // [B][cf_stride] index of the first piece of every chunk (nchunk + 1 used)
-    int cf_stride;
-    int P;                    // pieces per prompt (row length of `pieces`)
+    int S;                    // shots of a prompt; -1: no shot boundaries, chunk ends alone cut the keys
+    int P;                    // pieces a unit has room for
     int nchunk, chunk_keys;   // chunks per unit; keys per chunk (a multiple of 128)
     int L, Hkv, N, W, R, Rpad;
     int total_items;          // U * nchunk
@@ -48,11 +50,11 @@ struct ScoreTcParams {
     int* err;             // error word (host-visible); set to 1 when a bounded wait gave up
     long long wait_cycles;    // limit of every bounded wait, in SM clock cycles
     long long* clk;           // optional (host-visible): SM cycle counter and nanosecond timer of CTA 0 at kernel start and end
-    // Item filter.  The fast kernel (score_fast.cuh) raises redo[item] and *redo_any when an item's
-    // sums left the fp32 range it works in; the exact kernel, given the same arrays, recomputes
-    // only those items and returns at once when there is none.  Both NULL: every item is done.
-    int* redo;            // [total_items]
-    int* redo_any;
+    // Item filter.  Each of the eight epilogue warps of the fast and streaming kernels writes its byte
+    // of redo[item]: 1 when a sum of its rows left the fp32 range it works in, else 0 (so the array
+    // needs no clearing); the exact kernel, given the same array, recomputes the items with any byte
+    // set and returns at once when there is none.  NULL: every item is done.
+    unsigned long long* redo;   // [total_items]
     int* repaired;        // host-visible count of items recomputed under the filter (diagnostic)
 };
 
@@ -508,12 +510,19 @@ __device__ __forceinline__ void mma_role(const Pipe<Cfg>& pp, const ScoreTcParam
 template <int D, int MB>
 __global__ void __launch_bounds__(ScoreTcCfg<D, MB>::kThreads, 1)
     score_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const int q_box_rows,
-                    const int k_box_rows, const ScoreTcParams p) {
+                    const int k_box_rows, const ScoreTcParams p, const __grid_constant__ ShotTable tab) {
     using Cfg = ScoreTcCfg<D, MB>;
     constexpr int TN = tc::kTileKeys;
     constexpr int NSL = Cfg::kSlices, SLW = TN / NSL, NCH = SLW / 32;     // slices, slice width, chunks per slice
     extern __shared__ unsigned char smem_raw[];
-    if (p.redo_any && *p.redo_any == 0) return;       // repair launch with nothing to repair
+    const long long total = p.total_items;
+    const int item_begin = (int)(total * blockIdx.x / gridDim.x);
+    const int item_end = (int)(total * (blockIdx.x + 1) / gridDim.x);
+    if (p.redo) {                                      // repair launch: nothing to repair in this CTA's items?
+        bool any = false;
+        for (int i = item_begin + threadIdx.x; i < item_end; i += blockDim.x) any |= p.redo[i] != 0;
+        if (!__syncthreads_or(any)) return;
+    }
     tc::stamp(p.clk, 0);
     tc::Pipe<Cfg> pp;
     tc::pipe_setup(pp, smem_raw, 16 / MB);
@@ -524,9 +533,6 @@ __global__ void __launch_bounds__(ScoreTcCfg<D, MB>::kThreads, 1)
     auto bar_tempty = [&](int a, int b) { return pp.tempty(a, b); };
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long total = p.total_items;
-    const int item_begin = (int)(total * blockIdx.x / gridDim.x);
-    const int item_end = (int)(total * (blockIdx.x + 1) / gridDim.x);
 
     if (warp == 0) {
         if (lane == 0) tc::producer_role<D, MB, true, false>(pp, &tmQ, &tmK, q_box_rows, k_box_rows, p, item_begin, item_end);
@@ -555,15 +561,13 @@ __global__ void __launch_bounds__(ScoreTcCfg<D, MB>::kThreads, 1)
             const int u = it / p.nchunk, j = it - u * p.nchunk;
             const int lo = j * p.chunk_keys, hi = min(p.N, lo + p.chunk_keys);
             const int nt = (hi - lo + TN - 1) / TN;
-            const int bprompt = u / units_per_prompt;
-            const int2* pcs = p.pieces + (size_t)bprompt * p.P;
-            int pi = p.chunk_first[(size_t)bprompt * p.cf_stride + j];
-            const int pi_last = p.chunk_first[(size_t)bprompt * p.cf_stride + j + 1];
-            int pend = pi < pi_last ? pcs[pi].y : 0x7fffffff;
+            const int* o = table_row(tab, u / units_per_prompt);
+            int sg = count_le_warp(o, p.S + 1, lo);            // segment of the current piece
+            int pend = o[sg];                                  // its end
             float m_ref = SHOTKV_NEG_INF, z = 0.f;
             const int plain_end = min(hi, p.N - p.W + 1);      // keys below this count for every window row
 
-            // piece `pi` is complete for this thread's columns: merge the row's slices, write, move on
+            // the current piece is complete for this thread's columns: merge the row's slices, write, move on
             auto flush = [&]() {
                 // slot of warpgroup g' and local row r: comb[parity][g'][r][m, z]; a row's slices are the
                 // NSL consecutive warpgroups starting at its leader (slice 0)
@@ -582,15 +586,15 @@ __global__ void __launch_bounds__(ScoreTcCfg<D, MB>::kThreads, 1)
                     float zz = z * ex2f(m_ref - mu);
 #pragma unroll
                     for (int s = 1; s < NSL; ++s) zz += slot[s * 256 + 1] * ex2f(slot[s * 256] - mu);
-                    const size_t o = ((size_t)u * p.P + pi) * p.Rpad + row;
+                    const size_t o = ((size_t)u * p.P + sg + j) * p.Rpad + row;
                     const bool live = row < p.R;        // padding rows: their Q was never loaded
                     p.part_m[o] = live ? mm : 0.f;
                     p.part_z[o] = live ? zz : 0.f;
                 }
                 z = 0.f;
                 ++nflush;
-                ++pi;
-                pend = pi < pi_last ? pcs[pi].y : 0x7fffffff;
+                ++sg;
+                pend = o[sg];
             };
 
             // 32 columns of this thread's row, starting at key kc0
@@ -609,7 +613,7 @@ __global__ void __launch_bounds__(ScoreTcCfg<D, MB>::kThreads, 1)
                     return;
                 }
                 tc::exp32(r, scale, neg);
-                const int pend2 = pi + 1 < pi_last ? pcs[pi + 1].y : 0x7fffffff;
+                const int pend2 = o[sg + 1];
                 if (pend2 >= kc0 + 32) {                                  // exactly one boundary: one predicated pass
                     float lo_s, hi_s;
                     tc::split32(r, pend - kc0, lo_s, hi_s);
@@ -663,7 +667,8 @@ __global__ void __launch_bounds__(ScoreTcCfg<D, MB>::kThreads, 1)
                 acc ^= 1;
             }
             if (!ok) break;
-            while (pi < pi_last) flush();
+            while (pend < hi) flush();                         // boundaries behind this slice's last column
+            flush();                                           // the piece that the item's end cuts
         }
     }
 

@@ -43,7 +43,7 @@ __device__ inline int block_exclusive_scan(int* a, int n, int* tmp) {
 //   mode 0: the longest prefix of the ranking that fits;  mode 1: every shot that still fits.
 // Shared memory: S floats + 3*S ints + (kSelectThreads+1) ints.
 __global__ void __launch_bounds__(kSelectThreads) select_shots_kernel(
-    const float* __restrict__ shot_scores, const int* __restrict__ off, int L, int N, int S, int budget_tokens,
+    const float* __restrict__ shot_scores, const __grid_constant__ ShotTable tab, int L, int N, int S, int budget_tokens,
     int mode, int Mcap, uint8_t* __restrict__ keep, int* __restrict__ kept_idx, int* __restrict__ kept_count) {
     extern __shared__ __align__(16) unsigned char sm[];
     float* sc = reinterpret_cast<float*>(sm);
@@ -51,8 +51,8 @@ __global__ void __launch_bounds__(kSelectThreads) select_shots_kernel(
     int* cum = order + S;                          // rank -> length, then scanned
     int* kl = cum + S;                             // shot -> kept length, then destination offset
     int* tmp = kl + S;
-    const int bl = blockIdx.x, b = bl / L, tid = threadIdx.x;
-    const int* o = off + (size_t)b * (S + 1);
+    const int bl = blockIdx.x, tid = threadIdx.x;
+    const int* o = table_row(tab, bl / L);
     const int pre = o[0], qst = o[S];
     const int always = pre + (N - qst);
     const int shot_budget = budget_tokens - always;

@@ -193,10 +193,7 @@ bool token_route(const shotkv_dims* d) {
 int pmax_of(const shotkv_dims* d) { return (token_route(d) ? 0 : d->S) + 2 + kMaxChunks + 1; }
 
 struct PrefillWs {
-    int* off;          // [B][S+1]
-    int2* pieces;      // [B][Pmax]
-    int* piece_seg;    // [B][Pmax]
-    int* chunk_first;  // [B][kMaxChunks + 1]
+    int* off;          // [B][S+4]  the shot boundaries, when they are too many for the launch parameters
     float* part_m;     // [U][Pmax][Rpad]
     float* part_z;
     float* item_m;     // [U * kMaxChunks][Rpad] per (work item, row): the reference its pieces share and the sum of their z
@@ -205,7 +202,7 @@ struct PrefillWs {
     float* row_invz;
     float* unit_shot;  // [U][S]
     float* imp;        // [U][N] per-token importances of the fused call's per-token route (absent otherwise)
-    int* redo;         // [kMaxGroups + U * kMaxChunks] per group of units: one word "some item is marked", then one word per item the exact kernel must recompute
+    unsigned long long* redo;   // [U * kMaxChunks] not 0 for the items the exact kernel must recompute
     size_t total;
 };
 
@@ -214,10 +211,7 @@ PrefillWs carve(const shotkv_dims* d, void* base) {
     const size_t U = (size_t)d->B * d->L * d->Hkv, P = pmax_of(d), R = rpad_of(d);
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t at = o; o += align_up(bytes); return (unsigned char*)base + at; };
-    w.off = (int*)take((size_t)d->B * (d->S + 1) * 4);
-    w.pieces = (int2*)take((size_t)d->B * P * 8);
-    w.piece_seg = (int*)take((size_t)d->B * P * 4);
-    w.chunk_first = (int*)take((size_t)d->B * (kMaxChunks + 1) * 4);
+    w.off = (int*)take((size_t)d->B * (d->S + 1 + kTableEnd) * 4);
     w.part_m = (float*)take(U * P * R * 4);
     w.part_z = (float*)take(U * P * R * 4);
     w.item_m = (float*)take(U * kMaxChunks * R * 4);
@@ -226,7 +220,7 @@ PrefillWs carve(const shotkv_dims* d, void* base) {
     w.row_invz = (float*)take(U * R * 4);
     w.unit_shot = (float*)take(U * (size_t)(d->S > 0 ? d->S : 1) * 4);
     w.imp = (float*)take(token_route(d) ? U * (size_t)d->N * 4 : 0);
-    w.redo = (int*)take((U * kMaxChunks + kMaxGroups) * 4);
+    w.redo = (unsigned long long*)take(U * kMaxChunks * 8);
     w.total = o;
     return w;
 }
@@ -255,6 +249,8 @@ int upload_small(shotkv_ctx* ctx, void* dst, const void* src, size_t bytes, cuda
 // take equal runs of consecutive items.  The split that minimises the busiest CTA's tile count
 // wins; each extra chunk costs one more piece per unit, so ties go to fewer chunks.
 struct ChunkPlan { int nchunk, chunk_keys; };
+// Pieces a unit has room for: the piece of segment s in chunk j has index s + j (see score_tc.cuh).
+int pieces_of(int S, const ChunkPlan& plan) { return S + 1 + plan.nchunk; }
 ChunkPlan plan_chunks(const shotkv_dims* d, int sm_count) {
     const long long U = (long long)d->B * d->L * d->Hkv;
     const int tiles = (d->N + 127) / 128;
@@ -276,25 +272,21 @@ ChunkPlan plan_chunks(const shotkv_dims* d, int sm_count) {
 }
 
 // Cuts [0, N) of every prompt into pieces at the chunk ends and, when offsets are given, at the
-// segment boundaries (segment 0 = before the first shot, i+1 = shot i, S+1 = the question).
-// piece_seg records each piece's segment (S+2 marks list padding); chunk_first[b][j] is the index
-// of the first piece of chunk j.  Returns pieces per prompt (the same for all after padding).
+// segment boundaries (segment 0 = before the first shot, i+1 = shot i, S+1 = the question): the list
+// that shotkv_plan_pieces reports.  seg records each piece's segment (S+2 marks list padding).
+// Returns pieces per prompt (the same for all after padding).
 int build_pieces(const shotkv_dims* d, const int32_t* off, const ChunkPlan& plan, std::vector<int2>& pieces,
-                 std::vector<int>& seg, std::vector<int>& chunk_first) {
+                 std::vector<int>& seg) {
     std::vector<std::vector<int2>> pp(d->B);
     std::vector<std::vector<int>> ss(d->B);
-    chunk_first.assign((size_t)d->B * (kMaxChunks + 1), 0);
     size_t P = 0;
     for (int b = 0; b < d->B; ++b) {
-        int* cf = chunk_first.data() + (size_t)b * (kMaxChunks + 1);
-        int next_chunk = 0;
         auto add_range = [&](int lo, int hi, int s) {
             int x = lo;
             while (x < hi) {
                 const int j = x / plan.chunk_keys;
                 const int cend = (j + 1) * plan.chunk_keys;
                 const int y = cend < hi ? cend : hi;
-                while (next_chunk <= j) cf[next_chunk++] = (int)pp[b].size();
                 pp[b].push_back(make_int2(x, y));
                 ss[b].push_back(s);
                 x = y;
@@ -308,7 +300,6 @@ int build_pieces(const shotkv_dims* d, const int32_t* off, const ChunkPlan& plan
         } else {
             add_range(0, d->N, 0);
         }
-        while (next_chunk <= plan.nchunk) cf[next_chunk++] = (int)pp[b].size();
         if (pp[b].size() > P) P = pp[b].size();
     }
     if (P == 0) P = 1;
@@ -320,6 +311,37 @@ int build_pieces(const shotkv_dims* d, const int32_t* off, const ChunkPlan& plan
             seg[(size_t)b * P + i] = ss[b][i];
         }
     return (int)P;
+}
+
+// The boundaries of the call's prompts as the kernels take them: in the launch parameters when they
+// fit, else from a copy at `device` made on `stream`.  `walked`: the scoring pass walks along the rows
+// and needs the closing entries; selection alone takes the caller's layout as it is.
+int prepare_table(shotkv_ctx* ctx, const shotkv_dims* d, const int32_t* off_host, bool walked, int* device, ShotTable& t,
+                  cudaStream_t stream) {
+    const int row = d->S + 1;
+    t.stride = walked ? row + kTableEnd : row;
+    const size_t entries = (size_t)d->B * t.stride;
+    t.ptr = entries > (size_t)kTableArgs ? device : nullptr;
+    if (t.ptr && !walked) return upload_small(ctx, device, off_host, entries * 4, stream);
+    std::vector<int> big(t.ptr ? entries : 0);
+    int* to = t.ptr ? big.data() : t.data;
+    for (int b = 0; b < d->B; ++b, to += t.stride) {
+        memcpy(to, off_host + (size_t)b * row, (size_t)row * 4);
+        for (int i = row; i < t.stride; ++i) to[i] = kNoBound;
+    }
+    return t.ptr ? upload_small(ctx, device, big.data(), entries * 4, stream) : SHOTKV_OK;
+}
+// The table of the prompts from b0 on.
+void advance_table(ShotTable& t, int prompts, const ShotTable& whole, size_t b0) {
+    t.stride = whole.stride;
+    t.ptr = whole.ptr ? whole.ptr + b0 * whole.stride : nullptr;
+    if (!t.ptr) memcpy(t.data, whole.data + b0 * whole.stride, (size_t)prompts * whole.stride * 4);
+}
+// The table of a scoring pass over plain chunks: no boundaries.
+void empty_table(ShotTable& t) {
+    t.ptr = nullptr;
+    t.stride = 0;
+    for (int i = 0; i < kTableEnd; ++i) t.data[i] = kNoBound;
 }
 
 int set_device(shotkv_ctx* ctx) {
@@ -349,11 +371,11 @@ void* resolve_encode_tiled() {
 
 template <int D, int MB>
 int launch_score_tc_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorMap& tmK, int qbox, int kbox,
-                      const ScoreTcParams& sp, cudaStream_t stream) {
+                      const ScoreTcParams& sp, const ShotTable& tab, cudaStream_t stream) {
     constexpr int smem = ScoreTcCfg<D, MB>::kSmemBytes;
     int grid = sp.total_items < ctx->sm_count ? sp.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    score_tc_kernel<D, MB><<<grid, ScoreTcCfg<D, MB>::kThreads, smem, stream>>>(tmQ, tmK, qbox, kbox, sp);
+    score_tc_kernel<D, MB><<<grid, ScoreTcCfg<D, MB>::kThreads, smem, stream>>>(tmQ, tmK, qbox, kbox, sp, tab);
     LAUNCH_CHECK(ctx);
     return SHOTKV_OK;
 }
@@ -363,22 +385,22 @@ constexpr int kPolyEvery = 5;
 
 template <int D>
 int launch_score_fast_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorMap& tmK, int qbox, int kbox,
-                        const ScoreTcParams& sp, cudaStream_t stream) {
+                        const ScoreTcParams& sp, const ShotTable& tab, cudaStream_t stream) {
     constexpr int smem = ScoreFastCfg<D>::kSmemBytes;
     int grid = sp.total_items < ctx->sm_count ? sp.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    score_fast_kernel<D, kPolyEvery><<<grid, ScoreFastCfg<D>::kThreads, smem, stream>>>(tmQ, tmK, qbox, kbox, sp);
+    score_fast_kernel<D, kPolyEvery><<<grid, ScoreFastCfg<D>::kThreads, smem, stream>>>(tmQ, tmK, qbox, kbox, sp, tab);
     LAUNCH_CHECK(ctx);
     return SHOTKV_OK;
 }
 
 template <int D>
 int launch_score_stream_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorMap& tmK, int qbox, int kbox,
-                          const ScoreTcParams& sp, cudaStream_t stream) {
+                          const ScoreTcParams& sp, const ShotTable& tab, cudaStream_t stream) {
     using Cfg = ScoreStreamCfg<D>;
     int grid = sp.total_items < ctx->sm_count ? sp.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    score_stream_kernel<D, kPolyEvery><<<grid, Cfg::kThreads, Cfg::kSmemBytes, stream>>>(tmQ, tmK, qbox, kbox, sp);
+    score_stream_kernel<D, kPolyEvery><<<grid, Cfg::kThreads, Cfg::kSmemBytes, stream>>>(tmQ, tmK, qbox, kbox, sp, tab);
     LAUNCH_CHECK(ctx);
     return SHOTKV_OK;
 }
@@ -390,7 +412,7 @@ struct TcSetup {
     int qbox, kbox;
     ScoreTcParams sp;
 };
-int tc_setup(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q, const shotkv_bf16* K, const PrefillWs& w, int P,
+int tc_setup(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q, const shotkv_bf16* K, const PrefillWs& w, int S,
              const ChunkPlan& plan, TcSetup& t) {
     EncodeTiledFn enc = (EncodeTiledFn)ctx->encode_tiled;
     if (!enc) return fail(ctx, SHOTKV_ERR_CUDA, "cuTensorMapEncodeTiled is not available from this driver");
@@ -418,10 +440,8 @@ int tc_setup(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q, const 
     }
     ScoreTcParams& sp = t.sp;
     sp = ScoreTcParams{};
-    sp.pieces = w.pieces;
-    sp.chunk_first = w.chunk_first;
-    sp.cf_stride = kMaxChunks + 1;
-    sp.P = P;
+    sp.S = S;
+    sp.P = pieces_of(S, plan);
     sp.nchunk = plan.nchunk;
     sp.chunk_keys = plan.chunk_keys;
     sp.L = d->L; sp.Hkv = d->Hkv; sp.N = d->N; sp.W = d->W; sp.R = R; sp.Rpad = rpad_of(d);
@@ -451,7 +471,7 @@ int launch_colsum_tc(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q
                      float* imp, cudaStream_t stream) {
     TcSetup t;
     const ChunkPlan plan = plan_chunks(d, ctx->sm_count);
-    int rc = tc_setup(ctx, d, Q, K, w, 0, plan, t);
+    int rc = tc_setup(ctx, d, Q, K, w, -1, plan, t);
     if (rc) return rc;
     ColsumTcParams cp{};
     cp.base = t.sp;
@@ -461,10 +481,11 @@ int launch_colsum_tc(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q
     return big ? launch_colsum_tc_t<64, 2>(ctx, t, cp, stream) : launch_colsum_tc_t<64, 1>(ctx, t, cp, stream);
 }
 
+// The scoring pass; S = -1: chunk ends alone cut the keys (`tab` is not read).
 int launch_score_tc(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q, const shotkv_bf16* K, const PrefillWs& w,
-                    int P, const ChunkPlan& plan, cudaStream_t stream) {
+                    int S, const ShotTable& tab, const ChunkPlan& plan, cudaStream_t stream) {
     TcSetup t;
-    int rc0 = tc_setup(ctx, d, Q, K, w, P, plan, t);
+    int rc0 = tc_setup(ctx, d, Q, K, w, S, plan, t);
     if (rc0) return rc0;
     const CUtensorMap& tmQ = t.tmQ;
     const CUtensorMap& tmK = t.tmK;
@@ -476,16 +497,14 @@ int launch_score_tc(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q,
     if (ctx->scoring_mode == SHOTKV_SCORING_FAST) {
         // fast kernel first; it marks the items whose sums left its range, and the exact kernel
         // below then redoes exactly those (returning at once when there is none)
-        sp.redo_any = w.redo;
-        sp.redo = w.redo + 1;
-        CUDA_TRY(ctx, cudaMemsetAsync(w.redo, 0, ((size_t)sp.total_items + 1) * 4, stream));
-        if (d->d == 128) rc = big ? launch_score_stream_t<128>(ctx, tmQ, tmK, qbox, kbox, sp, stream) : launch_score_fast_t<128>(ctx, tmQ, tmK, qbox, kbox, sp, stream);
-        else rc = big ? launch_score_stream_t<64>(ctx, tmQ, tmK, qbox, kbox, sp, stream) : launch_score_fast_t<64>(ctx, tmQ, tmK, qbox, kbox, sp, stream);
+        sp.redo = w.redo;
+        if (d->d == 128) rc = big ? launch_score_stream_t<128>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream) : launch_score_fast_t<128>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream);
+        else rc = big ? launch_score_stream_t<64>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream) : launch_score_fast_t<64>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream);
         if (rc) return rc;
         sp.clk = nullptr;
     }
-    if (d->d == 128) return big ? launch_score_tc_t<128, 2>(ctx, tmQ, tmK, qbox, kbox, sp, stream) : launch_score_tc_t<128, 1>(ctx, tmQ, tmK, qbox, kbox, sp, stream);
-    return big ? launch_score_tc_t<64, 2>(ctx, tmQ, tmK, qbox, kbox, sp, stream) : launch_score_tc_t<64, 1>(ctx, tmQ, tmK, qbox, kbox, sp, stream);
+    if (d->d == 128) return big ? launch_score_tc_t<128, 2>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream) : launch_score_tc_t<128, 1>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream);
+    return big ? launch_score_tc_t<64, 2>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream) : launch_score_tc_t<64, 1>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream);
 }
 
 int check_ws(shotkv_ctx* ctx, const shotkv_dims* d, void* ws, size_t ws_bytes) {
@@ -496,55 +515,33 @@ int check_ws(shotkv_ctx* ctx, const shotkv_dims* d, void* ws, size_t ws_bytes) {
     return SHOTKV_OK;
 }
 
-// Builds the piece lists of every prompt for `plan` and uploads them with the chunk index.
-int prepare_pieces(shotkv_ctx* ctx, const shotkv_dims* d, const int32_t* off_host, const ChunkPlan& plan, const PrefillWs& w,
-                   int* P_out, cudaStream_t stream) {
-    std::vector<int2> pieces;
-    std::vector<int> seg, chunk_first;
-    const int P = build_pieces(d, off_host, plan, pieces, seg, chunk_first);
-    if (P > pmax_of(d)) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "internal: piece count %d exceeds bound %d", P, pmax_of(d));
-    int rc = upload_small(ctx, w.pieces, pieces.data(), pieces.size() * sizeof(int2), stream);
-    if (rc) return rc;
-    rc = upload_small(ctx, w.piece_seg, seg.data(), seg.size() * sizeof(int), stream);
-    if (rc) return rc;
-    rc = upload_small(ctx, w.chunk_first, chunk_first.data(), chunk_first.size() * sizeof(int), stream);
-    if (rc) return rc;
-    *P_out = P;
-    return SHOTKV_OK;
-}
-
 // What the scoring pass just left in `w`, as the reductions read it.
-PartialView partial_view(const shotkv_ctx* ctx, const shotkv_dims* d, const PrefillWs& w, int P, const ChunkPlan& plan) {
+PartialView partial_view(const shotkv_ctx* ctx, const shotkv_dims* d, const PrefillWs& w, int S, const ChunkPlan& plan) {
     PartialView v{};
     v.part_m = w.part_m; v.part_z = w.part_z; v.item_m = w.item_m; v.item_z = w.item_z;
     v.all_exact = ctx->scoring_mode == SHOTKV_SCORING_EXACT ? 1 : 0;
-    v.redo = v.all_exact ? nullptr : w.redo + 1;
-    v.chunk_first = w.chunk_first;
-    v.cf_stride = kMaxChunks + 1;
+    v.redo = v.all_exact ? nullptr : w.redo;
     v.nchunk = plan.nchunk;
-    v.P = P;
+    v.chunk_keys = plan.chunk_keys;
+    v.N = d->N;
+    v.S = S;
+    v.P = pieces_of(S, plan);
     v.Rpad = rpad_of(d);
     return v;
 }
 
-// STATS pass over `pieces` followed by the per-row reduction; leaves part_m/part_z (and for the
-// token path row_m/row_invz) in the workspace.
+// The scoring pass on plain chunks and the per-row reduction: leaves row_m / row_invz in the workspace.
 int run_stats(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q, const shotkv_bf16* K, const PrefillWs& w,
-              const int32_t* off_host, bool need_rows, int* P_out, cudaStream_t stream) {
+              cudaStream_t stream) {
     const ChunkPlan plan = plan_chunks(d, ctx->sm_count);
-    int P = 0;
-    int rc = prepare_pieces(ctx, d, off_host, plan, w, &P, stream);
-    if (rc) return rc;
-    const int U = d->B * d->L * d->Hkv;
+    ShotTable none;
+    empty_table(none);
     prof_mark(ctx, stream);
-    rc = launch_score_tc(ctx, d, Q, K, w, P, plan, stream);
+    const int rc = launch_score_tc(ctx, d, Q, K, w, -1, none, plan, stream);
     if (rc) return rc;
     prof_mark(ctx, stream);
-    if (need_rows) {
-        row_stats_kernel<<<U, 256, 0, stream>>>(partial_view(ctx, d, w, P, plan), d->L * d->Hkv, (d->H / d->Hkv) * d->W, w.row_m, w.row_invz);
-        LAUNCH_CHECK(ctx);
-    }
-    *P_out = P;
+    row_stats_kernel<<<d->B * d->L * d->Hkv, 256, 0, stream>>>(partial_view(ctx, d, w, -1, plan), (d->H / d->Hkv) * d->W, w.row_m, w.row_invz);
+    LAUNCH_CHECK(ctx);
     return SHOTKV_OK;
 }
 
@@ -593,14 +590,10 @@ GroupView group_view(const shotkv_dims* d, const GroupSplit& gs, int g) {
     v.u0 = v.bl0 * d->Hkv;
     return v;
 }
-// The group's slices of the workspace arrays (P = pieces per prompt as uploaded).
-PrefillWs group_ws(const PrefillWs& w, const shotkv_dims* d, const GroupView& v, int g, int P) {
+// The group's slices of the workspace arrays (P = pieces a unit has room for).
+PrefillWs group_ws(const PrefillWs& w, const shotkv_dims* d, const GroupView& v, int P) {
     PrefillWs x = w;
     const size_t R = rpad_of(d);
-    x.off = w.off + v.b0 * (d->S + 1);
-    x.pieces = w.pieces + v.b0 * P;
-    x.piece_seg = w.piece_seg + v.b0 * P;
-    x.chunk_first = w.chunk_first + v.b0 * (kMaxChunks + 1);
     x.part_m = w.part_m + v.u0 * P * R;
     x.part_z = w.part_z + v.u0 * P * R;
     x.item_m = w.item_m + v.u0 * kMaxChunks * R;
@@ -608,14 +601,14 @@ PrefillWs group_ws(const PrefillWs& w, const shotkv_dims* d, const GroupView& v,
     x.row_m = w.row_m + v.u0 * R;
     x.row_invz = w.row_invz + v.u0 * R;
     x.unit_shot = w.unit_shot + v.u0 * (size_t)(d->S > 0 ? d->S : 1);
-    x.redo = w.redo + g + v.u0 * kMaxChunks;
+    x.redo = w.redo + v.u0 * kMaxChunks;
     return x;
 }
 
-int run_select(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_policy* p, const PrefillWs& w, float* shot_scores,
+int run_select(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_policy* p, const ShotTable& tab, float* shot_scores,
                uint8_t* keep, int32_t* kept_idx, int32_t* kept_count, int32_t Mcap, cudaStream_t stream) {
     const size_t smem = (size_t)d->S * 16 + (kSelectThreads + 1) * 4 + 16;
-    select_shots_kernel<<<d->B * d->L, kSelectThreads, smem, stream>>>(shot_scores, w.off, d->L, d->N, d->S, budget_of(d, p),
+    select_shots_kernel<<<d->B * d->L, kSelectThreads, smem, stream>>>(shot_scores, tab, d->L, d->N, d->S, budget_of(d, p),
                                                                      p->select_mode, Mcap, keep, kept_idx, kept_count);
     LAUNCH_CHECK(ctx);
     return SHOTKV_OK;
@@ -800,8 +793,7 @@ int shotkv_prefill_score(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv_
     if ((rc = check_ws(ctx, dims, ws, ws_bytes))) return rc;
     cudaStream_t stream = (cudaStream_t)stream_;
     const PrefillWs w = carve(dims, ws);
-    int P = 0;
-    if ((rc = run_stats(ctx, dims, Qwin, K, w, nullptr, true, &P, stream))) return rc;
+    if ((rc = run_stats(ctx, dims, Qwin, K, w, stream))) return rc;
     return launch_colsum_tc(ctx, dims, Qwin, K, w, token_importance, stream);
 }
 
@@ -823,13 +815,14 @@ int shotkv_select_shots(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv_p
     if ((rc = check_ws(ctx, dims, ws, ws_bytes))) return rc;
     cudaStream_t stream = (cudaStream_t)stream_;
     const PrefillWs w = carve(dims, ws);
-    if ((rc = upload_small(ctx, w.off, offsets_host, (size_t)dims->B * (dims->S + 1) * 4, stream))) return rc;
+    ShotTable tab;
+    if ((rc = prepare_table(ctx, dims, offsets_host, false, w.off, tab, stream))) return rc;
     if (token_importance && dims->S > 0) {
         dim3 grid((dims->S + kShotsPerCta - 1) / kShotsPerCta, dims->B * dims->L);
-        shot_score_from_tokens_kernel<<<grid, 32 * kShotsPerCta, 0, stream>>>(token_importance, w.off, dims->L, dims->Hkv, dims->N, dims->S, shot_scores);
+        shot_score_from_tokens_kernel<<<grid, 32 * kShotsPerCta, 0, stream>>>(token_importance, tab, dims->L, dims->Hkv, dims->N, dims->S, shot_scores);
         LAUNCH_CHECK(ctx);
     }
-    if ((rc = run_select(ctx, dims, policy, w, shot_scores, keep, kept_idx, kept_count, Mcap, stream))) return rc;
+    if ((rc = run_select(ctx, dims, policy, tab, shot_scores, keep, kept_idx, kept_count, Mcap, stream))) return rc;
     if (orc > 0) fail(ctx, orc, "always-kept tokens (%d) exceed the budget (%d) for some prompt", worst, budget_of(dims, policy));
     return orc;
 }
@@ -878,16 +871,17 @@ int shotkv_select_shots_static(shotkv_ctx* ctx, const shotkv_dims* dims, const s
     const int need = budget_of(dims, policy) > worst ? budget_of(dims, policy) : worst;
     if (Mcap < need) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "Mcap = %d but %d rows may be kept", Mcap, need);
     cudaStream_t stream = (cudaStream_t)stream_;
-    PrefillWs w{};
-    if ((rc = static_offsets_ptr(ctx, &w.off))) return rc;
+    int32_t* off = nullptr;
+    if ((rc = static_offsets_ptr(ctx, &off))) return rc;
     // every entry the kernels read is overwritten here, so nothing of an earlier call survives
-    if ((rc = upload_small(ctx, w.off, offsets_host, (size_t)entries * 4, stream))) return rc;
+    ShotTable tab;
+    if ((rc = prepare_table(ctx, dims, offsets_host, false, off, tab, stream))) return rc;
     if (token_importance && dims->S > 0) {
         dim3 grid((dims->S + kShotsPerCta - 1) / kShotsPerCta, dims->B * dims->L);
-        shot_score_from_tokens_kernel<<<grid, 32 * kShotsPerCta, 0, stream>>>(token_importance, w.off, dims->L, dims->Hkv, dims->N, dims->S, shot_scores);
+        shot_score_from_tokens_kernel<<<grid, 32 * kShotsPerCta, 0, stream>>>(token_importance, tab, dims->L, dims->Hkv, dims->N, dims->S, shot_scores);
         LAUNCH_CHECK(ctx);
     }
-    if ((rc = run_select(ctx, dims, policy, w, shot_scores, keep, kept_idx, kept_count, Mcap, stream))) return rc;
+    if ((rc = run_select(ctx, dims, policy, tab, shot_scores, keep, kept_idx, kept_count, Mcap, stream))) return rc;
     if (orc > 0) fail(ctx, orc, "always-kept tokens (%d) exceed the budget (%d) for some prompt", worst, budget_of(dims, policy));
     return orc;
 }
@@ -957,13 +951,13 @@ int prefill_compress_impl(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv
     const int S = dims->S, R = (dims->H / dims->Hkv) * dims->W, Rpad = rpad_of(dims);
     const size_t S1 = S > 0 ? S : 1, row = dims->d;
 
-    // tables of all prompts once, cut for the work partition of one (full) group
+    // the boundaries of all prompts once, and the work partition of one (full) group
     const GroupSplit gs = plan_groups(ctx, dims, before_group != nullptr);
     const GroupView first = group_view(dims, gs, 0);
     const ChunkPlan plan = plan_chunks(&first.d, ctx->sm_count);
-    if ((rc = upload_small(ctx, w.off, offsets_host, (size_t)dims->B * (S + 1) * 4, stream))) return rc;
-    int P = 0;
-    if ((rc = prepare_pieces(ctx, dims, offsets_host, plan, w, &P, stream))) return rc;
+    ShotTable whole;
+    if ((rc = prepare_table(ctx, dims, offsets_host, true, w.off, whole, stream))) return rc;
+    const int P = pieces_of(S, plan);
     const size_t msm = ((size_t)P + 2 * Rpad) * 4;     // shot_mass_kernel: row statistics and one mass per piece
     if (S > 0) {
         if (msm > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "too many shots for the single-pass path (S = %d)", S);
@@ -980,7 +974,9 @@ int prefill_compress_impl(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv
     };
     for (int g = 0; g < gs.n; ++g) {
         const GroupView v = group_view(dims, gs, g);
-        const PrefillWs wg = group_ws(w, dims, v, g, P);
+        const PrefillWs wg = group_ws(w, dims, v, P);
+        ShotTable tab;
+        advance_table(tab, v.d.B, whole, v.b0);
         const shotkv_dims* dg = &v.d;
         const int Ug = dg->B * dg->L * dg->Hkv;
         const shotkv_bf16* Kg = K + v.u0 * dims->N * row;
@@ -990,7 +986,7 @@ int prefill_compress_impl(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv
         int32_t* count_g = kept_count + v.bl0;
         if (before_group && (rc = (*before_group)(v, stream))) return bail(rc);
         prof_gmark(ctx, g, 0, stream);
-        if ((rc = launch_score_tc(ctx, dg, Qwin + v.bl0 * dims->H * dims->W * row, Kg, wg, P, plan, stream))) return bail(rc);
+        if ((rc = launch_score_tc(ctx, dg, Qwin + v.bl0 * dims->H * dims->W * row, Kg, wg, S, tab, plan, stream))) return bail(rc);
         prof_gmark(ctx, g, 1, stream);
         if (forked) {
             if (cudaEventRecord(ctx->ev_fork[g], stream) != cudaSuccess || cudaStreamWaitEvent(tail, ctx->ev_fork[g], 0) != cudaSuccess)
@@ -999,19 +995,19 @@ int prefill_compress_impl(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv
         }
         prof_gmark(ctx, g, 2, tail);
         if (S > 0) {
-            const PartialView pv = partial_view(ctx, dg, wg, P, plan);
+            const PartialView pv = partial_view(ctx, dg, wg, S, plan);
             if (Rpad == 128)
-                shot_mass_kernel<128><<<Ug, 128, msm, tail>>>(pv, wg.piece_seg, R, dg->L, dg->Hkv, S, wg.unit_shot);
+                shot_mass_kernel<128><<<Ug, 128, msm, tail>>>(pv, tab, R, dg->L, dg->Hkv, S, wg.unit_shot);
             else
-                shot_mass_kernel<256><<<Ug, 256, msm, tail>>>(pv, wg.piece_seg, R, dg->L, dg->Hkv, S, wg.unit_shot);
+                shot_mass_kernel<256><<<Ug, 256, msm, tail>>>(pv, tab, R, dg->L, dg->Hkv, S, wg.unit_shot);
             ctx->launches += 1;
             if (cudaGetLastError() != cudaSuccess) return bail(fail(ctx, SHOTKV_ERR_CUDA, "per-shot reduction failed to launch"));
-            shot_score_from_mass_kernel<<<dg->B * dg->L, 128, 0, tail>>>(wg.unit_shot, wg.off, dg->L, dg->Hkv, S, scores_g);
+            shot_score_from_mass_kernel<<<dg->B * dg->L, 128, 0, tail>>>(wg.unit_shot, tab, dg->L, dg->Hkv, S, scores_g);
             ctx->launches += 1;
             if (cudaGetLastError() != cudaSuccess) return bail(fail(ctx, SHOTKV_ERR_CUDA, "per-shot score kernel failed to launch"));
         }
         prof_gmark(ctx, g, 3, tail);
-        if ((rc = run_select(ctx, dg, policy, wg, scores_g, keep + v.bl0 * S1, idx_g, count_g, Mcap, tail))) return bail(rc);
+        if ((rc = run_select(ctx, dg, policy, tab, scores_g, keep + v.bl0 * S1, idx_g, count_g, Mcap, tail))) return bail(rc);
         prof_gmark(ctx, g, 4, tail);
         if ((rc = run_compact(ctx, dg, Kg, Vg, idx_g, count_g, Mcap, Kc + v.u0 * (size_t)Mcap * row, Vc + v.u0 * (size_t)Mcap * row, tail))) return bail(rc);
         prof_gmark(ctx, g, 5, tail);
@@ -1294,8 +1290,8 @@ int32_t shotkv_plan_pieces(const shotkv_dims* dims, const int32_t* offsets_host,
     if (sm_count < 1) return SHOTKV_ERR_INVALID_ARG;
     const ChunkPlan plan = plan_chunks(dims, sm_count);
     std::vector<int2> pieces;
-    std::vector<int> seg, chunk_first;
-    const int P = build_pieces(dims, offsets_host, plan, pieces, seg, chunk_first);
+    std::vector<int> seg;
+    const int P = build_pieces(dims, offsets_host, plan, pieces, seg);
     if (nchunk) *nchunk = plan.nchunk;
     if (chunk_keys) *chunk_keys = plan.chunk_keys;
     if (pieces_out) {
