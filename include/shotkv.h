@@ -343,8 +343,8 @@ SHOTKV_API int shotkv_set_pipeline_groups(shotkv_ctx* ctx, int groups);
  * events on their stream at their stage boundaries; the last 64 calls are retained.  */
 SHOTKV_API int shotkv_profile_enable(shotkv_ctx* ctx, int enable);
 /* Stage durations in milliseconds of the profiled call made `calls_back` calls ago (0 = latest);
- * waits for that call to finish.  Prefill: {scoring kernel, per-shot reduce, select, compact},
- * each summed over the groups of a pipelined call (stages of different groups overlap, so the
+ * waits for that call to finish.  Prefill: {scoring kernel, per-shot reduce, select, compact} (reduce
+ * and select are one kernel in the single-pass form: its time is the reduce's, select is about 0), each summed over the groups of a pipelined call (stages of different groups overlap, so the
  * sum can exceed the call's duration); decode: {score kernel, accumulate+evict, -1, -1}.  Returns the number of stages or a negative
  * error. */
 SHOTKV_API int shotkv_profile_read(shotkv_ctx* ctx, int calls_back, float* stage_ms /* [4] */);

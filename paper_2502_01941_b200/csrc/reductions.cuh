@@ -13,10 +13,11 @@
 // of a unit has index s + j.
 // An item is "exact" when every item is (`all_exact`: the exact kernel did all the work) or when
 // its redo flag is set; its rows' statistics are then rebuilt from its pieces.
-// row_stats_kernel, shot_mass_kernel, shot_score_from_mass_kernel, shot_score_from_tokens_kernel:
-// fixed-order reductions of those partials, and of per-token importances.
+// row_stats_kernel, reduce_select_kernel, shot_score_from_tokens_kernel: fixed-order reductions of
+// those partials, and of per-token importances.
 #pragma once
 #include "common.cuh"
+#include "select_compact.cuh"
 
 namespace shotkv {
 
@@ -64,135 +65,280 @@ __device__ __forceinline__ void row_stats_of(const PartialView& v, const int* o,
     }
 }
 
-// Per (unit, row): m = max over the unit's keys, Z = sum exp2(x - m); stores m and 1/Z (0 for
-// padding rows and rows without weight).
+// Per (unit, row) of a scoring pass on plain chunks: m = max over the unit's keys, Z = sum exp2(x - m);
+// stores m and 1/Z (0 for padding rows and rows without weight).  The maximum first, then the sum, so
+// that the items' loads are in flight together (merged one by one: 4.8 and 6.4 us on 256 and 128 units).
 __global__ void row_stats_kernel(const PartialView v, int R, float* __restrict__ row_m, float* __restrict__ row_invz) {
-    const int u = blockIdx.x;
-    for (int r = threadIdx.x; r < v.Rpad; r += blockDim.x) {
-        float m = 0.f, z = 0.f;
-        if (r < R) row_stats_of(v, nullptr, u, r, m, z);   // (plain items: S = -1)  padding rows carry no weight; their partials may be anything
-        row_m[(size_t)u * v.Rpad + r] = (r < R && m != SHOTKV_NEG_INF) ? m : 0.f;
-        row_invz[(size_t)u * v.Rpad + r] = (r < R && z > 0.f) ? 1.f / z : 0.f;
+    const int u = blockIdx.x, r = threadIdx.x;                  // one thread per padded row
+    bool any = false;
+    for (int j = r; j < v.nchunk; j += blockDim.x) any |= item_is_exact(v, u * v.nchunk + j);
+    any = __syncthreads_or(any);
+    float m = SHOTKV_NEG_INF, z = 0.f;
+    if (r < R) {                                                // padding rows carry no weight; their partials may be anything
+        if (any) {
+            row_stats_of(v, nullptr, u, r, m, z);               // S = -1: the pieces are the items
+        } else {
+            const float* im = v.item_m + (size_t)u * v.nchunk * v.Rpad + r;
+            const float* iz = v.item_z + (size_t)u * v.nchunk * v.Rpad + r;
+#pragma unroll 8
+            for (int j = 0; j < v.nchunk; ++j) m = fmaxf(m, im[(size_t)j * v.Rpad]);
+            const float mu = m == SHOTKV_NEG_INF ? 0.f : m;
+#pragma unroll 8
+            for (int j = 0; j < v.nchunk; ++j) z += iz[(size_t)j * v.Rpad] * ex2f(im[(size_t)j * v.Rpad] - mu);
+        }
     }
+    row_m[(size_t)u * v.Rpad + r] = (r < R && m != SHOTKV_NEG_INF) ? m : 0.f;
+    row_invz[(size_t)u * v.Rpad + r] = (r < R && z > 0.f) ? 1.f / z : 0.f;
 }
 
-// Per unit: the mass every row puts on every shot, normalised and summed over the rows:
-//   unit_shot[u][i] = sum_r ( sum_{pieces q of shot i} z_q[r] * exp2(m_q[r] - m[r]) ) / Z[r]
-// Phase 1, one thread per row: the row's (m, 1/Z) from the item statistics, left in shared
-// memory.  Phase 2, one warp per piece: the lanes read the piece's z over the rows four at a
-// time, weight them, and one shuffle reduction gives the piece's mass; the weight
-// exp2(m_item[r] - m[r]) / Z[r] is the same for all pieces of an item and is formed once per
-// item, so an ordinary piece costs one read of its z and eight multiply-adds per lane (an exact
-// item's pieces carry their own references and pay one exp2 per row).  Phase 3 adds the pieces of
-// each shot in index order.  Shared memory: P + 2 * THREADS floats.
-template <int THREADS>
-__global__ void __launch_bounds__(THREADS) shot_mass_kernel(const PartialView v, const __grid_constant__ ShotTable tab, int R,
-                                                           int L, int Hkv, int S, float* __restrict__ unit_shot) {
-    constexpr int NW = THREADS / 32, NH = THREADS / 128;
-    static_assert(THREADS == 128 || THREADS == 256, "one thread per padded window row");
-    extern __shared__ __align__(16) float sm_mass[];
-    float* row_m = sm_mass;                      // [THREADS]
-    float* row_w = row_m + THREADS;              // [THREADS]  1/Z, 0 for rows without weight
-    float* piece_mass = row_w + THREADS;         // [P]
-    const int u = blockIdx.x;
-    const int b = u / (L * Hkv);
-    const int r = threadIdx.x, warp = r >> 5, lane = r & 31;
-    const int* o = table_row(tab, b);
-    __shared__ int2 range[64];                   // first and last piece of every item
-    for (int j = r; j < v.nchunk; j += THREADS) range[j] = make_int2(first_piece(v, o, j), last_piece(v, o, j));
-    {
-        float m = SHOTKV_NEG_INF, z = 0.f;
-        if (r < R) row_stats_of(v, o, u, r, m, z);
-        row_m[r] = m == SHOTKV_NEG_INF ? 0.f : m;
-        row_w[r] = (r < R && z > 0.f) ? 1.f / z : 0.f;
-    }
+// One (b, l): the mass every window row puts on every shot, normalised and summed over the rows and
+// the kv heads,
+//   mass[h][i] = sum_r ( sum_{pieces q of shot i} z_q[r] * exp2(m_q[r] - m[r]) ) / Z[r]
+//   Score(s_i) = (1/k_i) * sum_h mass[h][i]                             (prefill score equation)
+// then the selection.  A cluster of CTAs shares the kv heads of a (b, l), CTA c taking heads c,
+// c + cluster size, ...; each leaves its masses in the leader's shared memory and ends, and the leader
+// adds them in a fixed order and selects.  In one kernel because the three steps are latency, not work:
+// separate kernels for the masses (one CTA a unit, items and pieces one after the other), the sum
+// over heads and the selection took 20 + 2.3 + 5.5 us on one layer of 4K and 38 + 2.6 + 8.4 us on
+// 4 x 32 layers of 32K, where reading the partials (115 MB) is 18 us of memory time.
+//
+// Per head: (1) a thread (two, with 128 rows) per row merges the item statistics into the row's
+// (m, 1/Z): the maximum first, then the sum, so that the items' loads are all in flight at once.
+// (2) Every warp takes a run of consecutive pieces, its lanes the rows four at a time; the weight
+// exp2(m_item[r] - m[r]) / Z[r] is the same for all pieces of an item and is formed when the run
+// enters the item (an exact item's pieces carry their own references and pay one exp2 per row); one
+// shuffle reduction gives the piece's mass.  (3) The pieces of each shot are added in index order.
+// All sums have a fixed order.
+constexpr int kReduceThreads = kSelectThreads;
+constexpr int kReduceCluster = 8;                  // most CTAs that share the kv heads of a (b, l)
+
+// Shared memory: boundaries; masses of the shots, one row per CTA of the cluster (the leader's copy is
+// read); row statistics, piece masses and piece -> item (reused by the selection).
+__host__ __device__ constexpr size_t reduce_smem_bytes(int Rpad, int P, int S, int ranks) {
+    const size_t pieces = (size_t)(P + 3) / 4 * 4 * 4 + (size_t)(P + 15) / 16 * 16;
+    const size_t work = (size_t)Rpad * 16 + pieces, select = select_smem_bytes(S);
+    return bounds_smem_bytes(S) + ranks * ((size_t)(S + 3) / 4 * 4 * 4) + (work > select ? work : select);
+}
+
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Stores to the first CTA of the cluster: `p` is the address of the same variable in this CTA.
+__device__ __forceinline__ void store_to_leader(float* p, float v) {
+    uint32_t a;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(smem_u32(p)));
+    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+
+template <int ROWS>
+__global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const PartialView v, const __grid_constant__ ShotTable tab,
+                                                                      int R, int Hkv, int ranks,
+                                                                      float* __restrict__ shot_scores, const SelectArgs a) {
+    constexpr int NW = kReduceThreads / 32, NH = ROWS / 128, PARTS = kReduceThreads / ROWS;
+    constexpr unsigned char kNoItem = 255;
+    static_assert(ROWS == 128 || ROWS == 256, "padded window rows");
+    extern __shared__ __align__(16) unsigned char sm[];
+    __shared__ int2 range[64];                     // first and last piece of every item
+    __shared__ int exact[64];
+    const int S = v.S, np = v.P;
+    const int s4 = (S + 3) / 4 * 4;
+    int* o = reinterpret_cast<int*>(sm);
+    float* masses = reinterpret_cast<float*>(sm + bounds_smem_bytes(S));   // [ranks][s4]
+    unsigned char* work = reinterpret_cast<unsigned char*>(masses + (size_t)ranks * s4);
+    float* row_m = reinterpret_cast<float*>(work); // [2][ROWS] maxima of the parts, then [ROWS]
+    float* row_w = row_m + 2 * ROWS;               // [2][ROWS] sums of the parts, then [ROWS] 1/Z (0 for rows without weight)
+    float* piece_mass = row_w + 2 * ROWS;          // [P]
+    unsigned char* item_of = reinterpret_cast<unsigned char*>(piece_mass + (np + 3) / 4 * 4);   // [P]
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int bl = blockIdx.x / ranks, rank = blockIdx.x - bl * ranks;   // a cluster is the `ranks` CTAs of one (b, l)
+    float* mass = masses + rank * s4;              // of this CTA's heads
+
+    copy_bounds(o, tab, bl / a.L, S);
+    if (ranks > 1) cluster_arrive();               // (1) this CTA has begun: its shared memory may be written to
     __syncthreads();
-    // rows 4*lane .. 4*lane+3 (and the same 128 further on when there are 256 rows)
-    float4 rm[NH], rw[NH];
-#pragma unroll
-    for (int h = 0; h < NH; ++h) {
-        rm[h] = reinterpret_cast<const float4*>(row_m)[h * 32 + lane];
-        rw[h] = reinterpret_cast<const float4*>(row_w)[h * 32 + lane];
-    }
-    const float* pm = v.part_m + (size_t)u * v.P * v.Rpad;
-    const float* pz = v.part_z + (size_t)u * v.P * v.Rpad;
-    for (int j = 0; j < v.nchunk; ++j) {
-        const int item = u * v.nchunk + j;
-        const bool exact = item_is_exact(v, item);
-        float4 f[NH];                            // ordinary item: exp2(m_item - m) / Z of this lane's rows
-        if (!exact) {
-#pragma unroll
-            for (int h = 0; h < NH; ++h) {
-                const float4 mi = reinterpret_cast<const float4*>(v.item_m + (size_t)item * v.Rpad)[h * 32 + lane];
-                // a row without weight (padding, or nothing but underflow) has w = 0 and gets factor 0
-                f[h].x = rw[h].x > 0.f ? ex2f(mi.x - rm[h].x) * rw[h].x : 0.f;
-                f[h].y = rw[h].y > 0.f ? ex2f(mi.y - rm[h].y) * rw[h].y : 0.f;
-                f[h].z = rw[h].z > 0.f ? ex2f(mi.z - rm[h].z) * rw[h].z : 0.f;
-                f[h].w = rw[h].w > 0.f ? ex2f(mi.w - rm[h].w) * rw[h].w : 0.f;
+    for (int j = tid; j < v.nchunk; j += kReduceThreads) range[j] = make_int2(first_piece(v, o, j), last_piece(v, o, j));
+    for (int i = tid; i < S; i += kReduceThreads) mass[i] = 0.f;
+    for (int q = tid; q < np; q += kReduceThreads) item_of[q] = kNoItem;   // an index no piece has (a boundary on a chunk end)
+    __syncthreads();
+    for (int j = warp; j < v.nchunk; j += NW)
+        for (int q = range[j].x + lane; q <= range[j].y; q += 32) item_of[q] = (unsigned char)j;
+    const int q_first = range[0].x, q_count = range[v.nchunk - 1].y + 1 - q_first;
+
+    for (int h = rank; h < Hkv; h += ranks) {
+        const int u = bl * Hkv + h;
+        bool any = false;
+        for (int j = tid; j < v.nchunk; j += kReduceThreads) {
+            const bool e = item_is_exact(v, u * v.nchunk + j);
+            exact[j] = e;
+            any |= e;
+        }
+        any = __syncthreads_or(any);
+        {   // row statistics
+            const int r = tid % ROWS, part = tid / ROWS;
+            const float* im = v.item_m + (size_t)u * v.nchunk * v.Rpad + r;
+            const float* iz = v.item_z + (size_t)u * v.nchunk * v.Rpad + r;
+            float m = SHOTKV_NEG_INF, z = 0.f;
+            if (!any) {
+#pragma unroll 8
+                for (int j = part; j < v.nchunk; j += PARTS) m = fmaxf(m, im[(size_t)j * v.Rpad]);
+            } else if (part == 0) {
+                row_stats_of(v, o, u, r, m, z);
+            }
+            if (PARTS > 1) {
+                row_m[part * ROWS + r] = m;
+                __syncthreads();
+                m = fmaxf(row_m[r], row_m[ROWS + r]);
+            }
+            const float mu = m == SHOTKV_NEG_INF ? 0.f : m;
+            if (!any) {
+#pragma unroll 8
+                for (int j = part; j < v.nchunk; j += PARTS) z += iz[(size_t)j * v.Rpad] * ex2f(im[(size_t)j * v.Rpad] - mu);
+            }
+            if (PARTS > 1) {
+                row_w[part * ROWS + r] = z;
+                __syncthreads();
+                z = row_w[r] + row_w[ROWS + r];
+                __syncthreads();
+            }
+            if (part == 0) {
+                row_m[r] = mu;
+                row_w[r] = (r < R && z > 0.f) ? 1.f / z : 0.f;   // padding rows carry no weight
             }
         }
-        for (int q = range[j].x + warp; q <= range[j].y; q += NW) {
-            float a = 0.f;
+        __syncthreads();
+        // rows 4*lane .. 4*lane+3 (and the same 128 further on when there are 256 rows)
+        float4 rm[NH], rw[NH], f[NH];
 #pragma unroll
-            for (int h = 0; h < NH; ++h) {
-                const float4 z4 = reinterpret_cast<const float4*>(pz + (size_t)q * v.Rpad)[h * 32 + lane];
-                if (exact) {
-                    const float4 m4 = reinterpret_cast<const float4*>(pm + (size_t)q * v.Rpad)[h * 32 + lane];
-                    a += rw[h].x > 0.f ? z4.x * ex2f(m4.x - rm[h].x) * rw[h].x : 0.f;
-                    a += rw[h].y > 0.f ? z4.y * ex2f(m4.y - rm[h].y) * rw[h].y : 0.f;
-                    a += rw[h].z > 0.f ? z4.z * ex2f(m4.z - rm[h].z) * rw[h].z : 0.f;
-                    a += rw[h].w > 0.f ? z4.w * ex2f(m4.w - rm[h].w) * rw[h].w : 0.f;
-                } else {
-                    a = fmaf(z4.x, f[h].x, a);
-                    a = fmaf(z4.y, f[h].y, a);
-                    a = fmaf(z4.z, f[h].z, a);
-                    a = fmaf(z4.w, f[h].w, a);
+        for (int k = 0; k < NH; ++k) {
+            rm[k] = reinterpret_cast<const float4*>(row_m)[k * 32 + lane];
+            rw[k] = reinterpret_cast<const float4*>(row_w)[k * 32 + lane];
+        }
+        const float* pm = v.part_m + (size_t)u * v.P * v.Rpad;
+        const float* pz = v.part_z + (size_t)u * v.P * v.Rpad;
+        // 2^(m - row's m) / Z of this lane's rows; a row without weight (padding, or nothing but
+        // underflow) gets factor 0 whatever its reference
+        auto weights = [&](const float* ref) {
+#pragma unroll
+            for (int k = 0; k < NH; ++k) {
+                const float4 mi = reinterpret_cast<const float4*>(ref)[k * 32 + lane];
+                f[k].x = rw[k].x > 0.f ? ex2f(mi.x - rm[k].x) * rw[k].x : 0.f;
+                f[k].y = rw[k].y > 0.f ? ex2f(mi.y - rm[k].y) * rw[k].y : 0.f;
+                f[k].z = rw[k].z > 0.f ? ex2f(mi.z - rm[k].z) * rw[k].z : 0.f;
+                f[k].w = rw[k].w > 0.f ? ex2f(mi.w - rm[k].w) * rw[k].w : 0.f;
+            }
+        };
+        constexpr int AHEAD = 4 / NH;              // pieces whose z a warp has in flight
+        const int q0 = q_first + q_count * warp / NW, q1 = q_first + q_count * (warp + 1) / NW;
+        int item = kNoItem;
+        for (int q = q0; q < q1; q += AHEAD) {
+            float4 z4[AHEAD][NH];
+#pragma unroll
+            for (int n = 0; n < AHEAD; ++n)
+                if (q + n < q1)
+#pragma unroll
+                    for (int k = 0; k < NH; ++k) z4[n][k] = reinterpret_cast<const float4*>(pz + (size_t)(q + n) * v.Rpad)[k * 32 + lane];
+#pragma unroll
+            for (int n = 0; n < AHEAD; ++n) {
+                const int j = q + n < q1 ? item_of[q + n] : kNoItem;
+                if (j == kNoItem) continue;
+                if (exact[j]) weights(pm + (size_t)(q + n) * v.Rpad);
+                else if (j != item) weights(v.item_m + ((size_t)u * v.nchunk + j) * v.Rpad);
+                item = exact[j] ? kNoItem : j;
+                float s = 0.f;
+#pragma unroll
+                for (int k = 0; k < NH; ++k) {
+                    s = fmaf(z4[n][k].x, f[k].x, s);
+                    s = fmaf(z4[n][k].y, f[k].y, s);
+                    s = fmaf(z4[n][k].z, f[k].z, s);
+                    s = fmaf(z4[n][k].w, f[k].w, s);
                 }
+                s = warp_sum(s);
+                if (lane == 0) piece_mass[q + n] = s;
             }
-            a = warp_sum(a);
-            if (lane == 0) piece_mass[q] = a;
         }
+        __syncthreads();
+        for (int i = tid; i < S; i += kReduceThreads) {
+            float s = 0.f;
+            for (int j = o[i] / v.chunk_keys, last = (o[i + 1] - 1) / v.chunk_keys; j <= last; ++j) s += piece_mass[i + 1 + j];
+            mass[i] += s;
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < S; i += THREADS) {
-        float s = 0.f;
-        for (int j = o[i] / v.chunk_keys, last = (o[i + 1] - 1) / v.chunk_keys; j <= last; ++j) s += piece_mass[i + 1 + j];
-        unit_shot[(size_t)u * S + i] = s;
+    if (ranks > 1) {
+        cluster_wait();                            // (1) the leader has begun
+        if (rank != 0)
+            for (int i = tid; i < S; i += kReduceThreads) store_to_leader(mass + i, mass[i]);
+        cluster_arrive();                          // (2) this CTA's masses are with the leader
+    }
+    if (rank == 0) {
+        if (ranks > 1) cluster_wait();             // (2)
+        float* scores = shot_scores + (size_t)bl * S;
+        select_body<kReduceThreads>(a, bl, o, work, [&](int i) {
+            float s = 0.f;
+            for (int c = 0; c < ranks; ++c) s += masses[c * s4 + i];
+            s /= (float)(o[i + 1] - o[i]);
+            scores[i] = s;
+            return s;
+        });
     }
 }
 
-// Score(s_i) = (1/k_i) * sum over the kv heads of the unit masses (prefill score equation).
-__global__ void shot_score_from_mass_kernel(const float* __restrict__ unit_shot, const __grid_constant__ ShotTable tab, int L,
-                                            int Hkv, int S, float* __restrict__ shot_scores) {
-    const int bl = blockIdx.x;
-    const int* o = table_row(tab, bl / L);
-    for (int i = threadIdx.x; i < S; i += blockDim.x) {
-        float s = 0.f;
-        for (int h = 0; h < Hkv; ++h) s += unit_shot[((size_t)bl * Hkv + h) * S + i];
-        shot_scores[(size_t)bl * S + i] = s / (float)(o[i + 1] - o[i]);
-    }
-}
-
-// Score(s_i) from per-token importance: one warp per (b, l, shot), eight shots per CTA; every
-// lane sums a fixed subset of the shot's (kv head, token) pairs and the lanes are added by
-// shuffles, so the order is fixed.  (One CTA per shot spent most of its time being launched once
-// the units are sentence-sized and number in the thousands.)
-constexpr int kShotsPerCta = 8;
-__global__ void __launch_bounds__(32 * kShotsPerCta) shot_score_from_tokens_kernel(const float* __restrict__ imp,
-                                                                                   const __grid_constant__ ShotTable tab, int L,
-                                                                                   int Hkv, int N, int S,
-                                                                                   float* __restrict__ shot_scores) {
-    const int i = blockIdx.x * kShotsPerCta + (threadIdx.x >> 5), bl = blockIdx.y, lane = threadIdx.x & 31;
+// Score(s_i) from per-token importance.  Latency-bound: the importances come from L2, so what counts
+// is how many loads are in flight.  WPS warps share a shot, eight warps a CTA:
+//   WPS = 1  short units, thousands of them: a lane has up to eight heads' loads in flight
+//   WPS = 8  few long units: a warp takes every eighth head, and a lane up to eight tokens of it
+// Every lane sums a fixed subset of the shot's (kv head, token) pairs; lanes are added by shuffles and
+// warps in order.  Measured (32 layers of 643 sentences | 16 layers of 24 shots of 340 tokens): one
+// warp a shot and one load at a time 20 | 15 us; WPS = 1 15.7 | 19.7 us; WPS = 8 - | 5 us.
+constexpr int kTokenWarps = 8;
+constexpr int kLongShot = 96;                  // mean length from which eight warps share a shot
+template <int WPS>
+__global__ void __launch_bounds__(32 * kTokenWarps) shot_score_from_tokens_kernel(const float* __restrict__ imp,
+                                                                                  const __grid_constant__ ShotTable tab, int L,
+                                                                                  int Hkv, int N, int S,
+                                                                                  float* __restrict__ shot_scores) {
+    static_assert(WPS == 1 || WPS == kTokenWarps, "a warp or the whole CTA to a shot");
+    constexpr int AHEAD = 8;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, bl = blockIdx.y;
+    const int i = WPS == 1 ? blockIdx.x * kTokenWarps + warp : blockIdx.x;
     if (i >= S) return;
     const int* o = table_row(tab, bl / L);
     const int lo = o[i], hi = o[i + 1];
-    float a = 0.f;
-    for (int h = 0; h < Hkv; ++h) {
-        const float* row = imp + ((size_t)bl * Hkv + h) * N;
-        for (int t = lo + lane; t < hi; t += 32) a += row[t];
+    const float* base = imp + (size_t)bl * Hkv * N;
+    float a[AHEAD];
+#pragma unroll
+    for (int k = 0; k < AHEAD; ++k) a[k] = 0.f;
+    if (WPS == 1) {
+        for (int h0 = 0; h0 < Hkv; h0 += AHEAD)
+            for (int t = lo + lane; t < hi; t += 32)
+#pragma unroll
+                for (int k = 0; k < AHEAD; ++k)
+                    if (h0 + k < Hkv) a[k] += base[(size_t)(h0 + k) * N + t];
+    } else {
+        for (int h = warp; h < Hkv; h += kTokenWarps)
+            for (int t0 = lo; t0 < hi; t0 += 32 * AHEAD)
+#pragma unroll
+                for (int k = 0; k < AHEAD; ++k) {
+                    const int t = t0 + k * 32 + lane;
+                    if (t < hi) a[k] += base[(size_t)h * N + t];
+                }
     }
-    a = warp_sum(a);
-    if (lane == 0) shot_scores[(size_t)bl * S + i] = a / (float)(hi - lo);
+    float s = warp_sum(((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7])));
+    if (WPS > 1) {
+        __shared__ float part[kTokenWarps];
+        if (lane == 0) part[warp] = s;
+        __syncthreads();
+        s = 0.f;
+        for (int w = 0; w < kTokenWarps; ++w) s += part[w];
+        if (threadIdx.x == 0) shot_scores[(size_t)bl * S + i] = s / (float)(hi - lo);
+    } else if (lane == 0) {
+        shot_scores[(size_t)bl * S + i] = s / (float)(hi - lo);
+    }
 }
 
 }  // namespace shotkv

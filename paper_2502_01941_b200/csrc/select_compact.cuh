@@ -6,115 +6,228 @@ namespace shotkv {
 
 constexpr int kSelectThreads = 256;
 
-// Exclusive prefix sum over n ints in shared memory, in place; returns the total.  All threads
-// of the CTA must call it.  Each thread scans a contiguous slice, slices are combined serially
-// through `tmp` (kSelectThreads ints): n is at most a few thousand, latency is irrelevant here.
-__device__ inline int block_exclusive_scan(int* a, int n, int* tmp) {
-    const int tid = threadIdx.x;
-    const int per = (n + kSelectThreads - 1) / kSelectThreads;
+// Exclusive prefix sum over n ints in shared memory, in place; returns the total.  All NT threads
+// of the CTA must call it.  Each thread sums a contiguous slice, a warp scans its slices by shuffles
+// and every thread adds up the warps before its own (`tmp`: NT / 32 ints).
+template <int NT = kSelectThreads>
+__device__ __forceinline__ int block_exclusive_scan(int* a, int n, int* tmp) {
+    constexpr int NW = NT / 32;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int per = (n + NT - 1) / NT;
     const int lo = min(tid * per, n), hi = min(lo + per, n);
     int s = 0;
     for (int i = lo; i < hi; ++i) s += a[i];
-    tmp[tid] = s;
-    __syncthreads();
-    if (tid == 0) {
-        int run = 0;
-        for (int i = 0; i < kSelectThreads; ++i) {
-            const int v = tmp[i];
-            tmp[i] = run;
-            run += v;
-        }
-        tmp[kSelectThreads] = run;
+    int inc = s;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int v = __shfl_up_sync(0xffffffffu, inc, d);
+        if (lane >= d) inc += v;
     }
+    if (lane == 31) tmp[warp] = inc;
     __syncthreads();
-    int run = tmp[tid];
+    int run = inc - s, total = 0;
+#pragma unroll
+    for (int w = 0; w < NW; ++w) {
+        const int v = tmp[w];
+        if (w < warp) run += v;
+        total += v;
+    }
     for (int i = lo; i < hi; ++i) {
         const int v = a[i];
         a[i] = run;
         run += v;
     }
     __syncthreads();
-    return tmp[kSelectThreads];
+    return total;
 }
 
-// One CTA per (b, l).  Ranks the S shots by (score descending, index ascending), keeps whole
-// shots while they fit the budget left after the always-kept tokens, and writes the kept token
-// positions in ascending order.
-//   mode 0: the longest prefix of the ranking that fits;  mode 1: every shot that still fits.
-// Shared memory: S floats + 3*S ints + (kSelectThreads+1) ints.
-__global__ void __launch_bounds__(kSelectThreads) select_shots_kernel(
-    const float* __restrict__ shot_scores, const __grid_constant__ ShotTable tab, int L, int N, int S, int budget_tokens,
-    int mode, int Mcap, uint8_t* __restrict__ keep, int* __restrict__ kept_idx, int* __restrict__ kept_count) {
-    extern __shared__ __align__(16) unsigned char sm[];
-    float* sc = reinterpret_cast<float*>(sm);
-    int* order = reinterpret_cast<int*>(sc + S);   // rank -> shot
-    int* cum = order + S;                          // rank -> length, then scanned
-    int* kl = cum + S;                             // shot -> kept length, then destination offset
-    int* tmp = kl + S;
-    const int bl = blockIdx.x, tid = threadIdx.x;
-    const int* o = table_row(tab, bl / L);
-    const int pre = o[0], qst = o[S];
-    const int always = pre + (N - qst);
-    const int shot_budget = budget_tokens - always;
+// What one (b, l) selects from and where the result goes.
+struct SelectArgs {
+    int L, N, S, budget_tokens, mode, Mcap;
+    uint8_t* keep;       // [B*L][S]
+    int* kept_idx;       // [B*L][Mcap]
+    int* kept_count;     // [B*L]
+};
 
-    for (int i = tid; i < S; i += kSelectThreads) {
-        const float v = shot_scores[(size_t)bl * S + i];
-        sc[i] = v == v ? v : SHOTKV_NEG_INF;     // a NaN score ranks last instead of breaking the total order
-    }
-    __syncthreads();
-    for (int i = tid; i < S; i += kSelectThreads) {
-        const float v = sc[i];
-        int rank = 0;
-        for (int j = 0; j < S; ++j) {
-            const float w = sc[j];
-            rank += (w > v) || (w == v && j < i);
+// Up to this many shots are ranked by counting the better ones, one thread a shot, four scores a
+// shared-memory read; beyond it the S^2 comparisons weigh more than a bitonic sort, and the CTA has
+// four times the threads.
+constexpr int kRankByCount = kSelectThreads, kSortThreads = 1024;
+
+__host__ __device__ constexpr int select_sort_size(int S) {
+    int n = 2 * kRankByCount;
+    while (n < S) n *= 2;
+    return n;
+}
+// Shared memory of select_body, in bytes: scores and ranking, or sort keys; lengths; destinations.
+__host__ __device__ constexpr size_t select_smem_bytes(int S) {
+    const size_t s4 = (size_t)(S + 3) / 4 * 4;
+    return (S <= kRankByCount ? 2 * s4 * 4 : (size_t)select_sort_size(S) * 8) + 2 * s4 * 4 + 128;
+}
+
+// Bitonic sort of n = a power of two >= 64 keys in shared memory, ascending, by the NT threads of a
+// CTA.  Exchanges over fewer than 32 places run inside a warp, on registers, so that only the longer
+// ones cost a barrier each (1,024 keys: 21 barriers instead of 55).
+template <int NT>
+__device__ __forceinline__ void block_sort(unsigned long long* key, int n) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    auto in_warp = [&](int k_from, int k_to) {
+        for (int x0 = warp * 32; x0 < n; x0 += NT) {
+            const int x = x0 + lane;
+            unsigned long long v = key[x];
+            for (int k = k_from; k <= k_to; k <<= 1)
+                for (int j = min(k >> 1, 16); j > 0; j >>= 1) {
+                    const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, j);
+                    const bool low = (x & j) == 0, up = (x & k) == 0;
+                    if ((w < v) == (low == up) && w != v) v = w;      // the lower place of an ascending pair takes the smaller
+                }
+            key[x] = v;
         }
-        order[rank] = i;
-        cum[rank] = o[i + 1] - o[i];
+        __syncthreads();
+    };
+    in_warp(2, 32);
+    for (int k = 64; k <= n; k <<= 1) {
+        for (int j = k >> 1; j >= 32; j >>= 1) {
+            for (int t = threadIdx.x; t < n / 2; t += NT) {
+                const int x = 2 * t - (t & (j - 1)), y = x + j;       // y has bit j, x has not
+                const unsigned long long kx = key[x], ky = key[y];
+                if ((kx > ky) == ((x & k) == 0)) {
+                    key[x] = ky;
+                    key[y] = kx;
+                }
+            }
+            __syncthreads();
+        }
+        in_warp(k, k);
+    }
+}
+
+// Ranks the S shots by (score descending, index ascending), keeps whole shots while they fit the
+// budget left after the always-kept tokens, and writes the kept token positions in ascending order.
+//   mode 0: the longest prefix of the ranking that fits;  mode 1: every shot that still fits.
+// Run by a whole CTA of NT threads (at least S of them where shots are ranked by counting); score(i)
+// gives shot i's score (each i is asked for once, by one thread); `o` the prompt's boundaries, in
+// shared memory; `sm` select_smem_bytes(S) bytes, 16-byte aligned.  What bounds it is latency: every
+// step is a handful of barriers and shared-memory round trips, so none of them may be serial in S.
+template <int NT, class Score>
+__device__ __forceinline__ void select_body(const SelectArgs& a, int bl, const int* o, unsigned char* sm, Score&& score) {
+    const int S = a.S, s4 = (S + 3) / 4 * 4, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const bool counted = S <= kRankByCount;
+    const int nsort = counted ? 0 : select_sort_size(S);
+    float* sc = reinterpret_cast<float*>(sm);                               // counted: scores
+    int* order = reinterpret_cast<int*>(sm) + s4;                           // counted: rank -> shot
+    unsigned long long* key = reinterpret_cast<unsigned long long*>(sm);    // sorted: (score descending, shot)
+    int* cum = reinterpret_cast<int*>(sm + (counted ? 2 * (size_t)s4 * 4 : (size_t)nsort * 8));   // rank -> length, then scanned
+    int* kl = cum + s4;                                                     // shot -> kept length, then destination
+    int* tmp = kl + s4;
+    const int pre = o[0], qst = o[S];
+    const int always = pre + (a.N - qst);
+    const int shot_budget = a.budget_tokens - always;
+
+    if (counted) {
+        if (tid < s4) {
+            const float v = tid < S ? score(tid) : SHOTKV_NEG_INF;
+            sc[tid] = v == v ? v : SHOTKV_NEG_INF;     // a NaN score ranks last instead of breaking the total order
+        }
+        __syncthreads();
+        if (tid < S) {
+            const float v = sc[tid];
+            int rank = 0;
+            for (int j = 0; j < S; j += 4) {           // the padding behind the last shot never counts: -inf, larger index
+                const float4 w = *reinterpret_cast<const float4*>(sc + j);
+                rank += (w.x > v) || (w.x == v && j < tid);
+                rank += (w.y > v) || (w.y == v && j + 1 < tid);
+                rank += (w.z > v) || (w.z == v && j + 2 < tid);
+                rank += (w.w > v) || (w.w == v && j + 3 < tid);
+            }
+            order[rank] = tid;
+            cum[rank] = o[tid + 1] - o[tid];
+        }
+    } else {
+        for (int i = tid; i < nsort; i += NT) {
+            unsigned long long k = ~0ull;
+            if (i < S) {
+                float v = score(i);
+                v = (v == v ? v : SHOTKV_NEG_INF) + 0.f;                    // NaN last; -0 and +0 are equal
+                const unsigned b = __float_as_uint(v);
+                const unsigned up = b & 0x80000000u ? ~b : b | 0x80000000u;  // ascending with the score
+                k = (unsigned long long)~up << 32 | (unsigned)i;
+            }
+            key[i] = k;
+        }
+        __syncthreads();
+        block_sort<NT>(key, nsort);
+        for (int r = tid; r < S; r += NT) {
+            const int i = (int)(unsigned)key[r];
+            cum[r] = o[i + 1] - o[i];
+        }
     }
     __syncthreads();
-    if (mode == 0) {
-        block_exclusive_scan(cum, S, tmp);
-        for (int r = tid; r < S; r += kSelectThreads) {
-            const int i = order[r];
+    auto shot_at = [&](int r) { return counted ? order[r] : (int)(unsigned)key[r]; };
+    if (a.mode == 0) {
+        block_exclusive_scan<NT>(cum, S, tmp);
+        for (int r = tid; r < S; r += NT) {
+            const int i = shot_at(r);
             const int len = o[i + 1] - o[i];
             kl[i] = (cum[r] + len <= shot_budget) ? len : 0;
         }
-    } else {
-        if (tid == 0) {
-            int used = 0;
-            for (int r = 0; r < S; ++r) {
-                const int i = order[r];
-                const int len = cum[r];
-                if (used + len <= shot_budget) {
-                    kl[i] = len;
-                    used += len;
-                } else {
-                    kl[i] = 0;
-                }
+    } else if (warp == 0) {
+        // one warp walks the ranking, 32 shots at a time, and hops from one that fits to the next
+        int left = shot_budget;
+        for (int r0 = 0; r0 < S; r0 += 32) {
+            const int r = r0 + lane;
+            const int len = r < S ? cum[r] : 0x7fffffff;
+            unsigned ahead = 0xffffffffu, kept = 0;                          // shots not passed yet; shots kept
+            for (;;) {
+                const unsigned fit = __ballot_sync(0xffffffffu, len <= left) & ahead;
+                if (!fit) break;
+                const int f = __ffs(fit) - 1;
+                kept |= 1u << f;
+                ahead = f == 31 ? 0u : ~0u << (f + 1);
+                left -= __shfl_sync(0xffffffffu, len, f);
             }
+            if (r < S) kl[shot_at(r)] = (kept >> lane) & 1u ? len : 0;
         }
     }
     __syncthreads();
-    for (int i = tid; i < S; i += kSelectThreads) keep[(size_t)bl * S + i] = kl[i] > 0;
+    for (int i = tid; i < S; i += NT) a.keep[(size_t)bl * S + i] = kl[i] > 0;
     __syncthreads();
-    const int kept_shot_tokens = block_exclusive_scan(kl, S, tmp);
+    const int kept_shot_tokens = block_exclusive_scan<NT>(kl, S, tmp);
     const int total = always + kept_shot_tokens;
-    int* out = kept_idx + (size_t)bl * Mcap;
-    if (tid == 0) kept_count[bl] = total;
-    for (int t = tid; t < pre && t < Mcap; t += kSelectThreads) out[t] = t;
-    const int warp = tid >> 5, lane = tid & 31;
-    for (int i = warp; i < S; i += kSelectThreads / 32) {
-        if (keep[(size_t)bl * S + i]) {
-            const int dst = pre + kl[i], lo = o[i], len = o[i + 1] - o[i];
-            for (int t = lane; t < len; t += 32)
-                if (dst + t < Mcap) out[dst + t] = lo + t;
-        }
+    int* out = a.kept_idx + (size_t)bl * a.Mcap;
+    if (tid == 0) a.kept_count[bl] = total;
+    for (int t = tid; t < pre && t < a.Mcap; t += NT) out[t] = t;
+    for (int i = warp; i < S; i += NT / 32) {
+        const int at = kl[i], len = (i + 1 < S ? kl[i + 1] : kept_shot_tokens) - at;   // 0 unless the shot is kept
+        const int dst = pre + at, lo = o[i];
+        for (int t = lane; t < len; t += 32)
+            if (dst + t < a.Mcap) out[dst + t] = lo + t;
     }
     const int qdst = pre + kept_shot_tokens;
-    for (int t = tid; t < N - qst; t += kSelectThreads)
-        if (qdst + t < Mcap) out[qdst + t] = qst + t;
-    for (int t = total + tid; t < Mcap; t += kSelectThreads) out[t] = -1;
+    for (int t = tid; t < a.N - qst; t += NT)
+        if (qdst + t < a.Mcap) out[qdst + t] = qst + t;
+    for (int t = total + tid; t < a.Mcap; t += NT) out[t] = -1;
+}
+
+// The boundaries of a prompt, copied to shared memory by the whole CTA (the caller puts the barrier).
+__device__ __forceinline__ void copy_bounds(int* to, const ShotTable& tab, int b, int S) {
+    const int* o = table_row(tab, b);
+    for (int i = threadIdx.x; i <= S; i += blockDim.x) to[i] = o[i];
+}
+__host__ __device__ constexpr size_t bounds_smem_bytes(int S) { return (size_t)(S + 4) / 4 * 4 * 4; }
+
+// Selection from scores already in memory: one CTA per (b, l), NT = kSelectThreads where shots are
+// ranked by counting, kSortThreads beyond; bounds_smem_bytes(S) + select_smem_bytes(S) of shared memory.
+template <int NT>
+__global__ void __launch_bounds__(NT) select_shots_kernel(const float* __restrict__ shot_scores, const __grid_constant__ ShotTable tab,
+                                                         const SelectArgs a) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    const int bl = blockIdx.x;
+    int* o = reinterpret_cast<int*>(sm);
+    copy_bounds(o, tab, bl / a.L, a.S);
+    __syncthreads();
+    const float* scores = shot_scores + (size_t)bl * a.S;
+    select_body<NT>(a, bl, o, sm + bounds_smem_bytes(a.S), [&](int i) { return scores[i]; });
 }
 
 // Row gather: Kc[u][j] = K[u][kept_idx[bl][j]], same for V.  Rows are D bf16 = D/8 16-byte

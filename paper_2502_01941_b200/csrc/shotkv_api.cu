@@ -200,7 +200,6 @@ struct PrefillWs {
     float* item_z;
     float* row_m;      // [U][Rpad]
     float* row_invz;
-    float* unit_shot;  // [U][S]
     float* imp;        // [U][N] per-token importances of the fused call's per-token route (absent otherwise)
     unsigned long long* redo;   // [U * kMaxChunks] not 0 for the items the exact kernel must recompute
     size_t total;
@@ -218,7 +217,6 @@ PrefillWs carve(const shotkv_dims* d, void* base) {
     w.item_z = (float*)take(U * kMaxChunks * R * 4);
     w.row_m = (float*)take(U * R * 4);
     w.row_invz = (float*)take(U * R * 4);
-    w.unit_shot = (float*)take(U * (size_t)(d->S > 0 ? d->S : 1) * 4);
     w.imp = (float*)take(token_route(d) ? U * (size_t)d->N * 4 : 0);
     w.redo = (unsigned long long*)take(U * kMaxChunks * 8);
     w.total = o;
@@ -540,7 +538,7 @@ int run_stats(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q, const
     const int rc = launch_score_tc(ctx, d, Q, K, w, -1, none, plan, stream);
     if (rc) return rc;
     prof_mark(ctx, stream);
-    row_stats_kernel<<<d->B * d->L * d->Hkv, 256, 0, stream>>>(partial_view(ctx, d, w, -1, plan), (d->H / d->Hkv) * d->W, w.row_m, w.row_invz);
+    row_stats_kernel<<<d->B * d->L * d->Hkv, rpad_of(d), 0, stream>>>(partial_view(ctx, d, w, -1, plan), (d->H / d->Hkv) * d->W, w.row_m, w.row_invz);
     LAUNCH_CHECK(ctx);
     return SHOTKV_OK;
 }
@@ -600,18 +598,64 @@ PrefillWs group_ws(const PrefillWs& w, const shotkv_dims* d, const GroupView& v,
     x.item_z = w.item_z + v.u0 * kMaxChunks * R;
     x.row_m = w.row_m + v.u0 * R;
     x.row_invz = w.row_invz + v.u0 * R;
-    x.unit_shot = w.unit_shot + v.u0 * (size_t)(d->S > 0 ? d->S : 1);
     x.redo = w.redo + v.u0 * kMaxChunks;
     return x;
 }
 
-int run_select(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_policy* p, const ShotTable& tab, float* shot_scores,
-               uint8_t* keep, int32_t* kept_idx, int32_t* kept_count, int32_t Mcap, cudaStream_t stream) {
-    const size_t smem = (size_t)d->S * 16 + (kSelectThreads + 1) * 4 + 16;
-    select_shots_kernel<<<d->B * d->L, kSelectThreads, smem, stream>>>(shot_scores, tab, d->L, d->N, d->S, budget_of(d, p),
-                                                                     p->select_mode, Mcap, keep, kept_idx, kept_count);
+SelectArgs select_args(const shotkv_dims* d, const shotkv_policy* p, uint8_t* keep, int32_t* kept_idx, int32_t* kept_count,
+                       int32_t Mcap) {
+    return SelectArgs{d->L, d->N, d->S, budget_of(d, p), p->select_mode, Mcap, keep, kept_idx, kept_count};
+}
+
+int run_select(shotkv_ctx* ctx, const shotkv_dims* d, const ShotTable& tab, const float* shot_scores, const SelectArgs& sa,
+               cudaStream_t stream) {
+    const size_t smem = bounds_smem_bytes(d->S) + select_smem_bytes(d->S);
+    if (d->S <= kRankByCount) select_shots_kernel<kSelectThreads><<<d->B * d->L, kSelectThreads, smem, stream>>>(shot_scores, tab, sa);
+    else select_shots_kernel<kSortThreads><<<d->B * d->L, kSortThreads, smem, stream>>>(shot_scores, tab, sa);
     LAUNCH_CHECK(ctx);
     return SHOTKV_OK;
+}
+
+// Per-shot scores from per-token importances.
+int run_token_scores(shotkv_ctx* ctx, const shotkv_dims* d, const float* imp, const ShotTable& tab, float* shot_scores, cudaStream_t stream) {
+    const int bl = d->B * d->L;
+    if ((long long)d->N >= (long long)kLongShot * d->S)
+        shot_score_from_tokens_kernel<kTokenWarps><<<dim3(d->S, bl), 32 * kTokenWarps, 0, stream>>>(imp, tab, d->L, d->Hkv, d->N, d->S, shot_scores);
+    else
+        shot_score_from_tokens_kernel<1><<<dim3((d->S + kTokenWarps - 1) / kTokenWarps, bl), 32 * kTokenWarps, 0, stream>>>(imp, tab, d->L, d->Hkv, d->N, d->S, shot_scores);
+    LAUNCH_CHECK(ctx);
+    return SHOTKV_OK;
+}
+
+// Per-shot scores from the scoring pass's partials, and the selection.
+template <int ROWS>
+int run_reduce_select_t(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView& pv, const ShotTable& tab, float* shot_scores,
+                        const SelectArgs& sa, cudaStream_t stream) {
+    // a row of masses per CTA of the cluster: with thousands of shots fewer CTAs share the heads, so
+    // that two still fit an SM (one from about 4,000 shots on)
+    int ranks = d->Hkv < kReduceCluster ? d->Hkv : kReduceCluster;
+    while (ranks > 1 && reduce_smem_bytes(ROWS, pv.P, d->S, ranks) > kBigSmem / 2) ranks = (ranks + 1) / 2;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = ranks;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = dim3(d->B * d->L * ranks);
+    lc.blockDim = dim3(kReduceThreads);
+    lc.dynamicSmemBytes = reduce_smem_bytes(ROWS, pv.P, d->S, ranks);
+    lc.stream = stream;
+    lc.attrs = at;
+    lc.numAttrs = 1;
+    if (lc.dynamicSmemBytes > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "too many shots for the single-pass path (S = %d)", d->S);
+    CUDA_TRY(ctx, cudaLaunchKernelEx(&lc, reduce_select_kernel<ROWS>, pv, tab, (d->H / d->Hkv) * d->W, (int)d->Hkv, ranks, shot_scores, sa));
+    ctx->launches += 1;
+    return SHOTKV_OK;
+}
+int run_reduce_select(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView& pv, const ShotTable& tab, float* shot_scores,
+                      const SelectArgs& sa, cudaStream_t stream) {
+    if (d->S == 0) return run_select(ctx, d, tab, shot_scores, sa, stream);
+    return pv.Rpad == 128 ? run_reduce_select_t<128>(ctx, d, pv, tab, shot_scores, sa, stream)
+                          : run_reduce_select_t<256>(ctx, d, pv, tab, shot_scores, sa, stream);
 }
 
 int run_compact(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* K, const shotkv_bf16* V, const int32_t* kept_idx,
@@ -649,7 +693,8 @@ cudaError_t set_kernel_attributes() {
     if (e == cudaSuccess) e = set_tc_attributes<128, 2>();
     if (e == cudaSuccess) e = set_tc_attributes<64, 1>();
     if (e == cudaSuccess) e = set_tc_attributes<64, 2>();
-    const void* small[] = {(const void*)select_shots_kernel, (const void*)shot_mass_kernel<128>, (const void*)shot_mass_kernel<256>,
+    const void* small[] = {(const void*)select_shots_kernel<kSelectThreads>, (const void*)select_shots_kernel<kSortThreads>,
+                           (const void*)reduce_select_kernel<128>, (const void*)reduce_select_kernel<256>,
                            (const void*)decode_score_kernel<128>, (const void*)decode_score_kernel<64>,
                            (const void*)decode_attend_kernel<128>, (const void*)decode_attend_kernel<64>,
                            (const void*)decode_rank_kernel};
@@ -817,12 +862,8 @@ int shotkv_select_shots(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv_p
     const PrefillWs w = carve(dims, ws);
     ShotTable tab;
     if ((rc = prepare_table(ctx, dims, offsets_host, false, w.off, tab, stream))) return rc;
-    if (token_importance && dims->S > 0) {
-        dim3 grid((dims->S + kShotsPerCta - 1) / kShotsPerCta, dims->B * dims->L);
-        shot_score_from_tokens_kernel<<<grid, 32 * kShotsPerCta, 0, stream>>>(token_importance, tab, dims->L, dims->Hkv, dims->N, dims->S, shot_scores);
-        LAUNCH_CHECK(ctx);
-    }
-    if ((rc = run_select(ctx, dims, policy, tab, shot_scores, keep, kept_idx, kept_count, Mcap, stream))) return rc;
+    if (token_importance && dims->S > 0 && (rc = run_token_scores(ctx, dims, token_importance, tab, shot_scores, stream))) return rc;
+    if ((rc = run_select(ctx, dims, tab, shot_scores, select_args(dims, policy, keep, kept_idx, kept_count, Mcap), stream))) return rc;
     if (orc > 0) fail(ctx, orc, "always-kept tokens (%d) exceed the budget (%d) for some prompt", worst, budget_of(dims, policy));
     return orc;
 }
@@ -876,12 +917,8 @@ int shotkv_select_shots_static(shotkv_ctx* ctx, const shotkv_dims* dims, const s
     // every entry the kernels read is overwritten here, so nothing of an earlier call survives
     ShotTable tab;
     if ((rc = prepare_table(ctx, dims, offsets_host, false, off, tab, stream))) return rc;
-    if (token_importance && dims->S > 0) {
-        dim3 grid((dims->S + kShotsPerCta - 1) / kShotsPerCta, dims->B * dims->L);
-        shot_score_from_tokens_kernel<<<grid, 32 * kShotsPerCta, 0, stream>>>(token_importance, tab, dims->L, dims->Hkv, dims->N, dims->S, shot_scores);
-        LAUNCH_CHECK(ctx);
-    }
-    if ((rc = run_select(ctx, dims, policy, tab, shot_scores, keep, kept_idx, kept_count, Mcap, stream))) return rc;
+    if (token_importance && dims->S > 0 && (rc = run_token_scores(ctx, dims, token_importance, tab, shot_scores, stream))) return rc;
+    if ((rc = run_select(ctx, dims, tab, shot_scores, select_args(dims, policy, keep, kept_idx, kept_count, Mcap), stream))) return rc;
     if (orc > 0) fail(ctx, orc, "always-kept tokens (%d) exceed the budget (%d) for some prompt", worst, budget_of(dims, policy));
     return orc;
 }
@@ -948,7 +985,7 @@ int prefill_compress_impl(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv
     if ((rc = check_ws(ctx, dims, ws, ws_bytes))) return rc;
     cudaStream_t stream = (cudaStream_t)stream_;
     const PrefillWs w = carve(dims, ws);
-    const int S = dims->S, R = (dims->H / dims->Hkv) * dims->W, Rpad = rpad_of(dims);
+    const int S = dims->S;
     const size_t S1 = S > 0 ? S : 1, row = dims->d;
 
     // the boundaries of all prompts once, and the work partition of one (full) group
@@ -958,10 +995,6 @@ int prefill_compress_impl(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv
     ShotTable whole;
     if ((rc = prepare_table(ctx, dims, offsets_host, true, w.off, whole, stream))) return rc;
     const int P = pieces_of(S, plan);
-    const size_t msm = ((size_t)P + 2 * Rpad) * 4;     // shot_mass_kernel: row statistics and one mass per piece
-    if (S > 0) {
-        if (msm > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "too many shots for the single-pass path (S = %d)", S);
-    }
     prof_begin(ctx);
     const bool forked = gs.n > 1;
     cudaStream_t tail = forked ? ctx->aux : stream;
@@ -978,7 +1011,6 @@ int prefill_compress_impl(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv
         ShotTable tab;
         advance_table(tab, v.d.B, whole, v.b0);
         const shotkv_dims* dg = &v.d;
-        const int Ug = dg->B * dg->L * dg->Hkv;
         const shotkv_bf16* Kg = K + v.u0 * dims->N * row;
         const shotkv_bf16* Vg = V + v.u0 * dims->N * row;
         float* scores_g = shot_scores + v.bl0 * S1;
@@ -994,20 +1026,9 @@ int prefill_compress_impl(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv
             handed = true;
         }
         prof_gmark(ctx, g, 2, tail);
-        if (S > 0) {
-            const PartialView pv = partial_view(ctx, dg, wg, S, plan);
-            if (Rpad == 128)
-                shot_mass_kernel<128><<<Ug, 128, msm, tail>>>(pv, tab, R, dg->L, dg->Hkv, S, wg.unit_shot);
-            else
-                shot_mass_kernel<256><<<Ug, 256, msm, tail>>>(pv, tab, R, dg->L, dg->Hkv, S, wg.unit_shot);
-            ctx->launches += 1;
-            if (cudaGetLastError() != cudaSuccess) return bail(fail(ctx, SHOTKV_ERR_CUDA, "per-shot reduction failed to launch"));
-            shot_score_from_mass_kernel<<<dg->B * dg->L, 128, 0, tail>>>(wg.unit_shot, tab, dg->L, dg->Hkv, S, scores_g);
-            ctx->launches += 1;
-            if (cudaGetLastError() != cudaSuccess) return bail(fail(ctx, SHOTKV_ERR_CUDA, "per-shot score kernel failed to launch"));
-        }
-        prof_gmark(ctx, g, 3, tail);
-        if ((rc = run_select(ctx, dg, policy, tab, scores_g, keep + v.bl0 * S1, idx_g, count_g, Mcap, tail))) return bail(rc);
+        if ((rc = run_reduce_select(ctx, dg, partial_view(ctx, dg, wg, S, plan), tab, scores_g,
+                                    select_args(dg, policy, keep + v.bl0 * S1, idx_g, count_g, Mcap), tail))) return bail(rc);
+        prof_gmark(ctx, g, 3, tail);                    // reduction and selection are one kernel: the selection's own stage is empty
         prof_gmark(ctx, g, 4, tail);
         if ((rc = run_compact(ctx, dg, Kg, Vg, idx_g, count_g, Mcap, Kc + v.u0 * (size_t)Mcap * row, Vc + v.u0 * (size_t)Mcap * row, tail))) return bail(rc);
         prof_gmark(ctx, g, 5, tail);

@@ -1,0 +1,62 @@
+"""The kernel that reduces the scoring pass's partials and selects, and the ranking shared with
+shotkv_select_shots: sizes on both sides of every branch (ranking by counting or by sorting, shots
+to a warp, kv heads to a cluster)."""
+import numpy as np
+import pytest
+import torch
+
+import paper_2502_01941_b200 as skv
+from oracle import shotkv_oracle as O
+from paper_2502_01941_b200 import workloads as wl
+import parity as P
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = skv.Context(0)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("S", [1, 2, 31, 33, 255, 256, 257, 511, 512, 513, 1025, 8192])
+def test_ranking_with_ties(ctx, S):
+    """Whole numbers, so that many scores tie (index order decides), zeros of both signs among them."""
+    B, L, W = 2, 2, 4
+    rng = np.random.default_rng(S)
+    off = np.concatenate([np.zeros((B, 1), np.int64) + 3, 3 + np.cumsum(rng.integers(1, 9, size=(B, S)), axis=1)], axis=1).astype(np.int32)
+    N = int(off[:, -1].max()) + 20
+    dims = skv.make_dims(B, L, 4, 2, 64, N, W, S)
+    sc = rng.integers(-3, 4, size=(B, L, S)).astype(np.float32)
+    sc[sc == 0] = np.where(rng.random((sc == 0).sum()) < 0.5, np.float32(-0.0), np.float32(0.0))
+    for mode in (0, 1):
+        pol = skv.make_policy(r_p=0.45, select_mode=mode)
+        Mcap = skv.shotkv_kept_capacity(dims, pol, off)
+        out = skv.alloc_prefill_outputs(dims, Mcap)
+        out["shot_scores"].copy_(torch.from_numpy(sc))
+        skv.shotkv_select_shots(ctx, dims, pol, None, off, out["shot_scores"], out["keep"], out["kept_idx"], out["kept_count"], Mcap,
+                                out["ws"])
+        torch.cuda.synchronize()
+        for b in range(B):
+            for l in range(L):
+                keep, idx, _ = O.select_shots(sc[b, l], off[b], N, 0.45, mode)
+                np.testing.assert_array_equal(out["keep"][b, l].cpu().numpy(), keep)
+                n = int(out["kept_count"][b, l])
+                assert n == len(idx)
+                np.testing.assert_array_equal(out["kept_idx"][b, l, :n].cpu().numpy(), idx)
+                assert (out["kept_idx"][b, l, n:] == -1).all()
+
+
+@pytest.mark.parametrize("Hkv,G,W", [(1, 4, 32), (3, 2, 16), (8, 4, 64), (9, 1, 8), (17, 3, 64)])
+@pytest.mark.parametrize("mode", [skv.SCORING_FAST, skv.SCORING_EXACT], ids=["fast", "exact"])
+def test_heads_to_a_cluster(ctx, Hkv, G, W, mode):
+    cfg = wl.PrefillConfig("heads", B=2, L=1, H=Hkv * G, Hkv=Hkv, d=64, N=2305, W=W, S=17, shot_dist="uniform", shot_lo=64,
+                           shot_hi=192, question_len=129, r_p=0.4, cfg_id=62)
+    Q, K, V, off = wl.prefill_batch(cfg, "cuda")
+    skv.shotkv_set_scoring_mode(ctx, mode)
+    try:
+        gpu = P.gpu_prefill(ctx, P.dims_of(cfg), Q, K, V, off, cfg.r_p, 0, "fused")
+    finally:
+        skv.shotkv_set_scoring_mode(ctx, skv.SCORING_FAST)
+    assert P.check_all_units(gpu, Q, K, V, off, cfg.r_p) <= 1
