@@ -16,29 +16,65 @@ struct DecodeParams {
     __nv_bfloat16* Vd;            // [U][Dcap][d]
     float* partial;               // [U][Dcap]
     int H, Hkv, G, Mcap, Dcap, n_old;
+    int nsplit;                   // CTAs (a cluster) that share a unit's keys
     float scale_log2;
     const __nv_bfloat16* Vc;      // [U][Mcap][d]   (attention-output variant only)
     float* out;                   // [B][L][H][d]   (attention-output variant only)
 };
 
-// One CTA per (sequence, layer, kv head).  Each warp takes 16 keys at a time straight from
-// global memory: thread (g, t) of a warp reads 16 contiguous bytes of key rows g and g+8 per
-// 32-dim block, which serve as the A fragments of two m16n8k16 MMAs whose B operand is the
-// group's (up to 8) query rows held in registers with the same k-index permutation.  The logits
+// ---- a unit's keys shared by a cluster -------------------------------------------------------
+// A unit (sequence, layer, kv head) whose batch is too small to fill the GPU is shared by a cluster of
+// p.nsplit CTAs: blocks of 16 keys go round the warps of all of them.  Every CTA sends its (m, z) per
+// query row to all others and each then knows the whole row's maximum and sum.
+constexpr int kMaxSplit = 8;
+
+// Which CTA of the cluster has key i, NW warps to a CTA.
+__device__ __forceinline__ int split_of_key(int i, int NW, int nsplit) { return ((i >> 4) / NW) % nsplit; }
+
+// Every CTA's (m, z) of the 8 query rows (`own`, [8][2], in shared memory behind a barrier) to all
+// CTAs' `table` [nsplit][8][2]; returns when all have arrived.  Preceded by a cluster_arrive at the
+// start of the kernel (a CTA's memory may be written once it has begun).  What the CTA wrote to its own
+// shared memory before may be read by the others afterwards; they must be done before it ends.
+__device__ __forceinline__ void exchange_stats(const float* own, float* table, int rank, int nsplit) {
+    cluster_wait();
+    for (int i = threadIdx.x; i < 16 * nsplit; i += blockDim.x) cluster_store(table + rank * 16 + (i & 15), i >> 4, own[i & 15]);
+    cluster_arrive();
+    cluster_wait();
+}
+// The row's maximum and 1 / sum over the whole cluster.
+__device__ __forceinline__ void merge_stats(const float* table, int nsplit, int row, float& m, float& iz) {
+    m = SHOTKV_NEG_INF;
+    for (int c = 0; c < nsplit; ++c) m = fmaxf(m, table[c * 16 + row * 2]);
+    float z = 0.f;
+    for (int c = 0; c < nsplit; ++c) z += table[c * 16 + row * 2 + 1] * ex2f(table[c * 16 + row * 2] - m);
+    iz = z > 0.f ? 1.f / z : 0.f;
+}
+
+// One CTA, or a cluster of p.nsplit, per (sequence, layer, kv head).  Each warp takes 16 keys at a
+// time straight from global memory: thread (g, t) of a warp reads 16 contiguous bytes of key rows g
+// and g+8 per 32-dim block, which serve as the A fragments of two m16n8k16 MMAs whose B operand is
+// the group's (up to 8) query rows held in registers with the same k-index permutation.  The logits
 // of the decode entries are parked in shared memory until the softmax statistics over all keys
 // (kept prefill keys + decode keys) are known.
-template <int D>
+// SPLIT = false is the same for whole units, nsplit = 1: with the stride of the loop a constant the
+// compiler unrolls it and keeps more loads in flight (8 sequences x 32 layers: 245 us a step against 273).
+template <int D, bool SPLIT>
 __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p) {
     constexpr int NB = D / 32;     // 32-dim blocks
     constexpr int VPR = D / 8;     // 16-byte vectors per row
     extern __shared__ __align__(16) unsigned char dsm[];
     float* sdec = reinterpret_cast<float*>(dsm);             // [8][Dcap]
     float* sred = sdec + 8 * p.Dcap;                         // [8 warps][8 rows][2]
-    float* sfin = sred + 8 * 8 * 2;                          // [8 rows][2]  (m, 1/Z)
+    float* sfin = sred + 8 * 8 * 2;                          // [8 rows][2]  (m, z) of this CTA, then (m, 1/Z)
+    float* stab = sfin + 16;                                 // [nsplit][8 rows][2]  (m, z) of the cluster's CTAs
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, t4 = lane & 3;
-    const int u = blockIdx.x;
+    const int nsplit = SPLIT ? p.nsplit : 1;
+    const int u = blockIdx.x / nsplit, rank = blockIdx.x - u * nsplit;
+    if (SPLIT) cluster_arrive();
+    grid_wait();
+    grid_release();
     const int bl = u / p.Hkv, hk = u - bl * p.Hkv;
     const int M = min(p.kept_count[bl], p.Mcap);
     const int n = p.n_old + 1;
@@ -50,7 +86,8 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p)
     const uint4* vnew_u = reinterpret_cast<const uint4*>(p.v_new + (size_t)u * D);
 
     // append the new token's key and value as decode entry n_old
-    if (tid < VPR) Kd_u[(size_t)p.n_old * VPR + tid] = knew_u[tid];
+    if (rank != 0) {
+    } else if (tid < VPR) Kd_u[(size_t)p.n_old * VPR + tid] = knew_u[tid];
     else if (tid < 2 * VPR) Vd_u[(size_t)p.n_old * VPR + (tid - VPR)] = vnew_u[tid - VPR];
 
     // query rows of this group as B fragments (row g of the fragment = query head hk*G+g)
@@ -62,7 +99,7 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p)
     }
 
     float m0 = SHOTKV_NEG_INF, m1 = SHOTKV_NEG_INF, z0 = 0.f, z1 = 0.f;   // query rows 2*t4, 2*t4+1
-    for (int base = warp * 16; base < Ktot; base += 8 * 16) {
+    for (int base = (rank * 8 + warp) * 16; base < Ktot; base += nsplit * 8 * 16) {
         const int ia = base + g, ib = base + g + 8;
         const bool va = ia < Ktot, vb = ib < Ktot;
         auto row_ptr = [&](int i, bool valid) -> const uint4* {
@@ -138,13 +175,20 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p)
     if (tid < 8) {
         float m = SHOTKV_NEG_INF;
         for (int w = 0; w < 8; ++w) m = fmaxf(m, sred[(w * 8 + tid) * 2]);
+        const float mu = m == SHOTKV_NEG_INF ? 0.f : m;      // a CTA of a cluster may have had no keys
         float z = 0.f;
-        for (int w = 0; w < 8; ++w) z += sred[(w * 8 + tid) * 2 + 1] * ex2f(sred[(w * 8 + tid) * 2] - m);
+        for (int w = 0; w < 8; ++w) z += sred[(w * 8 + tid) * 2 + 1] * ex2f(sred[(w * 8 + tid) * 2] - mu);
         sfin[tid * 2] = m;
-        sfin[tid * 2 + 1] = z > 0.f ? 1.f / z : 0.f;
+        sfin[tid * 2 + 1] = SPLIT ? z : (z > 0.f ? 1.f / z : 0.f);
     }
     __syncthreads();
+    if (SPLIT) {
+        exchange_stats(sfin, stab, rank, nsplit);
+        if (tid < 8) merge_stats(stab, nsplit, tid, sfin[tid * 2], sfin[tid * 2 + 1]);
+        __syncthreads();
+    }
     for (int j = tid; j < n; j += 256) {
+        if (SPLIT && split_of_key(M + j, 8, nsplit) != rank) continue;
         float s = 0.f;
         for (int r = 0; r < p.G; ++r) s += ex2f(sdec[r * p.Dcap + j] - sfin[r * 2]) * sfin[r * 2 + 1];
         p.partial[(size_t)u * p.Dcap + j] = s;
@@ -219,13 +263,17 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     extern __shared__ __align__(16) unsigned char dsm[];
     float* sdec = reinterpret_cast<float*>(dsm);             // [8][Dcap]
     float* sred = sdec + 8 * p.Dcap;                         // [NW warps][8 rows][2]
-    float* sfin = sred + NW * 8 * 2;                         // [8 rows][2]  (m, 1/Z)
-    unsigned char* ring = reinterpret_cast<unsigned char*>(sfin + 16);   // [NW][NS][keys | values][16 rows][D bf16]; later [NW][8 rows][D] floats
+    float* sfin = sred + NW * 8 * 2;                         // [8 rows][2]  (m, z) of this CTA, then (m, 1/Z)
+    float* stab = sfin + 16;                                 // [kMaxSplit][8 rows][2]  (m, z) of the cluster's CTAs
+    unsigned char* ring = reinterpret_cast<unsigned char*>(stab + kMaxSplit * 16);   // [NW][NS][keys | values][16 rows][D bf16]; later [NW][8 rows][D] floats
     float* sO = reinterpret_cast<float*>(ring);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, t4 = lane & 3;
-    const int u = blockIdx.x;
+    const int u = blockIdx.x / p.nsplit, rank = blockIdx.x - u * p.nsplit;
+    if (p.nsplit > 1) cluster_arrive();
+    grid_wait();
+    grid_release();
     const int bl = u / p.Hkv, hk = u - bl * p.Hkv;
     const int M = min(p.kept_count[bl], p.Mcap);
     const int n = p.n_old + 1;
@@ -238,7 +286,8 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     const uint4* Vc_u = reinterpret_cast<const uint4*>(p.Vc + (size_t)u * p.Mcap * D);
 
     // append the new token's key and value as decode entry n_old
-    if (tid < VPR) Kd_u[(size_t)p.n_old * VPR + tid] = knew_u[tid];
+    if (rank != 0) {
+    } else if (tid < VPR) Kd_u[(size_t)p.n_old * VPR + tid] = knew_u[tid];
     else if (tid < 2 * VPR) Vd_u[(size_t)p.n_old * VPR + (tid - VPR)] = vnew_u[tid - VPR];
 
     // query row g of the group as A fragments (rows 8..15 of the 16-row operand are zero)
@@ -282,14 +331,14 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     float m = SHOTKV_NEG_INF, z = 0.f;
     // blocks are requested NS - 1 ahead; one copy group per block, empty past the end, so that
     // "at most NS - 1 groups pending" always means this block's rows have landed
-    constexpr int STRIDE = NW * 16;
+    const int first = (rank * NW + warp) * 16, STRIDE = p.nsplit * NW * 16;
     int stage = 0;
 #pragma unroll
     for (int k = 0; k < NS - 1; ++k) {
-        if (warp * 16 + k * STRIDE < Ktot) fetch_block(warp * 16 + k * STRIDE, k);
+        if (first + k * STRIDE < Ktot) fetch_block(first + k * STRIDE, k);
         else cp_async_commit();
     }
-    for (int base = warp * 16; base < Ktot; base += STRIDE) {
+    for (int base = first; base < Ktot; base += STRIDE) {
         __syncwarp();                                       // every lane has read the stage the next copy overwrites
         {
             const int nb = base + (NS - 1) * STRIDE;
@@ -381,106 +430,163 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     if (tid < 8) {
         float mm = SHOTKV_NEG_INF;
         for (int w = 0; w < NW; ++w) mm = fmaxf(mm, sred[(w * 8 + tid) * 2]);
+        const float mu = mm == SHOTKV_NEG_INF ? 0.f : mm;    // a CTA of a cluster may have had no keys
         float zz = 0.f;
-        for (int w = 0; w < NW; ++w) zz += sred[(w * 8 + tid) * 2 + 1] * ex2f(sred[(w * 8 + tid) * 2] - mm);
+        for (int w = 0; w < NW; ++w) zz += sred[(w * 8 + tid) * 2 + 1] * ex2f(sred[(w * 8 + tid) * 2] - mu);
         sfin[tid * 2] = mm;
-        sfin[tid * 2 + 1] = zz > 0.f ? 1.f / zz : 0.f;
+        sfin[tid * 2 + 1] = p.nsplit > 1 ? zz : (zz > 0.f ? 1.f / zz : 0.f);
     }
     __syncthreads();
+    float* out = p.out + ((size_t)bl * p.H + (size_t)hk * p.G) * D;
+    // the warps' outputs, relative to the CTA's maximum; alone, the CTA has the rows' whole sums already
     for (int idx = tid; idx < p.G * D; idx += NT) {
-        const int r = idx / D, dim = idx - r * D;
+        const int r = idx / D;
         const float mm = sfin[r * 2];
         float o = 0.f;
         for (int w = 0; w < NW; ++w) {
             const float mw = sred[(w * 8 + r) * 2];
-            if (mw != SHOTKV_NEG_INF) o += sO[(w * 8 + r) * D + dim] * ex2f(mw - mm);
+            if (mw != SHOTKV_NEG_INF) o += sO[w * 8 * D + idx] * ex2f(mw - mm);
         }
-        p.out[((size_t)bl * p.H + (size_t)hk * p.G + r) * D + dim] = o * sfin[r * 2 + 1];
+        if (p.nsplit > 1) sO[idx] = o;                       // read above by this thread alone
+        else out[idx] = o * sfin[r * 2 + 1];
+    }
+    if (p.nsplit > 1) {
+        __syncthreads();
+        exchange_stats(sfin, stab, rank, p.nsplit);          // and all CTAs' outputs may be read
+        if (tid < 8) merge_stats(stab, p.nsplit, tid, sfin[tid * 2], sfin[tid * 2 + 1]);
+        __syncthreads();
+        // each CTA adds up its share of the output elements
+        for (int idx = rank * NT + tid; idx < p.G * D; idx += p.nsplit * NT) {
+            const int r = idx / D;
+            const float mm = sfin[r * 2];
+            float o = 0.f;
+            for (int c = 0; c < p.nsplit; ++c) o += cluster_load(sO + idx, c) * ex2f(stab[c * 16 + r * 2] - mm);
+            out[idx] = o * sfin[r * 2 + 1];
+        }
+        cluster_arrive();                                    // done with the others' memory
     }
     for (int j = tid; j < n; j += NT) {
+        if (p.nsplit > 1 && split_of_key(M + j, NW, p.nsplit) != rank) continue;
         float s = 0.f;
         for (int r = 0; r < p.G; ++r) s += ex2f(sdec[r * p.Dcap + j] - sfin[r * 2]) * sfin[r * 2 + 1];
         p.partial[(size_t)u * p.Dcap + j] = s;
     }
+    if (p.nsplit > 1) cluster_wait();                        // the others are done with this CTA's
 }
 
-// acc[bl][j] += sum over kv heads of partial (fixed order); the new entry starts from 0.
-__global__ void decode_accumulate_kernel(const float* __restrict__ partial, int Hkv, int Dcap, int n_old, int T_old,
-                                         float* __restrict__ acc, int* __restrict__ born) {
+// The rest of a step for one (b, l): acc[j] += sum over kv heads of the entries' weights (fixed order,
+// a new entry starts from 0), and, every so many steps, the eviction: the k entries greatest in (acc
+// descending, index ascending) are kept, acc, born and the K and V rows moved up in place.  Entries
+// born at or after `protect_from` rank before all others (an option beyond the paper's rule; a value
+// above every step number protects nothing).
+struct DecodeFinishParams {
+    const float* partial;         // [U][Dcap]
+    float* acc;                   // [B*L][Dcap]
+    int* born;                    // [B*L][Dcap]
+    __nv_bfloat16* Kd;            // [U][Dcap][d]
+    __nv_bfloat16* Vd;            // [U][Dcap][d]
+    int Hkv, Dcap, n, T_old;      // n entries, the new one included
+    int k, protect_from;          // entries to keep
+    int ranks;                    // CTAs (a cluster) per (b, l), heads rank, rank + ranks, ... each
+};
+__device__ __forceinline__ float accumulated(const DecodeFinishParams& p, int bl, int j) {
+    const float* part = p.partial + (size_t)bl * p.Hkv * p.Dcap + j;
+    float s = 0.f;
+#pragma unroll 8
+    for (int h = 0; h < p.Hkv; ++h) s += part[(size_t)h * p.Dcap];
+    return (j == p.n - 1 ? 0.f : p.acc[(size_t)bl * p.Dcap + j]) + s;
+}
+
+// A step without eviction.
+__global__ void __launch_bounds__(128) decode_accumulate_kernel(const DecodeFinishParams p) {
     const int bl = blockIdx.x;
-    for (int j = threadIdx.x; j <= n_old; j += blockDim.x) {
-        float s = 0.f;
-        for (int h = 0; h < Hkv; ++h) s += partial[((size_t)bl * Hkv + h) * Dcap + j];
-        const float prev = j == n_old ? 0.f : acc[(size_t)bl * Dcap + j];
-        acc[(size_t)bl * Dcap + j] = prev + s;
-        if (j == n_old) born[(size_t)bl * Dcap + j] = T_old;
+    grid_wait();
+    grid_release();
+    for (int j = threadIdx.x; j < p.n; j += blockDim.x) {
+        p.acc[(size_t)bl * p.Dcap + j] = accumulated(p, bl, j);
+        if (j == p.n - 1) p.born[(size_t)bl * p.Dcap + j] = p.T_old;
     }
 }
 
-// Top-k of the n decode entries of one (b, l) by (acc descending, index ascending); writes the
-// kept positions in ascending order and compacts acc and born.  Shared: n floats + 3n ints + scan.
-// Entries born at or after `protect_from` rank before all others (an option beyond the paper's
-// rule; pass a value above every step number to protect nothing).
-__global__ void __launch_bounds__(kSelectThreads) decode_rank_kernel(float* __restrict__ acc, int* __restrict__ born,
-                                                                    int Dcap, int n, int k, int protect_from,
-                                                                    int* __restrict__ keep_pos) {
+// A step with eviction.  Every CTA of the cluster adds up and ranks all entries for itself (a few
+// hundred: cheaper than handing the ranking round), so one barrier is all the cluster needs: nobody
+// writes acc and born before all have read them.  Then each moves the rows of its heads, as many at a
+// time as a thread keeps 16-byte vectors in flight; the source of row j is at or after j, so a pass
+// that first loads its rows and then, after a barrier, stores them never overwrites a later source.
+// Latency-bound: as three kernels (sum, ranking, rows) the end of a cycle took 2.5 + 4.8 + 2.4 us on one
+// small layer and 5 + 6.4 + 39 us on 8 sequences x 32 layers.
+// Shared memory: decode_evict_smem_bytes(n).
+__host__ __device__ constexpr size_t decode_evict_smem_bytes(int n) {
+    return rank_smem_bytes(n) + 5 * ((size_t)(n + 3) / 4 * 4 * 4) + 128;
+}
+template <int D>
+__global__ void __launch_bounds__(kSelectThreads) decode_evict_kernel(const DecodeFinishParams p) {
+    constexpr int NT = kSelectThreads, VPR = D / 8, RPP = NT / VPR, Q = 4;   // 16-byte vectors a row, rows a pass per vector in flight
     extern __shared__ __align__(16) unsigned char sm[];
-    float* a = reinterpret_cast<float*>(sm);
-    int* bs = reinterpret_cast<int*>(a + n);
-    int* kf = bs + n;     // keep flag
-    int* ds = kf + n;     // keep flag, then its exclusive scan = destination
-    int* tmp = ds + n;
-    const int bl = blockIdx.x, tid = threadIdx.x;
-    for (int j = tid; j < n; j += kSelectThreads) {
-        const float v = acc[(size_t)bl * Dcap + j];
-        a[j] = v == v ? v : SHOTKV_NEG_INF;      // keep the order total even if a score is NaN
-        bs[j] = born[(size_t)bl * Dcap + j];
+    __shared__ int first_gone;
+    const int n = p.n, n4 = (n + 3) / 4 * 4;
+    float* a = reinterpret_cast<float*>(sm + rank_smem_bytes(n));   // accumulated scores
+    int* bs = reinterpret_cast<int*>(a + n4);      // born
+    int* kf = bs + n4;                             // kept?
+    int* ds = kf + n4;                             // its exclusive scan = destination
+    int* kp = ds + n4;                             // destination -> source
+    int* tmp = kp + n4;
+    const int tid = threadIdx.x;
+    const int bl = blockIdx.x / p.ranks, rank = blockIdx.x - bl * p.ranks;
+    if (tid == 0) first_gone = n;
+    grid_wait();
+    grid_release();
+    for (int j = tid; j < n; j += NT) {
+        const float v = accumulated(p, bl, j);
+        a[j] = v == v ? v : SHOTKV_NEG_INF;        // keep the order total even if a score is NaN
+        bs[j] = j < n - 1 ? p.born[(size_t)bl * p.Dcap + j] : p.T_old;
     }
+    if (p.ranks > 1) cluster_arrive();
     __syncthreads();
     const float top = __int_as_float(0x7f800000);
-    for (int j = tid; j < n; j += kSelectThreads) {
-        const float v = bs[j] >= protect_from ? top : a[j];
-        int rank = 0;
-        for (int i = 0; i < n; ++i) {
-            const float w = bs[i] >= protect_from ? top : a[i];
-            rank += (w > v) || (w == v && i < j);
-        }
-        kf[j] = ds[j] = rank < k;
-    }
+    rank_all<NT>(n, sm, [&](int j) { return bs[j] >= p.protect_from ? top : a[j]; },
+                 [&](int r, int j) {
+                     kf[j] = ds[j] = r < p.k;
+                     if (r >= p.k) atomicMin(&first_gone, j);
+                 });
     __syncthreads();
-    block_exclusive_scan(ds, n, tmp);
-    for (int j = tid; j < n; j += kSelectThreads) {
-        if (kf[j]) {
-            const int dst = ds[j];
-            keep_pos[(size_t)bl * Dcap + dst] = j;
-            acc[(size_t)bl * Dcap + dst] = a[j];
-            born[(size_t)bl * Dcap + dst] = bs[j];
+    block_exclusive_scan<NT>(ds, n, tmp);
+    for (int j = tid; j < n; j += NT)
+        if (kf[j]) kp[ds[j]] = j;
+    if (p.ranks > 1) cluster_wait();               // all CTAs have read acc and born
+    __syncthreads();
+    if (rank == 0)
+        for (int j = tid; j < p.k; j += NT) {
+            p.acc[(size_t)bl * p.Dcap + j] = a[kp[j]];
+            p.born[(size_t)bl * p.Dcap + j] = bs[kp[j]];
         }
-    }
-}
-
-// In-place compaction of the decode K or V rows of one (b, l, kv head): row j <- row keep_pos[j].
-// keep_pos is ascending with keep_pos[j] >= j, so a pass that first loads 256/VPR source rows and
-// then, after a barrier, stores them at rows [c, c+256/VPR) never overwrites a later source.
-template <int D>
-__global__ void __launch_bounds__(256) decode_compact_kernel(__nv_bfloat16* Kd, __nv_bfloat16* Vd,
-                                                            const int* __restrict__ keep_pos, int Hkv, int Dcap,
-                                                            int k) {
-    constexpr int VPR = D / 8;
-    constexpr int ROWS = 256 / VPR;
-    const int u = blockIdx.x;
-    const int bl = u / Hkv;
-    uint4* X = reinterpret_cast<uint4*>((blockIdx.y == 0 ? Kd : Vd) + (size_t)u * Dcap * D);
-    const int* kp = keep_pos + (size_t)bl * Dcap;
-    const int row_in = threadIdx.x / VPR, v = threadIdx.x % VPR;
-    for (int c = 0; c < k; c += ROWS) {
-        const int j = c + row_in;
-        uint4 val = make_uint4(0, 0, 0, 0);
-        const bool ok = j < k;
-        if (ok) val = X[(size_t)kp[j] * VPR + v];
-        __syncthreads();
-        if (ok) X[(size_t)j * VPR + v] = val;
-        __syncthreads();
+    const int row_in = tid / VPR, vec = tid % VPR;
+    for (int h = rank; h < p.Hkv; h += p.ranks) {
+        uint4* Ku = reinterpret_cast<uint4*>(p.Kd + ((size_t)bl * p.Hkv + h) * p.Dcap * D);
+        uint4* Vu = reinterpret_cast<uint4*>(p.Vd + ((size_t)bl * p.Hkv + h) * p.Dcap * D);
+        for (int c = first_gone; c < p.k; c += RPP * Q) {      // the rows before the first evicted entry stay
+            uint4 kk[Q], vv[Q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int j = c + q * RPP + row_in;
+                kk[q] = vv[q] = make_uint4(0, 0, 0, 0);
+                if (j < p.k) {
+                    const size_t at = (size_t)kp[j] * VPR + vec;
+                    kk[q] = Ku[at];
+                    vv[q] = Vu[at];
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int j = c + q * RPP + row_in;
+                if (j < p.k) {
+                    Ku[(size_t)j * VPR + vec] = kk[q];
+                    Vu[(size_t)j * VPR + vec] = vv[q];
+                }
+            }
+            __syncthreads();
+        }
     }
 }
 

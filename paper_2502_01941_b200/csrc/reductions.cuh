@@ -120,21 +120,6 @@ __host__ __device__ constexpr size_t reduce_smem_bytes(int Rpad, int P, int S, i
     return bounds_smem_bytes(S) + ranks * ((size_t)(S + 3) / 4 * 4 * 4) + (work > select ? work : select);
 }
 
-__device__ __forceinline__ void cluster_arrive() {
-    __syncwarp();
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait() {
-    __syncwarp();
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// Stores to the first CTA of the cluster: `p` is the address of the same variable in this CTA.
-__device__ __forceinline__ void store_to_leader(float* p, float v) {
-    uint32_t a;
-    asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(a) : "r"(smem_u32(p)));
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
-}
-
 template <int ROWS>
 __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const PartialView v, const __grid_constant__ ShotTable tab,
                                                                       int R, int Hkv, int ranks,
@@ -272,7 +257,7 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
     if (ranks > 1) {
         cluster_wait();                            // (1) the leader has begun
         if (rank != 0)
-            for (int i = tid; i < S; i += kReduceThreads) store_to_leader(mass + i, mass[i]);
+            for (int i = tid; i < S; i += kReduceThreads) cluster_store(mass + i, 0, mass[i]);
         cluster_arrive();                          // (2) this CTA's masses are with the leader
     }
     if (rank == 0) {

@@ -59,10 +59,19 @@ __host__ __device__ constexpr int select_sort_size(int S) {
     while (n < S) n *= 2;
     return n;
 }
-// Shared memory of select_body, in bytes: scores and ranking, or sort keys; lengths; destinations.
+// Shared memory of rank_all for n values, and of select_body for S shots, in bytes (multiples of 16).
+__host__ __device__ constexpr size_t rank_smem_bytes(int n) {
+    return n <= kRankByCount ? (size_t)(n + 3) / 4 * 4 * 4 : (size_t)select_sort_size(n) * 8;
+}
 __host__ __device__ constexpr size_t select_smem_bytes(int S) {
-    const size_t s4 = (size_t)(S + 3) / 4 * 4;
-    return (S <= kRankByCount ? 2 * s4 * 4 : (size_t)select_sort_size(S) * 8) + 2 * s4 * 4 + 128;
+    return rank_smem_bytes(S) + 2 * ((size_t)(S + 3) / 4 * 4 * 4) + 128;
+}
+
+// Sort key of (value descending, index ascending); v is not NaN.
+__device__ __forceinline__ unsigned long long rank_key(float v, int i) {
+    const unsigned b = __float_as_uint(v + 0.f);                            // -0 and +0 are equal
+    const unsigned up = b & 0x80000000u ? ~b : b | 0x80000000u;             // ascending with the value
+    return (unsigned long long)~up << 32 | (unsigned)i;
 }
 
 // Bitonic sort of n = a power of two >= 64 keys in shared memory, ascending, by the NT threads of a
@@ -102,6 +111,49 @@ __device__ __forceinline__ void block_sort(unsigned long long* key, int n) {
     }
 }
 
+// Ranks n values by (value descending, index ascending), NaN last: emit(rank, i) is called once for
+// every i, by some thread of the CTA; value(i) is asked for once, by one thread.  NT threads (at least
+// n of them where values are ranked by counting), all of which call; `sm` rank_smem_bytes(n) bytes,
+// 16-byte aligned.  The caller puts the barrier behind it.
+template <int NT, class Value, class Emit>
+__device__ __forceinline__ void rank_all(int n, unsigned char* sm, Value&& value, Emit&& emit) {
+    const int tid = threadIdx.x;
+    if (n <= kRankByCount) {
+        float* sc = reinterpret_cast<float*>(sm);
+        if (tid < (n + 3) / 4 * 4) {
+            const float v = tid < n ? value(tid) : SHOTKV_NEG_INF;
+            sc[tid] = v == v ? v : SHOTKV_NEG_INF;     // a NaN ranks last instead of breaking the total order
+        }
+        __syncthreads();
+        if (tid < n) {
+            const float v = sc[tid];
+            int rank = 0;
+            for (int j = 0; j < n; j += 4) {           // the padding behind the last value never counts: -inf, larger index
+                const float4 w = *reinterpret_cast<const float4*>(sc + j);
+                rank += (w.x > v) || (w.x == v && j < tid);
+                rank += (w.y > v) || (w.y == v && j + 1 < tid);
+                rank += (w.z > v) || (w.z == v && j + 2 < tid);
+                rank += (w.w > v) || (w.w == v && j + 3 < tid);
+            }
+            emit(rank, tid);
+        }
+    } else {
+        unsigned long long* key = reinterpret_cast<unsigned long long*>(sm);
+        const int ns = select_sort_size(n);
+        for (int i = tid; i < ns; i += NT) {
+            unsigned long long k = ~0ull;
+            if (i < n) {
+                const float v = value(i);
+                k = rank_key(v == v ? v : SHOTKV_NEG_INF, i);
+            }
+            key[i] = k;
+        }
+        __syncthreads();
+        block_sort<NT>(key, ns);
+        for (int r = tid; r < n; r += NT) emit(r, (int)(unsigned)key[r]);
+    }
+}
+
 // Ranks the S shots by (score descending, index ascending), keeps whole shots while they fit the
 // budget left after the always-kept tokens, and writes the kept token positions in ascending order.
 //   mode 0: the longest prefix of the ranking that fits;  mode 1: every shot that still fits.
@@ -112,62 +164,23 @@ __device__ __forceinline__ void block_sort(unsigned long long* key, int n) {
 template <int NT, class Score>
 __device__ __forceinline__ void select_body(const SelectArgs& a, int bl, const int* o, unsigned char* sm, Score&& score) {
     const int S = a.S, s4 = (S + 3) / 4 * 4, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const bool counted = S <= kRankByCount;
-    const int nsort = counted ? 0 : select_sort_size(S);
-    float* sc = reinterpret_cast<float*>(sm);                               // counted: scores
-    int* order = reinterpret_cast<int*>(sm) + s4;                           // counted: rank -> shot
-    unsigned long long* key = reinterpret_cast<unsigned long long*>(sm);    // sorted: (score descending, shot)
-    int* cum = reinterpret_cast<int*>(sm + (counted ? 2 * (size_t)s4 * 4 : (size_t)nsort * 8));   // rank -> length, then scanned
-    int* kl = cum + s4;                                                     // shot -> kept length, then destination
-    int* tmp = kl + s4;
+    int* order = reinterpret_cast<int*>(sm + rank_smem_bytes(S));           // rank -> shot
+    int* cum = order + s4;                                                  // rank -> length, then scanned
+    int* kl = reinterpret_cast<int*>(sm);                                   // shot -> kept length, then destination (once ranked)
+    int* tmp = cum + s4;
     const int pre = o[0], qst = o[S];
     const int always = pre + (a.N - qst);
     const int shot_budget = a.budget_tokens - always;
 
-    if (counted) {
-        if (tid < s4) {
-            const float v = tid < S ? score(tid) : SHOTKV_NEG_INF;
-            sc[tid] = v == v ? v : SHOTKV_NEG_INF;     // a NaN score ranks last instead of breaking the total order
-        }
-        __syncthreads();
-        if (tid < S) {
-            const float v = sc[tid];
-            int rank = 0;
-            for (int j = 0; j < S; j += 4) {           // the padding behind the last shot never counts: -inf, larger index
-                const float4 w = *reinterpret_cast<const float4*>(sc + j);
-                rank += (w.x > v) || (w.x == v && j < tid);
-                rank += (w.y > v) || (w.y == v && j + 1 < tid);
-                rank += (w.z > v) || (w.z == v && j + 2 < tid);
-                rank += (w.w > v) || (w.w == v && j + 3 < tid);
-            }
-            order[rank] = tid;
-            cum[rank] = o[tid + 1] - o[tid];
-        }
-    } else {
-        for (int i = tid; i < nsort; i += NT) {
-            unsigned long long k = ~0ull;
-            if (i < S) {
-                float v = score(i);
-                v = (v == v ? v : SHOTKV_NEG_INF) + 0.f;                    // NaN last; -0 and +0 are equal
-                const unsigned b = __float_as_uint(v);
-                const unsigned up = b & 0x80000000u ? ~b : b | 0x80000000u;  // ascending with the score
-                k = (unsigned long long)~up << 32 | (unsigned)i;
-            }
-            key[i] = k;
-        }
-        __syncthreads();
-        block_sort<NT>(key, nsort);
-        for (int r = tid; r < S; r += NT) {
-            const int i = (int)(unsigned)key[r];
-            cum[r] = o[i + 1] - o[i];
-        }
-    }
+    rank_all<NT>(S, sm, score, [&](int rank, int i) {
+        order[rank] = i;
+        cum[rank] = o[i + 1] - o[i];
+    });
     __syncthreads();
-    auto shot_at = [&](int r) { return counted ? order[r] : (int)(unsigned)key[r]; };
     if (a.mode == 0) {
         block_exclusive_scan<NT>(cum, S, tmp);
         for (int r = tid; r < S; r += NT) {
-            const int i = shot_at(r);
+            const int i = order[r];
             const int len = o[i + 1] - o[i];
             kl[i] = (cum[r] + len <= shot_budget) ? len : 0;
         }
@@ -186,7 +199,7 @@ __device__ __forceinline__ void select_body(const SelectArgs& a, int bl, const i
                 ahead = f == 31 ? 0u : ~0u << (f + 1);
                 left -= __shfl_sync(0xffffffffu, len, f);
             }
-            if (r < S) kl[shot_at(r)] = (kept >> lane) & 1u ? len : 0;
+            if (r < S) kl[order[r]] = (kept >> lane) & 1u ? len : 0;
         }
     }
     __syncthreads();

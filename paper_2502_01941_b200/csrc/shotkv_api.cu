@@ -12,6 +12,7 @@
 #include <cstring>
 #include <functional>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "colsum_tc.cuh"
@@ -109,6 +110,35 @@ int fail(shotkv_ctx* ctx, int code, const char* fmt, ...) {
         (ctx)->launches += 1;                \
         CUDA_TRY(ctx, cudaGetLastError());   \
     } while (0)
+
+// Launches `kernel` with thread-block clusters of `cluster` CTAs (1: none) and, with `early`, as a
+// programmatic dependent of what precedes it on the stream: it may begin before that has ended and
+// orders itself by grid_wait (common.cuh), so only a kernel that calls it may be launched so.
+template <class... P, class... A>
+int launch(shotkv_ctx* ctx, void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, int cluster, bool early,
+           A&&... args) {
+    cudaLaunchAttribute at[2] = {};
+    cudaLaunchConfig_t lc{};
+    lc.gridDim = grid;
+    lc.blockDim = dim3(threads);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = stream;
+    lc.attrs = at;
+    if (cluster > 1) {
+        at[lc.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        at[lc.numAttrs].val.clusterDim.x = cluster;
+        at[lc.numAttrs].val.clusterDim.y = at[lc.numAttrs].val.clusterDim.z = 1;
+        ++lc.numAttrs;
+    }
+    if (early) {
+        at[lc.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        at[lc.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+        ++lc.numAttrs;
+    }
+    CUDA_TRY(ctx, cudaLaunchKernelEx(&lc, kernel, std::forward<A>(args)...));
+    ctx->launches += 1;
+    return SHOTKV_OK;
+}
 
 // Records the next stage boundary of the current profiled call (no-op unless profiling is on).
 void prof_begin(shotkv_ctx* ctx) {
@@ -635,21 +665,10 @@ int run_reduce_select_t(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView
     // that two still fit an SM (one from about 4,000 shots on)
     int ranks = d->Hkv < kReduceCluster ? d->Hkv : kReduceCluster;
     while (ranks > 1 && reduce_smem_bytes(ROWS, pv.P, d->S, ranks) > kBigSmem / 2) ranks = (ranks + 1) / 2;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = ranks;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    cudaLaunchConfig_t lc{};
-    lc.gridDim = dim3(d->B * d->L * ranks);
-    lc.blockDim = dim3(kReduceThreads);
-    lc.dynamicSmemBytes = reduce_smem_bytes(ROWS, pv.P, d->S, ranks);
-    lc.stream = stream;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    if (lc.dynamicSmemBytes > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "too many shots for the single-pass path (S = %d)", d->S);
-    CUDA_TRY(ctx, cudaLaunchKernelEx(&lc, reduce_select_kernel<ROWS>, pv, tab, (d->H / d->Hkv) * d->W, (int)d->Hkv, ranks, shot_scores, sa));
-    ctx->launches += 1;
-    return SHOTKV_OK;
+    const size_t smem = reduce_smem_bytes(ROWS, pv.P, d->S, ranks);
+    if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "too many shots for the single-pass path (S = %d)", d->S);
+    return launch(ctx, reduce_select_kernel<ROWS>, dim3(d->B * d->L * ranks), kReduceThreads, smem, stream, ranks, false, pv, tab,
+                  (d->H / d->Hkv) * d->W, (int)d->Hkv, ranks, shot_scores, sa);
 }
 int run_reduce_select(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView& pv, const ShotTable& tab, float* shot_scores,
                       const SelectArgs& sa, cudaStream_t stream) {
@@ -695,9 +714,10 @@ cudaError_t set_kernel_attributes() {
     if (e == cudaSuccess) e = set_tc_attributes<64, 2>();
     const void* small[] = {(const void*)select_shots_kernel<kSelectThreads>, (const void*)select_shots_kernel<kSortThreads>,
                            (const void*)reduce_select_kernel<128>, (const void*)reduce_select_kernel<256>,
-                           (const void*)decode_score_kernel<128>, (const void*)decode_score_kernel<64>,
+                           (const void*)decode_score_kernel<128, true>, (const void*)decode_score_kernel<64, true>,
+                           (const void*)decode_score_kernel<128, false>, (const void*)decode_score_kernel<64, false>,
                            (const void*)decode_attend_kernel<128>, (const void*)decode_attend_kernel<64>,
-                           (const void*)decode_rank_kernel};
+                           (const void*)decode_evict_kernel<128>, (const void*)decode_evict_kernel<64>};
     for (const void* f : small)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kBigSmem);
     // the fused decode step wants three CTAs of ~74 KB each on an SM: ask for the largest shared-memory carve-out
@@ -1207,13 +1227,29 @@ int shotkv_decode_init(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv_po
 
 namespace {
 
+// CTAs that share a unit's keys: as many (a power of two) as still fit the GPU together, `per_sm` to an
+// SM, and leave every warp at least kMinSplitBlocks blocks of 16 keys.
+constexpr int kMinSplitBlocks = 2;
+int decode_split(const shotkv_ctx* ctx, long long U, long long keys, int warps, int per_sm) {
+    int n = 1;
+    while (n < kMaxSplit && U * n * 2 <= (long long)ctx->sm_count * per_sm && keys >= (long long)n * 2 * warps * 16 * kMinSplitBlocks) n *= 2;
+    return n;
+}
+
 template <int D>
-int launch_decode_attend(shotkv_ctx* ctx, const DecodeParams& p, int U, cudaStream_t stream) {
+int launch_decode_attend(shotkv_ctx* ctx, DecodeParams& p, int U, cudaStream_t stream) {
     using Cfg = AttendCfg<D>;
-    const size_t smem = ((size_t)8 * p.Dcap + Cfg::kWarps * 8 * 2 + 16) * 4 + Cfg::kRingBytes;
+    const size_t smem = ((size_t)8 * p.Dcap + Cfg::kWarps * 8 * 2 + 16 + kMaxSplit * 16) * 4 + Cfg::kRingBytes;
     if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "Dcap too large for the attention-output step");
-    decode_attend_kernel<D><<<U, Cfg::kWarps * 32, smem, stream>>>(p);
-    return SHOTKV_OK;
+    p.nsplit = decode_split(ctx, U, (long long)p.Mcap + p.n_old + 1, Cfg::kWarps, 3);
+    return launch(ctx, decode_attend_kernel<D>, dim3(U * p.nsplit), Cfg::kWarps * 32, smem, stream, p.nsplit, true, p);
+}
+template <int D>
+int launch_decode_score(shotkv_ctx* ctx, DecodeParams& p, int U, cudaStream_t stream) {
+    const size_t smem = ((size_t)8 * p.Dcap + 8 * 8 * 2 + 16 + kMaxSplit * 16) * 4;
+    p.nsplit = decode_split(ctx, U, (long long)p.Mcap + p.n_old + 1, 8, 4);
+    return p.nsplit > 1 ? launch(ctx, decode_score_kernel<D, true>, dim3(U * p.nsplit), 256, smem, stream, p.nsplit, true, p)
+                        : launch(ctx, decode_score_kernel<D, false>, dim3(U), 256, smem, stream, 1, true, p);
 }
 
 // One decode step; with `attn_out` the score kernel is the variant that also writes the attention output.
@@ -1229,57 +1265,45 @@ int decode_step_impl(shotkv_ctx* ctx, shotkv_decode_state* st, const shotkv_bf16
     cudaStream_t stream = (cudaStream_t)stream_;
     const shotkv_dims& d = st->dims;
     const int BL = d.B * d.L, U = BL * d.Hkv;
-    float* partial = (float*)st->ws;
-    int* keep_pos = (int*)((unsigned char*)st->ws + align_up((size_t)U * st->Dcap * 4));
 
     DecodeParams p{};
     p.q = (const __nv_bfloat16*)q; p.k_new = (const __nv_bfloat16*)k_new; p.v_new = (const __nv_bfloat16*)v_new;
     p.Kc = (const __nv_bfloat16*)Kc; p.kept_count = kept_count;
-    p.Kd = (__nv_bfloat16*)st->Kd; p.Vd = (__nv_bfloat16*)st->Vd; p.partial = partial;
+    p.Kd = (__nv_bfloat16*)st->Kd; p.Vd = (__nv_bfloat16*)st->Vd; p.partial = (float*)st->ws;
     p.H = d.H; p.Hkv = d.Hkv; p.G = d.H / d.Hkv; p.Mcap = st->Mcap; p.Dcap = st->Dcap; p.n_old = st->n_dec;
     p.scale_log2 = kLog2e / sqrtf((float)d.d);
     p.Vc = (const __nv_bfloat16*)Vc; p.out = attn_out;
-    const size_t smem = (size_t)8 * st->Dcap * 4 + (8 * 8 * 2 + 16) * 4;
     prof_begin(ctx);
     prof_mark(ctx, stream);
-    if (attn_out) {
-        rc = d.d == 128 ? launch_decode_attend<128>(ctx, p, U, stream) : launch_decode_attend<64>(ctx, p, U, stream);
-        if (rc) return rc;
-    } else if (d.d == 128) {
-        decode_score_kernel<128><<<U, 256, smem, stream>>>(p);
-    } else {
-        decode_score_kernel<64><<<U, 256, smem, stream>>>(p);
-    }
-    LAUNCH_CHECK(ctx);
+    if (attn_out) rc = d.d == 128 ? launch_decode_attend<128>(ctx, p, U, stream) : launch_decode_attend<64>(ctx, p, U, stream);
+    else rc = d.d == 128 ? launch_decode_score<128>(ctx, p, U, stream) : launch_decode_score<64>(ctx, p, U, stream);
+    if (rc) return rc;
     prof_mark(ctx, stream);
-    decode_accumulate_kernel<<<BL, 128, 0, stream>>>(partial, d.Hkv, st->Dcap, st->n_dec, st->T, st->acc, st->born);
-    LAUNCH_CHECK(ctx);
-    st->n_dec += 1;
-    st->T += 1;
-    if (st->T % st->policy.recompress_every == 0) {
-        const int n = st->n_dec;
-        int k = (int)std::floor((double)st->policy.r_d * (double)st->T);
+
+    DecodeFinishParams f{};
+    f.partial = p.partial; f.acc = st->acc; f.born = st->born; f.Kd = p.Kd; f.Vd = p.Vd;
+    f.Hkv = d.Hkv; f.Dcap = st->Dcap; f.n = st->n_dec + 1; f.T_old = st->T;
+    const int T = st->T + 1;
+    f.k = f.n;
+    if (T % st->policy.recompress_every == 0) {
+        f.k = (int)std::floor((double)st->policy.r_d * (double)T);
         // entries of the last protect_recent steps are all still present (they were protected at every
         // earlier eviction too) and are kept whatever their score; the others share what is left of k
-        const int prot = st->policy.protect_recent < st->T ? st->policy.protect_recent : st->T;
-        if (k < prot) k = prot;
-        if (k > n) k = n;
-        if (k < n) {
-            const size_t rs = (size_t)n * 16 + (kSelectThreads + 1) * 4 + 16;
-            decode_rank_kernel<<<BL, kSelectThreads, rs, stream>>>(st->acc, st->born, st->Dcap, n, k,
-                                                                   prot > 0 ? st->T - prot : 0x7fffffff, keep_pos);
-            LAUNCH_CHECK(ctx);
-            if (k > 0) {
-                dim3 grid(U, 2);
-                if (d.d == 128)
-                    decode_compact_kernel<128><<<grid, 256, 0, stream>>>((__nv_bfloat16*)st->Kd, (__nv_bfloat16*)st->Vd, keep_pos, d.Hkv, st->Dcap, k);
-                else
-                    decode_compact_kernel<64><<<grid, 256, 0, stream>>>((__nv_bfloat16*)st->Kd, (__nv_bfloat16*)st->Vd, keep_pos, d.Hkv, st->Dcap, k);
-                LAUNCH_CHECK(ctx);
-            }
-            st->n_dec = k;
-        }
+        const int prot = st->policy.protect_recent < T ? st->policy.protect_recent : T;
+        if (f.k < prot) f.k = prot;
+        if (f.k > f.n) f.k = f.n;
+        f.protect_from = prot > 0 ? T - prot : 0x7fffffff;
     }
+    if (f.k < f.n) {
+        f.ranks = d.Hkv < kReduceCluster ? d.Hkv : kReduceCluster;
+        rc = d.d == 128 ? launch(ctx, decode_evict_kernel<128>, dim3(BL * f.ranks), kSelectThreads, decode_evict_smem_bytes(f.n), stream, f.ranks, true, f)
+                        : launch(ctx, decode_evict_kernel<64>, dim3(BL * f.ranks), kSelectThreads, decode_evict_smem_bytes(f.n), stream, f.ranks, true, f);
+    } else {
+        rc = launch(ctx, decode_accumulate_kernel, dim3(BL), 128, 0, stream, 1, true, f);
+    }
+    if (rc) return rc;
+    st->T = T;
+    st->n_dec = f.k;
     prof_mark(ctx, stream);
     return SHOTKV_OK;
 }

@@ -1,0 +1,32 @@
+"""Units shared by a cluster of CTAs and the fused end of an eviction cycle, against the oracle: one to
+eight CTAs to a unit, CTAs without a single key, heads that do not divide by the cluster, regions on
+both sides of the ranking by counting (256 entries) and by sorting."""
+import numpy as np
+import pytest
+
+import paper_2502_01941_b200 as skv
+from paper_2502_01941_b200 import workloads as wl
+from test_decode_gpu import lockstep
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    c = skv.Context(0)
+    yield c
+    c.close()
+
+
+@pytest.mark.parametrize("attend", [False, True], ids=["plain", "attend"])
+@pytest.mark.parametrize("Hkv,G,d,M,count", [(1, 4, 128, 2048, 2048), (1, 8, 64, 2047, 1), (2, 3, 128, 2049, 0), (2, 4, 64, 500, 400),
+                                             (8, 4, 128, 1100, 1023), (9, 1, 64, 700, 513), (96, 1, 64, 1500, 1400)])
+def test_unit_shared_by_a_cluster(ctx, Hkv, G, d, M, count, attend):
+    cfg = wl.DecodeConfig("split", B=1, L=1, H=Hkv * G, Hkv=Hkv, d=d, steps=14, r_d=0.5, recompress_every=4, cfg_id=71)
+    assert lockstep(ctx, cfg, M, [(0, 0)], np.full((1, 1), count, np.int32), attend=attend) <= 1
+
+
+@pytest.mark.parametrize("every", [255, 256, 257, 300, 530])
+def test_eviction_of_a_large_region(ctx, every):
+    cfg = wl.DecodeConfig("evict", B=1, L=1, H=4, Hkv=2, d=64, steps=every + 3, r_d=0.6, recompress_every=every, cfg_id=72)
+    assert lockstep(ctx, cfg, 40, [(0, 0)]) <= 2
