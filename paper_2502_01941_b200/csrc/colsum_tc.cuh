@@ -104,6 +104,7 @@ __global__ void __launch_bounds__(ColsumTcCfg<D, MB>::kThreads, 1)
     constexpr int TN = tc::kTileKeys, ROWS = Cfg::kRows, RG = ROWS / 2, NCH = RG / 32;
     const ScoreTcParams& p = cp.base;
     extern __shared__ unsigned char smem_raw[];
+    grid_release();
     tc::Pipe<Cfg> pp;
     tc::pipe_setup(pp, smem_raw, Cfg::kEpiWarps, 4 * 2 * 2, 2);     // extra barriers: [quad][slot][full, empty]
     float4* cst = reinterpret_cast<float4*>(tc::pipe_scratch(pp, smem_raw));    // [8 warps][RG / 2]
@@ -124,6 +125,7 @@ __global__ void __launch_bounds__(ColsumTcCfg<D, MB>::kThreads, 1)
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncthreads();
     }
+    grid_wait();
 
     if (warp == 0) {
         if (lane == 0) tc::producer_role<D, MB, false, true>(pp, &tmQ, &tmK, q_box_rows, k_box_rows, p, item_begin, item_end);

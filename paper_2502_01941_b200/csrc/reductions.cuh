@@ -70,6 +70,8 @@ __device__ __forceinline__ void row_stats_of(const PartialView& v, const int* o,
 // that the items' loads are in flight together (merged one by one: 4.8 and 6.4 us on 256 and 128 units).
 __global__ void row_stats_kernel(const PartialView v, int R, float* __restrict__ row_m, float* __restrict__ row_invz) {
     const int u = blockIdx.x, r = threadIdx.x;                  // one thread per padded row
+    grid_release();
+    grid_wait();
     bool any = false;
     for (int j = r; j < v.nchunk; j += blockDim.x) any |= item_is_exact(v, u * v.nchunk + j);
     any = __syncthreads_or(any);
@@ -143,6 +145,8 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
     const int bl = blockIdx.x / ranks, rank = blockIdx.x - bl * ranks;   // a cluster is the `ranks` CTAs of one (b, l)
     float* mass = masses + rank * s4;              // of this CTA's heads
 
+    grid_release();
+    if (tab.ptr) grid_wait();                      // boundaries among the launch parameters are there already
     copy_bounds(o, tab, bl / a.L, S);
     if (ranks > 1) cluster_arrive();               // (1) this CTA has begun: its shared memory may be written to
     __syncthreads();
@@ -152,6 +156,7 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
     __syncthreads();
     for (int j = warp; j < v.nchunk; j += NW)
         for (int q = range[j].x + lane; q <= range[j].y; q += 32) item_of[q] = (unsigned char)j;
+    grid_wait();
     const int q_first = range[0].x, q_count = range[v.nchunk - 1].y + 1 - q_first;
 
     for (int h = rank; h < Hkv; h += ranks) {
@@ -291,7 +296,9 @@ __global__ void __launch_bounds__(32 * kTokenWarps) shot_score_from_tokens_kerne
     constexpr int AHEAD = 8;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, bl = blockIdx.y;
     const int i = WPS == 1 ? blockIdx.x * kTokenWarps + warp : blockIdx.x;
+    grid_release();
     if (i >= S) return;
+    grid_wait();
     const int* o = table_row(tab, bl / L);
     const int lo = o[i], hi = o[i + 1];
     const float* base = imp + (size_t)bl * Hkv * N;

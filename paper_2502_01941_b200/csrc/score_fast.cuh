@@ -176,13 +176,15 @@ __global__ void __launch_bounds__(ScoreFastCfg<D>::kThreads, 1)
     constexpr int TN = tc::kTileKeys, MB = 1;
     constexpr int NSL = Cfg::kSlices, SLW = TN / NSL, NCH = SLW / 32, RD = Cfg::kRingDepth;
     extern __shared__ unsigned char smem_raw[];
-    tc::stamp(p.clk, 0);
+    grid_release();
     tc::Pipe<Cfg> pp;
     tc::pipe_setup(pp, smem_raw, Cfg::kEpiWarps, Cfg::kRings * Cfg::kRingDepth * 2, 2);
     float* comb = tc::pipe_scratch(pp, smem_raw);     // [ring][slot][lane][m, z]
     float4* mtab = reinterpret_cast<float4*>(reinterpret_cast<unsigned char*>(comb) + Cfg::kCombBytes);   // split masks
     tc::build_split_masks(mtab);
     __syncthreads();
+    grid_wait();
+    tc::stamp(p.clk, 0);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long total = p.total_items;

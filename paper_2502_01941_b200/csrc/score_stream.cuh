@@ -77,12 +77,14 @@ __global__ void __launch_bounds__(ScoreStreamCfg<D>::kThreads, 1)
     using Cfg = ScoreStreamCfg<D>;
     constexpr int TN = tc::kTileKeys, MB = 2;
     extern __shared__ unsigned char smem_raw[];
-    tc::stamp(p.clk, 0);
+    grid_release();
     tc::Pipe<Cfg> pp;
     tc::pipe_setup(pp, smem_raw, 4, 0, 2);
     float4* mtab = reinterpret_cast<float4*>(tc::pipe_scratch(pp, smem_raw));   // split masks
     tc::build_split_masks(mtab);
     __syncthreads();
+    grid_wait();
+    tc::stamp(p.clk, 0);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long total = p.total_items;

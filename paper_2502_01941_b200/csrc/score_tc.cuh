@@ -518,6 +518,8 @@ __global__ void __launch_bounds__(ScoreTcCfg<D, MB>::kThreads, 1)
     const long long total = p.total_items;
     const int item_begin = (int)(total * blockIdx.x / gridDim.x);
     const int item_end = (int)(total * (blockIdx.x + 1) / gridDim.x);
+    grid_release();
+    grid_wait();
     if (p.redo) {                                      // repair launch: nothing to repair in this CTA's items?
         bool any = false;
         for (int i = item_begin + threadIdx.x; i < item_end; i += blockDim.x) any |= p.redo[i] != 0;

@@ -237,6 +237,8 @@ __global__ void __launch_bounds__(NT) select_shots_kernel(const float* __restric
     extern __shared__ __align__(16) unsigned char sm[];
     const int bl = blockIdx.x;
     int* o = reinterpret_cast<int*>(sm);
+    grid_release();
+    grid_wait();
     copy_bounds(o, tab, bl / a.L, a.S);
     __syncthreads();
     const float* scores = shot_scores + (size_t)bl * a.S;
@@ -254,6 +256,8 @@ __global__ void __launch_bounds__(256) compact_kv_kernel(const uint4* __restrict
     constexpr int VPR = D / 8;                 // 16-byte vectors per row
     constexpr int ROWS = 256 / VPR * 4;        // rows per CTA per pass
     const int bl = blockIdx.z, h = blockIdx.y;
+    grid_release();
+    grid_wait();
     const int count = min(kept_count[bl], Mcap);
     const int row_in = threadIdx.x / VPR, v = threadIdx.x % VPR;
     const size_t u = (size_t)bl * Hkv + h;

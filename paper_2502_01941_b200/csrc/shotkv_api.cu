@@ -280,17 +280,20 @@ struct ChunkPlan { int nchunk, chunk_keys; };
 // Pieces a unit has room for: the piece of segment s in chunk j has index s + j (see score_tc.cuh).
 int pieces_of(int S, const ChunkPlan& plan) { return S + 1 + plan.nchunk; }
 ChunkPlan plan_chunks(const shotkv_dims* d, int sm_count) {
-    const long long U = (long long)d->B * d->L * d->Hkv;
-    const int tiles = (d->N + 127) / 128;
+    const int U = d->B * d->L * d->Hkv;                       // below 2^23 (check_dims): all of this fits 32 bits,
+    const int tiles = (d->N + 127) / 128;                     // whose divisions cost a third of the 64-bit ones
     ChunkPlan best{1, tiles * 128};
     long long best_cost = -1;
+    int last_ct = 0;
     for (int want = 1; want <= kMaxChunks && want <= tiles; ++want) {
         const int ct = (tiles + want - 1) / want;             // tiles per chunk
+        if (ct == last_ct) continue;                          // the same split as the one before
+        last_ct = ct;
         const int nchunk = (tiles + ct - 1) / ct;
-        const long long items = U * nchunk;
-        const long long ctas = items < sm_count ? items : sm_count;
-        const long long per_cta = (items + ctas - 1) / ctas;
-        const long long cost = per_cta * (ct * 16 + 3);       // a tile plus a small per-item overhead, in 1/16 tiles
+        const int items = U * nchunk;
+        const int ctas = items < sm_count ? items : sm_count;
+        const int per_cta = (items + ctas - 1) / ctas;
+        const long long cost = (long long)per_cta * (ct * 16 + 3);   // a tile plus a small per-item overhead, in 1/16 tiles
         if (best_cost < 0 || cost < best_cost) {
             best_cost = cost;
             best = ChunkPlan{nchunk, ct * 128};
@@ -403,9 +406,7 @@ int launch_score_tc_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorMap
     constexpr int smem = ScoreTcCfg<D, MB>::kSmemBytes;
     int grid = sp.total_items < ctx->sm_count ? sp.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    score_tc_kernel<D, MB><<<grid, ScoreTcCfg<D, MB>::kThreads, smem, stream>>>(tmQ, tmK, qbox, kbox, sp, tab);
-    LAUNCH_CHECK(ctx);
-    return SHOTKV_OK;
+    return launch(ctx, score_tc_kernel<D, MB>, dim3(grid), ScoreTcCfg<D, MB>::kThreads, smem, stream, 1, true, tmQ, tmK, qbox, kbox, sp, tab);
 }
 
 // Column pairs, of every 16, whose exponentials run on the FMA pipe instead of the special-function unit.
@@ -417,9 +418,7 @@ int launch_score_fast_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorM
     constexpr int smem = ScoreFastCfg<D>::kSmemBytes;
     int grid = sp.total_items < ctx->sm_count ? sp.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    score_fast_kernel<D, kPolyEvery><<<grid, ScoreFastCfg<D>::kThreads, smem, stream>>>(tmQ, tmK, qbox, kbox, sp, tab);
-    LAUNCH_CHECK(ctx);
-    return SHOTKV_OK;
+    return launch(ctx, score_fast_kernel<D, kPolyEvery>, dim3(grid), ScoreFastCfg<D>::kThreads, smem, stream, 1, true, tmQ, tmK, qbox, kbox, sp, tab);
 }
 
 template <int D>
@@ -428,9 +427,7 @@ int launch_score_stream_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtenso
     using Cfg = ScoreStreamCfg<D>;
     int grid = sp.total_items < ctx->sm_count ? sp.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    score_stream_kernel<D, kPolyEvery><<<grid, Cfg::kThreads, Cfg::kSmemBytes, stream>>>(tmQ, tmK, qbox, kbox, sp, tab);
-    LAUNCH_CHECK(ctx);
-    return SHOTKV_OK;
+    return launch(ctx, score_stream_kernel<D, kPolyEvery>, dim3(grid), Cfg::kThreads, Cfg::kSmemBytes, stream, 1, true, tmQ, tmK, qbox, kbox, sp, tab);
 }
 
 // Tensor maps of Q (2-D: d x rows) and K (3-D: d x N x units), 64-element boxes with 128-byte swizzle, and the
@@ -489,9 +486,7 @@ int launch_colsum_tc_t(shotkv_ctx* ctx, const TcSetup& t, const ColsumTcParams& 
     constexpr int smem = ColsumTcCfg<D, MB>::kSmemBytes;
     int grid = cp.base.total_items < ctx->sm_count ? cp.base.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    colsum_tc_kernel<D, MB, kPolyEvery><<<grid, ColsumTcCfg<D, MB>::kThreads, smem, stream>>>(t.tmQ, t.tmK, t.qbox, t.kbox, cp);
-    LAUNCH_CHECK(ctx);
-    return SHOTKV_OK;
+    return launch(ctx, colsum_tc_kernel<D, MB, kPolyEvery>, dim3(grid), ColsumTcCfg<D, MB>::kThreads, smem, stream, 1, true, t.tmQ, t.tmK, t.qbox, t.kbox, cp);
 }
 
 // Second pass of the per-token path: token_importance from the row statistics in the workspace.
@@ -568,9 +563,8 @@ int run_stats(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q, const
     const int rc = launch_score_tc(ctx, d, Q, K, w, -1, none, plan, stream);
     if (rc) return rc;
     prof_mark(ctx, stream);
-    row_stats_kernel<<<d->B * d->L * d->Hkv, rpad_of(d), 0, stream>>>(partial_view(ctx, d, w, -1, plan), (d->H / d->Hkv) * d->W, w.row_m, w.row_invz);
-    LAUNCH_CHECK(ctx);
-    return SHOTKV_OK;
+    return launch(ctx, row_stats_kernel, dim3(d->B * d->L * d->Hkv), rpad_of(d), 0, stream, 1, true, partial_view(ctx, d, w, -1, plan),
+                  (d->H / d->Hkv) * d->W, w.row_m, w.row_invz);
 }
 
 // ---- the fused call's pipeline over groups of units ---------------------------------------------
@@ -640,21 +634,19 @@ SelectArgs select_args(const shotkv_dims* d, const shotkv_policy* p, uint8_t* ke
 int run_select(shotkv_ctx* ctx, const shotkv_dims* d, const ShotTable& tab, const float* shot_scores, const SelectArgs& sa,
                cudaStream_t stream) {
     const size_t smem = bounds_smem_bytes(d->S) + select_smem_bytes(d->S);
-    if (d->S <= kRankByCount) select_shots_kernel<kSelectThreads><<<d->B * d->L, kSelectThreads, smem, stream>>>(shot_scores, tab, sa);
-    else select_shots_kernel<kSortThreads><<<d->B * d->L, kSortThreads, smem, stream>>>(shot_scores, tab, sa);
-    LAUNCH_CHECK(ctx);
-    return SHOTKV_OK;
+    return d->S <= kRankByCount
+               ? launch(ctx, select_shots_kernel<kSelectThreads>, dim3(d->B * d->L), kSelectThreads, smem, stream, 1, true, shot_scores, tab, sa)
+               : launch(ctx, select_shots_kernel<kSortThreads>, dim3(d->B * d->L), kSortThreads, smem, stream, 1, true, shot_scores, tab, sa);
 }
 
 // Per-shot scores from per-token importances.
 int run_token_scores(shotkv_ctx* ctx, const shotkv_dims* d, const float* imp, const ShotTable& tab, float* shot_scores, cudaStream_t stream) {
     const int bl = d->B * d->L;
-    if ((long long)d->N >= (long long)kLongShot * d->S)
-        shot_score_from_tokens_kernel<kTokenWarps><<<dim3(d->S, bl), 32 * kTokenWarps, 0, stream>>>(imp, tab, d->L, d->Hkv, d->N, d->S, shot_scores);
-    else
-        shot_score_from_tokens_kernel<1><<<dim3((d->S + kTokenWarps - 1) / kTokenWarps, bl), 32 * kTokenWarps, 0, stream>>>(imp, tab, d->L, d->Hkv, d->N, d->S, shot_scores);
-    LAUNCH_CHECK(ctx);
-    return SHOTKV_OK;
+    return (long long)d->N >= (long long)kLongShot * d->S
+               ? launch(ctx, shot_score_from_tokens_kernel<kTokenWarps>, dim3(d->S, bl), 32 * kTokenWarps, 0, stream, 1, true, imp, tab,
+                        (int)d->L, (int)d->Hkv, (int)d->N, (int)d->S, shot_scores)
+               : launch(ctx, shot_score_from_tokens_kernel<1>, dim3((d->S + kTokenWarps - 1) / kTokenWarps, bl), 32 * kTokenWarps, 0, stream,
+                        1, true, imp, tab, (int)d->L, (int)d->Hkv, (int)d->N, (int)d->S, shot_scores);
 }
 
 // Per-shot scores from the scoring pass's partials, and the selection.
@@ -667,7 +659,7 @@ int run_reduce_select_t(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView
     while (ranks > 1 && reduce_smem_bytes(ROWS, pv.P, d->S, ranks) > kBigSmem / 2) ranks = (ranks + 1) / 2;
     const size_t smem = reduce_smem_bytes(ROWS, pv.P, d->S, ranks);
     if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "too many shots for the single-pass path (S = %d)", d->S);
-    return launch(ctx, reduce_select_kernel<ROWS>, dim3(d->B * d->L * ranks), kReduceThreads, smem, stream, ranks, false, pv, tab,
+    return launch(ctx, reduce_select_kernel<ROWS>, dim3(d->B * d->L * ranks), kReduceThreads, smem, stream, ranks, true, pv, tab,
                   (d->H / d->Hkv) * d->W, (int)d->Hkv, ranks, shot_scores, sa);
 }
 int run_reduce_select(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView& pv, const ShotTable& tab, float* shot_scores,
@@ -684,12 +676,11 @@ int run_compact(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* K, con
     if (gx < 1) gx = 1;
     dim3 grid(gx, d->Hkv, d->B * d->L);
     if (grid.z > 65535) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "B*L must be <= 65535");
-    if (d->d == 128)
-        compact_kv_kernel<128><<<grid, 256, 0, stream>>>((const uint4*)K, (const uint4*)V, kept_idx, kept_count, d->Hkv, d->N, Mcap, (uint4*)Kc, (uint4*)Vc);
-    else
-        compact_kv_kernel<64><<<grid, 256, 0, stream>>>((const uint4*)K, (const uint4*)V, kept_idx, kept_count, d->Hkv, d->N, Mcap, (uint4*)Kc, (uint4*)Vc);
-    LAUNCH_CHECK(ctx);
-    return SHOTKV_OK;
+    // begun early only where one wave of CTAs does all of it: with more, the waiting CTAs gained nothing and
+    // 4 x 32 layers of 32K lost 2 % (3,590 us a call against 3,525)
+    const bool early = (long long)grid.x * grid.y * grid.z <= 8LL * ctx->sm_count;
+    return launch(ctx, d->d == 128 ? compact_kv_kernel<128> : compact_kv_kernel<64>, grid, 256, 0, stream, 1, early, (const uint4*)K, (const uint4*)V,
+                  kept_idx, kept_count, (int)d->Hkv, (int)d->N, (int)Mcap, (uint4*)Kc, (uint4*)Vc);
 }
 
 // Dynamic shared-memory limits of every kernel that may need more than the 48 KB default.  A
