@@ -114,31 +114,70 @@ def lib() -> C.CDLL:
 
 
 # ------------------------------------------------------------------ marshalling helpers
-def _ptr(t, *, device=None, dtype=None, name="tensor"):
-    if t is None:
-        return None
+# A call on a small layer is a few launches of two microseconds each, so what happens here counts: the
+# checks below are one attribute each, pointers go to ctypes as plain ints, and the current stream is
+# asked for by its handle.
+def _bad(t, dtype, cuda, name):
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name}: expected a torch tensor")
     if not t.is_contiguous():
         raise ValueError(f"{name}: must be contiguous")
     if dtype is not None and t.dtype != dtype:
         raise TypeError(f"{name}: expected {dtype}, got {t.dtype}")
-    if device == "cuda" and not t.is_cuda:
+    if cuda:
         raise ValueError(f"{name}: must be a CUDA tensor")
-    if device == "cpu" and t.is_cuda:
-        raise ValueError(f"{name}: must be a host tensor")
-    return C.c_void_p(t.data_ptr())
+    raise ValueError(f"{name}: must be a host tensor")
+
+
+def _dev(t, dtype, name):
+    """Address of a contiguous CUDA tensor of `dtype`; None stays None."""
+    if t is None:
+        return None
+    if isinstance(t, torch.Tensor) and t.dtype is dtype and t.is_cuda and t.is_contiguous():
+        return t.data_ptr()
+    _bad(t, dtype, True, name)
+
+
+def _host(t, dtype, name):
+    """Address of a contiguous host tensor of `dtype`; None stays None."""
+    if t is None:
+        return None
+    if isinstance(t, torch.Tensor) and t.dtype is dtype and not t.is_cuda and t.is_contiguous():
+        return t.data_ptr()
+    _bad(t, dtype, False, name)
+
+
+def _raw(t, name):
+    """Address and bytes of a contiguous CUDA tensor of any type (workspaces)."""
+    if isinstance(t, torch.Tensor) and t.is_cuda and t.is_contiguous():
+        return t.data_ptr(), t.nbytes
+    _bad(t, None, True, name)
 
 
 def _offsets(off) -> np.ndarray:
-    a = np.ascontiguousarray(off.cpu().numpy() if isinstance(off, torch.Tensor) else off, dtype=np.int32)
-    return a
+    if type(off) is np.ndarray and off.dtype == np.int32 and off.flags.c_contiguous:
+        return off
+    return np.ascontiguousarray(off.cpu().numpy() if isinstance(off, torch.Tensor) else off, dtype=np.int32)
 
 
-def _stream(stream) -> C.c_void_p:
+def _stream(stream):
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
+        return _current_stream()
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
+
+
+def _current_stream() -> int:
+    """Handle of torch's current stream on the current device."""
+    if _raw_stream is not None and torch.cuda.is_initialized():
+        return _raw_stream(_raw_device())
+    return torch.cuda.current_stream().cuda_stream
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+_raw_device = getattr(torch._C, "_cuda_getDevice", None)
+if _raw_device is None:
+    _raw_stream = None
+_BF16, _F32, _I32, _U8 = torch.bfloat16, torch.float32, torch.int32, torch.uint8
 
 
 def make_dims(B, L, H, Hkv, d, N, W, S) -> Dims:
@@ -195,13 +234,13 @@ def shotkv_budget_tokens(dims: Dims, policy: Policy) -> int:
 
 def shotkv_kept_capacity(dims: Dims, policy: Policy, offsets) -> int:
     o = _offsets(offsets)
-    return int(lib().shotkv_kept_capacity(C.byref(dims), C.byref(policy), o.ctypes.data_as(C.c_void_p)))
+    return int(lib().shotkv_kept_capacity(C.byref(dims), C.byref(policy), o.ctypes.data))
 
 
 def shotkv_validate(dims: Dims, policy: Policy | None = None, offsets=None) -> int:
     o = _offsets(offsets) if offsets is not None else None
     return int(lib().shotkv_validate(C.byref(dims), C.byref(policy) if policy is not None else None,
-                                     o.ctypes.data_as(C.c_void_p) if o is not None else None))
+                                     o.ctypes.data if o is not None else None))
 
 
 def shotkv_workspace_bytes(dims: Dims) -> int:
@@ -209,10 +248,10 @@ def shotkv_workspace_bytes(dims: Dims) -> int:
 
 
 def shotkv_prefill_score(ctx: Context, dims: Dims, Qwin, K, token_importance, ws, stream=None) -> int:
-    rc = lib().shotkv_prefill_score(ctx._h, C.byref(dims), _ptr(Qwin, device="cuda", dtype=torch.bfloat16, name="Qwin"),
-                                    _ptr(K, device="cuda", dtype=torch.bfloat16, name="K"),
-                                    _ptr(token_importance, device="cuda", dtype=torch.float32, name="token_importance"),
-                                    _ptr(ws, device="cuda", name="ws"), ws.numel() * ws.element_size(), _stream(stream))
+    rc = lib().shotkv_prefill_score(ctx._h, C.byref(dims), _dev(Qwin, _BF16, "Qwin"),
+                                    _dev(K, _BF16, "K"),
+                                    _dev(token_importance, _F32, "token_importance"),
+                                    *_raw(ws, "ws"), _stream(stream))
     return ctx.check(rc)
 
 
@@ -220,13 +259,13 @@ def shotkv_select_shots(ctx: Context, dims: Dims, policy: Policy, token_importan
                         kept_idx, kept_count, Mcap: int, ws, stream=None) -> int:
     o = _offsets(offsets)
     rc = lib().shotkv_select_shots(ctx._h, C.byref(dims), C.byref(policy),
-                                   _ptr(token_importance, device="cuda", dtype=torch.float32, name="token_importance"),
-                                   o.ctypes.data_as(C.c_void_p),
-                                   _ptr(shot_scores, device="cuda", dtype=torch.float32, name="shot_scores"),
-                                   _ptr(keep, device="cuda", dtype=torch.uint8, name="keep"),
-                                   _ptr(kept_idx, device="cuda", dtype=torch.int32, name="kept_idx"),
-                                   _ptr(kept_count, device="cuda", dtype=torch.int32, name="kept_count"),
-                                   int(Mcap), _ptr(ws, device="cuda", name="ws"), ws.numel() * ws.element_size(),
+                                   _dev(token_importance, _F32, "token_importance"),
+                                   o.ctypes.data,
+                                   _dev(shot_scores, _F32, "shot_scores"),
+                                   _dev(keep, _U8, "keep"),
+                                   _dev(kept_idx, _I32, "kept_idx"),
+                                   _dev(kept_count, _I32, "kept_count"),
+                                   int(Mcap), *_raw(ws, "ws"),
                                    _stream(stream))
     return ctx.check(rc)
 
@@ -238,23 +277,23 @@ def shotkv_select_shots_static(ctx: Context, dims: Dims, policy: Policy, token_i
     B*(S+1) <= 65536).  Calls on one device must not overlap on the GPU."""
     o = _offsets(offsets)
     rc = lib().shotkv_select_shots_static(ctx._h, C.byref(dims), C.byref(policy),
-                                          _ptr(token_importance, device="cuda", dtype=torch.float32, name="token_importance"),
-                                          o.ctypes.data_as(C.c_void_p),
-                                          _ptr(shot_scores, device="cuda", dtype=torch.float32, name="shot_scores"),
-                                          _ptr(keep, device="cuda", dtype=torch.uint8, name="keep"),
-                                          _ptr(kept_idx, device="cuda", dtype=torch.int32, name="kept_idx"),
-                                          _ptr(kept_count, device="cuda", dtype=torch.int32, name="kept_count"),
+                                          _dev(token_importance, _F32, "token_importance"),
+                                          o.ctypes.data,
+                                          _dev(shot_scores, _F32, "shot_scores"),
+                                          _dev(keep, _U8, "keep"),
+                                          _dev(kept_idx, _I32, "kept_idx"),
+                                          _dev(kept_count, _I32, "kept_count"),
                                           int(Mcap), _stream(stream))
     return ctx.check(rc)
 
 
 def shotkv_compact_kv(ctx: Context, dims: Dims, K, V, kept_idx, kept_count, Mcap: int, Kc, Vc, stream=None) -> int:
-    rc = lib().shotkv_compact_kv(ctx._h, C.byref(dims), _ptr(K, device="cuda", dtype=torch.bfloat16, name="K"),
-                                 _ptr(V, device="cuda", dtype=torch.bfloat16, name="V"),
-                                 _ptr(kept_idx, device="cuda", dtype=torch.int32, name="kept_idx"),
-                                 _ptr(kept_count, device="cuda", dtype=torch.int32, name="kept_count"), int(Mcap),
-                                 _ptr(Kc, device="cuda", dtype=torch.bfloat16, name="Kc"),
-                                 _ptr(Vc, device="cuda", dtype=torch.bfloat16, name="Vc"), _stream(stream))
+    rc = lib().shotkv_compact_kv(ctx._h, C.byref(dims), _dev(K, _BF16, "K"),
+                                 _dev(V, _BF16, "V"),
+                                 _dev(kept_idx, _I32, "kept_idx"),
+                                 _dev(kept_count, _I32, "kept_count"), int(Mcap),
+                                 _dev(Kc, _BF16, "Kc"),
+                                 _dev(Vc, _BF16, "Vc"), _stream(stream))
     return ctx.check(rc)
 
 
@@ -264,15 +303,15 @@ def shotkv_prefill_compress(ctx: Context, dims: Dims, policy: Policy, Qwin, K, V
     o = _offsets(offsets)
     rc = lib().shotkv_prefill_compress(
         ctx._h, C.byref(dims), C.byref(policy),
-        _ptr(Qwin, device="cuda", dtype=torch.bfloat16, name="Qwin"), _ptr(K, device="cuda", dtype=torch.bfloat16, name="K"),
-        _ptr(V, device="cuda", dtype=torch.bfloat16, name="V"), o.ctypes.data_as(C.c_void_p),
-        _ptr(shot_scores, device="cuda", dtype=torch.float32, name="shot_scores"),
-        _ptr(keep, device="cuda", dtype=torch.uint8, name="keep"),
-        _ptr(kept_idx, device="cuda", dtype=torch.int32, name="kept_idx"),
-        _ptr(kept_count, device="cuda", dtype=torch.int32, name="kept_count"), int(Mcap),
-        _ptr(Kc, device="cuda", dtype=torch.bfloat16, name="Kc"), _ptr(Vc, device="cuda", dtype=torch.bfloat16, name="Vc"),
-        _ptr(token_importance, device="cuda", dtype=torch.float32, name="token_importance"), int(flags),
-        _ptr(ws, device="cuda", name="ws"), ws.numel() * ws.element_size(), _stream(stream))
+        _dev(Qwin, _BF16, "Qwin"), _dev(K, _BF16, "K"),
+        _dev(V, _BF16, "V"), o.ctypes.data,
+        _dev(shot_scores, _F32, "shot_scores"),
+        _dev(keep, _U8, "keep"),
+        _dev(kept_idx, _I32, "kept_idx"),
+        _dev(kept_count, _I32, "kept_count"), int(Mcap),
+        _dev(Kc, _BF16, "Kc"), _dev(Vc, _BF16, "Vc"),
+        _dev(token_importance, _F32, "token_importance"), int(flags),
+        *_raw(ws, "ws"), _stream(stream))
     return ctx.check(rc)
 
 
@@ -286,16 +325,16 @@ def shotkv_prefill_compress_host(ctx: Context, dims: Dims, policy: Policy, Qwin_
     o = _offsets(offsets)
     rc = lib().shotkv_prefill_compress_host(
         ctx._h, C.byref(dims), C.byref(policy),
-        _ptr(Qwin_host, device="cpu", dtype=torch.bfloat16, name="Qwin_host"),
-        _ptr(K_host, device="cpu", dtype=torch.bfloat16, name="K_host"),
-        _ptr(V_host, device="cpu", dtype=torch.bfloat16, name="V_host"), o.ctypes.data_as(C.c_void_p),
-        _ptr(shot_scores_host, device="cpu", dtype=torch.float32, name="shot_scores_host"),
-        _ptr(keep_host, device="cpu", dtype=torch.uint8, name="keep_host"),
-        _ptr(kept_idx_host, device="cpu", dtype=torch.int32, name="kept_idx_host"),
-        _ptr(kept_count_host, device="cpu", dtype=torch.int32, name="kept_count_host"), int(Mcap),
-        _ptr(Kc_host, device="cpu", dtype=torch.bfloat16, name="Kc_host"),
-        _ptr(Vc_host, device="cpu", dtype=torch.bfloat16, name="Vc_host"),
-        _ptr(arena, device="cuda", name="arena"), arena.numel() * arena.element_size(), _stream(stream))
+        _host(Qwin_host, _BF16, "Qwin_host"),
+        _host(K_host, _BF16, "K_host"),
+        _host(V_host, _BF16, "V_host"), o.ctypes.data,
+        _host(shot_scores_host, _F32, "shot_scores_host"),
+        _host(keep_host, _U8, "keep_host"),
+        _host(kept_idx_host, _I32, "kept_idx_host"),
+        _host(kept_count_host, _I32, "kept_count_host"), int(Mcap),
+        _host(Kc_host, _BF16, "Kc_host"),
+        _host(Vc_host, _BF16, "Vc_host"),
+        *_raw(arena, "arena"), _stream(stream))
     return ctx.check(rc)
 
 
@@ -310,34 +349,34 @@ def shotkv_decode_capacity(policy: Policy, steps: int) -> int:
 def shotkv_decode_init(ctx: Context, dims: Dims, policy: Policy, Dcap: int, Mcap: int, Kd, Vd, acc, born, ws) -> DecodeState:
     st = DecodeState()
     rc = lib().shotkv_decode_init(ctx._h, C.byref(dims), C.byref(policy), int(Dcap), int(Mcap),
-                                  _ptr(Kd, device="cuda", dtype=torch.bfloat16, name="Kd"),
-                                  _ptr(Vd, device="cuda", dtype=torch.bfloat16, name="Vd"),
-                                  _ptr(acc, device="cuda", dtype=torch.float32, name="acc"),
-                                  _ptr(born, device="cuda", dtype=torch.int32, name="born"),
-                                  _ptr(ws, device="cuda", name="ws"), ws.numel() * ws.element_size(), C.byref(st))
+                                  _dev(Kd, _BF16, "Kd"),
+                                  _dev(Vd, _BF16, "Vd"),
+                                  _dev(acc, _F32, "acc"),
+                                  _dev(born, _I32, "born"),
+                                  *_raw(ws, "ws"), C.byref(st))
     ctx.check(rc)
     st._keepalive = (Kd, Vd, acc, born, ws)
     return st
 
 
 def shotkv_decode_step(ctx: Context, state: DecodeState, q, k_new, v_new, Kc, kept_count, stream=None) -> int:
-    rc = lib().shotkv_decode_step(ctx._h, C.byref(state), _ptr(q, device="cuda", dtype=torch.bfloat16, name="q"),
-                                  _ptr(k_new, device="cuda", dtype=torch.bfloat16, name="k_new"),
-                                  _ptr(v_new, device="cuda", dtype=torch.bfloat16, name="v_new"),
-                                  _ptr(Kc, device="cuda", dtype=torch.bfloat16, name="Kc"),
-                                  _ptr(kept_count, device="cuda", dtype=torch.int32, name="kept_count"), _stream(stream))
+    rc = lib().shotkv_decode_step(ctx._h, C.byref(state), _dev(q, _BF16, "q"),
+                                  _dev(k_new, _BF16, "k_new"),
+                                  _dev(v_new, _BF16, "v_new"),
+                                  _dev(Kc, _BF16, "Kc"),
+                                  _dev(kept_count, _I32, "kept_count"), _stream(stream))
     return ctx.check(rc)
 
 
 def shotkv_decode_step_attend(ctx: Context, state: DecodeState, q, k_new, v_new, Kc, Vc, kept_count, attn_out,
                               stream=None) -> int:
-    rc = lib().shotkv_decode_step_attend(ctx._h, C.byref(state), _ptr(q, device="cuda", dtype=torch.bfloat16, name="q"),
-                                         _ptr(k_new, device="cuda", dtype=torch.bfloat16, name="k_new"),
-                                         _ptr(v_new, device="cuda", dtype=torch.bfloat16, name="v_new"),
-                                         _ptr(Kc, device="cuda", dtype=torch.bfloat16, name="Kc"),
-                                         _ptr(Vc, device="cuda", dtype=torch.bfloat16, name="Vc"),
-                                         _ptr(kept_count, device="cuda", dtype=torch.int32, name="kept_count"),
-                                         _ptr(attn_out, device="cuda", dtype=torch.float32, name="attn_out"), _stream(stream))
+    rc = lib().shotkv_decode_step_attend(ctx._h, C.byref(state), _dev(q, _BF16, "q"),
+                                         _dev(k_new, _BF16, "k_new"),
+                                         _dev(v_new, _BF16, "v_new"),
+                                         _dev(Kc, _BF16, "Kc"),
+                                         _dev(Vc, _BF16, "Vc"),
+                                         _dev(kept_count, _I32, "kept_count"),
+                                         _dev(attn_out, _F32, "attn_out"), _stream(stream))
     return ctx.check(rc)
 
 
@@ -347,7 +386,7 @@ def shotkv_plan_pieces(dims: Dims, offsets=None, sm_count: int = 148):
     cap = dims.S + 80
     out = np.zeros((dims.B, cap, 3), dtype=np.int32)
     nchunk, ck = C.c_int32(), C.c_int32()
-    P = int(lib().shotkv_plan_pieces(C.byref(dims), o.ctypes.data_as(C.c_void_p) if o is not None else None, int(sm_count),
+    P = int(lib().shotkv_plan_pieces(C.byref(dims), o.ctypes.data if o is not None else None, int(sm_count),
                                      C.byref(nchunk), C.byref(ck), out.ctypes.data_as(C.c_void_p), cap))
     if P < 0:
         raise ShotKVError(P, "shotkv_plan_pieces rejected its arguments")
