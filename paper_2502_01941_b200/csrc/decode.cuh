@@ -56,6 +56,7 @@ __device__ __forceinline__ void merge_stats(const float* table, int nsplit, int 
 // the group's (up to 8) query rows held in registers with the same k-index permutation.  The logits
 // of the decode entries are parked in shared memory until the softmax statistics over all keys
 // (kept prefill keys + decode keys) are known.
+// A shared unit leaves few warps to an SM, so each asks for its next block before it computes this one.
 // SPLIT = false is the same for whole units, nsplit = 1: with the stride of the loop a constant the
 // compiler unrolls it and keeps more loads in flight (8 sequences x 32 layers: 245 us a step against 273).
 template <int D, bool SPLIT>
@@ -98,23 +99,44 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p)
         for (int kb = 0; kb < NB; ++kb) qf[kb] = g < p.G ? qrow[kb * 4 + t4] : make_uint4(0, 0, 0, 0);
     }
 
-    float m0 = SHOTKV_NEG_INF, m1 = SHOTKV_NEG_INF, z0 = 0.f, z1 = 0.f;   // query rows 2*t4, 2*t4+1
-    for (int base = (rank * 8 + warp) * 16; base < Ktot; base += nsplit * 8 * 16) {
-        const int ia = base + g, ib = base + g + 8;
-        const bool va = ia < Ktot, vb = ib < Ktot;
-        auto row_ptr = [&](int i, bool valid) -> const uint4* {
-            if (!valid) return knew_u;                     // any readable row; the result is masked
-            if (i < M) return Kc_u + (size_t)i * VPR;
-            const int j = i - M;
-            return j == p.n_old ? knew_u : Kd_u + (size_t)j * VPR;
-        };
-        const uint4* pa = row_ptr(ia, va);
-        const uint4* pb = row_ptr(ib, vb);
-        uint4 a_lo[NB], a_hi[NB];
+    auto row_ptr = [&](int i, bool valid) -> const uint4* {
+        if (!valid) return knew_u;                         // any readable row; the result is masked
+        if (i < M) return Kc_u + (size_t)i * VPR;
+        const int j = i - M;
+        return j == p.n_old ? knew_u : Kd_u + (size_t)j * VPR;
+    };
+    // a block's 16 key rows: this lane's 16-byte pieces of rows base + g and base + 8 + g
+    uint4 a_lo[NB], a_hi[NB], n_lo[NB], n_hi[NB];          // this block and, where units are shared, the next
+    auto load = [&](int base, uint4 (&lo)[NB], uint4 (&hi)[NB]) {
+        const uint4 *pa, *pb;
+        if (SPLIT && base + 16 <= M) {                     // all of it kept prefill rows: one run of memory (whole
+            pa = Kc_u + (size_t)(base + g) * VPR;          // units: the branch would cost the unrolled loop 2.6 %)
+            pb = pa + 8 * VPR;
+        } else {
+            pa = row_ptr(base + g, base + g < Ktot);
+            pb = row_ptr(base + 8 + g, base + 8 + g < Ktot);
+        }
 #pragma unroll
         for (int kb = 0; kb < NB; ++kb) {
-            a_lo[kb] = pa[kb * 4 + t4];
-            a_hi[kb] = pb[kb * 4 + t4];
+            lo[kb] = pa[kb * 4 + t4];
+            hi[kb] = pb[kb * 4 + t4];
+        }
+    };
+    float m0 = SHOTKV_NEG_INF, m1 = SHOTKV_NEG_INF, z0 = 0.f, z1 = 0.f;   // query rows 2*t4, 2*t4+1
+    const int first = (rank * 8 + warp) * 16;
+    if (SPLIT && first < Ktot) load(first, n_lo, n_hi);
+    for (int base = first; base < Ktot; base += nsplit * 8 * 16) {
+        const int ia = base + g, ib = base + g + 8;
+        const bool va = ia < Ktot, vb = ib < Ktot;
+        if (SPLIT) {
+#pragma unroll
+            for (int kb = 0; kb < NB; ++kb) {
+                a_lo[kb] = n_lo[kb];
+                a_hi[kb] = n_hi[kb];
+            }
+            if (base + nsplit * 8 * 16 < Ktot) load(base + nsplit * 8 * 16, n_lo, n_hi);
+        } else {
+            load(base, a_lo, a_hi);
         }
         float c[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -200,6 +222,9 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p)
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int bytes) {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(bytes) : "memory");
 }
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
@@ -253,6 +278,11 @@ struct AttendCfg {
 // remainder: relative error 2^-17) in two MMAs per 16 dimensions, and ldmatrix.trans turns the
 // value rows into the A fragments of V^T.  Online softmax per warp with a running maximum per
 // query row (lanes that share g); the warps' (m, z, O) are merged at the end in warp order.
+// With few CTAs on an SM what bounds it is the chain of one block in one warp (0.7 us before, 0.5 now): the
+// copies of a block that is all prefill rows take their addresses from one pointer and immediate offsets,
+// masks and parked logits are left to the blocks that need them, and the first product runs as four chains
+// of MMAs.  32 steps of 8 sequences x 32 layers 16.25 -> 15.93 ms, a step of 4 sequences x 1 layer 17.0 -> 15.9 us,
+// one unit of 8,000 keys 20.0 -> 15.5 us.
 template <int D>
 __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_kernel(const DecodeParams p) {
     using Cfg = AttendCfg<D>;
@@ -301,10 +331,25 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     // this warp's ring.  A lane copies chunk (lane % VPR) of rows lane / VPR + k * (32 / VPR); rows
     // past the end are filled with zeros (a weight of zero must not meet a stray NaN).
     const uint32_t wring = smem_u32(ring) + (uint32_t)(warp * NS * Cfg::kStageBytes);
+    // offsets of this lane's first copies in a stage: row lane / VPR, chunk lane % VPR permuted as above (the
+    // row's low bits of later copies enter the values' permutation by exclusive or)
+    const uint32_t kdst = (uint32_t)((lane / VPR) * Cfg::kRowBytes + (((lane % VPR) ^ (((lane / VPR) & 1) << 2)) << 4));
+    const uint32_t vdst = (uint32_t)(Cfg::kTileBytes + (lane / VPR) * Cfg::kRowBytes + (((lane % VPR) ^ ((lane / VPR) & 7)) << 4));
     auto fetch_block = [&](int base, int stage) {
         constexpr int RPI = 32 / VPR;                       // rows per warp-wide copy
         const int c = lane % VPR;
         const uint32_t st = wring + (uint32_t)(stage * Cfg::kStageBytes);
+        if (base + 16 <= M) {                               // all of it kept prefill rows: one run of memory
+            const uint4* ks = Kc_u + (size_t)base * VPR + lane;
+            const uint4* vs = Vc_u + (size_t)base * VPR + lane;
+#pragma unroll
+            for (int k = 0; k < 16 / RPI; ++k) {
+                cp_async16(st + kdst + (uint32_t)(k * RPI * Cfg::kRowBytes), ks + k * 32);
+                cp_async16(st + (vdst ^ (uint32_t)(((k * RPI) & 7) << 4)) + (uint32_t)(k * RPI * Cfg::kRowBytes), vs + k * 32);
+            }
+            cp_async_commit();
+            return;
+        }
 #pragma unroll
         for (int k = 0; k < 16 / RPI; ++k) {
             const int rr = lane / VPR + k * RPI;
@@ -349,7 +394,8 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
         __syncwarp();
         const uint32_t st = wring + (uint32_t)(stage * Cfg::kStageBytes);
         // keys base+g and base+8+g as B fragments
-        float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};   // keys base+0..7 and base+8..15
+        // keys base+0..7 and base+8..15, each in two chains of MMAs so that none is longer than NB
+        float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f}, s2[4] = {0.f, 0.f, 0.f, 0.f}, s3[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int kb = 0; kb < NB; ++kb) {
             const uint32_t off = (uint32_t)(((kb * 4 + t4) ^ ((g & 1) << 2)) << 4);
@@ -359,22 +405,20 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
             const uint32_t a0[4] = {qf[kb].x, 0u, qf[kb].y, 0u};
             const uint32_t a1[4] = {qf[kb].z, 0u, qf[kb].w, 0u};
             mma_bf16_16816(s0, a0, ka.x, ka.y);
-            mma_bf16_16816(s0, a1, ka.z, ka.w);
             mma_bf16_16816(s1, a0, kb8.x, kb8.y);
-            mma_bf16_16816(s1, a1, kb8.z, kb8.w);
+            mma_bf16_16816(s2, a1, ka.z, ka.w);
+            mma_bf16_16816(s3, a1, kb8.z, kb8.w);
         }
         // this lane: row g, keys base + {2*t4, 2*t4+1, 8+2*t4, 9+2*t4}
         const int k0 = base + 2 * t4;
-        float x[4];
-        x[0] = k0 < Ktot ? s0[0] * p.scale_log2 : SHOTKV_NEG_INF;
-        x[1] = k0 + 1 < Ktot ? s0[1] * p.scale_log2 : SHOTKV_NEG_INF;
-        x[2] = k0 + 8 < Ktot ? s1[0] * p.scale_log2 : SHOTKV_NEG_INF;
-        x[3] = k0 + 9 < Ktot ? s1[1] * p.scale_log2 : SHOTKV_NEG_INF;
-        if (g < p.G) {
+        float x[4] = {(s0[0] + s2[0]) * p.scale_log2, (s0[1] + s2[1]) * p.scale_log2, (s1[0] + s3[0]) * p.scale_log2,
+                      (s1[1] + s3[1]) * p.scale_log2};
+        if (base + 16 > M) {                                // decode entries, or the end of the keys
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int key = k0 + (q & 1) + (q >> 1) * 8;
-                if (key >= M && key < Ktot) sdec[g * p.Dcap + (key - M)] = x[q];
+                if (key >= Ktot) x[q] = SHOTKV_NEG_INF;
+                else if (g < p.G && key >= M) sdec[g * p.Dcap + (key - M)] = x[q];
             }
         }
         float bm = fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3]));

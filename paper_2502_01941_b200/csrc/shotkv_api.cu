@@ -83,6 +83,8 @@ struct shotkv_ctx {
     long long wait_cycles = tc::kWaitCycles;   // limit of every bounded device-side wait
     int32_t* static_offsets = nullptr;         // device address of the built-in boundary table (looked up on first use)
     void* encode_tiled = nullptr;              // cuTensorMapEncodeTiled, resolved at creation
+    int room_attend[2][kMaxSplit + 1] = {};    // clusters of n CTAs the device runs at a time, d = 64 and 128 (asked at creation)
+    int room_score[2][kMaxSplit + 1] = {};
 };
 
 namespace {
@@ -683,6 +685,13 @@ int run_compact(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* K, con
                   kept_idx, kept_count, (int)d->Hkv, (int)d->N, (int)Mcap, (uint4*)Kc, (uint4*)Vc);
 }
 
+// Dynamic shared memory of the decode kernels for decode regions of Dcap rows.
+template <int D>
+size_t attend_smem(int Dcap) {
+    return ((size_t)8 * Dcap + AttendCfg<D>::kWarps * 8 * 2 + 16 + kMaxSplit * 16) * 4 + AttendCfg<D>::kRingBytes;
+}
+size_t score_smem(int Dcap) { return ((size_t)8 * Dcap + 8 * 8 * 2 + 16 + kMaxSplit * 16) * 4; }
+
 // Dynamic shared-memory limits of every kernel that may need more than the 48 KB default.  A
 // function attribute belongs to the device's context, so it is set once when a shotkv_ctx is
 // created on that device, never on a launch path.
@@ -715,6 +724,35 @@ cudaError_t set_kernel_attributes() {
     const void* wide[] = {(const void*)decode_attend_kernel<128>, (const void*)decode_attend_kernel<64>};
     for (const void* f : wide)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    return e;
+}
+
+// How many clusters of n decode CTAs the device runs at the same time, with decode regions of kRoomRows rows
+// (larger ones take more shared memory; the figure then is an estimate that costs a second wave at worst).
+constexpr int kRoomRows = 320;
+template <class K>
+cudaError_t ask_room(K* kernel, int threads, size_t smem, int* room) {
+    for (int n = 2; n <= kMaxSplit; ++n) {
+        cudaLaunchAttribute at[1] = {};
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = n;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cudaLaunchConfig_t lc{};
+        lc.gridDim = dim3(n * 1024);
+        lc.blockDim = dim3(threads);
+        lc.dynamicSmemBytes = smem;
+        lc.attrs = at;
+        lc.numAttrs = 1;
+        const cudaError_t e = cudaOccupancyMaxActiveClusters(&room[n], kernel, &lc);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+cudaError_t ask_decode_room(shotkv_ctx* ctx) {
+    cudaError_t e = ask_room(decode_attend_kernel<64>, AttendCfg<64>::kWarps * 32, attend_smem<64>(kRoomRows), ctx->room_attend[0]);
+    if (e == cudaSuccess) e = ask_room(decode_attend_kernel<128>, AttendCfg<128>::kWarps * 32, attend_smem<128>(kRoomRows), ctx->room_attend[1]);
+    if (e == cudaSuccess) e = ask_room(decode_score_kernel<64, true>, 256, score_smem(kRoomRows), ctx->room_score[0]);
+    if (e == cudaSuccess) e = ask_room(decode_score_kernel<128, true>, 256, score_smem(kRoomRows), ctx->room_score[1]);
     return e;
 }
 
@@ -764,7 +802,7 @@ int shotkv_create(shotkv_ctx** out, int device) {
                                                                  // words 8-15: four 64-bit clock stamps of the last scoring launch
     ctx->sm_count = prop.multiProcessorCount;
     ctx->encode_tiled = resolve_encode_tiled();
-    if (set_kernel_attributes() != cudaSuccess) {
+    if (set_kernel_attributes() != cudaSuccess || ask_decode_room(ctx) != cudaSuccess) {
         shotkv_destroy(ctx);
         return SHOTKV_ERR_CUDA;
     }
@@ -1218,27 +1256,28 @@ int shotkv_decode_init(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv_po
 
 namespace {
 
-// CTAs that share a unit's keys: as many (a power of two) as still fit the GPU together, `per_sm` to an
-// SM, and leave every warp at least kMinSplitBlocks blocks of 16 keys.
+// CTAs that share a unit's keys: as many as still run at the same time for all units (`room[n]` clusters of
+// n CTAs do: a cluster stays within a group of SMs, so it is fewer than the SMs' slots / n) and leave every
+// warp at least kMinSplitBlocks blocks of 16 keys.
 constexpr int kMinSplitBlocks = 2;
-int decode_split(const shotkv_ctx* ctx, long long U, long long keys, int warps, int per_sm) {
-    int n = 1;
-    while (n < kMaxSplit && U * n * 2 <= (long long)ctx->sm_count * per_sm && keys >= (long long)n * 2 * warps * 16 * kMinSplitBlocks) n *= 2;
+int decode_split(const int* room, long long U, long long keys, int warps) {
+    int n = kMaxSplit;
+    while (n > 1 && (U > room[n] || keys < (long long)n * warps * 16 * kMinSplitBlocks)) --n;
     return n;
 }
 
 template <int D>
 int launch_decode_attend(shotkv_ctx* ctx, DecodeParams& p, int U, cudaStream_t stream) {
     using Cfg = AttendCfg<D>;
-    const size_t smem = ((size_t)8 * p.Dcap + Cfg::kWarps * 8 * 2 + 16 + kMaxSplit * 16) * 4 + Cfg::kRingBytes;
+    const size_t smem = attend_smem<D>(p.Dcap);
     if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "Dcap too large for the attention-output step");
-    p.nsplit = decode_split(ctx, U, (long long)p.Mcap + p.n_old + 1, Cfg::kWarps, 3);
+    p.nsplit = decode_split(ctx->room_attend[D == 128], U, (long long)p.Mcap + p.n_old + 1, Cfg::kWarps);
     return launch(ctx, decode_attend_kernel<D>, dim3(U * p.nsplit), Cfg::kWarps * 32, smem, stream, p.nsplit, true, p);
 }
 template <int D>
 int launch_decode_score(shotkv_ctx* ctx, DecodeParams& p, int U, cudaStream_t stream) {
-    const size_t smem = ((size_t)8 * p.Dcap + 8 * 8 * 2 + 16 + kMaxSplit * 16) * 4;
-    p.nsplit = decode_split(ctx, U, (long long)p.Mcap + p.n_old + 1, 8, 4);
+    const size_t smem = score_smem(p.Dcap);
+    p.nsplit = decode_split(ctx->room_score[D == 128], U, (long long)p.Mcap + p.n_old + 1, 8);
     return p.nsplit > 1 ? launch(ctx, decode_score_kernel<D, true>, dim3(U * p.nsplit), 256, smem, stream, p.nsplit, true, p)
                         : launch(ctx, decode_score_kernel<D, false>, dim3(U), 256, smem, stream, 1, true, p);
 }
