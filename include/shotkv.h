@@ -333,7 +333,7 @@ SHOTKV_API int shotkv_selftest_bounded_wait(shotkv_ctx* ctx, int64_t limit_cycle
 SHOTKV_API int shotkv_last_scoring_clock(const shotkv_ctx* ctx, int64_t* cycles, int64_t* nanoseconds);
 
 /* Groups the single-pass form of shotkv_prefill_compress pipelines its units in: 0 (default)
- * chooses -- one group for device buffers, one per 256 MB of K (at most 4) for the host-buffer
+ * chooses -- one group for device buffers, one per 16 MB of K (at most 4) for the host-buffer
  * variant, where the groups overlap uploads with write-backs --, 1 runs every step on the
  * caller's stream, 2..4 force that many groups where there are enough prompts (or layers).  A
  * tuning and testing knob; the paper has no counterpart.  */

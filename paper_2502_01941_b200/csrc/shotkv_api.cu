@@ -34,7 +34,10 @@ constexpr int kStageSlots = 4;
 constexpr size_t kStageSlotBytes = 1u << 20;
 constexpr int kProfSlots = 64;
 constexpr int kMaxGroups = 4;         // most groups the fused prefill call pipelines its units in
-constexpr double kMinGroupKBytes = 256.0 * 1024 * 1024;   // least K a group of the automatic split holds
+// Least K a group of the automatic split holds.  A group costs its launches (10 us) and saves its share of the
+// write-back, which runs beside the next group's upload: K of 4 MB in 1, 2, 4 groups 211, 222, 250 us; 34 MB
+// in 1 or 2 1,152 and 1,046; 134 MB in 1, 2, 4 3,702, 3,474 and 3,346.
+constexpr double kMinGroupKBytes = 16.0 * 1024 * 1024;
 constexpr int kErrWords = 16;          // ints of host-mapped memory the kernels report through
 constexpr int kBigSmem = 200 * 1024;   // dynamic shared memory the small kernels are allowed (set once per context)
 
