@@ -415,7 +415,11 @@ int launch_score_tc_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorMap
 }
 
 // Column pairs, of every 16, whose exponentials run on the FMA pipe instead of the special-function unit.
-constexpr int kPolyEvery = 5;
+// The larger share takes fewer cycles and more energy: with 256 window rows the scoring pass runs at the
+// power cap for as long as it runs (5, 4, 3, 2, 1, 0 pairs: 4 x 32 layers of 32K 3,570, 3,550, 3,530, 3,580,
+// 3,630, 3,705 us a call), with 128 it waits for memory as much as for power (32 layers of 16K 395, -, 397,
+// 398, 399, 402).
+constexpr int kPolyEvery = 5, kPolyEveryStream = 3;
 
 template <int D>
 int launch_score_fast_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorMap& tmK, int qbox, int kbox,
@@ -432,7 +436,7 @@ int launch_score_stream_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtenso
     using Cfg = ScoreStreamCfg<D>;
     int grid = sp.total_items < ctx->sm_count ? sp.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    return launch(ctx, score_stream_kernel<D, kPolyEvery>, dim3(grid), Cfg::kThreads, Cfg::kSmemBytes, stream, 1, true, tmQ, tmK, qbox, kbox, sp, tab);
+    return launch(ctx, score_stream_kernel<D, kPolyEveryStream>, dim3(grid), Cfg::kThreads, Cfg::kSmemBytes, stream, 1, true, tmQ, tmK, qbox, kbox, sp, tab);
 }
 
 // Tensor maps of Q (2-D: d x rows) and K (3-D: d x N x units), 64-element boxes with 128-byte swizzle, and the
@@ -705,7 +709,7 @@ cudaError_t set_tc_attributes() {
     if (e == cudaSuccess && MB == 1)
         e = cudaFuncSetAttribute(score_fast_kernel<D, kPolyEvery>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreFastCfg<D>::kSmemBytes);
     if (e == cudaSuccess && MB == 2)
-        e = cudaFuncSetAttribute(score_stream_kernel<D, kPolyEvery>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreStreamCfg<D>::kSmemBytes);
+        e = cudaFuncSetAttribute(score_stream_kernel<D, kPolyEveryStream>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreStreamCfg<D>::kSmemBytes);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(colsum_tc_kernel<D, MB, kPolyEvery>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColsumTcCfg<D, MB>::kSmemBytes);
     return e;

@@ -1,0 +1,30 @@
+"""A key far above its work item's reference, at columns that each scoring kernel exponentiates on the
+FMA pipe (column pairs 3 and 5 of a 32-column chunk) and on the special-function unit (pair 0): the item
+must be recomputed and the result must match."""
+import numpy as np
+import pytest
+
+import paper_2502_01941_b200 as skv
+from paper_2502_01941_b200 import workloads as wl
+import parity as P
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("H,W", [(16, 16), (32, 64)], ids=["32_rows", "256_rows"])
+@pytest.mark.parametrize("col", [0, 7, 10])
+def test_out_of_range_column_on_either_pipe(col, H, W):
+    ctx = skv.Context(0)
+    cfg = wl.PrefillConfig("outlier", B=1, L=8, H=H, Hkv=8, d=64, N=2048, W=W, S=6, shot_dist="uniform", shot_lo=200,
+                           shot_hi=400, question_len=100, r_p=0.5, cfg_id=23)
+    Q, K, V, off = wl.prefill_batch(cfg, "cuda")
+    Q[..., 0], K[..., 0] = 8.0, 0.0
+    t = 3 * 128 + 32 + col
+    K[0, 0, :, t, 0] = 2000.0                 # logit 8 * 2000 / sqrt(64) = 2000
+    gpu = P.gpu_prefill(ctx, P.dims_of(cfg), Q, K, V, off, cfg.r_p, 0, "fused")
+    assert skv.shotkv_repaired_items(ctx) == cfg.Hkv
+    s = int(np.searchsorted(off[0], t, side="right")) - 1
+    k = int(off[0, s + 1] - off[0, s])
+    np.testing.assert_allclose(gpu["shot_scores"][0, 0, s].item(), cfg.H * cfg.W / k, rtol=1e-4)
+    P.check_all_units(gpu, Q, K, V, off, cfg.r_p)
+    ctx.close()
