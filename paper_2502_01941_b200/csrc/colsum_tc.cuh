@@ -105,6 +105,7 @@ __global__ void __launch_bounds__(ColsumTcCfg<D, MB>::kThreads, 1)
     const ScoreTcParams& p = cp.base;
     extern __shared__ unsigned char smem_raw[];
     grid_release();
+    tc::prefetch_maps(&tmQ, &tmK);
     tc::Pipe<Cfg> pp;
     tc::pipe_setup(pp, smem_raw, Cfg::kEpiWarps, 4 * 2 * 2, 2);     // extra barriers: [quad][slot][full, empty]
     float4* cst = reinterpret_cast<float4*>(tc::pipe_scratch(pp, smem_raw));    // [8 warps][RG / 2]

@@ -127,6 +127,7 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
                                                                       int R, int Hkv, int ranks,
                                                                       float* __restrict__ shot_scores, const SelectArgs a) {
     constexpr int NW = kReduceThreads / 32, NH = ROWS / 128, PARTS = kReduceThreads / ROWS;
+    constexpr int AHEAD = 4 / NH, FIRST = 4;       // pieces whose z a warp has in flight; items whose statistics a thread has
     constexpr unsigned char kNoItem = 255;
     static_assert(ROWS == 128 || ROWS == 256, "padded window rows");
     extern __shared__ __align__(16) unsigned char sm[];
@@ -161,6 +162,30 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
 
     for (int h = rank; h < Hkv; h += ranks) {
         const int u = bl * Hkv + h;
+        // everything the common case needs is asked for at once: the items' flags, the first statistics of
+        // this thread's row, and the first pieces of this warp
+        const int r = tid % ROWS, part = tid / ROWS;
+        const float* im = v.item_m + (size_t)u * v.nchunk * v.Rpad + r;
+        const float* iz = v.item_z + (size_t)u * v.nchunk * v.Rpad + r;
+        const float* pm = v.part_m + (size_t)u * v.P * v.Rpad;
+        const float* pz = v.part_z + (size_t)u * v.P * v.Rpad;
+        const int q0 = q_first + q_count * warp / NW, q1 = q_first + q_count * (warp + 1) / NW;
+        float m_first[FIRST], z_first[FIRST];
+        float4 z4[AHEAD][NH];
+#pragma unroll
+        for (int n = 0; n < FIRST; ++n) {
+            const int j = part + n * PARTS;
+            m_first[n] = j < v.nchunk ? im[(size_t)j * v.Rpad] : SHOTKV_NEG_INF;
+            z_first[n] = j < v.nchunk ? iz[(size_t)j * v.Rpad] : 0.f;
+        }
+        auto load_pieces = [&](int q) {
+#pragma unroll
+            for (int n = 0; n < AHEAD; ++n)
+                if (q + n < q1)
+#pragma unroll
+                    for (int k = 0; k < NH; ++k) z4[n][k] = reinterpret_cast<const float4*>(pz + (size_t)(q + n) * v.Rpad)[k * 32 + lane];
+        };
+        load_pieces(q0);
         bool any = false;
         for (int j = tid; j < v.nchunk; j += kReduceThreads) {
             const bool e = item_is_exact(v, u * v.nchunk + j);
@@ -169,13 +194,12 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
         }
         any = __syncthreads_or(any);
         {   // row statistics
-            const int r = tid % ROWS, part = tid / ROWS;
-            const float* im = v.item_m + (size_t)u * v.nchunk * v.Rpad + r;
-            const float* iz = v.item_z + (size_t)u * v.nchunk * v.Rpad + r;
             float m = SHOTKV_NEG_INF, z = 0.f;
             if (!any) {
-#pragma unroll 8
-                for (int j = part; j < v.nchunk; j += PARTS) m = fmaxf(m, im[(size_t)j * v.Rpad]);
+#pragma unroll
+                for (int n = 0; n < FIRST; ++n) m = fmaxf(m, m_first[n]);
+#pragma unroll 4
+                for (int j = part + FIRST * PARTS; j < v.nchunk; j += PARTS) m = fmaxf(m, im[(size_t)j * v.Rpad]);
             } else if (part == 0) {
                 row_stats_of(v, o, u, r, m, z);
             }
@@ -186,8 +210,10 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
             }
             const float mu = m == SHOTKV_NEG_INF ? 0.f : m;
             if (!any) {
-#pragma unroll 8
-                for (int j = part; j < v.nchunk; j += PARTS) z += iz[(size_t)j * v.Rpad] * ex2f(im[(size_t)j * v.Rpad] - mu);
+#pragma unroll
+                for (int n = 0; n < FIRST; ++n) z += z_first[n] * ex2f(m_first[n] - mu);
+#pragma unroll 4
+                for (int j = part + FIRST * PARTS; j < v.nchunk; j += PARTS) z += iz[(size_t)j * v.Rpad] * ex2f(im[(size_t)j * v.Rpad] - mu);
             }
             if (PARTS > 1) {
                 row_w[part * ROWS + r] = z;
@@ -208,8 +234,6 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
             rm[k] = reinterpret_cast<const float4*>(row_m)[k * 32 + lane];
             rw[k] = reinterpret_cast<const float4*>(row_w)[k * 32 + lane];
         }
-        const float* pm = v.part_m + (size_t)u * v.P * v.Rpad;
-        const float* pz = v.part_z + (size_t)u * v.P * v.Rpad;
         // 2^(m - row's m) / Z of this lane's rows; a row without weight (padding, or nothing but
         // underflow) gets factor 0 whatever its reference
         auto weights = [&](const float* ref) {
@@ -222,16 +246,9 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
                 f[k].w = rw[k].w > 0.f ? ex2f(mi.w - rm[k].w) * rw[k].w : 0.f;
             }
         };
-        constexpr int AHEAD = 4 / NH;              // pieces whose z a warp has in flight
-        const int q0 = q_first + q_count * warp / NW, q1 = q_first + q_count * (warp + 1) / NW;
         int item = kNoItem;
         for (int q = q0; q < q1; q += AHEAD) {
-            float4 z4[AHEAD][NH];
-#pragma unroll
-            for (int n = 0; n < AHEAD; ++n)
-                if (q + n < q1)
-#pragma unroll
-                    for (int k = 0; k < NH; ++k) z4[n][k] = reinterpret_cast<const float4*>(pz + (size_t)(q + n) * v.Rpad)[k * 32 + lane];
+            if (q != q0) load_pieces(q);
 #pragma unroll
             for (int n = 0; n < AHEAD; ++n) {
                 const int j = q + n < q1 ? item_of[q + n] : kNoItem;

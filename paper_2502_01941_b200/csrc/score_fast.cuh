@@ -177,6 +177,7 @@ __global__ void __launch_bounds__(ScoreFastCfg<D>::kThreads, 1)
     constexpr int NSL = Cfg::kSlices, SLW = TN / NSL, NCH = SLW / 32, RD = Cfg::kRingDepth;
     extern __shared__ unsigned char smem_raw[];
     grid_release();
+    tc::prefetch_maps(&tmQ, &tmK);
     tc::Pipe<Cfg> pp;
     tc::pipe_setup(pp, smem_raw, Cfg::kEpiWarps, Cfg::kRings * Cfg::kRingDepth * 2, 2);
     float* comb = tc::pipe_scratch(pp, smem_raw);     // [ring][slot][lane][m, z]

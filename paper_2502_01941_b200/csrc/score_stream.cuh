@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(ScoreStreamCfg<D>::kThreads, 1)
     constexpr int TN = tc::kTileKeys, MB = 2;
     extern __shared__ unsigned char smem_raw[];
     grid_release();
+    tc::prefetch_maps(&tmQ, &tmK);
     tc::Pipe<Cfg> pp;
     tc::pipe_setup(pp, smem_raw, 4, 0, 2);
     float4* mtab = reinterpret_cast<float4*>(tc::pipe_scratch(pp, smem_raw));   // split masks

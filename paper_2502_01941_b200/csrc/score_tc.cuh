@@ -170,6 +170,14 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map
         : "memory");
 }
 
+// The two tensor maps into the descriptor cache, ahead of the first copy that needs them (they are launch
+// parameters, so this may come before grid_wait).
+__device__ __forceinline__ void prefetch_maps(const CUtensorMap* a, const CUtensorMap* b) {
+    if (threadIdx.x == 0) {
+        asm volatile("prefetch.tensormap [%0];" ::"l"(a) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"(b) : "memory");
+    }
+}
 __device__ __forceinline__ void tmem_alloc(uint32_t slot, uint32_t cols) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(slot), "r"(cols) : "memory");
 }

@@ -258,22 +258,28 @@ __global__ void __launch_bounds__(256) compact_kv_kernel(const uint4* __restrict
     const int bl = blockIdx.z, h = blockIdx.y;
     grid_release();
     grid_wait();
-    const int count = min(kept_count[bl], Mcap);
+    const int* idx = kept_idx + (size_t)bl * Mcap;
     const int row_in = threadIdx.x / VPR, v = threadIdx.x % VPR;
+    // the first pass's indices and the count are asked for together (the index rows hold Mcap entries)
+    int src[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int j = blockIdx.x * ROWS + q * (256 / VPR) + row_in;
+        src[q] = j < Mcap ? idx[j] : -1;
+    }
+    const int count = min(kept_count[bl], Mcap);
     const size_t u = (size_t)bl * Hkv + h;
     const uint4* Ku = K + u * N * VPR;
     const uint4* Vu = V + u * N * VPR;
     uint4* Kcu = Kc + u * Mcap * VPR;
     uint4* Vcu = Vc + u * Mcap * VPR;
-    const int* idx = kept_idx + (size_t)bl * Mcap;
     for (int j0 = blockIdx.x * ROWS; j0 < count; j0 += gridDim.x * ROWS) {
         uint4 kk[4], vv[4];
-        int src[4];
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int j = j0 + q * (256 / VPR) + row_in;
-            src[q] = j < count ? idx[j] : -1;
-            if (src[q] >= N) src[q] = -1;
+            if (j0 != blockIdx.x * ROWS) src[q] = j < count ? idx[j] : -1;
+            if (j >= count || src[q] >= N) src[q] = -1;
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q)
