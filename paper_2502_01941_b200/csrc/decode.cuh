@@ -28,9 +28,6 @@ struct DecodeParams {
 // query row to all others and each then knows the whole row's maximum and sum.
 constexpr int kMaxSplit = 8;
 
-// Which CTA of the cluster has key i, NW warps to a CTA.
-__device__ __forceinline__ int split_of_key(int i, int NW, int nsplit) { return ((i >> 4) / NW) % nsplit; }
-
 // Every CTA's (m, z) of the 8 query rows (`own`, [8][2], in shared memory behind a barrier) to all
 // CTAs' `table` [nsplit][8][2]; returns when all have arrived.  Preceded by a cluster_arrive at the
 // start of the kernel (a CTA's memory may be written once it has begun).  What the CTA wrote to its own
@@ -209,11 +206,19 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p)
         if (tid < 8) merge_stats(stab, nsplit, tid, sfin[tid * 2], sfin[tid * 2 + 1]);
         __syncthreads();
     }
-    for (int j = tid; j < n; j += 256) {
-        if (SPLIT && split_of_key(M + j, 8, nsplit) != rank) continue;
+    auto weight = [&](int j) {
         float s = 0.f;
         for (int r = 0; r < p.G; ++r) s += ex2f(sdec[r * p.Dcap + j] - sfin[r * 2]) * sfin[r * 2 + 1];
         p.partial[(size_t)u * p.Dcap + j] = s;
+    };
+    if (SPLIT) {                                           // the decode entries among this warp's blocks
+        const int stride = nsplit * 8 * 16;
+        for (int base = first + max(0, (M - 15 - first + stride - 1) / stride) * stride; base < Ktot; base += stride) {
+            const int j = base + lane - M;
+            if (lane < 16 && j >= 0 && j < n) weight(j);
+        }
+    } else {
+        for (int j = tid; j < n; j += 256) weight(j);
     }
 }
 
@@ -305,15 +310,39 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     grid_wait();
     grid_release();
     const int bl = u / p.Hkv, hk = u - bl * p.Hkv;
-    const int M = min(p.kept_count[bl], p.Mcap);
+    const int kept = p.kept_count[bl];
+    const uint4* Kc_u = reinterpret_cast<const uint4*>(p.Kc + (size_t)u * p.Mcap * D);
+    const uint4* Vc_u = reinterpret_cast<const uint4*>(p.Vc + (size_t)u * p.Mcap * D);
+    // this warp's ring.  A lane copies chunk (lane % VPR) of rows lane / VPR + k * (32 / VPR) of a block;
+    // kdst and vdst are its first copies' offsets in a stage, permuted as above (the row's low bits of later
+    // copies enter the values' permutation by exclusive or)
+    constexpr int RPI = 32 / VPR;                            // rows per warp-wide copy
+    const uint32_t wring = smem_u32(ring) + (uint32_t)(warp * NS * Cfg::kStageBytes);
+    const uint32_t kdst = (uint32_t)((lane / VPR) * Cfg::kRowBytes + (((lane % VPR) ^ (((lane / VPR) & 1) << 2)) << 4));
+    const uint32_t vdst = (uint32_t)(Cfg::kTileBytes + (lane / VPR) * Cfg::kRowBytes + (((lane % VPR) ^ ((lane / VPR) & 7)) << 4));
+    auto fetch_prefill = [&](int base, int stage) {          // 16 prefill rows: one run of memory
+        const uint32_t st = wring + (uint32_t)(stage * Cfg::kStageBytes);
+        const uint4* ks = Kc_u + (size_t)base * VPR + lane;
+        const uint4* vs = Vc_u + (size_t)base * VPR + lane;
+#pragma unroll
+        for (int k = 0; k < 16 / RPI; ++k) {
+            cp_async16(st + kdst + (uint32_t)(k * RPI * Cfg::kRowBytes), ks + k * 32);
+            cp_async16(st + (vdst ^ (uint32_t)(((k * RPI) & 7) << 4)) + (uint32_t)(k * RPI * Cfg::kRowBytes), vs + k * 32);
+        }
+        cp_async_commit();
+    };
+    // the first block is asked for before the kept count is there: rows below Mcap can be read, and where the
+    // count turns out to end before them they are fetched again
+    const int first = (rank * NW + warp) * 16;
+    const bool ahead = first + 16 <= p.Mcap;
+    if (ahead) fetch_prefill(first, 0);
+    const int M = min(kept, p.Mcap);
     const int n = p.n_old + 1;
     const int Ktot = M + n;
-    const uint4* Kc_u = reinterpret_cast<const uint4*>(p.Kc + (size_t)u * p.Mcap * D);
     uint4* Kd_u = reinterpret_cast<uint4*>(p.Kd + (size_t)u * p.Dcap * D);
     uint4* Vd_u = reinterpret_cast<uint4*>(p.Vd + (size_t)u * p.Dcap * D);
     const uint4* knew_u = reinterpret_cast<const uint4*>(p.k_new + (size_t)u * D);
     const uint4* vnew_u = reinterpret_cast<const uint4*>(p.v_new + (size_t)u * D);
-    const uint4* Vc_u = reinterpret_cast<const uint4*>(p.Vc + (size_t)u * p.Mcap * D);
 
     // append the new token's key and value as decode entry n_old
     if (rank != 0) {
@@ -328,28 +357,15 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
         for (int kb = 0; kb < NB; ++kb) qf[kb] = g < p.G ? qrow[kb * 4 + t4] : make_uint4(0, 0, 0, 0);
     }
 
-    // this warp's ring.  A lane copies chunk (lane % VPR) of rows lane / VPR + k * (32 / VPR); rows
-    // past the end are filled with zeros (a weight of zero must not meet a stray NaN).
-    const uint32_t wring = smem_u32(ring) + (uint32_t)(warp * NS * Cfg::kStageBytes);
-    // offsets of this lane's first copies in a stage: row lane / VPR, chunk lane % VPR permuted as above (the
-    // row's low bits of later copies enter the values' permutation by exclusive or)
-    const uint32_t kdst = (uint32_t)((lane / VPR) * Cfg::kRowBytes + (((lane % VPR) ^ (((lane / VPR) & 1) << 2)) << 4));
-    const uint32_t vdst = (uint32_t)(Cfg::kTileBytes + (lane / VPR) * Cfg::kRowBytes + (((lane % VPR) ^ ((lane / VPR) & 7)) << 4));
+    // a block with decode entries in it, or past the end: rows past the end are filled with zeros (a weight of
+    // zero must not meet a stray NaN)
     auto fetch_block = [&](int base, int stage) {
-        constexpr int RPI = 32 / VPR;                       // rows per warp-wide copy
-        const int c = lane % VPR;
-        const uint32_t st = wring + (uint32_t)(stage * Cfg::kStageBytes);
-        if (base + 16 <= M) {                               // all of it kept prefill rows: one run of memory
-            const uint4* ks = Kc_u + (size_t)base * VPR + lane;
-            const uint4* vs = Vc_u + (size_t)base * VPR + lane;
-#pragma unroll
-            for (int k = 0; k < 16 / RPI; ++k) {
-                cp_async16(st + kdst + (uint32_t)(k * RPI * Cfg::kRowBytes), ks + k * 32);
-                cp_async16(st + (vdst ^ (uint32_t)(((k * RPI) & 7) << 4)) + (uint32_t)(k * RPI * Cfg::kRowBytes), vs + k * 32);
-            }
-            cp_async_commit();
+        if (base + 16 <= M) {
+            fetch_prefill(base, stage);
             return;
         }
+        const int c = lane % VPR;
+        const uint32_t st = wring + (uint32_t)(stage * Cfg::kStageBytes);
 #pragma unroll
         for (int k = 0; k < 16 / RPI; ++k) {
             const int rr = lane / VPR + k * RPI;
@@ -376,10 +392,18 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     float m = SHOTKV_NEG_INF, z = 0.f;
     // blocks are requested NS - 1 ahead; one copy group per block, empty past the end, so that
     // "at most NS - 1 groups pending" always means this block's rows have landed
-    const int first = (rank * NW + warp) * 16, STRIDE = p.nsplit * NW * 16;
+    const int STRIDE = p.nsplit * NW * 16;
     int stage = 0;
+    if (ahead && first + 16 > M) {                          // not all prefill rows after all
+        cp_async_wait<0>();
+        __syncwarp();
+    }
+    if (!ahead || first + 16 > M) {
+        if (first < Ktot) fetch_block(first, 0);
+        else cp_async_commit();
+    }
 #pragma unroll
-    for (int k = 0; k < NS - 1; ++k) {
+    for (int k = 1; k < NS - 1; ++k) {
         if (first + k * STRIDE < Ktot) fetch_block(first + k * STRIDE, k);
         else cp_async_commit();
     }
@@ -509,11 +533,14 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
         }
         cluster_arrive();                                    // done with the others' memory
     }
-    for (int j = tid; j < n; j += NT) {
-        if (p.nsplit > 1 && split_of_key(M + j, NW, p.nsplit) != rank) continue;
-        float s = 0.f;
-        for (int r = 0; r < p.G; ++r) s += ex2f(sdec[r * p.Dcap + j] - sfin[r * 2]) * sfin[r * 2 + 1];
-        p.partial[(size_t)u * p.Dcap + j] = s;
+    // the decode entries among this warp's blocks: their weights summed over the query rows
+    for (int base = first + max(0, (M - 15 - first + STRIDE - 1) / STRIDE) * STRIDE; base < Ktot; base += STRIDE) {
+        const int j = base + lane - M;
+        if (lane < 16 && j >= 0 && j < n) {
+            float s = 0.f;
+            for (int r = 0; r < p.G; ++r) s += ex2f(sdec[r * p.Dcap + j] - sfin[r * 2]) * sfin[r * 2 + 1];
+            p.partial[(size_t)u * p.Dcap + j] = s;
+        }
     }
     if (p.nsplit > 1) cluster_wait();                        // the others are done with this CTA's
 }
@@ -542,11 +569,12 @@ __device__ __forceinline__ float accumulated(const DecodeFinishParams& p, int bl
 }
 
 // A step without eviction.
-__global__ void __launch_bounds__(128) decode_accumulate_kernel(const DecodeFinishParams p) {
-    const int bl = blockIdx.x;
+constexpr int kAccumulateThreads = 128;         // one entry a thread
+__global__ void __launch_bounds__(kAccumulateThreads) decode_accumulate_kernel(const DecodeFinishParams p) {
+    const int bl = blockIdx.x, j = blockIdx.y * kAccumulateThreads + threadIdx.x;
     grid_wait();
     grid_release();
-    for (int j = threadIdx.x; j < p.n; j += blockDim.x) {
+    if (j < p.n) {
         p.acc[(size_t)bl * p.Dcap + j] = accumulated(p, bl, j);
         if (j == p.n - 1) p.born[(size_t)bl * p.Dcap + j] = p.T_old;
     }

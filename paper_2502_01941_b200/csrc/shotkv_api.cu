@@ -1336,7 +1336,7 @@ int decode_step_impl(shotkv_ctx* ctx, shotkv_decode_state* st, const shotkv_bf16
         rc = d.d == 128 ? launch(ctx, decode_evict_kernel<128>, dim3(BL * f.ranks), kSelectThreads, decode_evict_smem_bytes(f.n), stream, f.ranks, true, f)
                         : launch(ctx, decode_evict_kernel<64>, dim3(BL * f.ranks), kSelectThreads, decode_evict_smem_bytes(f.n), stream, f.ranks, true, f);
     } else {
-        rc = launch(ctx, decode_accumulate_kernel, dim3(BL), 128, 0, stream, 1, true, f);
+        rc = launch(ctx, decode_accumulate_kernel, dim3(BL, (f.n + kAccumulateThreads - 1) / kAccumulateThreads), kAccumulateThreads, 0, stream, 1, true, f);
     }
     if (rc) return rc;
     st->T = T;
