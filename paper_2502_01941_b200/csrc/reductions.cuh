@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
 constexpr int kTokenWarps = 8;
 constexpr int kLongShot = 96;                  // mean length from which eight warps share a shot
 template <int WPS>
-__global__ void __launch_bounds__(32 * kTokenWarps) shot_score_from_tokens_kernel(const float* __restrict__ imp,
+__global__ void __launch_bounds__(32 * kTokenWarps, 4) shot_score_from_tokens_kernel(const float* __restrict__ imp,
                                                                                   const __grid_constant__ ShotTable tab, int L,
                                                                                   int Hkv, int N, int S,
                                                                                   float* __restrict__ shot_scores) {

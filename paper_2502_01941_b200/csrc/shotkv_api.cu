@@ -490,12 +490,16 @@ int tc_setup(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q, const 
     return SHOTKV_OK;
 }
 
-template <int D, int MB>
-int launch_colsum_tc_t(shotkv_ctx* ctx, const TcSetup& t, const ColsumTcParams& cp, cudaStream_t stream) {
+template <int D, int MB, bool FULL>
+int launch_colsum_tc_f(shotkv_ctx* ctx, const TcSetup& t, const ColsumTcParams& cp, cudaStream_t stream) {
     constexpr int smem = ColsumTcCfg<D, MB>::kSmemBytes;
     int grid = cp.base.total_items < ctx->sm_count ? cp.base.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    return launch(ctx, colsum_tc_kernel<D, MB, kPolyEvery>, dim3(grid), ColsumTcCfg<D, MB>::kThreads, smem, stream, 1, true, t.tmQ, t.tmK, t.qbox, t.kbox, cp);
+    return launch(ctx, colsum_tc_kernel<D, MB, kPolyEvery, FULL>, dim3(grid), ColsumTcCfg<D, MB>::kThreads, smem, stream, 1, true, t.tmQ, t.tmK, t.qbox, t.kbox, cp);
+}
+template <int D, int MB>
+int launch_colsum_tc_t(shotkv_ctx* ctx, const TcSetup& t, const ColsumTcParams& cp, cudaStream_t stream) {
+    return cp.base.R > 128 * MB - 32 ? launch_colsum_tc_f<D, MB, true>(ctx, t, cp, stream) : launch_colsum_tc_f<D, MB, false>(ctx, t, cp, stream);
 }
 
 // Second pass of the per-token path: token_importance from the row statistics in the workspace.
@@ -711,7 +715,9 @@ cudaError_t set_tc_attributes() {
     if (e == cudaSuccess && MB == 2)
         e = cudaFuncSetAttribute(score_stream_kernel<D, kPolyEveryStream>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreStreamCfg<D>::kSmemBytes);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(colsum_tc_kernel<D, MB, kPolyEvery>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColsumTcCfg<D, MB>::kSmemBytes);
+        e = cudaFuncSetAttribute(colsum_tc_kernel<D, MB, kPolyEvery, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColsumTcCfg<D, MB>::kSmemBytes);
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(colsum_tc_kernel<D, MB, kPolyEvery, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColsumTcCfg<D, MB>::kSmemBytes);
     return e;
 }
 cudaError_t set_kernel_attributes() {

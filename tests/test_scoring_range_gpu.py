@@ -28,3 +28,17 @@ def test_out_of_range_column_on_either_pipe(col, H, W):
     np.testing.assert_allclose(gpu["shot_scores"][0, 0, s].item(), cfg.H * cfg.W / k, rtol=1e-4)
     P.check_all_units(gpu, Q, K, V, off, cfg.r_p)
     ctx.close()
+
+
+@pytest.mark.parametrize("G,W", [(1, 1), (1, 31), (2, 16), (1, 33), (3, 32), (1, 97), (4, 32), (3, 43), (4, 56), (5, 45), (4, 64)])
+def test_token_importance_at_edges_of_32_row_chunks(G, W):
+    """Window rows (1, 31, 32, 33, 96, 97, 128, 129, 224, 225, 256) on both sides of the second pass's 32-row
+    chunks: chunks without a row are left out."""
+    ctx = skv.Context(0)
+    cfg = wl.PrefillConfig("chunks", B=1, L=1, H=2 * G, Hkv=2, d=128, N=1411, W=W, S=5, shot_dist="uniform", shot_lo=100,
+                           shot_hi=400, question_len=211, r_p=0.5, cfg_id=24)
+    Q, K, V, off = wl.prefill_batch(cfg, "cuda")
+    gpu = P.gpu_prefill(ctx, P.dims_of(cfg), Q, K, V, off, cfg.r_p, 0, "calls")
+    assert gpu["token_importance"] is not None
+    P.check_all_units(gpu, Q, K, V, off, cfg.r_p, check_tokens=True)
+    ctx.close()
