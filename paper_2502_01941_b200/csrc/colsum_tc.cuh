@@ -11,10 +11,11 @@
 //
 // Epilogue: eight warps in two groups; a warp owns 32 keys (its tensor-memory lanes), a group
 // half of the window rows.  Per row the constants (-M_r, 1/Z_r) come from shared memory as
-// broadcast reads.  The second group hands its partial sums to the first through a two-slot
+// broadcast reads.  A chunk of 32 rows is asked for from tensor memory before the one ahead of it is
+// computed (32 layers of 16K in sentences 640 -> 628 us a call).  The second group hands its partial sums to the first through a two-slot
 // shared-memory ring guarded by mbarriers; the first adds them in a fixed order and stores.
 #pragma once
-#include "score_fast.cuh"
+#include "score_stream.cuh"
 
 namespace shotkv {
 
@@ -189,20 +190,13 @@ __global__ void __launch_bounds__(ColsumTcCfg<D, MB>::kThreads, 1)
                 const uint32_t taddr = pp.tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)(acc * ROWS + r0);
                 const bool plain = lo + t * TN + TN <= p.N - p.W + 1;       // every key of the tile counts for every row
                 uint64_t s2[2] = {0ull, 0ull};
-                uint32_t r[32];
-                if (!FULL && nch == 0) {                            // no window rows in this group's half
+                auto release = [&]() {
+                    tc::fence_before_sync();
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive(pp.tempty(acc, 0));
-                }
-#pragma unroll 1
-                for (int c = 0; c < nch; ++c) {
-                    tc::tmem_ld32_sync(r, taddr + c * 32);
-                    if (c == nch - 1) {
-                        tc::fence_before_sync();
-                        __syncwarp();
-                        if (lane == 0) tc::mbar_arrive(pp.tempty(acc, 0));
-                    }
-                    // alpha of the pair of rows (2 jp, 2 jp + 1) at this thread's key, times 1/Z, added to the sums
+                };
+                // the 32 rows of chunk c in r: alpha of every pair of rows at this thread's key, times 1/Z, added up
+                auto chunk = [&](const uint32_t (&r)[32], int c) {
                     auto pair_term = [&](int jp, bool masked) {
                         const float4 k4 = cu[c * 16 + jp];
                         uint64_t e2;
@@ -227,6 +221,22 @@ __global__ void __launch_bounds__(ColsumTcCfg<D, MB>::kThreads, 1)
                     } else {
 #pragma unroll
                         for (int jp = 0; jp < 16; ++jp) pair_term(jp, true);
+                    }
+                };
+                uint32_t ra[32], rb[32];
+                if (!FULL && nch == 0) release();                   // no window rows in this group's half
+                else tc::tmem_ld32_issue(ra, taddr);
+#pragma unroll 1
+                for (int c = 0; c < nch; c += 2) {
+                    tc::tmem_ld_wait(ra);
+                    if (c + 1 < nch) tc::tmem_ld32_issue(rb, taddr + (c + 1) * 32);
+                    else release();
+                    chunk(ra, c);
+                    if (c + 1 < nch) {
+                        tc::tmem_ld_wait(rb);
+                        if (c + 2 < nch) tc::tmem_ld32_issue(ra, taddr + (c + 2) * 32);
+                        else release();
+                        chunk(rb, c + 1);
                     }
                 }
                 float sum;
