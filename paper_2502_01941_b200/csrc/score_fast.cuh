@@ -52,6 +52,37 @@ struct ScoreFastCfg {
 
 namespace tc {
 
+// 32 consecutive fp32 columns of this thread's tensor-memory lane, requested but not waited for:
+// the registers are not defined until tmem_ld_wait has been passed with the same array.
+__device__ __forceinline__ void tmem_ld32_issue(uint32_t (&v)[32], uint32_t taddr) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
+        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]), "=r"(v[8]),
+          "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]), "=r"(v[16]),
+          "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]),
+          "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(taddr)
+        : "memory");
+}
+// Waits for every tensor-memory load this thread has requested.  The array is passed as a
+// read-write operand so that no use of its registers can be moved above the wait.
+__device__ __forceinline__ void tmem_ld_wait(uint32_t (&v)[32]) {
+    asm volatile(
+        "tcgen05.wait::ld.sync.aligned;"
+        : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7]), "+r"(v[8]),
+          "+r"(v[9]), "+r"(v[10]), "+r"(v[11]), "+r"(v[12]), "+r"(v[13]), "+r"(v[14]), "+r"(v[15]), "+r"(v[16]),
+          "+r"(v[17]), "+r"(v[18]), "+r"(v[19]), "+r"(v[20]), "+r"(v[21]), "+r"(v[22]), "+r"(v[23]), "+r"(v[24]),
+          "+r"(v[25]), "+r"(v[26]), "+r"(v[27]), "+r"(v[28]), "+r"(v[29]), "+r"(v[30]), "+r"(v[31])
+        :
+        : "memory");
+}
+
+}  // namespace tc
+
+namespace tc {
+
 constexpr float kRefShift = 32.f;        // the first tile's row maximum is exponentiated to 2^-32
 constexpr float kRedoAbove = 1e30f;      // a partial sum at or above this sends its item to the exact kernel
 
@@ -354,13 +385,16 @@ __global__ void __launch_bounds__(ScoreFastCfg<D>::kThreads, 1)
                 if (kc0 + SLW <= min(pend, plain_end)) {
                     // most tiles: every column of the slice counts for every row (it lies before the
                     // item's end and before the first window position) and no piece ends inside it.
-                    // One short loop without further branches.
-#pragma unroll 1
-                    for (int c = 0; c < NCH; ++c) {
-                        tc::tmem_ld32_sync(r, taddr + c * 32);
-                        tc::expacc32<PE>(r, scale, neg, z);
-                    }
+                    // The second chunk is asked for before the first is computed (32 layers of 16K 387.5 ->
+                    // 383.5 us a call).
+                    static_assert(NCH == 2, "a slice is two chunks");
+                    uint32_t rb[32];
+                    tc::tmem_ld32_sync(r, taddr);
+                    tc::tmem_ld32_issue(rb, taddr + 32);
+                    tc::expacc32<PE>(r, scale, neg, z);
+                    tc::tmem_ld_wait(rb);
                     release();
+                    tc::expacc32<PE>(rb, scale, neg, z);
                 } else {
 #pragma unroll 1
                     for (int c = 0; c < NCH; ++c) {
