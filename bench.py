@@ -732,7 +732,7 @@ def main():
                          "units of 10-40 tokens (the document-QA adaptation), or fixed chunks of 16 tokens")
     ap.add_argument("--chunk-tokens", type=int, default=16, help="chunk length for --units chunks")
     ap.add_argument("--scoring", default="fast", choices=sorted(SCORING_MODES),
-                    help="scoring kernel: the default pair (fast kernel + exact repair) or the exact kernel alone")
+                    help="scoring kernel: the default (fast kernel with exact repair) or the exact kernel alone")
     ap.add_argument("--groups", type=int, default=0, choices=[0, 1, 2, 3, 4],
                     help="groups of units the fused call pipelines (0: the library's choice; 1: no overlap of steps)")
     ap.add_argument("--no-tokens", action="store_true", help="skip the per-token-importance form of the step")

@@ -6,12 +6,12 @@
 //   item_m, item_z [U*nchunk][Rpad]   per (item, row) the reference exponent m all of the item's
 //                              pieces share, and the sum of their z -- written by the kernels that
 //                              fix one reference per item (score_fast.cuh, score_stream.cuh)
-//   part_m [U][P][Rpad]       per (piece, row) reference -- written only by the exact kernel
-//                              (score_tc.cuh), whose running maximum moves inside an item
-//   redo   [U*nchunk]         not 0 for the items the exact kernel recomputed after the fast one
+//   part_m [U][P][Rpad]       per (piece, row) reference -- written only by the epilogue of
+//                              score_tc.cuh, whose running maximum moves inside an item
+//   redo   [U*nchunk]         not 0 for the items that were recomputed with a running maximum
 // The piece of segment s (0 = before the first shot, i + 1 = shot i, S + 1 = the question) in item j
 // of a unit has index s + j.
-// An item is "exact" when every item is (`all_exact`: the exact kernel did all the work) or when
+// An item is "exact" when every item is (`all_exact`: the kernel of score_tc.cuh did all the work) or when
 // its redo flag is set; its rows' statistics are then rebuilt from its pieces.
 // row_stats_kernel, reduce_select_kernel, shot_score_from_tokens_kernel: fixed-order reductions of
 // those partials, and of per-token importances.

@@ -16,9 +16,8 @@
 //     of the item is exponentiated against the same m.  fp32 leaves about 2^+158 above that point
 //     and 2^-94 below it; what underflows is below 2^-94 of a term the row's own softmax
 //     denominator contains, so it cannot matter to any score.  What overflows is caught: a
-//     partial sum that is not below 1e30 marks its item in `redo`, and a second launch (the exact
-//     kernel of score_tc.cuh with the same flags) recomputes marked items with a true running
-//     maximum.
+//     partial sum that is not below 1e30 marks its item in `redo`, and at the end of the kernel the
+//     CTA recomputes the items it marked with a true running maximum (repair_items of score_tc.cuh).
 //   * One ex2 per logit is the ceiling of the special-function unit (16 lanes per clock per SM),
 //     so PE of every 16 column pairs take their exponentials on the FMA pipe instead: round to nearest
 //     integer n by the magic-number addition, a cubic in the remainder f in [-1/2, 1/2]
@@ -84,7 +83,7 @@ __device__ __forceinline__ void tmem_ld_wait(uint32_t (&v)[32]) {
 namespace tc {
 
 constexpr float kRefShift = 32.f;        // the first tile's row maximum is exponentiated to 2^-32
-constexpr float kRedoAbove = 1e30f;      // a partial sum at or above this sends its item to the exact kernel
+constexpr float kRedoAbove = 1e30f;      // a partial sum at or above this has its item recomputed
 
 // 2^x on the FMA pipe for two logits at a time, x = s * scale + neg.  One saturating
 // multiply-add per logit maps x from [-126, 128] onto y in [0, 1] and so does the scaling, the
@@ -202,7 +201,7 @@ __device__ __forceinline__ void peel_chunk(uint32_t (&r)[32], float scale, float
 template <int D, int PE>
 __global__ void __launch_bounds__(ScoreFastCfg<D>::kThreads, 1)
     score_fast_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const int q_box_rows,
-                      const int k_box_rows, const ScoreTcParams p, const __grid_constant__ ShotTable tab) {
+                      const int k_box_rows, const __grid_constant__ ScoreTcParams p, const __grid_constant__ ShotTable tab) {
     using Cfg = ScoreFastCfg<D>;
     constexpr int TN = tc::kTileKeys, MB = 1;
     constexpr int NSL = Cfg::kSlices, SLW = TN / NSL, NCH = SLW / 32, RD = Cfg::kRingDepth;
@@ -252,7 +251,7 @@ __global__ void __launch_bounds__(ScoreFastCfg<D>::kThreads, 1)
             // load's latency never sits between a piece end and the next comparison
             const int* next = o + sg + 1;
             int pend = next[-1], pend_n = next[0];
-            // this warp's flag of the item: set when a sum leaves the range (the exact kernel redoes the item)
+            // this warp's flag of the item: set when a sum leaves the range (the item is then recomputed below)
             unsigned char* flag = reinterpret_cast<unsigned char*>(p.redo + it) + (warp - 4);
             if (lane == 0) *flag = 0;
             __syncwarp();
@@ -274,9 +273,9 @@ __global__ void __launch_bounds__(ScoreFastCfg<D>::kThreads, 1)
                 }
                 const int slot = nflush & (RD - 1);
                 const uint32_t par = (uint32_t)(nflush / RD) & 1u;
-                // out of range (or not a number): the exact kernel redoes the item.  Tested on this
+                // out of range (or not a number): the item is recomputed below.  Tested on this
                 // slice's own sum, before any rescaling by another slice's reference could hide it.
-                if (live && !(zz < tc::kRedoAbove)) *flag = 1;
+                if (live && !(zz < tc::kRedoAbove)) *flag = 1, *pp.repair_flag() = 1;
                 if (slice != 0) {
                     const int ring = (blk * 4 + quad) * (NSL - 1) + (slice - 1);
                     const int rs = ring * RD + slot;
@@ -419,6 +418,8 @@ __global__ void __launch_bounds__(ScoreFastCfg<D>::kThreads, 1)
     tc::fence_before_sync();
     __syncthreads();
     tc::stamp(p.clk, 1);
+    if (*pp.repair_flag() && !*pp.abort_flag)
+        tc::repair_items<D, MB, Cfg::kEpiWarps, Cfg>(smem_raw, &tmQ, &tmK, q_box_rows, k_box_rows, p, tab);
     if (warp == 0) {
         __syncwarp();
         tc::fence_after_sync();

@@ -1,7 +1,7 @@
 // Window attention scoring for units of more than 128 window rows (two 128-row blocks of Q), the
 // kernel the prefill path runs first on them: the TMA producer, MMA issuers, work items and
-// per-(piece, window row) outputs (m, z) of score_tc.cuh, the fixed reference exponent with
-// exact-kernel repair and the two-pipe exponentials of score_fast.cuh, and an epilogue that never
+// per-(piece, window row) outputs (m, z) of score_tc.cuh, the fixed reference exponent, the repair at the
+// end and the two-pipe exponentials of score_fast.cuh, and an epilogue that never
 // waits for tensor memory.
 //
 // Eight epilogue warps, one per (row block, tensor-memory lane quarter); a thread is one whole
@@ -43,7 +43,7 @@ struct ScoreStreamCfg {
 template <int D, int PE>
 __global__ void __launch_bounds__(ScoreStreamCfg<D>::kThreads, 1)
     score_stream_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const int q_box_rows,
-                        const int k_box_rows, const ScoreTcParams p, const __grid_constant__ ShotTable tab) {
+                        const int k_box_rows, const __grid_constant__ ScoreTcParams p, const __grid_constant__ ShotTable tab) {
     using Cfg = ScoreStreamCfg<D>;
     constexpr int TN = tc::kTileKeys, MB = 2;
     extern __shared__ unsigned char smem_raw[];
@@ -89,7 +89,7 @@ __global__ void __launch_bounds__(ScoreStreamCfg<D>::kThreads, 1)
             // end of the current piece, and of the one after it (fetched one piece ahead)
             const int* next = o + sg + 1;
             int pend = next[-1], pend_n = next[0];
-            // this warp's flag of the item: set when a sum leaves the range (the exact kernel redoes the item)
+            // this warp's flag of the item: set when a sum leaves the range (the item is then recomputed below)
             if (lane == 0) reinterpret_cast<unsigned char*>(p.redo + it)[warp - 4] = 0;
             __syncwarp();
             float m_ref = SHOTKV_NEG_INF, neg = 0.f;       // reference exponent of this (row, item); neg = -m_ref
@@ -104,7 +104,10 @@ __global__ void __launch_bounds__(ScoreStreamCfg<D>::kThreads, 1)
                 tc::unpack2(z[0], s0, s1);
                 tc::unpack2(z[1], s2, s3);
                 const float zz = (s0 + s1) + (s2 + s3);
-                if (live && !(zz < tc::kRedoAbove)) reinterpret_cast<unsigned char*>(p.redo + it)[warp - 4] = 1;   // out of range, or not a number
+                if (live && !(zz < tc::kRedoAbove)) {      // out of range, or not a number
+                    reinterpret_cast<unsigned char*>(p.redo + it)[warp - 4] = 1;
+                    *pp.repair_flag() = 1;
+                }
                 *out_z = live ? zz : 0.f;
                 out_z += p.Rpad;
                 zsum += zz;
@@ -223,6 +226,8 @@ __global__ void __launch_bounds__(ScoreStreamCfg<D>::kThreads, 1)
     tc::fence_before_sync();
     __syncthreads();
     tc::stamp(p.clk, 1);
+    if (*pp.repair_flag() && !*pp.abort_flag)
+        tc::repair_items<D, MB, Cfg::kEpiWarps, Cfg>(smem_raw, &tmQ, &tmK, q_box_rows, k_box_rows, p, tab);
     if (warp == 0) {
         __syncwarp();
         tc::fence_after_sync();

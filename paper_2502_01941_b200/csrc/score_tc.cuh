@@ -2,8 +2,9 @@
 // tensor memory) with K streamed by TMA: the exact scoring kernel (a running maximum per row),
 // and the parts every tensor-core pass of this library shares -- PTX wrappers, the shared-memory
 // and barrier map (tc::Pipe), the TMA producer and the MMA issuer (tc::producer_role,
-// tc::mma_role).  The prefill path runs score_fast.cuh first and this kernel as its repair
-// launch; with SHOTKV_SCORING_EXACT this kernel does all the work.
+// tc::mma_role).  The prefill path runs score_fast.cuh or score_stream.cuh, which come back to the
+// epilogue of this file (tc::repair_items) for the items whose sums left their range; with
+// SHOTKV_SCORING_EXACT the kernel of this file does all the work.
 //
 // Persistent CTAs, one per SM, each owning a contiguous range of work items.  An item is one
 // (unit, chunk): unit = prompt x layer x kv head, chunk = a run of whole 128-key tiles of that
@@ -50,12 +51,11 @@ struct ScoreTcParams {
     int* err;             // error word (host-visible); set to 1 when a bounded wait gave up
     long long wait_cycles;    // limit of every bounded wait, in SM clock cycles
     long long* clk;           // optional (host-visible): SM cycle counter and nanosecond timer of CTA 0 at kernel start and end
-    // Item filter.  Each of the eight epilogue warps of the fast and streaming kernels writes its byte
-    // of redo[item]: 1 when a sum of its rows left the fp32 range it works in, else 0 (so the array
-    // needs no clearing); the exact kernel, given the same array, recomputes the items with any byte
-    // set and returns at once when there is none.  NULL: every item is done.
+    // Each of the eight epilogue warps of the fast and streaming kernels writes its byte of redo[item]:
+    // 1 when a sum of its rows left the fp32 range it works in, else 0 (so the array needs no clearing).
+    // The items with any byte set are recomputed with a running maximum at the end of the same kernel.
     unsigned long long* redo;   // [total_items]
-    int* repaired;        // host-visible count of items recomputed under the filter (diagnostic)
+    int* repaired;        // host-visible count of items recomputed (diagnostic)
 };
 
 template <int D, int MB>
@@ -68,8 +68,8 @@ struct ScoreTcCfg {
     static constexpr int kBarBytes = 1024;
     static constexpr int kCombBytes = 2 * 4 * 128 * 2 * 4;   // [parity][slice][row][m, z]
     static constexpr int kSmemBytes = kQBytes + kStages * kStageBytes + kBarBytes + kCombBytes + 1024;
-    static constexpr int kSlices = 4 / MB;                    // column slices of a tile, one per epilogue warpgroup
-    static constexpr int kThreads = 128 + 16 * 32;            // producer, MMA issuer, two idle warps; 16 epilogue warps
+    static constexpr int kEpiWarps = 16;
+    static constexpr int kThreads = 128 + kEpiWarps * 32;     // producer, MMA issuer, two idle warps; epilogue
 };
 
 namespace tc {
@@ -342,8 +342,41 @@ struct Pipe {
     __device__ __forceinline__ uint32_t tempty(int a, int b) const { return sBar + 8u * (2 * NST + 6 + a * 2 + b); }
     __device__ __forceinline__ uint32_t tmem_slot() const { return sBar + 8u * (2 * NST + 10); }
     __device__ __forceinline__ uint32_t extra_bar(int i) const { return sBar + 256u + 8u * i; }
+    // set by an epilogue warp that marked an item for recomputation; read behind a barrier of the CTA
+    __device__ __forceinline__ volatile int* repair_flag() const { return abort_flag + 1; }
 };
 
+// One thread: the barriers at their initial state (arguments as for pipe_setup).
+template <class Cfg>
+__device__ __forceinline__ void pipe_init_barriers(const Pipe<Cfg>& pp, int tempty_arrivals, int extra, int mma_threads) {
+    for (int s = 0; s < Cfg::kStages; ++s) {
+        mbar_init(pp.full(s), 1);
+        mbar_init(pp.empty(s), 1);
+    }
+    mbar_init(pp.qfull(), 1);
+    mbar_init(pp.qempty(), mma_threads);
+    for (int a = 0; a < 2; ++a)
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(pp.tfull(a, b), 1);
+            mbar_init(pp.tempty(a, b), tempty_arrivals);
+        }
+    for (int i = 0; i < extra; ++i) mbar_init(pp.extra_bar(i), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+// Where everything lies in the CTA's shared memory; returns the word that holds the address of its tensor memory.
+template <class Cfg>
+__device__ __forceinline__ volatile uint32_t* pipe_map(Pipe<Cfg>& pp, unsigned char* smem_raw) {
+    const uint32_t raw_addr = smem_u32(smem_raw);
+    const uint32_t base = (raw_addr + 1023u) & ~1023u;
+    unsigned char* gbase = smem_raw + (base - raw_addr);
+    pp.sQ = base;
+    pp.sK = base + Cfg::kQBytes;
+    pp.sBar = pp.sK + Cfg::kStages * Cfg::kStageBytes;
+    volatile uint32_t* tmem_slot_g = reinterpret_cast<volatile uint32_t*>(gbase + (pp.tmem_slot() - base));
+    pp.abort_flag = reinterpret_cast<volatile int*>(gbase + (pp.tmem_slot() - base) + 4);
+    return tmem_slot_g;
+}
 // Barrier set-up, tensor-memory allocation and the CTA-wide hand-over of its address.  Called by
 // every thread; `tempty_arrivals` = epilogue warps that release one (buffer, row block).
 // `extra` further barriers of one arrival each are initialised from pp.extra_bar(0) on.
@@ -351,30 +384,11 @@ struct Pipe {
 template <class Cfg>
 __device__ __forceinline__ void pipe_setup(Pipe<Cfg>& pp, unsigned char* smem_raw, int tempty_arrivals, int extra = 0,
                                            int mma_threads = 1) {
-    constexpr int NST = Cfg::kStages;
-    const uint32_t raw_addr = smem_u32(smem_raw);
-    const uint32_t base = (raw_addr + 1023u) & ~1023u;
-    unsigned char* gbase = smem_raw + (base - raw_addr);
-    pp.sQ = base;
-    pp.sK = base + Cfg::kQBytes;
-    pp.sBar = pp.sK + NST * Cfg::kStageBytes;
-    volatile uint32_t* tmem_slot_g = reinterpret_cast<volatile uint32_t*>(gbase + (pp.tmem_slot() - base));
-    pp.abort_flag = reinterpret_cast<volatile int*>(gbase + (pp.tmem_slot() - base) + 4);
+    volatile uint32_t* tmem_slot_g = pipe_map(pp, smem_raw);
     if (threadIdx.x == 0) {
-        for (int s = 0; s < NST; ++s) {
-            mbar_init(pp.full(s), 1);
-            mbar_init(pp.empty(s), 1);
-        }
-        mbar_init(pp.qfull(), 1);
-        mbar_init(pp.qempty(), mma_threads);
-        for (int a = 0; a < 2; ++a)
-            for (int b = 0; b < 2; ++b) {
-                mbar_init(pp.tfull(a, b), 1);
-                mbar_init(pp.tempty(a, b), tempty_arrivals);
-            }
-        for (int i = 0; i < extra; ++i) mbar_init(pp.extra_bar(i), 1);
         *pp.abort_flag = 0;
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        *pp.repair_flag() = 0;
+        pipe_init_barriers(pp, tempty_arrivals, extra, mma_threads);
     }
     if ((threadIdx.x >> 5) == 0) {
         tmem_alloc(pp.tmem_slot(), 512);
@@ -393,7 +407,7 @@ __device__ __forceinline__ float* pipe_scratch(const Pipe<Cfg>& pp, unsigned cha
 }
 
 // One thread: the unit's window queries (once per unit) and K tiles of 128 keys into the ring.
-// FILTERED: skip the items whose redo flag is clear (the exact kernel's repair launches).
+// FILTERED: skip the items whose redo flag is clear (repair_items).
 // QKMAJOR: lay Q out k-block major (all rows of one 64-element k block contiguous), as a B
 // operand of more than 128 rows needs; otherwise row-block major (each 128-row block contiguous).
 template <int D, int MB, bool FILTERED, bool QKMAJOR, class Cfg>
@@ -405,7 +419,7 @@ __device__ __forceinline__ void producer_role(const Pipe<Cfg>& pp, const CUtenso
     uint32_t ephase = 1, qephase = 1;
     bool ok = true;
     for (int it = item_begin; it < item_end && ok; ++it) {
-        if (FILTERED && p.redo && !p.redo[it]) continue;
+        if (FILTERED && !p.redo[it]) continue;
         const int u = it / p.nchunk, j = it - u * p.nchunk;
         const int lo = j * p.chunk_keys, hi = min(p.N, lo + p.chunk_keys);
         const int nt = (hi - lo + TN - 1) / TN;
@@ -470,7 +484,7 @@ __device__ __forceinline__ void mma_role(const Pipe<Cfg>& pp, const ScoreTcParam
     uint32_t fphase = 0, qfphase = 0, tephase0 = 1, tephase1 = 1;
     bool ok = true;
     for (int it = item_begin; it < item_end && ok; ++it) {
-        if (FILTERED && p.redo && !p.redo[it]) continue;
+        if (FILTERED && !p.redo[it]) continue;
         const int u = it / p.nchunk, j = it - u * p.nchunk;
         const int lo = j * p.chunk_keys, hi = min(p.N, lo + p.chunk_keys);
         const int nt = (hi - lo + TN - 1) / TN;
@@ -513,6 +527,188 @@ __device__ __forceinline__ void mma_role(const Pipe<Cfg>& pp, const ScoreTcParam
     }
 }
 
+// The epilogue with a true running maximum, run by the EW warps from warp 4 on: a thread is one window
+// row and one of 4 * MB / EW-th parts (a column slice) of every tile.  `comb`: the scratch in which a row's
+// slices are merged, [parity][warpgroup][row][m, z] (not used when a thread owns whole rows).
+// FILTERED: skip the items whose redo flag is clear.
+template <int D, int MB, int EW, bool FILTERED, class Cfg>
+__device__ __forceinline__ void exact_epilogue(const Pipe<Cfg>& pp, float* comb, const ScoreTcParams& p, const ShotTable& tab,
+                                               int item_begin, int item_end) {
+    constexpr int TN = kTileKeys;
+    constexpr int NSL = EW / 4 / MB, SLW = TN / NSL, NCH = SLW / 32;      // slices, slice width, chunks per slice
+    // a warp may touch the 32 tensor-memory lanes given by its index modulo 4; any four
+    // consecutive warps cover all 128 rows of a block
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int g = (warp - 4) >> 2, quad = warp & 3;
+    const int blk = g / NSL;                           // 128-row block of Q
+    const int slice = g % NSL;                         // column slice of every tile
+    const int lrow = quad * 32 + lane;
+    const int row = blk * 128 + lrow;
+    const int plim = row < p.R ? p.N - p.W + (row % p.W) : p.N - 1;
+    const float scale = p.scale_log2;
+    const int units_per_prompt = p.L * p.Hkv;
+    int acc = 0, nflush = 0, ndone = 0;
+    uint32_t tfphase0 = 0, tfphase1 = 0;
+    bool ok = true;
+    for (int it = item_begin; it < item_end && ok; ++it) {
+        if (FILTERED) {
+            if (!p.redo[it]) continue;
+            ++ndone;
+        }
+        const int u = it / p.nchunk, j = it - u * p.nchunk;
+        const int lo = j * p.chunk_keys, hi = min(p.N, lo + p.chunk_keys);
+        const int nt = (hi - lo + TN - 1) / TN;
+        const int* o = table_row(tab, u / units_per_prompt);
+        int sg = count_le_warp(o, p.S + 1, lo);            // segment of the current piece
+        int pend = o[sg];                                  // its end
+        float m_ref = SHOTKV_NEG_INF, z = 0.f;
+        const int plain_end = min(hi, p.N - p.W + 1);      // keys below this count for every window row
+
+        // the current piece is complete for this thread's columns: merge the row's slices, write, move on
+        auto flush = [&]() {
+            // slot of warpgroup g' and local row r: comb[parity][g'][r][m, z]; a row's slices are the
+            // NSL consecutive warpgroups starting at its leader (slice 0)
+            float* slot = comb + (nflush & 1) * (EW / 4 * 256) + (g - slice) * 256 + lrow * 2;
+            if (slice != 0) {
+                slot[slice * 256] = m_ref;
+                slot[slice * 256 + 1] = z;
+            }
+            if (NSL > 1) {
+                if (blk == 0) asm volatile("bar.sync 1, %0;" ::"n"(NSL * 128) : "memory");
+                else asm volatile("bar.sync 2, %0;" ::"n"(NSL * 128) : "memory");
+            }
+            if (slice == 0) {
+                float mm = m_ref;
+#pragma unroll
+                for (int s = 1; s < NSL; ++s) mm = fmaxf(mm, slot[s * 256]);
+                const float mu = mm == SHOTKV_NEG_INF ? 0.f : mm;
+                float zz = z * ex2f(m_ref - mu);
+#pragma unroll
+                for (int s = 1; s < NSL; ++s) zz += slot[s * 256 + 1] * ex2f(slot[s * 256] - mu);
+                const size_t o = ((size_t)u * p.P + sg + j) * p.Rpad + row;
+                const bool live = row < p.R;        // padding rows: their Q was never loaded
+                p.part_m[o] = live ? mm : 0.f;
+                p.part_z[o] = live ? zz : 0.f;
+            }
+            z = 0.f;
+            ++nflush;
+            ++sg;
+            pend = o[sg];
+        };
+
+        // 32 columns of this thread's row, starting at key kc0
+        auto chunk = [&](uint32_t (&r)[32], int kc0) {
+            while (pend <= kc0) flush();
+            const int lim = min(hi, plim + 1) - kc0;                 // columns of the chunk that count
+            if (!__all_sync(0xffffffffu, lim >= 32)) mask32(r, lim);   // end of the keys, or the causal window
+            const float cm = max32(r) * scale;
+            if (cm > m_ref + 8.f) {                                   // also the first time (m_ref = -inf, z = 0)
+                z *= ex2f(m_ref - cm);
+                m_ref = cm;
+            }
+            const float neg = m_ref == SHOTKV_NEG_INF ? 0.f : -m_ref;
+            if (pend >= kc0 + 32) {                                   // no piece ends inside the chunk
+                z += expsum32(r, scale, neg);
+                return;
+            }
+            exp32(r, scale, neg);
+            const int pend2 = o[sg + 1];
+            if (pend2 >= kc0 + 32) {                                  // exactly one boundary: one predicated pass
+                float lo_s, hi_s;
+                split32(r, pend - kc0, lo_s, hi_s);
+                z += lo_s;
+                flush();
+                z = hi_s;
+            } else {                                                  // several short pieces: general walk
+                int start = 0;
+                while (pend < kc0 + 32) {
+                    const int e = pend - kc0;
+                    z += range32(r, start, e);
+                    start = e;
+                    flush();
+                }
+                z += range32(r, start, 32);
+            }
+        };
+
+        for (int t = 0; t < nt; ++t) {
+            const uint32_t tph = acc ? tfphase1 : tfphase0;
+            ok = lane == 0 ? mbar_wait(pp.tfull(acc, blk), tph, pp.abort_flag, p.err, p.wait_cycles) : true;   // one poller per warp
+            ok = __shfl_sync(0xffffffffu, ok, 0);
+            if (!ok) break;
+            if (acc) tfphase1 ^= 1; else tfphase0 ^= 1;
+            fence_after_sync();
+            const int kc0 = lo + t * TN + slice * SLW;
+            const uint32_t taddr = pp.tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)((acc * MB + blk) * TN + slice * SLW);
+            while (pend <= kc0) flush();
+            uint32_t r[32];
+#pragma unroll
+            for (int c = 0; c < NCH; ++c) {
+                tmem_ld32_sync(r, taddr + c * 32);
+                if (c == NCH - 1) {                                   // the last of this tile's accumulators are in registers
+                    fence_before_sync();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(pp.tempty(acc, blk));
+                }
+                // most chunks: every column counts for every row (it lies before the item's end and
+                // before the first window position) and no piece ends at or inside the chunk
+                if (kc0 + c * 32 + 32 <= min(pend, plain_end)) {
+                    const float cm = max32(r) * scale;
+                    if (cm > m_ref + 8.f) {
+                        z *= ex2f(m_ref - cm);
+                        m_ref = cm;
+                    }
+                    z += expsum32(r, scale, -m_ref);
+                } else {
+                    chunk(r, kc0 + c * 32);
+                }
+            }
+            acc ^= 1;
+        }
+        if (!ok) break;
+        while (pend < hi) flush();                         // boundaries behind this slice's last column
+        flush();                                           // the piece that the item's end cuts
+    }
+    // one addition across the bus a CTA (one for every item took 0.85 us each, more than the item itself)
+    if (FILTERED && warp == 4 && lane == 0) atomicAdd(p.repaired, ndone);
+}
+
+// Barriers of the repair pass, behind those of the pass before it (which may still be receiving the
+// last commits): bytes from the start of the barrier area.
+constexpr uint32_t kRepairBars = 512;
+
+// The end of the fast and streaming kernels, for a CTA that marked an item of its own: recomputes its
+// marked items with a running maximum, over the same shared memory, tensor memory and output arrays.
+// Called by all threads behind a barrier of the CTA, once every accumulator of the pass before has been
+// read.  Inside the kernel that found them: as a launch of its own (which nearly always found nothing to do) it cost
+// one layer of a 4K prompt 22.4 us a call against 18.5, one small layer of 512 tokens 20.2 against 16.2.  Not inlined, and handed nothing that
+// would have to be kept through the pass before it: the streaming kernel has no register to spare.
+template <int D, int MB, int EW, class Cfg>
+__device__ __noinline__ void repair_items(unsigned char* smem_raw, const CUtensorMap* tmQ, const CUtensorMap* tmK, int q_box_rows,
+                                          int k_box_rows, const ScoreTcParams& p, const ShotTable& tab) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long total = p.total_items;
+    const int item_begin = (int)(total * blockIdx.x / gridDim.x);
+    const int item_end = (int)(total * (blockIdx.x + 1) / gridDim.x);
+    Pipe<Cfg> pp;
+    pp.tmem_base = *pipe_map(pp, smem_raw);
+    float* comb = pipe_scratch(pp, smem_raw);
+    pp.sBar += kRepairBars;
+    if (threadIdx.x == 0) pipe_init_barriers(pp, EW / MB, 0, 1);
+    fence_before_sync();
+    __syncthreads();
+    fence_after_sync();
+    if (warp == 0) {
+        if (lane == 0) producer_role<D, MB, true, false>(pp, tmQ, tmK, q_box_rows, k_box_rows, p, item_begin, item_end);
+    } else if (warp == 1) {
+        if (lane == 0) mma_role<D, MB, true, 1>(pp, p, item_begin, item_end, 0);
+    } else if (warp >= 4) {
+        exact_epilogue<D, MB, EW, true>(pp, comb, p, tab, item_begin, item_end);
+    }
+    fence_before_sync();
+    __syncthreads();
+}
+
 }  // namespace tc
 
 template <int D, int MB>
@@ -520,166 +716,23 @@ __global__ void __launch_bounds__(ScoreTcCfg<D, MB>::kThreads, 1)
     score_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK, const int q_box_rows,
                     const int k_box_rows, const ScoreTcParams p, const __grid_constant__ ShotTable tab) {
     using Cfg = ScoreTcCfg<D, MB>;
-    constexpr int TN = tc::kTileKeys;
-    constexpr int NSL = Cfg::kSlices, SLW = TN / NSL, NCH = SLW / 32;     // slices, slice width, chunks per slice
     extern __shared__ unsigned char smem_raw[];
     const long long total = p.total_items;
     const int item_begin = (int)(total * blockIdx.x / gridDim.x);
     const int item_end = (int)(total * (blockIdx.x + 1) / gridDim.x);
     grid_release();
     grid_wait();
-    if (p.redo) {                                      // repair launch: nothing to repair in this CTA's items?
-        bool any = false;
-        for (int i = item_begin + threadIdx.x; i < item_end; i += blockDim.x) any |= p.redo[i] != 0;
-        if (!__syncthreads_or(any)) return;
-    }
     tc::stamp(p.clk, 0);
     tc::Pipe<Cfg> pp;
-    tc::pipe_setup(pp, smem_raw, 16 / MB);
-    float* comb = tc::pipe_scratch(pp, smem_raw);     // [2][4][128][2]
-    const uint32_t tmem_base = pp.tmem_base;
-    volatile int* abort_flag = pp.abort_flag;
-    auto bar_tfull = [&](int a, int b) { return pp.tfull(a, b); };
-    auto bar_tempty = [&](int a, int b) { return pp.tempty(a, b); };
+    tc::pipe_setup(pp, smem_raw, Cfg::kEpiWarps / MB);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-
     if (warp == 0) {
-        if (lane == 0) tc::producer_role<D, MB, true, false>(pp, &tmQ, &tmK, q_box_rows, k_box_rows, p, item_begin, item_end);
+        if (lane == 0) tc::producer_role<D, MB, false, false>(pp, &tmQ, &tmK, q_box_rows, k_box_rows, p, item_begin, item_end);
     } else if (warp == 1) {
-        if (lane == 0) tc::mma_role<D, MB, true, 1>(pp, p, item_begin, item_end, 0);
+        if (lane == 0) tc::mma_role<D, MB, false, 1>(pp, p, item_begin, item_end, 0);
     } else if (warp >= 4) {
-        // ------------------------------------------------------------------ epilogue
-        // a warp may touch the 32 tensor-memory lanes given by its index modulo 4; any four
-        // consecutive warps cover all 128 rows of a block
-        const int g = (warp - 4) >> 2, quad = warp & 3;
-        const int blk = MB == 2 ? (g >> 1) : 0;            // 128-row block of Q
-        const int slice = MB == 2 ? (g & 1) : g;           // column slice of every tile
-        const int lrow = quad * 32 + lane;
-        const int row = blk * 128 + lrow;
-        const int plim = row < p.R ? p.N - p.W + (row % p.W) : p.N - 1;
-        const float scale = p.scale_log2;
-        const int units_per_prompt = p.L * p.Hkv;
-        int acc = 0, nflush = 0;
-        uint32_t tfphase0 = 0, tfphase1 = 0;
-        bool ok = true;
-        for (int it = item_begin; it < item_end && ok; ++it) {
-            if (p.redo) {
-                if (!p.redo[it]) continue;
-                if (warp == 4 && lane == 0) atomicAdd(p.repaired, 1);
-            }
-            const int u = it / p.nchunk, j = it - u * p.nchunk;
-            const int lo = j * p.chunk_keys, hi = min(p.N, lo + p.chunk_keys);
-            const int nt = (hi - lo + TN - 1) / TN;
-            const int* o = table_row(tab, u / units_per_prompt);
-            int sg = count_le_warp(o, p.S + 1, lo);            // segment of the current piece
-            int pend = o[sg];                                  // its end
-            float m_ref = SHOTKV_NEG_INF, z = 0.f;
-            const int plain_end = min(hi, p.N - p.W + 1);      // keys below this count for every window row
-
-            // the current piece is complete for this thread's columns: merge the row's slices, write, move on
-            auto flush = [&]() {
-                // slot of warpgroup g' and local row r: comb[parity][g'][r][m, z]; a row's slices are the
-                // NSL consecutive warpgroups starting at its leader (slice 0)
-                float* slot = comb + (nflush & 1) * 1024 + (g - slice) * 256 + lrow * 2;
-                if (slice != 0) {
-                    slot[slice * 256] = m_ref;
-                    slot[slice * 256 + 1] = z;
-                }
-                if (blk == 0) asm volatile("bar.sync 1, %0;" ::"n"(NSL * 128) : "memory");
-                else asm volatile("bar.sync 2, %0;" ::"n"(NSL * 128) : "memory");
-                if (slice == 0) {
-                    float mm = m_ref;
-#pragma unroll
-                    for (int s = 1; s < NSL; ++s) mm = fmaxf(mm, slot[s * 256]);
-                    const float mu = mm == SHOTKV_NEG_INF ? 0.f : mm;
-                    float zz = z * ex2f(m_ref - mu);
-#pragma unroll
-                    for (int s = 1; s < NSL; ++s) zz += slot[s * 256 + 1] * ex2f(slot[s * 256] - mu);
-                    const size_t o = ((size_t)u * p.P + sg + j) * p.Rpad + row;
-                    const bool live = row < p.R;        // padding rows: their Q was never loaded
-                    p.part_m[o] = live ? mm : 0.f;
-                    p.part_z[o] = live ? zz : 0.f;
-                }
-                z = 0.f;
-                ++nflush;
-                ++sg;
-                pend = o[sg];
-            };
-
-            // 32 columns of this thread's row, starting at key kc0
-            auto chunk = [&](uint32_t (&r)[32], int kc0) {
-                while (pend <= kc0) flush();
-                const int lim = min(hi, plim + 1) - kc0;                 // columns of the chunk that count
-                if (!__all_sync(0xffffffffu, lim >= 32)) tc::mask32(r, lim);   // end of the keys, or the causal window
-                const float cm = tc::max32(r) * scale;
-                if (cm > m_ref + 8.f) {                                   // also the first time (m_ref = -inf, z = 0)
-                    z *= ex2f(m_ref - cm);
-                    m_ref = cm;
-                }
-                const float neg = m_ref == SHOTKV_NEG_INF ? 0.f : -m_ref;
-                if (pend >= kc0 + 32) {                                   // no piece ends inside the chunk
-                    z += tc::expsum32(r, scale, neg);
-                    return;
-                }
-                tc::exp32(r, scale, neg);
-                const int pend2 = o[sg + 1];
-                if (pend2 >= kc0 + 32) {                                  // exactly one boundary: one predicated pass
-                    float lo_s, hi_s;
-                    tc::split32(r, pend - kc0, lo_s, hi_s);
-                    z += lo_s;
-                    flush();
-                    z = hi_s;
-                } else {                                                  // several short pieces: general walk
-                    int start = 0;
-                    while (pend < kc0 + 32) {
-                        const int e = pend - kc0;
-                        z += tc::range32(r, start, e);
-                        start = e;
-                        flush();
-                    }
-                    z += tc::range32(r, start, 32);
-                }
-            };
-
-            for (int t = 0; t < nt; ++t) {
-                const uint32_t tph = acc ? tfphase1 : tfphase0;
-                ok = lane == 0 ? tc::mbar_wait(bar_tfull(acc, blk), tph, abort_flag, p.err, p.wait_cycles) : true;   // one poller per warp
-                ok = __shfl_sync(0xffffffffu, ok, 0);
-                if (!ok) break;
-                if (acc) tfphase1 ^= 1; else tfphase0 ^= 1;
-                tc::fence_after_sync();
-                const int kc0 = lo + t * TN + slice * SLW;
-                const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16) + (uint32_t)((acc * MB + blk) * TN + slice * SLW);
-                while (pend <= kc0) flush();
-                uint32_t r[32];
-#pragma unroll
-                for (int c = 0; c < NCH; ++c) {
-                    tc::tmem_ld32_sync(r, taddr + c * 32);
-                    if (c == NCH - 1) {                                   // the last of this tile's accumulators are in registers
-                        tc::fence_before_sync();
-                        __syncwarp();
-                        if (lane == 0) tc::mbar_arrive(bar_tempty(acc, blk));
-                    }
-                    // most chunks: every column counts for every row (it lies before the item's end and
-                    // before the first window position) and no piece ends at or inside the chunk
-                    if (kc0 + c * 32 + 32 <= min(pend, plain_end)) {
-                        const float cm = tc::max32(r) * scale;
-                        if (cm > m_ref + 8.f) {
-                            z *= ex2f(m_ref - cm);
-                            m_ref = cm;
-                        }
-                        z += tc::expsum32(r, scale, -m_ref);
-                    } else {
-                        chunk(r, kc0 + c * 32);
-                    }
-                }
-                acc ^= 1;
-            }
-            if (!ok) break;
-            while (pend < hi) flush();                         // boundaries behind this slice's last column
-            flush();                                           // the piece that the item's end cuts
-        }
+        tc::exact_epilogue<D, MB, Cfg::kEpiWarps, false>(pp, tc::pipe_scratch(pp, smem_raw), p, tab, item_begin, item_end);
     }
 
     tc::fence_before_sync();
@@ -688,7 +741,7 @@ __global__ void __launch_bounds__(ScoreTcCfg<D, MB>::kThreads, 1)
     if (warp == 0) {
         __syncwarp();
         tc::fence_after_sync();
-        tc::tmem_dealloc(tmem_base, 512);
+        tc::tmem_dealloc(pp.tmem_base, 512);
     }
 }
 

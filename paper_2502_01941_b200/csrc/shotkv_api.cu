@@ -236,7 +236,7 @@ struct PrefillWs {
     float* row_m;      // [U][Rpad]
     float* row_invz;
     float* imp;        // [U][N] per-token importances of the fused call's per-token route (absent otherwise)
-    unsigned long long* redo;   // [U * kMaxChunks] not 0 for the items the exact kernel must recompute
+    unsigned long long* redo;   // [U * kMaxChunks] not 0 for the items recomputed with a running maximum
     size_t total;
 };
 
@@ -528,16 +528,11 @@ int launch_score_tc(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q,
     const int qbox = t.qbox, kbox = t.kbox;
     ScoreTcParams& sp = t.sp;
     const bool big = sp.Rpad == 256;
-    int rc = SHOTKV_OK;
-    sp.clk = (long long*)(ctx->err_dev + 8);        // the first launch below stamps its clocks; a repair launch after it does not
+    sp.clk = (long long*)(ctx->err_dev + 8);
     if (ctx->scoring_mode == SHOTKV_SCORING_FAST) {
-        // fast kernel first; it marks the items whose sums left its range, and the exact kernel
-        // below then redoes exactly those (returning at once when there is none)
         sp.redo = w.redo;
-        if (d->d == 128) rc = big ? launch_score_stream_t<128>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream) : launch_score_fast_t<128>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream);
-        else rc = big ? launch_score_stream_t<64>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream) : launch_score_fast_t<64>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream);
-        if (rc) return rc;
-        sp.clk = nullptr;
+        if (d->d == 128) return big ? launch_score_stream_t<128>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream) : launch_score_fast_t<128>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream);
+        return big ? launch_score_stream_t<64>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream) : launch_score_fast_t<64>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream);
     }
     if (d->d == 128) return big ? launch_score_tc_t<128, 2>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream) : launch_score_tc_t<128, 1>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream);
     return big ? launch_score_tc_t<64, 2>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream) : launch_score_tc_t<64, 1>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream);

@@ -42,3 +42,23 @@ def test_token_importance_at_edges_of_32_row_chunks(G, W):
     assert gpu["token_importance"] is not None
     P.check_all_units(gpu, Q, K, V, off, cfg.r_p, check_tokens=True)
     ctx.close()
+
+
+@pytest.mark.parametrize("d,H,W", [(64, 16, 16), (128, 16, 24), (128, 32, 33), (64, 32, 64)], ids=["32_rows", "48_rows", "132_rows", "256_rows"])
+def test_some_of_the_items_of_every_cta_out_of_range(d, H, W):
+    """More units than SMs, two layers of every three with a key out of range: a CTA recomputes some of its
+    items, of several units, and leaves the others as they are."""
+    ctx = skv.Context(0)
+    cfg = wl.PrefillConfig("outliers", B=2, L=24, H=H, Hkv=8, d=d, N=1100, W=W, S=4, shot_dist="uniform", shot_lo=150,
+                           shot_hi=300, question_len=100, r_p=0.5, cfg_id=25)
+    Q, K, V, off = wl.prefill_batch(cfg, "cuda")
+    Q[..., 0], K[..., 0] = 8.0, 0.0
+    _, chunk_keys, _ = skv.shotkv_plan_pieces(P.dims_of(cfg), off)
+    assert chunk_keys >= 256, "the case needs work items of at least two tiles"
+    t = min(chunk_keys, 1024) - 128 + 45         # in a later tile of every unit's first item
+    marked = [l for l in range(cfg.L) if l % 3 != 1]
+    K[:, marked, :, t, 0] = 250.0 * np.sqrt(d)   # logit 8 * 250 = 2000
+    gpu = P.gpu_prefill(ctx, P.dims_of(cfg), Q, K, V, off, cfg.r_p, 0, "fused")
+    assert skv.shotkv_repaired_items(ctx) == cfg.B * len(marked) * cfg.Hkv
+    P.check_all_units(gpu, Q, K, V, off, cfg.r_p)
+    ctx.close()
