@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libshotkv.so: argument marshalling only.
+"""Thin binding of libshotkv.so: argument marshalling only (ctypes, and for the calls made once per layer
+or per generated token the module built from csrc/marshal.cpp).
 
 Every function has the name and argument order of its C counterpart in
 `include/shotkv.h`; tensors are torch tensors whose data pointers are passed
@@ -12,6 +13,11 @@ import os
 
 import numpy as np
 import torch
+
+try:
+    from . import _marshal
+except ImportError:                     # not built: the ctypes path below serves every call
+    _marshal = None
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libshotkv.so")
@@ -61,11 +67,12 @@ class DecodeState(C.Structure):
 
 
 _lib = None
+_native = None      # _marshal, once it knows the library's functions
 
 
 def lib() -> C.CDLL:
     """Loads libshotkv.so (once).  Raises if it has not been built: there is no fallback."""
-    global _lib
+    global _lib, _native
     if _lib is not None:
         return _lib
     if not os.path.exists(LIB_PATH):
@@ -109,14 +116,20 @@ def lib() -> C.CDLL:
     for name, (res, args) in sig.items():
         fn = getattr(L, name)
         fn.restype, fn.argtypes = res, args
+    if _marshal is not None:
+        _marshal.init(Dims, Policy, DecodeState, *(C.cast(getattr(L, n), vp).value for n in (
+            "shotkv_prefill_score", "shotkv_select_shots", "shotkv_compact_kv", "shotkv_prefill_compress",
+            "shotkv_decode_step", "shotkv_decode_step_attend")))
+        _native = _marshal
     _lib = L
     return L
 
 
 # ------------------------------------------------------------------ marshalling helpers
 # A call on a small layer is a few launches of two microseconds each, so what happens here counts: the
-# checks below are one attribute each, pointers go to ctypes as plain ints, and the current stream is
-# asked for by its handle.
+# calls of a program's inner loops go through _native where their arguments are what it expects (it says
+# None where they are not), and the others' checks are one attribute each, with pointers as plain ints
+# and the current stream by its handle.
 def _bad(t, dtype, cuda, name):
     if not isinstance(t, torch.Tensor):
         raise TypeError(f"{name}: expected a torch tensor")
@@ -248,6 +261,10 @@ def shotkv_workspace_bytes(dims: Dims) -> int:
 
 
 def shotkv_prefill_score(ctx: Context, dims: Dims, Qwin, K, token_importance, ws, stream=None) -> int:
+    if _native is not None:
+        rc = _native.prefill_score(ctx._h, dims, Qwin, K, token_importance, ws, stream)
+        if rc is not None:
+            return ctx.check(rc)
     rc = lib().shotkv_prefill_score(ctx._h, C.byref(dims), _dev(Qwin, _BF16, "Qwin"),
                                     _dev(K, _BF16, "K"),
                                     _dev(token_importance, _F32, "token_importance"),
@@ -257,6 +274,11 @@ def shotkv_prefill_score(ctx: Context, dims: Dims, Qwin, K, token_importance, ws
 
 def shotkv_select_shots(ctx: Context, dims: Dims, policy: Policy, token_importance, offsets, shot_scores, keep,
                         kept_idx, kept_count, Mcap: int, ws, stream=None) -> int:
+    if _native is not None:
+        rc = _native.select_shots(ctx._h, dims, policy, token_importance, offsets, shot_scores, keep, kept_idx, kept_count,
+                                  Mcap, ws, stream)
+        if rc is not None:
+            return ctx.check(rc)
     o = _offsets(offsets)
     rc = lib().shotkv_select_shots(ctx._h, C.byref(dims), C.byref(policy),
                                    _dev(token_importance, _F32, "token_importance"),
@@ -288,6 +310,10 @@ def shotkv_select_shots_static(ctx: Context, dims: Dims, policy: Policy, token_i
 
 
 def shotkv_compact_kv(ctx: Context, dims: Dims, K, V, kept_idx, kept_count, Mcap: int, Kc, Vc, stream=None) -> int:
+    if _native is not None:
+        rc = _native.compact_kv(ctx._h, dims, K, V, kept_idx, kept_count, Mcap, Kc, Vc, stream)
+        if rc is not None:
+            return ctx.check(rc)
     rc = lib().shotkv_compact_kv(ctx._h, C.byref(dims), _dev(K, _BF16, "K"),
                                  _dev(V, _BF16, "V"),
                                  _dev(kept_idx, _I32, "kept_idx"),
@@ -300,6 +326,11 @@ def shotkv_compact_kv(ctx: Context, dims: Dims, K, V, kept_idx, kept_count, Mcap
 def shotkv_prefill_compress(ctx: Context, dims: Dims, policy: Policy, Qwin, K, V, offsets, shot_scores, keep,
                             kept_idx, kept_count, Mcap: int, Kc, Vc, token_importance, flags: int, ws,
                             stream=None) -> int:
+    if _native is not None:
+        rc = _native.prefill_compress(ctx._h, dims, policy, Qwin, K, V, offsets, shot_scores, keep, kept_idx, kept_count, Mcap,
+                                      Kc, Vc, token_importance, flags, ws, stream)
+        if rc is not None:
+            return ctx.check(rc)
     o = _offsets(offsets)
     rc = lib().shotkv_prefill_compress(
         ctx._h, C.byref(dims), C.byref(policy),
@@ -360,6 +391,10 @@ def shotkv_decode_init(ctx: Context, dims: Dims, policy: Policy, Dcap: int, Mcap
 
 
 def shotkv_decode_step(ctx: Context, state: DecodeState, q, k_new, v_new, Kc, kept_count, stream=None) -> int:
+    if _native is not None:
+        rc = _native.decode_step(ctx._h, state, q, k_new, v_new, Kc, kept_count, stream)
+        if rc is not None:
+            return ctx.check(rc)
     rc = lib().shotkv_decode_step(ctx._h, C.byref(state), _dev(q, _BF16, "q"),
                                   _dev(k_new, _BF16, "k_new"),
                                   _dev(v_new, _BF16, "v_new"),
@@ -370,6 +405,10 @@ def shotkv_decode_step(ctx: Context, state: DecodeState, q, k_new, v_new, Kc, ke
 
 def shotkv_decode_step_attend(ctx: Context, state: DecodeState, q, k_new, v_new, Kc, Vc, kept_count, attn_out,
                               stream=None) -> int:
+    if _native is not None:
+        rc = _native.decode_step_attend(ctx._h, state, q, k_new, v_new, Kc, Vc, kept_count, attn_out, stream)
+        if rc is not None:
+            return ctx.check(rc)
     rc = lib().shotkv_decode_step_attend(ctx._h, C.byref(state), _dev(q, _BF16, "q"),
                                          _dev(k_new, _BF16, "k_new"),
                                          _dev(v_new, _BF16, "v_new"),

@@ -1,14 +1,18 @@
-"""Builds libshotkv.so (the C-ABI library) in-tree with nvcc for sm_100a."""
+"""Builds in-tree libshotkv.so (the C-ABI library) with nvcc for sm_100a, and _marshal.so (the binding's
+argument marshalling) with the host compiler."""
 from __future__ import annotations
 
 import os
+import shutil
 import subprocess
 import sys
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libshotkv.so")
+MARSHAL_PATH = os.path.join(PKG_DIR, "_marshal.so")
 SOURCES = ["shotkv_api.cu"]
+MARSHAL_SOURCE = os.path.join(CSRC, "marshal.cpp")
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-O3", "-std=c++17", "-lineinfo",
     "-Xcompiler", "-fPIC,-fvisibility=hidden", "--expt-relaxed-constexpr",
@@ -23,28 +27,48 @@ def _nvcc() -> str:
     return "nvcc"
 
 
-def _stale() -> bool:
-    if not os.path.exists(LIB_PATH):
+def _stale(target: str, sources: list) -> bool:
+    if not os.path.exists(target):
         return True
-    t = os.path.getmtime(LIB_PATH)
-    deps = [os.path.join(CSRC, f) for f in os.listdir(CSRC)]
-    deps.append(os.path.join(PKG_DIR, "..", "include", "shotkv.h"))
-    return any(os.path.getmtime(p) > t for p in deps)
+    t = os.path.getmtime(target)
+    return any(os.path.getmtime(p) > t for p in sources + [os.path.join(PKG_DIR, "..", "include", "shotkv.h")])
+
+
+def _run(cmd: list, what: str) -> subprocess.CompletedProcess:
+    res = subprocess.run(cmd, capture_output=True, text=True)
+    if res.returncode != 0:
+        sys.stderr.write(res.stdout + res.stderr)
+        raise RuntimeError(f"{cmd[0]} failed building {what}")
+    return res
+
+
+def build_marshal(force: bool = False) -> str:
+    """Compile the marshalling module next to this file, against the installed torch; returns its path."""
+    if not force and not _stale(MARSHAL_PATH, [MARSHAL_SOURCE]):
+        return MARSHAL_PATH
+    import sysconfig
+
+    import torch
+    root = os.path.join(os.path.dirname(torch.__file__), "")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(shutil.which(_nvcc()) or _nvcc()))), "include")
+    include = [root + "include", root + "include/torch/csrc/api/include", cuda, sysconfig.get_paths()["include"]]
+    _run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
+          f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(x for i in include for x in ("-isystem", i)),
+          MARSHAL_SOURCE, "-o", MARSHAL_PATH, f"-L{root}lib", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"],
+         "_marshal.so")
+    return MARSHAL_PATH
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
     """Compile the CUDA sources into `libshotkv.so` next to this file; returns its path."""
-    if not force and not _stale():
+    build_marshal(force)
+    if not force and not _stale(LIB_PATH, [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".cpp")]):
         return LIB_PATH
     cmd = [_nvcc(), *NVCC_FLAGS]
     if verbose:
         cmd += ["-Xptxas", "-v"]
     cmd += [os.path.join(CSRC, s) for s in SOURCES]
-    cmd += ["-o", LIB_PATH]
-    res = subprocess.run(cmd, capture_output=True, text=True)
-    if res.returncode != 0:
-        sys.stderr.write(res.stdout + res.stderr)
-        raise RuntimeError("nvcc failed building libshotkv.so")
+    res = _run(cmd + ["-o", LIB_PATH], "libshotkv.so")
     if verbose:
         sys.stderr.write(res.stderr)
     return LIB_PATH
