@@ -50,7 +50,7 @@ struct ScoreTcParams {
     float* item_z;        //                     written by the kernels that fix a reference per item
     int* err;             // error word (host-visible); set to 1 when a bounded wait gave up
     long long wait_cycles;    // limit of every bounded wait, in SM clock cycles
-    long long* clk;           // optional (host-visible): SM cycle counter and nanosecond timer of CTA 0 at kernel start and end
+    long long* clk;           // optional: SM cycle counter and nanosecond timer of CTA 0 at kernel start and end
     // Each of the eight epilogue warps of the fast and streaming kernels writes its byte of redo[item]:
     // 1 when a sum of its rows left the fp32 range it works in, else 0 (so the array needs no clearing).
     // The items with any byte set are recomputed with a running maximum at the end of the same kernel.

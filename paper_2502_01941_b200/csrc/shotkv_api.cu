@@ -38,7 +38,7 @@ constexpr int kMaxGroups = 4;         // most groups the fused prefill call pipe
 // write-back, which runs beside the next group's upload: K of 4 MB in 1, 2, 4 groups 211, 222, 250 us; 34 MB
 // in 1 or 2 1,152 and 1,046; 134 MB in 1, 2, 4 3,702, 3,474 and 3,346.
 constexpr double kMinGroupKBytes = 16.0 * 1024 * 1024;
-constexpr int kErrWords = 16;          // ints of host-mapped memory the kernels report through
+constexpr int kErrWords = 8;           // ints of host-mapped memory the kernels report through
 constexpr int kBigSmem = 200 * 1024;   // dynamic shared memory the small kernels are allowed (set once per context)
 
 inline size_t align_up(size_t x, size_t a = 256) { return (x + a - 1) / a * a; }
@@ -81,6 +81,8 @@ struct shotkv_ctx {
     // error word that kernels with bounded waits raise; pinned host memory mapped into the device
     int* err_host = nullptr;
     int* err_dev = nullptr;
+    long long* clk = nullptr;                  // device memory: four clock stamps of the last scoring launch
+    bool scored = false;                       // there has been one
     int sm_count = 148;
     int scoring_mode = SHOTKV_SCORING_FAST;
     long long wait_cycles = tc::kWaitCycles;   // limit of every bounded device-side wait
@@ -528,7 +530,9 @@ int launch_score_tc(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q,
     const int qbox = t.qbox, kbox = t.kbox;
     ScoreTcParams& sp = t.sp;
     const bool big = sp.Rpad == 256;
-    sp.clk = (long long*)(ctx->err_dev + 8);
+    // in device memory: a store across the bus at the end of the kernel held up whatever waits for it by 0.6 us
+    sp.clk = ctx->clk;
+    ctx->scored = true;
     if (ctx->scoring_mode == SHOTKV_SCORING_FAST) {
         sp.redo = w.redo;
         if (d->d == 128) return big ? launch_score_stream_t<128>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream) : launch_score_fast_t<128>(ctx, tmQ, tmK, qbox, kbox, sp, tab, stream);
@@ -798,16 +802,16 @@ int shotkv_create(shotkv_ctx** out, int device) {
         shotkv_destroy(ctx);
         return SHOTKV_ERR_CUDA;
     }
-    bool ok = cudaStreamCreateWithFlags(&ctx->aux, cudaStreamNonBlocking) == cudaSuccess &&
+    bool ok = cudaMalloc((void**)&ctx->clk, 4 * sizeof(long long)) == cudaSuccess &&
+              cudaStreamCreateWithFlags(&ctx->aux, cudaStreamNonBlocking) == cudaSuccess &&
               cudaEventCreateWithFlags(&ctx->ev_join, cudaEventDisableTiming) == cudaSuccess;
     for (int i = 0; ok && i < kMaxGroups; ++i) ok = cudaEventCreateWithFlags(&ctx->ev_fork[i], cudaEventDisableTiming) == cudaSuccess;
     if (!ok) {
         shotkv_destroy(ctx);
         return SHOTKV_ERR_CUDA;
     }
-    for (int i = 0; i < kErrWords; ++i) ctx->err_host[i] = 0;   // word 0: a bounded wait gave up; word 1: work items the
-                                                                 // exact scoring kernel recomputed; words 2-5: self-test report;
-                                                                 // words 8-15: four 64-bit clock stamps of the last scoring launch
+    for (int i = 0; i < kErrWords; ++i) ctx->err_host[i] = 0;   // word 0: a bounded wait gave up; word 1: work items
+                                                                 // recomputed with a running maximum; words 2-5: self-test report
     ctx->sm_count = prop.multiProcessorCount;
     ctx->encode_tiled = resolve_encode_tiled();
     if (set_kernel_attributes() != cudaSuccess || ask_decode_room(ctx) != cudaSuccess) {
@@ -835,6 +839,7 @@ void shotkv_destroy(shotkv_ctx* ctx) {
         if (ctx->ev_fork[i]) cudaEventDestroy(ctx->ev_fork[i]);
     if (ctx->stage) cudaFreeHost(ctx->stage);
     if (ctx->err_host) cudaFreeHost(ctx->err_host);
+    if (ctx->clk) cudaFree(ctx->clk);
     for (int i = 0; i < kProfSlots; ++i) {
         for (int j = 0; j < 5; ++j)
             if (ctx->prof_ev[i][j]) cudaEventDestroy(ctx->prof_ev[i][j]);
@@ -1479,7 +1484,8 @@ uint64_t shotkv_launch_count(const shotkv_ctx* ctx) { return ctx ? ctx->launches
 
 int shotkv_last_scoring_clock(const shotkv_ctx* ctx, int64_t* cycles, int64_t* nanoseconds) {
     if (!ctx || !ctx->err_host || !cycles || !nanoseconds) return SHOTKV_ERR_INVALID_ARG;
-    const volatile long long* w = (const volatile long long*)(ctx->err_host + 8);
+    long long w[4] = {0, 0, 0, 0};
+    if (ctx->scored && cudaMemcpy(w, ctx->clk, sizeof w, cudaMemcpyDeviceToHost) != cudaSuccess) return SHOTKV_ERR_CUDA;
     *cycles = (int64_t)(w[2] - w[0]);
     *nanoseconds = (int64_t)(w[3] - w[1]);
     return SHOTKV_OK;
