@@ -151,11 +151,16 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
     copy_bounds(o, tab, bl / a.L, S);
     if (ranks > 1) cluster_arrive();               // (1) this CTA has begun: its shared memory may be written to
     __syncthreads();
+#pragma unroll 1
     for (int j = tid; j < v.nchunk; j += kReduceThreads) range[j] = make_int2(first_piece(v, o, j), last_piece(v, o, j));
+#pragma unroll 1
     for (int i = tid; i < S; i += kReduceThreads) mass[i] = 0.f;
+#pragma unroll 1
     for (int q = tid; q < np; q += kReduceThreads) item_of[q] = kNoItem;   // an index no piece has (a boundary on a chunk end)
     __syncthreads();
+#pragma unroll 1
     for (int j = warp; j < v.nchunk; j += NW)
+#pragma unroll 1
         for (int q = range[j].x + lane; q <= range[j].y; q += 32) item_of[q] = (unsigned char)j;
     grid_wait();
     const int q_first = range[0].x, q_count = range[v.nchunk - 1].y + 1 - q_first;
@@ -187,6 +192,7 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
         };
         load_pieces(q0);
         bool any = false;
+#pragma unroll 1
         for (int j = tid; j < v.nchunk; j += kReduceThreads) {
             const bool e = item_is_exact(v, u * v.nchunk + j);
             exact[j] = e;
@@ -253,9 +259,9 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
             for (int n = 0; n < AHEAD; ++n) {
                 const int j = q + n < q1 ? item_of[q + n] : kNoItem;
                 if (j == kNoItem) continue;
-                if (exact[j]) weights(pm + (size_t)(q + n) * v.Rpad);
-                else if (j != item) weights(v.item_m + ((size_t)u * v.nchunk + j) * v.Rpad);
-                item = exact[j] ? kNoItem : j;
+                const bool e = exact[j] != 0;
+                if (e || j != item) weights(e ? pm + (size_t)(q + n) * v.Rpad : v.item_m + ((size_t)u * v.nchunk + j) * v.Rpad);
+                item = e ? kNoItem : j;
                 float s = 0.f;
 #pragma unroll
                 for (int k = 0; k < NH; ++k) {
@@ -269,8 +275,10 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
             }
         }
         __syncthreads();
+#pragma unroll 1
         for (int i = tid; i < S; i += kReduceThreads) {
             float s = 0.f;
+#pragma unroll 1
             for (int j = o[i] / v.chunk_keys, last = (o[i + 1] - 1) / v.chunk_keys; j <= last; ++j) s += piece_mass[i + 1 + j];
             mass[i] += s;
         }
@@ -279,6 +287,7 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
     if (ranks > 1) {
         cluster_wait();                            // (1) the leader has begun
         if (rank != 0)
+#pragma unroll 1
             for (int i = tid; i < S; i += kReduceThreads) cluster_store(mass + i, 0, mass[i]);
         cluster_arrive();                          // (2) this CTA's masses are with the leader
     }
@@ -287,6 +296,7 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
         float* scores = shot_scores + (size_t)bl * S;
         select_body<kReduceThreads>(a, bl, o, work, [&](int i) {
             float s = 0.f;
+#pragma unroll 1
             for (int c = 0; c < ranks; ++c) s += masses[c * s4 + i];
             s /= (float)(o[i + 1] - o[i]);
             scores[i] = s;
