@@ -47,7 +47,7 @@ FALLBACK_BF16_TFLOPS_SUSTAINED = 1400.0  # the same, back to back under the powe
 # byte of the scoring kernel and of the two decode score kernels, taken on reduced copies of the
 # workloads (config 3 with B=1, L=8; config 4 with B=2) and scaled by the bytes of a full launch.
 # A ratio is set to None whenever its kernel has changed since its capture.
-SCORE_TC_TRAFFIC_RATIO = 1.042
+SCORE_TC_TRAFFIC_RATIO = 1.041
 SCORE_FAST_TRAFFIC_RATIO = 1.021      # the 128-row kernel on config 2 at full size
 DECODE_TRAFFIC_RATIO = 1.012
 DECODE_ATTEND_TRAFFIC_RATIO = 1.006
