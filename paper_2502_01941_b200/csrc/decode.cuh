@@ -34,6 +34,7 @@ constexpr int kMaxSplit = 8;
 // shared memory before may be read by the others afterwards; they must be done before it ends.
 __device__ __forceinline__ void exchange_stats(const float* own, float* table, int rank, int nsplit) {
     cluster_wait();
+#pragma unroll 1
     for (int i = threadIdx.x; i < 16 * nsplit; i += blockDim.x) cluster_store(table + rank * 16 + (i & 15), i >> 4, own[i & 15]);
     cluster_arrive();
     cluster_wait();
@@ -288,6 +289,8 @@ struct AttendCfg {
 // masks and parked logits are left to the blocks that need them, and the first product runs as four chains
 // of MMAs.  32 steps of 8 sequences x 32 layers 16.25 -> 15.93 ms, a step of 4 sequences x 1 layer 17.0 -> 15.9 us,
 // one unit of 8,000 keys 20.0 -> 15.5 us.
+// What follows the blocks runs once and its loops are not unrolled: code that runs once is fetched cold (32 steps
+// of one layer 439.2 -> 435.8 us).
 template <int D>
 __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_kernel(const DecodeParams p) {
     using Cfg = AttendCfg<D>;
@@ -507,6 +510,7 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     __syncthreads();
     float* out = p.out + ((size_t)bl * p.H + (size_t)hk * p.G) * D;
     // the warps' outputs, relative to the CTA's maximum; alone, the CTA has the rows' whole sums already
+#pragma unroll 1
     for (int idx = tid; idx < p.G * D; idx += NT) {
         const int r = idx / D;
         const float mm = sfin[r * 2];
@@ -524,6 +528,7 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
         if (tid < 8) merge_stats(stab, p.nsplit, tid, sfin[tid * 2], sfin[tid * 2 + 1]);
         __syncthreads();
         // each CTA adds up its share of the output elements
+#pragma unroll 1
         for (int idx = rank * NT + tid; idx < p.G * D; idx += p.nsplit * NT) {
             const int r = idx / D;
             const float mm = sfin[r * 2];
@@ -538,6 +543,7 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
         const int j = base + lane - M;
         if (lane < 16 && j >= 0 && j < n) {
             float s = 0.f;
+#pragma unroll 1
             for (int r = 0; r < p.G; ++r) s += ex2f(sdec[r * p.Dcap + j] - sfin[r * 2]) * sfin[r * 2 + 1];
             p.partial[(size_t)u * p.Dcap + j] = s;
         }
@@ -608,6 +614,7 @@ __global__ void __launch_bounds__(kSelectThreads) decode_evict_kernel(const Deco
     if (tid == 0) first_gone = n;
     grid_wait();
     grid_release();
+#pragma unroll 1
     for (int j = tid; j < n; j += NT) {
         const float v = accumulated(p, bl, j);
         a[j] = v == v ? v : SHOTKV_NEG_INF;        // keep the order total even if a score is NaN
@@ -623,11 +630,13 @@ __global__ void __launch_bounds__(kSelectThreads) decode_evict_kernel(const Deco
                  });
     __syncthreads();
     block_exclusive_scan<NT>(ds, n, tmp);
+#pragma unroll 1
     for (int j = tid; j < n; j += NT)
         if (kf[j]) kp[ds[j]] = j;
     if (p.ranks > 1) cluster_wait();               // all CTAs have read acc and born
     __syncthreads();
     if (rank == 0)
+#pragma unroll 1
         for (int j = tid; j < p.k; j += NT) {
             p.acc[(size_t)bl * p.Dcap + j] = a[kp[j]];
             p.born[(size_t)bl * p.Dcap + j] = bs[kp[j]];
