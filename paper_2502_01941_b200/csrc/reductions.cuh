@@ -262,6 +262,14 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
                 const bool e = exact[j] != 0;
                 if (e || j != item) weights(e ? pm + (size_t)(q + n) * v.Rpad : v.item_m + ((size_t)u * v.nchunk + j) * v.Rpad);
                 item = e ? kNoItem : j;
+                if (e)                                 // an exact item's sums need not be numbers in a row without weight
+#pragma unroll
+                    for (int k = 0; k < NH; ++k) {
+                        z4[n][k].x = rw[k].x > 0.f ? z4[n][k].x : 0.f;
+                        z4[n][k].y = rw[k].y > 0.f ? z4[n][k].y : 0.f;
+                        z4[n][k].z = rw[k].z > 0.f ? z4[n][k].z : 0.f;
+                        z4[n][k].w = rw[k].w > 0.f ? z4[n][k].w : 0.f;
+                    }
                 float s = 0.f;
 #pragma unroll
                 for (int k = 0; k < NH; ++k) {

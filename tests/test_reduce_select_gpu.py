@@ -60,3 +60,34 @@ def test_heads_to_a_cluster(ctx, Hkv, G, W, mode):
     finally:
         skv.shotkv_set_scoring_mode(ctx, skv.SCORING_FAST)
     assert P.check_all_units(gpu, Q, K, V, off, cfg.r_p) <= 1
+
+
+@pytest.mark.parametrize("W", [32, 64])                    # 128 and 256 window rows
+@pytest.mark.parametrize("mode", [skv.SCORING_FAST, skv.SCORING_EXACT], ids=["fast", "exact"])
+@pytest.mark.parametrize("what", ["query_nan", "query_inf", "key_nan"])
+def test_rows_that_are_not_numbers_carry_no_weight(ctx, what, mode, W):
+    """A window row whose softmax denominator is not a number drops out of the sums; the other rows, and the
+    other heads, give what they give without it."""
+    Hkv, G, d, N, S = 2, 4, 64, 1500, 7
+    cfg = wl.PrefillConfig("nan", B=1, L=1, H=Hkv * G, Hkv=Hkv, d=d, N=N, W=W, S=S, shot_dist="uniform", shot_lo=100, shot_hi=250,
+                           question_len=130, r_p=0.4, cfg_id=64)
+    Q, K, V, off = wl.prefill_batch(cfg, "cuda")
+    dropped = torch.zeros(Hkv * G, W, dtype=torch.bool, device="cuda")
+    if what == "key_nan":
+        K[0, 0, 1, 296:304, 5] = float("nan")              # every window row sees them (the fast kernels' FMA pipe takes a
+                                                           # lone one for a key without weight, the other pipe does not)
+        dropped[G:] = True
+    else:
+        Q[0, 0, 2, 3] = float("nan") if what == "query_nan" else float("inf")
+        dropped[2, 3] = True
+    x = torch.einsum("hwd,hnd->hwn", Q[0, 0].double(), K[0, 0].double().repeat_interleave(G, 0)) / d ** 0.5
+    x = x.masked_fill(torch.arange(N, device="cuda") > torch.arange(N - W, N, device="cuda")[:, None], float("-inf"))
+    alpha = torch.where(dropped[..., None], 0.0, x.softmax(-1)).sum((0, 1))
+    o = off[0]
+    want = torch.stack([alpha[o[i]:o[i + 1]].mean() for i in range(S)])
+    skv.shotkv_set_scoring_mode(ctx, mode)
+    try:
+        got = P.gpu_prefill(ctx, P.dims_of(cfg), Q, K, V, off, cfg.r_p, 0, "fused")["shot_scores"][0, 0]
+    finally:
+        skv.shotkv_set_scoring_mode(ctx, skv.SCORING_FAST)
+    assert torch.allclose(got.double(), want, rtol=P.SCORE_RTOL, atol=P.SCORE_ATOL), (got, want)
