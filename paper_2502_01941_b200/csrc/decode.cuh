@@ -532,8 +532,9 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
         for (int idx = rank * NT + tid; idx < p.G * D; idx += p.nsplit * NT) {
             const int r = idx / D;
             const float mm = sfin[r * 2];
+            const float mu = mm == SHOTKV_NEG_INF ? 0.f : mm;    // a row without a finite logit has no weight anywhere
             float o = 0.f;
-            for (int c = 0; c < p.nsplit; ++c) o += cluster_load(sO + idx, c) * ex2f(stab[c * 16 + r * 2] - mm);
+            for (int c = 0; c < p.nsplit; ++c) o += cluster_load(sO + idx, c) * ex2f(stab[c * 16 + r * 2] - mu);
             out[idx] = o * sfin[r * 2 + 1];
         }
         cluster_arrive();                                    // done with the others' memory

@@ -3,10 +3,11 @@ eight CTAs to a unit, CTAs without a single key, heads that do not divide by the
 both sides of the ranking by counting (256 entries) and by sorting."""
 import numpy as np
 import pytest
+import torch
 
 import paper_2502_01941_b200 as skv
 from paper_2502_01941_b200 import workloads as wl
-from test_decode_gpu import lockstep
+from test_decode_gpu import GpuDecoder, OUT_ATOL, OUT_RTOL, lockstep
 
 pytestmark = pytest.mark.gpu
 
@@ -30,3 +31,23 @@ def test_unit_shared_by_a_cluster(ctx, Hkv, G, d, M, count, attend):
 def test_eviction_of_a_large_region(ctx, every):
     cfg = wl.DecodeConfig("evict", B=1, L=1, H=4, Hkv=2, d=64, steps=every + 3, r_d=0.6, recompress_every=every, cfg_id=72)
     assert lockstep(ctx, cfg, 40, [(0, 0)]) <= 2
+
+
+@pytest.mark.parametrize("M", [40, 2048], ids=["whole_unit", "shared_unit"])
+def test_query_that_is_not_a_number_gives_no_output(ctx, M):
+    """The same output, zero, whether one CTA has the unit or a cluster shares it; other heads are as without it."""
+    cfg = wl.DecodeConfig("nan", B=1, L=1, H=8, Hkv=2, d=128, steps=4, r_d=0.5, recompress_every=4, cfg_id=74)
+    Kc, kept = wl.random_prefill_cache(cfg, M, "cuda")
+    Vc = wl.random_prefill_values(cfg, M, "cuda")
+    gpu = GpuDecoder(ctx, cfg, Kc, kept, Vc=Vc)
+    q, k, v = wl.decode_step_inputs(cfg, 0, "cuda")
+    q[0, 0, 2] = float("nan")
+    gpu.step(q, k, v)
+    torch.cuda.synchronize()
+    n = int(kept[0, 0])
+    keys = torch.cat([Kc[0, 0, :, :n], k[0, 0][:, None]], 1).double().repeat_interleave(4, 0)
+    vals = torch.cat([Vc[0, 0, :, :n], v[0, 0][:, None]], 1).double().repeat_interleave(4, 0)
+    want = ((q[0, 0].double()[:, None] * keys).sum(-1) / 128 ** 0.5).softmax(-1)[:, None] @ vals
+    want[2] = 0
+    err = (gpu.out[0, 0].double() - want[:, 0]).abs()
+    assert (err <= OUT_RTOL * want[:, 0].abs().amax(1, keepdim=True) + OUT_ATOL).all(), err.amax(1)
