@@ -76,7 +76,9 @@ __device__ __forceinline__ int count_le_warp(const int* o, int n, int x) {
 // it on the stream still runs.  Every such kernel passes grid_wait before it touches global memory:
 // it returns when the kernel before has finished and its writes are visible (and, that kernel having
 // waited too, everything before it).  grid_release lets the next kernel's CTAs begin, once all CTAs of
-// this one have called it or ended.
+// this one have called it or ended.  What such a kernel reads may still be written when it begins, so no
+// pointer it reads through is __restrict__ and no load takes the read-only path: either would let the compiler
+// move a load above the wait.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

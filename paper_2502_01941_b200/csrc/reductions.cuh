@@ -323,10 +323,9 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
 constexpr int kTokenWarps = 8;
 constexpr int kLongShot = 96;                  // mean length from which eight warps share a shot
 template <int WPS>
-__global__ void __launch_bounds__(32 * kTokenWarps, 4) shot_score_from_tokens_kernel(const float* __restrict__ imp,
+__global__ void __launch_bounds__(32 * kTokenWarps, 4) shot_score_from_tokens_kernel(const float* imp,
                                                                                   const __grid_constant__ ShotTable tab, int L,
-                                                                                  int Hkv, int N, int S,
-                                                                                  float* __restrict__ shot_scores) {
+                                                                                  int Hkv, int N, int S, float* shot_scores) {
     static_assert(WPS == 1 || WPS == kTokenWarps, "a warp or the whole CTA to a shot");
     constexpr int AHEAD = 8;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, bl = blockIdx.y;

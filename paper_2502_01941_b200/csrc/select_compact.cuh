@@ -298,7 +298,7 @@ __host__ __device__ constexpr size_t bounds_smem_bytes(int S) { return (size_t)(
 // Selection from scores already in memory: one CTA per (b, l), NT = kSelectThreads where shots are
 // ranked by counting, kSortThreads beyond; bounds_smem_bytes(S) + select_smem_bytes(S) of shared memory.
 template <int NT>
-__global__ void __launch_bounds__(NT) select_shots_kernel(const float* __restrict__ shot_scores, const __grid_constant__ ShotTable tab,
+__global__ void __launch_bounds__(NT) select_shots_kernel(const float* shot_scores, const __grid_constant__ ShotTable tab,
                                                          const SelectArgs a) {
     extern __shared__ __align__(16) unsigned char sm[];
     const int bl = blockIdx.x;
@@ -315,10 +315,8 @@ __global__ void __launch_bounds__(NT) select_shots_kernel(const float* __restric
 // vectors; consecutive lanes move consecutive vectors of a row, each thread keeps four
 // independent loads in flight.  grid = (row blocks, Hkv, B*L).
 template <int D>
-__global__ void __launch_bounds__(256) compact_kv_kernel(const uint4* __restrict__ K, const uint4* __restrict__ V,
-                                                        const int* __restrict__ kept_idx,
-                                                        const int* __restrict__ kept_count, int Hkv, int N, int Mcap,
-                                                        uint4* __restrict__ Kc, uint4* __restrict__ Vc) {
+__global__ void __launch_bounds__(256) compact_kv_kernel(const uint4* K, const uint4* V, const int* kept_idx, const int* kept_count,
+                                                        int Hkv, int N, int Mcap, uint4* Kc, uint4* Vc) {
     constexpr int VPR = D / 8;                 // 16-byte vectors per row
     constexpr int ROWS = 256 / VPR * 4;        // rows per CTA per pass
     const int bl = blockIdx.z, h = blockIdx.y;
@@ -350,8 +348,8 @@ __global__ void __launch_bounds__(256) compact_kv_kernel(const uint4* __restrict
 #pragma unroll
         for (int q = 0; q < 4; ++q)
             if (src[q] >= 0) {
-                kk[q] = __ldg(Ku + (size_t)src[q] * VPR + v);
-                vv[q] = __ldg(Vu + (size_t)src[q] * VPR + v);
+                kk[q] = Ku[(size_t)src[q] * VPR + v];
+                vv[q] = Vu[(size_t)src[q] * VPR + v];
             }
 #pragma unroll
         for (int q = 0; q < 4; ++q)
