@@ -253,6 +253,7 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
             }
         };
         int item = kNoItem;
+        bool odd = false;                              // a piece's mass is not a number
         for (int q = q0; q < q1; q += AHEAD) {
             if (q != q0) load_pieces(q);
 #pragma unroll
@@ -262,14 +263,6 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
                 const bool e = exact[j] != 0;
                 if (e || j != item) weights(e ? pm + (size_t)(q + n) * v.Rpad : v.item_m + ((size_t)u * v.nchunk + j) * v.Rpad);
                 item = e ? kNoItem : j;
-                if (e)                                 // an exact item's sums need not be numbers in a row without weight
-#pragma unroll
-                    for (int k = 0; k < NH; ++k) {
-                        z4[n][k].x = rw[k].x > 0.f ? z4[n][k].x : 0.f;
-                        z4[n][k].y = rw[k].y > 0.f ? z4[n][k].y : 0.f;
-                        z4[n][k].z = rw[k].z > 0.f ? z4[n][k].z : 0.f;
-                        z4[n][k].w = rw[k].w > 0.f ? z4[n][k].w : 0.f;
-                    }
                 float s = 0.f;
 #pragma unroll
                 for (int k = 0; k < NH; ++k) {
@@ -279,7 +272,21 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
                     s = fmaf(z4[n][k].w, f[k].w, s);
                 }
                 s = warp_sum(s);
+                odd |= s != s;
                 if (lane == 0) piece_mass[q + n] = s;
+            }
+        }
+        if (odd) {                                     // an exact item's sums need not be numbers in a row without weight: that row is left out
+            __syncwarp();
+#pragma unroll 1
+            for (int q = q0; q < q1; ++q) {
+                if (item_of[q] == kNoItem || piece_mass[q] == piece_mass[q]) continue;
+                float s = 0.f;
+#pragma unroll 1
+                for (int k = lane; k < ROWS; k += 32)
+                    if (row_w[k] > 0.f) s += pz[(size_t)q * v.Rpad + k] * (ex2f(pm[(size_t)q * v.Rpad + k] - row_m[k]) * row_w[k]);
+                s = warp_sum(s);
+                if (lane == 0) piece_mass[q] = s;
             }
         }
         __syncthreads();
