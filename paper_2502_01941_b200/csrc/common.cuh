@@ -82,6 +82,16 @@ __device__ __forceinline__ int count_le_warp(const int* o, int n, int x) {
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// 16 bytes at p, or zeros.  Written as one predicated instruction: a branch around each plain load of a row kept
+// the next one waiting behind it.
+__device__ __forceinline__ uint4 load_if(const uint4* p, bool valid) {
+    uint4 v = make_uint4(0, 0, 0, 0);
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %5, 0;\n\t@q ld.global.v4.u32 {%0, %1, %2, %3}, [%4];\n\t}"
+                 : "+r"(v.x), "+r"(v.y), "+r"(v.z), "+r"(v.w)
+                 : "l"(p), "r"((int)valid));
+    return v;
+}
+
 // Barrier of a thread-block cluster in two halves, for all threads of its CTAs.
 __device__ __forceinline__ void cluster_arrive() {
     __syncwarp();

@@ -346,11 +346,10 @@ __global__ void __launch_bounds__(256) compact_kv_kernel(const uint4* K, const u
             if (j >= count || src[q] >= N) src[q] = -1;
         }
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (src[q] >= 0) {
-                kk[q] = Ku[(size_t)src[q] * VPR + v];
-                vv[q] = Vu[(size_t)src[q] * VPR + v];
-            }
+        for (int q = 0; q < 4; ++q) {
+            kk[q] = load_if(Ku + (size_t)src[q] * VPR + v, src[q] >= 0);
+            vv[q] = load_if(Vu + (size_t)src[q] * VPR + v, src[q] >= 0);
+        }
 #pragma unroll
         for (int q = 0; q < 4; ++q)
             if (src[q] >= 0) {
