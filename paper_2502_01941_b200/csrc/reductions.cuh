@@ -13,6 +13,8 @@
 // of a unit has index s + j.
 // An item is "exact" when every item is (`all_exact`: the kernel of score_tc.cuh did all the work) or when
 // its redo flag is set; its rows' statistics are then rebuilt from its pieces.
+// A row whose z is not a number in some piece (a query or a key that is none) has the pair (m, z) = (NaN, 0) there: its
+// sum over the unit is then no number either, so the row gets weight 0, and its z may still be multiplied by it.
 // row_stats_kernel, reduce_select_kernel, shot_score_from_tokens_kernel: fixed-order reductions of
 // those partials, and of per-token importances.
 #pragma once
@@ -253,7 +255,6 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
             }
         };
         int item = kNoItem;
-        bool odd = false;                              // a piece's mass is not a number
         for (int q = q0; q < q1; q += AHEAD) {
             if (q != q0) load_pieces(q);
 #pragma unroll
@@ -272,21 +273,7 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
                     s = fmaf(z4[n][k].w, f[k].w, s);
                 }
                 s = warp_sum(s);
-                odd |= s != s;
                 if (lane == 0) piece_mass[q + n] = s;
-            }
-        }
-        if (odd) {                                     // an exact item's sums need not be numbers in a row without weight: that row is left out
-            __syncwarp();
-#pragma unroll 1
-            for (int q = q0; q < q1; ++q) {
-                if (item_of[q] == kNoItem || piece_mass[q] == piece_mass[q]) continue;
-                float s = 0.f;
-#pragma unroll 1
-                for (int k = lane; k < ROWS; k += 32)
-                    if (row_w[k] > 0.f) s += pz[(size_t)q * v.Rpad + k] * (ex2f(pm[(size_t)q * v.Rpad + k] - row_m[k]) * row_w[k]);
-                s = warp_sum(s);
-                if (lane == 0) piece_mass[q] = s;
             }
         }
         __syncthreads();

@@ -587,8 +587,9 @@ __device__ __forceinline__ void exact_epilogue(const Pipe<Cfg>& pp, float* comb,
                 for (int s = 1; s < NSL; ++s) zz += slot[s * 256 + 1] * ex2f(slot[s * 256] - mu);
                 const size_t o = ((size_t)u * p.P + sg + j) * p.Rpad + row;
                 const bool live = row < p.R;        // padding rows: their Q was never loaded
-                p.part_m[o] = live ? mm : 0.f;
-                p.part_z[o] = live ? zz : 0.f;
+                const bool number = zz < __int_as_float(0x7f800000);     // see reductions.cuh
+                p.part_m[o] = live ? (number ? mm : __int_as_float(0x7fffffff)) : 0.f;
+                p.part_z[o] = live && number ? zz : 0.f;
             }
             z = 0.f;
             ++nflush;
