@@ -382,6 +382,12 @@ void empty_table(ShotTable& t) {
     for (int i = 0; i < kTableEnd; ++i) t.data[i] = kNoBound;
 }
 
+// bf16 tensors are read and written as 16-byte vectors.
+template <class... P>
+bool aligned16(const P*... p) {
+    return ((... | (uintptr_t)p) & 15) == 0;
+}
+
 int set_device(shotkv_ctx* ctx) {
     if (!ctx) return SHOTKV_ERR_INVALID_ARG;
     CUDA_TRY(ctx, cudaSetDevice(ctx->device));
@@ -994,6 +1000,7 @@ int shotkv_compact_kv(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv_bf1
     const char* why = "";
     if ((rc = check_dims(dims, &why))) return fail(ctx, rc, "%s", why);
     if (!K || !V || !kept_idx || !kept_count || !Kc || !Vc) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "pointers must not be NULL");
+    if (!aligned16(K, V, Kc, Vc)) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "K, V, Kc and Vc must be 16-byte aligned");
     if (Mcap < 1) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "Mcap must be >= 1");
     return run_compact(ctx, dims, K, V, kept_idx, kept_count, Mcap, Kc, Vc, (cudaStream_t)stream_);
 }
@@ -1012,6 +1019,7 @@ int prefill_compress_impl(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv
     if (rc) return rc;
     const char* why = "";
     if ((rc = check_dims(dims, &why))) return fail(ctx, rc, "%s", why);
+    if (!aligned16(Qwin, K, V, Kc, Vc)) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "Qwin, K, V, Kc and Vc must be 16-byte aligned");
     const bool tokens = (flags & SHOTKV_FLAG_TOKEN_IMPORTANCE) != 0;
     if (tokens || token_route(dims)) {
         // per-token importances first (asked for, or many short units): the three public steps in
@@ -1252,6 +1260,7 @@ int shotkv_decode_init(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv_po
     if (Dcap < 1 || Dcap > 4096) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "Dcap must be in [1, 4096]");
     if (Mcap < 0) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "Mcap must be >= 0");
     if (!Kd || !Vd || !acc || !born || !ws) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "device pointers must not be NULL");
+    if (!aligned16(Kd, Vd)) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "Kd and Vd must be 16-byte aligned");
     if (ws_bytes < shotkv_decode_workspace_bytes(dims, Dcap))
         return fail(ctx, SHOTKV_ERR_WORKSPACE_TOO_SMALL, "decode workspace has %zu bytes, %zu needed", ws_bytes,
                     shotkv_decode_workspace_bytes(dims, Dcap));
@@ -1304,6 +1313,8 @@ int decode_step_impl(shotkv_ctx* ctx, shotkv_decode_state* st, const shotkv_bf16
     if (!st || !q || !k_new || !v_new || !kept_count) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "pointers must not be NULL");
     if (st->Mcap > 0 && !Kc) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "Kc must not be NULL when Mcap > 0");
     if (attn_out && st->Mcap > 0 && !Vc) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "Vc must not be NULL when Mcap > 0");
+    if (!aligned16(q, k_new, v_new)) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "q, k_new and v_new must be 16-byte aligned");
+    if (st->Mcap > 0 && !aligned16(Kc, attn_out ? Vc : nullptr)) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "Kc and Vc must be 16-byte aligned");
     if (st->n_dec + 1 > st->Dcap) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "decode region full: n_dec = %d, Dcap = %d", st->n_dec, st->Dcap);
     cudaStream_t stream = (cudaStream_t)stream_;
     const shotkv_dims& d = st->dims;
