@@ -9,15 +9,11 @@ library is missing or a call fails, a `ShotKVError` is raised.
 from __future__ import annotations
 
 import ctypes as C
+import importlib.util
 import os
 
 import numpy as np
 import torch
-
-try:
-    from . import _marshal
-except ImportError:                     # not built: the ctypes path below serves every call
-    _marshal = None
 
 _PKG = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_PKG, "libshotkv.so")
@@ -67,7 +63,7 @@ class DecodeState(C.Structure):
 
 
 _lib = None
-_native = None      # _marshal, once it knows the library's functions
+_native = None      # the marshalling module, once it knows the library's functions
 
 
 def lib() -> C.CDLL:
@@ -116,13 +112,29 @@ def lib() -> C.CDLL:
     for name, (res, args) in sig.items():
         fn = getattr(L, name)
         fn.restype, fn.argtypes = res, args
-    if _marshal is not None:
-        _marshal.init(Dims, Policy, DecodeState, *(C.cast(getattr(L, n), vp).value for n in (
+    m = _load_marshal()
+    if m is not None:
+        m.init(Dims, Policy, DecodeState, *(C.cast(getattr(L, n), vp).value for n in (
             "shotkv_prefill_score", "shotkv_select_shots", "shotkv_compact_kv", "shotkv_prefill_compress",
             "shotkv_decode_step", "shotkv_decode_step_attend")))
-        _native = _marshal
+        _native = m
     _lib = L
     return L
+
+
+def _load_marshal():
+    """The marshalling module built for this Python and torch, or None: the ctypes path serves every call."""
+    from .build import marshal_path
+    path = marshal_path()
+    if not os.path.exists(path):
+        return None
+    spec = importlib.util.spec_from_file_location(f"{__package__}._marshal", path)
+    try:
+        m = importlib.util.module_from_spec(spec)
+        spec.loader.exec_module(m)
+    except ImportError:
+        return None
+    return m
 
 
 # ------------------------------------------------------------------ marshalling helpers

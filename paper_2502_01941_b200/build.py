@@ -1,16 +1,16 @@
-"""Builds in-tree libshotkv.so (the C-ABI library) with nvcc for sm_100a, and _marshal.so (the binding's
-argument marshalling) with the host compiler."""
+"""Builds in-tree libshotkv.so (the C-ABI library) with nvcc for sm_100a, and the binding's argument
+marshalling module with the host compiler."""
 from __future__ import annotations
 
 import os
 import shutil
 import subprocess
 import sys
+import warnings
 
 PKG_DIR = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(PKG_DIR, "csrc")
 LIB_PATH = os.path.join(PKG_DIR, "libshotkv.so")
-MARSHAL_PATH = os.path.join(PKG_DIR, "_marshal.so")
 SOURCES = ["shotkv_api.cu"]
 MARSHAL_SOURCE = os.path.join(CSRC, "marshal.cpp")
 NVCC_FLAGS = [
@@ -42,10 +42,20 @@ def _run(cmd: list, what: str) -> subprocess.CompletedProcess:
     return res
 
 
+def marshal_path() -> str:
+    """Where the marshalling module for this Python and this torch lies.  It is compiled against the layout
+    of their objects, so both are part of its name and one built for others is never loaded."""
+    import sysconfig
+
+    import torch
+    return os.path.join(PKG_DIR, f"_marshal.torch-{torch.__version__}{sysconfig.get_config_var('EXT_SUFFIX')}")
+
+
 def build_marshal(force: bool = False) -> str:
     """Compile the marshalling module next to this file, against the installed torch; returns its path."""
-    if not force and not _stale(MARSHAL_PATH, [MARSHAL_SOURCE]):
-        return MARSHAL_PATH
+    path = marshal_path()
+    if not force and not _stale(path, [MARSHAL_SOURCE]):
+        return path
     import sysconfig
 
     import torch
@@ -54,14 +64,23 @@ def build_marshal(force: bool = False) -> str:
     include = [root + "include", root + "include/torch/csrc/api/include", cuda, sysconfig.get_paths()["include"]]
     _run([os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-shared", "-fPIC", "-fvisibility=hidden",
           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}", *(x for i in include for x in ("-isystem", i)),
-          MARSHAL_SOURCE, "-o", MARSHAL_PATH, f"-L{root}lib", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"],
-         "_marshal.so")
-    return MARSHAL_PATH
+          MARSHAL_SOURCE, "-o", path, f"-L{root}lib", "-ltorch_python", "-ltorch", "-ltorch_cpu", "-lc10", "-lc10_cuda"],
+         "the marshalling module")
+    return path
 
 
 def build_library(force: bool = False, verbose: bool = False) -> str:
-    """Compile the CUDA sources into `libshotkv.so` next to this file; returns its path."""
-    build_marshal(force)
+    """Compile the CUDA sources into `libshotkv.so` next to this file; returns its path.  The marshalling
+    module is built after it where that is possible: without it the binding goes through ctypes."""
+    path = _build_cuda(force, verbose)
+    try:
+        build_marshal(force)
+    except (ImportError, OSError, RuntimeError) as e:
+        warnings.warn(f"the marshalling module was not built ({e}); calls go through ctypes")
+    return path
+
+
+def _build_cuda(force: bool, verbose: bool) -> str:
     if not force and not _stale(LIB_PATH, [os.path.join(CSRC, f) for f in os.listdir(CSRC) if not f.endswith(".cpp")]):
         return LIB_PATH
     cmd = [_nvcc(), *NVCC_FLAGS]
