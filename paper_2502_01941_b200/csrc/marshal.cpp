@@ -7,6 +7,10 @@
 // binding.py then takes its own path, which converts what can be converted and names what cannot.
 #include <Python.h>
 #include <c10/cuda/CUDAStream.h>
+
+#include <optional>
+#include <utility>
+
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "../../include/shotkv.h"
@@ -125,21 +129,24 @@ struct Args {
 };
 
 // `body` reads its arguments and, when all were as expected, returns a call to make without the
-// interpreter's lock.
+// interpreter's lock.  Only the reading may throw (a tensor that cannot say where it lies): an exception out of
+// the call would be caught without the lock.
 template <class Body>
 PyObject* guarded(PyObject* const* a, Py_ssize_t n, Body&& body) {
+    using Call = decltype(body(std::declval<Args&>()));
+    std::optional<Call> call;
+    Args g{a, n};
     try {
-        Args g{a, n};
-        auto call = body(g);
-        if (!g.ok) Py_RETURN_NONE;
-        int rc;
-        Py_BEGIN_ALLOW_THREADS
-        rc = call();
-        Py_END_ALLOW_THREADS
-        return PyLong_FromLong(rc);
-    } catch (...) {                             // a tensor that cannot say where it lies
+        call.emplace(body(g));
+    } catch (...) {
         Py_RETURN_NONE;
     }
+    if (!g.ok) Py_RETURN_NONE;
+    int rc;
+    Py_BEGIN_ALLOW_THREADS
+    rc = (*call)();
+    Py_END_ALLOW_THREADS
+    return PyLong_FromLong(rc);
 }
 
 PyObject* prefill_score(PyObject*, PyObject* const* a, Py_ssize_t n) {

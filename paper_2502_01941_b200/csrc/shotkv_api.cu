@@ -11,6 +11,7 @@
 #include <cstdlib>
 #include <cstring>
 #include <functional>
+#include <memory>
 #include <new>
 #include <utility>
 #include <vector>
@@ -361,13 +362,14 @@ int prepare_table(shotkv_ctx* ctx, const shotkv_dims* d, const int32_t* off_host
     const size_t entries = (size_t)d->B * t.stride;
     t.ptr = entries > (size_t)kTableArgs ? device : nullptr;
     if (t.ptr && !walked) return upload_small(ctx, device, off_host, entries * 4, stream);
-    std::vector<int> big(t.ptr ? entries : 0);
-    int* to = t.ptr ? big.data() : t.data;
+    std::unique_ptr<int[]> big(t.ptr ? new (std::nothrow) int[entries] : nullptr);
+    if (t.ptr && !big) return fail(ctx, SHOTKV_ERR_INVALID_ARG, "no host memory for %zu shot boundaries", entries);
+    int* to = t.ptr ? big.get() : t.data;
     for (int b = 0; b < d->B; ++b, to += t.stride) {
         memcpy(to, off_host + (size_t)b * row, (size_t)row * 4);
         for (int i = row; i < t.stride; ++i) to[i] = kNoBound;
     }
-    return t.ptr ? upload_small(ctx, device, big.data(), entries * 4, stream) : SHOTKV_OK;
+    return t.ptr ? upload_small(ctx, device, big.get(), entries * 4, stream) : SHOTKV_OK;
 }
 // The table of the prompts from b0 on.
 void advance_table(ShotTable& t, int prompts, const ShotTable& whole, size_t b0) {
