@@ -1498,7 +1498,15 @@ uint64_t shotkv_launch_count(const shotkv_ctx* ctx) { return ctx ? ctx->launches
 int shotkv_last_scoring_clock(const shotkv_ctx* ctx, int64_t* cycles, int64_t* nanoseconds) {
     if (!ctx || !ctx->err_host || !cycles || !nanoseconds) return SHOTKV_ERR_INVALID_ARG;
     long long w[4] = {0, 0, 0, 0};
-    if (ctx->scored && cudaMemcpy(w, ctx->clk, sizeof w, cudaMemcpyDeviceToHost) != cudaSuccess) return SHOTKV_ERR_CUDA;
+    if (ctx->scored) {
+        // on the context's own stream, which waits for no other, and whatever the calling thread captures
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return SHOTKV_ERR_CUDA;
+        const bool ok = cudaMemcpyAsync(w, ctx->clk, sizeof w, cudaMemcpyDeviceToHost, ctx->aux) == cudaSuccess &&
+                        cudaStreamSynchronize(ctx->aux) == cudaSuccess;
+        cudaThreadExchangeStreamCaptureMode(&mode);
+        if (!ok) return SHOTKV_ERR_CUDA;
+    }
     *cycles = (int64_t)(w[2] - w[0]);
     *nanoseconds = (int64_t)(w[3] - w[1]);
     return SHOTKV_OK;

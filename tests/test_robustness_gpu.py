@@ -153,3 +153,26 @@ def test_boundary_table_larger_than_a_staging_slot(ctx):
         n = int(out["kept_count"][b, 0])
         assert n == len(idx)
         np.testing.assert_array_equal(out["kept_idx"][b, 0, :n].cpu().numpy(), idx)
+
+
+def test_scoring_clock_is_read_beside_other_work(ctx):
+    """The clock of a finished launch can be read while other streams are busy and while one is being captured."""
+    cfg = wl.CONFIGS[0]
+    Q, K, V, off = wl.prefill_batch(cfg, "cuda")
+    P.gpu_prefill(ctx, P.dims_of(cfg), Q, K, V, off, cfg.r_p, 0, "fused")
+    cycles, ns = skv.shotkv_last_scoring_clock(ctx)
+    assert cycles > 0 and ns > 0
+    done = torch.cuda.Event()
+    with torch.cuda.stream(torch.cuda.default_stream()):                 # the legacy stream, for half a second or so
+        torch.cuda._sleep(1_000_000_000)
+        done.record()
+    assert skv.shotkv_last_scoring_clock(ctx) == (cycles, ns)
+    assert not done.query()
+    torch.cuda.synchronize()
+    x, graph = torch.zeros(4, device="cuda"), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        x += 1
+        assert skv.shotkv_last_scoring_clock(ctx) == (cycles, ns)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert x.tolist() == [1.0] * 4
