@@ -307,38 +307,51 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
     }
 }
 
-// Score(s_i) from per-token importance.  Latency-bound: the importances come from L2, so what counts
-// is how many loads are in flight.  WPS warps share a shot, eight warps a CTA:
-//   WPS = 1  short units, thousands of them: a lane has up to eight heads' loads in flight
-//   WPS = 8  few long units: a warp takes every eighth head, and a lane up to eight tokens of it
+// Score(s_i) from per-token importance.  Latency-bound while the importances come from L2, so what counts is how
+// many loads are in flight, and how many warps where there are many shots.  Eight warps a CTA, in three forms:
+//   kHeadsAbreast  short units, thousands of them: a warp a shot, a lane has up to eight heads' loads in flight
+//   kTokensAhead   many long units: a warp a shot, head after head, four runs of 32 tokens in flight; few registers, so
+//                  that twice the warps of the other forms fit an SM
+//   kWholeCta      few long units: a CTA a shot, a warp takes every eighth head, and a lane up to eight tokens of it
 // Every lane sums a fixed subset of the shot's (kv head, token) pairs; lanes are added by shuffles and
-// warps in order.  Measured (32 layers of 643 sentences | 16 layers of 24 shots of 340 tokens): one
-// warp a shot and one load at a time 20 | 15 us; WPS = 1 15.7 | 19.7 us; WPS = 8 - | 5 us.
+// warps in order.
+enum TokenForm { kHeadsAbreast, kTokensAhead, kWholeCta };
 constexpr int kTokenWarps = 8;
-constexpr int kLongShot = 96;                  // mean length from which eight warps share a shot
-template <int WPS>
-__global__ void __launch_bounds__(32 * kTokenWarps, 4) shot_score_from_tokens_kernel(const float* imp,
-                                                                                  const __grid_constant__ ShotTable tab, int L,
-                                                                                  int Hkv, int N, int S, float* shot_scores) {
-    static_assert(WPS == 1 || WPS == kTokenWarps, "a warp or the whole CTA to a shot");
-    constexpr int AHEAD = 8;
+constexpr int kLongShot = 96;                  // mean length from which a unit is long
+template <TokenForm FORM>
+__global__ void __launch_bounds__(32 * kTokenWarps, FORM == kTokensAhead ? 8 : 4)
+    shot_score_from_tokens_kernel(const float* imp, const __grid_constant__ ShotTable tab, int L, int Hkv, int N, int S, float* shot_scores) {
+    constexpr int AHEAD = FORM == kTokensAhead ? 4 : 8;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, bl = blockIdx.y;
-    const int i = WPS == 1 ? blockIdx.x * kTokenWarps + warp : blockIdx.x;
+    const int i = FORM == kWholeCta ? blockIdx.x : blockIdx.x * kTokenWarps + warp;
     grid_release();
     if (i >= S) return;
     grid_wait();
     const int* o = table_row(tab, bl / L);
     const int lo = o[i], hi = o[i + 1];
     const float* base = imp + (size_t)bl * Hkv * N;
-    float a[AHEAD];
+    float a[8];
 #pragma unroll
-    for (int k = 0; k < AHEAD; ++k) a[k] = 0.f;
-    if (WPS == 1) {
+    for (int k = 0; k < 8; ++k) a[k] = 0.f;
+    if (FORM == kHeadsAbreast) {
         for (int h0 = 0; h0 < Hkv; h0 += AHEAD)
             for (int t = lo + lane; t < hi; t += 32)
 #pragma unroll
                 for (int k = 0; k < AHEAD; ++k)
                     if (h0 + k < Hkv) a[k] += base[(size_t)(h0 + k) * N + t];
+    } else if (FORM == kTokensAhead) {
+        for (int h = 0; h < Hkv; ++h) {
+            const float* row = base + (size_t)h * N;
+            int t = lo + lane;
+            for (; t + 32 * (AHEAD - 1) < hi; t += 32 * AHEAD) {
+                float v[AHEAD];
+#pragma unroll
+                for (int k = 0; k < AHEAD; ++k) v[k] = row[t + 32 * k];
+#pragma unroll
+                for (int k = 0; k < AHEAD; ++k) a[k] += v[k];
+            }
+            for (; t < hi; t += 32) a[0] += row[t];
+        }
     } else {
         for (int h = warp; h < Hkv; h += kTokenWarps)
             for (int t0 = lo; t0 < hi; t0 += 32 * AHEAD)
@@ -349,7 +362,7 @@ __global__ void __launch_bounds__(32 * kTokenWarps, 4) shot_score_from_tokens_ke
                 }
     }
     float s = warp_sum(((a[0] + a[1]) + (a[2] + a[3])) + ((a[4] + a[5]) + (a[6] + a[7])));
-    if (WPS > 1) {
+    if (FORM == kWholeCta) {
         __shared__ float part[kTokenWarps];
         if (lane == 0) part[warp] = s;
         __syncthreads();

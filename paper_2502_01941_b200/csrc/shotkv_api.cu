@@ -659,14 +659,22 @@ int run_select(shotkv_ctx* ctx, const shotkv_dims* d, const ShotTable& tab, cons
                : launch(ctx, select_shots_kernel<kSortThreads>, dim3(d->B * d->L), kSortThreads, smem, stream, 1, true, shot_scores, tab, sa);
 }
 
-// Per-shot scores from per-token importances.
+// Per-shot scores from per-token importances.  A CTA takes one long shot while there are at most two of them to an
+// SM for every head: a warp alone would have too long a chain of loads then, one head after the other; beyond, the
+// CTAs of one shot each cost their start and their barrier, and a warp a shot fills the GPU.
+// Measured, whole selection call, one CTA a shot | one warp a shot, us: 8 heads, shots of 330 tokens, 768 shots 9.4 |
+// 13.5, 2,048 14.3 | 14.8, 3,072 19.2 | 17.4, 12,288 96 | 49; 1 head, 768 8.6 | 7.0, 12,288 51 | 17; 8 heads, shots of
+// 1,300 tokens, 1,152 21.8 | 26.3, 3,072 80 | 55.
 int run_token_scores(shotkv_ctx* ctx, const shotkv_dims* d, const float* imp, const ShotTable& tab, float* shot_scores, cudaStream_t stream) {
     const int bl = d->B * d->L;
-    return (long long)d->N >= (long long)kLongShot * d->S
-               ? launch(ctx, shot_score_from_tokens_kernel<kTokenWarps>, dim3(d->S, bl), 32 * kTokenWarps, 0, stream, 1, true, imp, tab,
-                        (int)d->L, (int)d->Hkv, (int)d->N, (int)d->S, shot_scores)
-               : launch(ctx, shot_score_from_tokens_kernel<1>, dim3((d->S + kTokenWarps - 1) / kTokenWarps, bl), 32 * kTokenWarps, 0, stream,
-                        1, true, imp, tab, (int)d->L, (int)d->Hkv, (int)d->N, (int)d->S, shot_scores);
+    const bool is_long = (long long)d->N >= (long long)kLongShot * d->S;
+    const bool few = (long long)d->S * bl <= 2LL * ctx->sm_count * (d->Hkv < kTokenWarps ? d->Hkv : kTokenWarps);
+    const auto run = [&](auto* kernel, int per_cta) {
+        return launch(ctx, kernel, dim3((d->S + per_cta - 1) / per_cta, bl), 32 * kTokenWarps, 0, stream, 1, true, imp, tab, (int)d->L,
+                      (int)d->Hkv, (int)d->N, (int)d->S, shot_scores);
+    };
+    if (!is_long) return run(shot_score_from_tokens_kernel<kHeadsAbreast>, kTokenWarps);
+    return few ? run(shot_score_from_tokens_kernel<kWholeCta>, 1) : run(shot_score_from_tokens_kernel<kTokensAhead>, kTokenWarps);
 }
 
 // Per-shot scores from the scoring pass's partials, and the selection.

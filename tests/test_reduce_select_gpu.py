@@ -91,3 +91,24 @@ def test_rows_that_are_not_numbers_carry_no_weight(ctx, what, mode, W):
     finally:
         skv.shotkv_set_scoring_mode(ctx, skv.SCORING_FAST)
     assert torch.allclose(got.double(), want, rtol=P.SCORE_RTOL, atol=P.SCORE_ATOL), (got, want)
+
+
+@pytest.mark.parametrize("B,L,S,mean,Hkv", [(1, 1, 3, 200, 1), (1, 297, 1, 130, 1), (2, 40, 7, 97, 2), (1, 37, 65, 129, 8), (1, 2, 40, 33, 3),
+                                            (3, 200, 8, 300, 8), (1, 600, 4, 160, 9)])
+def test_scores_from_token_importances(ctx, B, L, S, mean, Hkv):
+    """Short units, few long ones and many long ones, on both sides of the lines between the kernel's forms, lengths
+    around a run of 32 tokens among them.  Two orders of up to 4,000 positive fp32 terms: 1e-5 relative."""
+    rng = np.random.default_rng(S)
+    lens = np.maximum(1, rng.integers(mean // 2, 3 * mean // 2, size=(B, S)) // 32 * 32 + rng.integers(-1, 2, size=(B, S)))
+    off = np.concatenate([np.full((B, 1), 5), 5 + np.cumsum(lens, 1)], 1).astype(np.int32)
+    N = int(off.max()) + 40
+    dims, pol = skv.make_dims(B, L, Hkv, Hkv, 64, N, 8, S), skv.make_policy(r_p=0.5)
+    Mcap = skv.shotkv_kept_capacity(dims, pol, off)
+    out = skv.alloc_prefill_outputs(dims, Mcap)
+    imp = torch.rand(B, L, Hkv, N, device="cuda", generator=torch.Generator("cuda").manual_seed(S))
+    skv.shotkv_select_shots(ctx, dims, pol, imp, off, out["shot_scores"], out["keep"], out["kept_idx"], out["kept_count"], Mcap, out["ws"])
+    total = torch.nn.functional.pad(imp.double().sum(2).cumsum(-1), (1, 0))
+    for b in range(B):
+        o = torch.from_numpy(off[b]).long().cuda()
+        want = (total[b][:, o[1:]] - total[b][:, o[:-1]]) / (o[1:] - o[:-1])
+        assert torch.allclose(out["shot_scores"][b].double(), want, rtol=1e-5, atol=0)
