@@ -430,6 +430,7 @@ int launch_score_tc_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorMap
 // 3,630, 3,705 us a call), with 128 it waits for memory as much as for power (32 layers of 16K 395, -, 397,
 // 398, 399, 402).
 constexpr int kPolyEvery = 5, kPolyEveryStream = 3;
+constexpr int kShortUnit = 64;        // mean length below which the streaming kernel takes its form for short units
 
 template <int D>
 int launch_score_fast_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorMap& tmK, int qbox, int kbox,
@@ -446,7 +447,9 @@ int launch_score_stream_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtenso
     using Cfg = ScoreStreamCfg<D>;
     int grid = sp.total_items < ctx->sm_count ? sp.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    return launch(ctx, score_stream_kernel<D, kPolyEveryStream>, dim3(grid), Cfg::kThreads, Cfg::kSmemBytes, stream, 1, true, tmQ, tmK, qbox, kbox, sp, tab);
+    const bool few_tokens = sp.S > 0 && (long long)sp.N < (long long)kShortUnit * sp.S;
+    return launch(ctx, few_tokens ? score_stream_kernel<D, kPolyEveryStream, true> : score_stream_kernel<D, kPolyEveryStream, false>, dim3(grid),
+                  Cfg::kThreads, Cfg::kSmemBytes, stream, 1, true, tmQ, tmK, qbox, kbox, sp, tab);
 }
 
 // Tensor maps of Q (2-D: d x rows) and K (3-D: d x N x units), 64-element boxes with 128-byte swizzle, and the
@@ -728,7 +731,9 @@ cudaError_t set_tc_attributes() {
     if (e == cudaSuccess && MB == 1)
         e = cudaFuncSetAttribute(score_fast_kernel<D, kPolyEvery>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreFastCfg<D>::kSmemBytes);
     if (e == cudaSuccess && MB == 2)
-        e = cudaFuncSetAttribute(score_stream_kernel<D, kPolyEveryStream>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreStreamCfg<D>::kSmemBytes);
+        e = cudaFuncSetAttribute(score_stream_kernel<D, kPolyEveryStream, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreStreamCfg<D>::kSmemBytes);
+    if (e == cudaSuccess && MB == 2)
+        e = cudaFuncSetAttribute(score_stream_kernel<D, kPolyEveryStream, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreStreamCfg<D>::kSmemBytes);
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(colsum_tc_kernel<D, MB, kPolyEvery, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColsumTcCfg<D, MB>::kSmemBytes);
     if (e == cudaSuccess)
