@@ -119,13 +119,15 @@ int fail(shotkv_ctx* ctx, int code, const char* fmt, ...) {
         CUDA_TRY(ctx, cudaGetLastError());   \
     } while (0)
 
-// Launches `kernel` with thread-block clusters of `cluster` CTAs (1: none) and, with `early`, as a
+// Launches `kernel` with thread-block clusters of `cluster` CTAs (1: none) and, with kEarly in `how`, as a
 // programmatic dependent of what precedes it on the stream: it may begin before that has ended and
-// orders itself by grid_wait (common.cuh), so only a kernel that calls it may be launched so.
+// orders itself by grid_wait (common.cuh), so only a kernel that calls it may be launched so.  With kWideShared the
+// SMs split their memory as far in favour of shared memory as they can, whatever the kernel itself needs.
+constexpr int kEarly = 1, kWideShared = 2;
 template <class... P, class... A>
-int launch(shotkv_ctx* ctx, void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, int cluster, bool early,
+int launch(shotkv_ctx* ctx, void (*kernel)(P...), dim3 grid, int threads, size_t smem, cudaStream_t stream, int cluster, int how,
            A&&... args) {
-    cudaLaunchAttribute at[2] = {};
+    cudaLaunchAttribute at[3] = {};
     cudaLaunchConfig_t lc{};
     lc.gridDim = grid;
     lc.blockDim = dim3(threads);
@@ -138,7 +140,12 @@ int launch(shotkv_ctx* ctx, void (*kernel)(P...), dim3 grid, int threads, size_t
         at[lc.numAttrs].val.clusterDim.y = at[lc.numAttrs].val.clusterDim.z = 1;
         ++lc.numAttrs;
     }
-    if (early) {
+    if (how & kWideShared) {
+        at[lc.numAttrs].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+        at[lc.numAttrs].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+        ++lc.numAttrs;
+    }
+    if (how & kEarly) {
         at[lc.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
         at[lc.numAttrs].val.programmaticStreamSerializationAllowed = 1;
         ++lc.numAttrs;
@@ -421,7 +428,7 @@ int launch_score_tc_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorMap
     constexpr int smem = ScoreTcCfg<D, MB>::kSmemBytes;
     int grid = sp.total_items < ctx->sm_count ? sp.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    return launch(ctx, score_tc_kernel<D, MB>, dim3(grid), ScoreTcCfg<D, MB>::kThreads, smem, stream, 1, true, tmQ, tmK, qbox, kbox, sp, tab);
+    return launch(ctx, score_tc_kernel<D, MB>, dim3(grid), ScoreTcCfg<D, MB>::kThreads, smem, stream, 1, kEarly, tmQ, tmK, qbox, kbox, sp, tab);
 }
 
 // Column pairs, of every 16, whose exponentials run on the FMA pipe instead of the special-function unit.
@@ -438,7 +445,7 @@ int launch_score_fast_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorM
     constexpr int smem = ScoreFastCfg<D>::kSmemBytes;
     int grid = sp.total_items < ctx->sm_count ? sp.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    return launch(ctx, score_fast_kernel<D, kPolyEvery>, dim3(grid), ScoreFastCfg<D>::kThreads, smem, stream, 1, true, tmQ, tmK, qbox, kbox, sp, tab);
+    return launch(ctx, score_fast_kernel<D, kPolyEvery>, dim3(grid), ScoreFastCfg<D>::kThreads, smem, stream, 1, kEarly, tmQ, tmK, qbox, kbox, sp, tab);
 }
 
 template <int D>
@@ -449,7 +456,7 @@ int launch_score_stream_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtenso
     if (grid < 1) grid = 1;
     const bool few_tokens = sp.S > 0 && (long long)sp.N < (long long)kShortUnit * sp.S;
     return launch(ctx, few_tokens ? score_stream_kernel<D, kPolyEveryStream, true> : score_stream_kernel<D, kPolyEveryStream, false>, dim3(grid),
-                  Cfg::kThreads, Cfg::kSmemBytes, stream, 1, true, tmQ, tmK, qbox, kbox, sp, tab);
+                  Cfg::kThreads, Cfg::kSmemBytes, stream, 1, kEarly, tmQ, tmK, qbox, kbox, sp, tab);
 }
 
 // Tensor maps of Q (2-D: d x rows) and K (3-D: d x N x units), 64-element boxes with 128-byte swizzle, and the
@@ -508,7 +515,7 @@ int launch_colsum_tc_f(shotkv_ctx* ctx, const TcSetup& t, const ColsumTcParams& 
     constexpr int smem = ColsumTcCfg<D, MB>::kSmemBytes;
     int grid = cp.base.total_items < ctx->sm_count ? cp.base.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    return launch(ctx, colsum_tc_kernel<D, MB, kPolyEvery, FULL>, dim3(grid), ColsumTcCfg<D, MB>::kThreads, smem, stream, 1, true, t.tmQ, t.tmK, t.qbox, t.kbox, cp);
+    return launch(ctx, colsum_tc_kernel<D, MB, kPolyEvery, FULL>, dim3(grid), ColsumTcCfg<D, MB>::kThreads, smem, stream, 1, kEarly, t.tmQ, t.tmK, t.qbox, t.kbox, cp);
 }
 template <int D, int MB>
 int launch_colsum_tc_t(shotkv_ctx* ctx, const TcSetup& t, const ColsumTcParams& cp, cudaStream_t stream) {
@@ -586,7 +593,7 @@ int run_stats(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q, const
     const int rc = launch_score_tc(ctx, d, Q, K, w, -1, none, plan, stream);
     if (rc) return rc;
     prof_mark(ctx, stream);
-    return launch(ctx, row_stats_kernel, dim3(d->B * d->L * d->Hkv), rpad_of(d), 0, stream, 1, true, partial_view(ctx, d, w, -1, plan),
+    return launch(ctx, row_stats_kernel, dim3(d->B * d->L * d->Hkv), rpad_of(d), 0, stream, 1, kEarly, partial_view(ctx, d, w, -1, plan),
                   (d->H / d->Hkv) * d->W, w.row_m, w.row_invz);
 }
 
@@ -658,8 +665,8 @@ int run_select(shotkv_ctx* ctx, const shotkv_dims* d, const ShotTable& tab, cons
                cudaStream_t stream) {
     const size_t smem = bounds_smem_bytes(d->S) + select_smem_bytes(d->S);
     return d->S <= kRankByCount
-               ? launch(ctx, select_shots_kernel<kSelectThreads>, dim3(d->B * d->L), kSelectThreads, smem, stream, 1, true, shot_scores, tab, sa)
-               : launch(ctx, select_shots_kernel<kSortThreads>, dim3(d->B * d->L), kSortThreads, smem, stream, 1, true, shot_scores, tab, sa);
+               ? launch(ctx, select_shots_kernel<kSelectThreads>, dim3(d->B * d->L), kSelectThreads, smem, stream, 1, kEarly, shot_scores, tab, sa)
+               : launch(ctx, select_shots_kernel<kSortThreads>, dim3(d->B * d->L), kSortThreads, smem, stream, 1, kEarly, shot_scores, tab, sa);
 }
 
 // Per-shot scores from per-token importances.  A CTA takes one long shot while there are at most two of them to an
@@ -673,7 +680,7 @@ int run_token_scores(shotkv_ctx* ctx, const shotkv_dims* d, const float* imp, co
     const bool is_long = (long long)d->N >= (long long)kLongShot * d->S;
     const bool few = (long long)d->S * bl <= 2LL * ctx->sm_count * (d->Hkv < kTokenWarps ? d->Hkv : kTokenWarps);
     const auto run = [&](auto* kernel, int per_cta) {
-        return launch(ctx, kernel, dim3((d->S + per_cta - 1) / per_cta, bl), 32 * kTokenWarps, 0, stream, 1, true, imp, tab, (int)d->L,
+        return launch(ctx, kernel, dim3((d->S + per_cta - 1) / per_cta, bl), 32 * kTokenWarps, 0, stream, 1, kEarly, imp, tab, (int)d->L,
                       (int)d->Hkv, (int)d->N, (int)d->S, shot_scores);
     };
     if (!is_long) return run(shot_score_from_tokens_kernel<kHeadsAbreast>, kTokenWarps);
@@ -690,7 +697,7 @@ int run_reduce_select_t(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView
     while (ranks > 1 && reduce_smem_bytes(ROWS, pv.P, d->S, ranks) > kBigSmem / 2) ranks = (ranks + 1) / 2;
     const size_t smem = reduce_smem_bytes(ROWS, pv.P, d->S, ranks);
     if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "too many shots for the single-pass path (S = %d)", d->S);
-    return launch(ctx, reduce_select_kernel<ROWS>, dim3(d->B * d->L * ranks), kReduceThreads, smem, stream, ranks, true, pv, tab,
+    return launch(ctx, reduce_select_kernel<ROWS>, dim3(d->B * d->L * ranks), kReduceThreads, smem, stream, ranks, kEarly, pv, tab,
                   (d->H / d->Hkv) * d->W, (int)d->Hkv, ranks, shot_scores, sa);
 }
 int run_reduce_select(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView& pv, const ShotTable& tab, float* shot_scores,
@@ -707,9 +714,10 @@ int run_compact(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* K, con
     if (gx < 1) gx = 1;
     dim3 grid(gx, d->Hkv, d->B * d->L);
     if (grid.z > 65535) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "B*L must be <= 65535");
-    // begun early only where one wave of CTAs does all of it: with more, the waiting CTAs gained nothing and
-    // 4 x 32 layers of 32K lost 2 % (3,590 us a call against 3,525)
-    const bool early = (long long)grid.x * grid.y * grid.z <= 8LL * ctx->sm_count;
+    // begun early only where one or two waves of CTAs do all of it (four fit an SM): 416 CTAs 22.3 us a call against 23.7,
+    // 624 26.5 against 28.2, 1,144 44.6 against 46.4; with more, the waiting CTAs gain nothing (1,248 and 1,664 the same
+    // either way) and 4 x 32 layers of 32K lost 2 % (3,590 against 3,525)
+    const int early = (long long)grid.x * grid.y * grid.z <= 8LL * ctx->sm_count ? kEarly : 0;
     return launch(ctx, d->d == 128 ? compact_kv_kernel<128> : compact_kv_kernel<64>, grid, 256, 0, stream, 1, early, (const uint4*)K, (const uint4*)V,
                   kept_idx, kept_count, (int)d->Hkv, (int)d->N, (int)Mcap, (uint4*)Kc, (uint4*)Vc);
 }
@@ -1303,20 +1311,31 @@ int decode_split(const int* room, long long U, long long keys, int warps) {
     return n;
 }
 
+// Whole units of the fused step, more of them than SMs and at most two to an SM, are one uneven wave: its time is that of
+// the SMs with most CTAs.  Begun early, it was placed while CTAs of the kernel before still held 32 SMs or so that
+// had another split of shared memory, and put three on others: 256 units of 3,276 keys 78 us a step, of 16,000 keys 350.
+// The kernels that end a step therefore ask for this kernel's split here, and this one for so much shared memory that
+// no third CTA fits: 71 and 310 us (288 units 88 -> 81 and 382 -> 365).
+constexpr size_t kNoThirdCta = 80 * 1024;
+bool two_to_an_sm(const shotkv_ctx* ctx, const DecodeParams& p, int U) {
+    return p.nsplit == 1 && U > ctx->sm_count && U <= 2 * ctx->sm_count;
+}
+
 template <int D>
 int launch_decode_attend(shotkv_ctx* ctx, DecodeParams& p, int U, cudaStream_t stream) {
     using Cfg = AttendCfg<D>;
-    const size_t smem = attend_smem<D>(p.Dcap);
+    size_t smem = attend_smem<D>(p.Dcap);
     if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "Dcap too large for the attention-output step");
     p.nsplit = decode_split(ctx->room_attend[D == 128], U, (long long)p.Mcap + p.n_old + 1, Cfg::kWarps);
-    return launch(ctx, decode_attend_kernel<D>, dim3(U * p.nsplit), Cfg::kWarps * 32, smem, stream, p.nsplit, true, p);
+    if (two_to_an_sm(ctx, p, U) && smem < kNoThirdCta) smem = kNoThirdCta;
+    return launch(ctx, decode_attend_kernel<D>, dim3(U * p.nsplit), Cfg::kWarps * 32, smem, stream, p.nsplit, kEarly, p);
 }
 template <int D>
 int launch_decode_score(shotkv_ctx* ctx, DecodeParams& p, int U, cudaStream_t stream) {
     const size_t smem = score_smem(p.Dcap);
     p.nsplit = decode_split(ctx->room_score[D == 128], U, (long long)p.Mcap + p.n_old + 1, 8);
-    return p.nsplit > 1 ? launch(ctx, decode_score_kernel<D, true>, dim3(U * p.nsplit), 256, smem, stream, p.nsplit, true, p)
-                        : launch(ctx, decode_score_kernel<D, false>, dim3(U), 256, smem, stream, 1, true, p);
+    return p.nsplit > 1 ? launch(ctx, decode_score_kernel<D, true>, dim3(U * p.nsplit), 256, smem, stream, p.nsplit, kEarly, p)
+                        : launch(ctx, decode_score_kernel<D, false>, dim3(U), 256, smem, stream, 1, kEarly, p);
 }
 
 // One decode step; with `attn_out` the score kernel is the variant that also writes the attention output.
@@ -1363,12 +1382,13 @@ int decode_step_impl(shotkv_ctx* ctx, shotkv_decode_state* st, const shotkv_bf16
         if (f.k > f.n) f.k = f.n;
         f.protect_from = prot > 0 ? T - prot : 0x7fffffff;
     }
+    const int how = kEarly | (attn_out && two_to_an_sm(ctx, p, U) ? kWideShared : 0);
     if (f.k < f.n) {
         f.ranks = d.Hkv < kReduceCluster ? d.Hkv : kReduceCluster;
-        rc = d.d == 128 ? launch(ctx, decode_evict_kernel<128>, dim3(BL * f.ranks), kSelectThreads, decode_evict_smem_bytes(f.n), stream, f.ranks, true, f)
-                        : launch(ctx, decode_evict_kernel<64>, dim3(BL * f.ranks), kSelectThreads, decode_evict_smem_bytes(f.n), stream, f.ranks, true, f);
+        rc = d.d == 128 ? launch(ctx, decode_evict_kernel<128>, dim3(BL * f.ranks), kSelectThreads, decode_evict_smem_bytes(f.n), stream, f.ranks, how, f)
+                        : launch(ctx, decode_evict_kernel<64>, dim3(BL * f.ranks), kSelectThreads, decode_evict_smem_bytes(f.n), stream, f.ranks, how, f);
     } else {
-        rc = launch(ctx, decode_accumulate_kernel, dim3(BL, (f.n + kAccumulateThreads - 1) / kAccumulateThreads), kAccumulateThreads, 0, stream, 1, true, f);
+        rc = launch(ctx, decode_accumulate_kernel, dim3(BL, (f.n + kAccumulateThreads - 1) / kAccumulateThreads), kAccumulateThreads, 0, stream, 1, how, f);
     }
     if (rc) return rc;
     st->T = T;

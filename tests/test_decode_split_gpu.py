@@ -51,3 +51,10 @@ def test_query_that_is_not_a_number_gives_no_output(ctx, M):
     want[2] = 0
     err = (gpu.out[0, 0].double() - want[:, 0]).abs()
     assert (err <= OUT_RTOL * want[:, 0].abs().amax(1, keepdim=True) + OUT_ATOL).all(), err.amax(1)
+
+
+@pytest.mark.parametrize("L", [19, 32, 37])
+def test_whole_units_two_to_an_sm(ctx, L):
+    """More units than SMs and at most two to an SM, an eviction among the steps."""
+    cfg = wl.DecodeConfig("pairs", B=1, L=L, H=32, Hkv=8, d=128, steps=9, r_d=0.5, recompress_every=4, cfg_id=75)
+    assert lockstep(ctx, cfg, 300, [(0, 0), (0, L - 1)], attend=True) <= 1
