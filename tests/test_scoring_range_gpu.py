@@ -65,13 +65,13 @@ def test_some_of_the_items_of_every_cta_out_of_range(d, H, W):
 
 
 @pytest.mark.parametrize("d", [64, 128])
-@pytest.mark.parametrize("mean", [20, 62, 66])
+@pytest.mark.parametrize("mean", [20, 50, 66])
 def test_out_of_range_among_short_units(mean, d):
     """Units on both sides of the length below which a piece's sum is not looked at for itself: the item of the one
     key out of range is recomputed and no other."""
     ctx = skv.Context(0)
     S = 1800 // mean
-    cfg = wl.PrefillConfig("short", B=1, L=4, H=32, Hkv=8, d=d, N=S * (mean - 6) + 150, W=64, S=S, shot_dist="uniform", shot_lo=mean - 6,
+    cfg = wl.PrefillConfig("short", B=1, L=4, H=32, Hkv=8, d=d, N=S * mean + 150, W=64, S=S, shot_dist="uniform", shot_lo=mean - 6,
                            shot_hi=mean + 6, question_len=150, r_p=0.5, cfg_id=27)
     Q, K, V, off = wl.prefill_batch(cfg, "cuda")
     Q[..., 0], K[..., 0] = 8.0, 0.0
