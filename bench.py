@@ -49,8 +49,8 @@ FALLBACK_BF16_TFLOPS_SUSTAINED = 1400.0  # the same, back to back under the powe
 # A ratio is set to None whenever its kernel has changed since its capture.
 SCORE_TC_TRAFFIC_RATIO = 1.041
 SCORE_FAST_TRAFFIC_RATIO = 1.021      # the 128-row kernel on config 2 at full size
-DECODE_TRAFFIC_RATIO = 1.012
-DECODE_ATTEND_TRAFFIC_RATIO = 1.006
+DECODE_TRAFFIC_RATIO = None
+DECODE_ATTEND_TRAFFIC_RATIO = None
 NOMINAL_HBM_GBS = 8000.0
 SUSTAIN_SECONDS = 2.5           # length of the sustained repeat of the step
 SCORING_MODES = {"fast": 0, "exact": 1}
@@ -325,7 +325,7 @@ def run_ours(args):
                   "frac": round(achieved_tf / tf_sustained, 4), "frac_of_burst_peak": round(achieved_tf / tf_burst, 4),
                   "floor_ms": round(flops / tf_sustained / 1e9, 4)}
     # one exponential per logit: 16 per clock per SM is what the special-function unit alone delivers
-    # (measured); the kernel takes 5 of every 16 column pairs on the FMA pipe instead, so this
+    # (measured); the kernel takes 3 or 5 of every 16 column pairs on the FMA pipe instead, so this
     # fraction may pass 1
     alu_rec = {"bound": "alu", "unit": "exp/clk/SM", "achieved": round(ex2_rate, 2), "peak": 16.0,
                "frac": round(ex2_rate / 16.0, 4), "at_sm_mhz": sm_mhz,

@@ -329,7 +329,8 @@ SHOTKV_API int shotkv_selftest_bounded_wait(shotkv_ctx* ctx, int64_t limit_cycle
  * ran for (its own cycle counter and the GPU's nanosecond timer, read at its start and end).  Their
  * quotient is the SM clock the kernel really ran at -- under a power cap that is not the clock a
  * sampler reads between kernels -- and cycles / tiles per SM is the kernel's cost per tile in the
- * unit its arithmetic is counted in.  Valid once the launch has finished (synchronise first).  */
+ * unit its arithmetic is counted in.  Valid once the launch has finished (synchronise first); waits for
+ * no other stream, and may be called while one is captured.  */
 SHOTKV_API int shotkv_last_scoring_clock(const shotkv_ctx* ctx, int64_t* cycles, int64_t* nanoseconds);
 
 /* Groups the single-pass form of shotkv_prefill_compress pipelines its units in: 0 (default)

@@ -17,9 +17,9 @@
 // epilogue takes the same cycles per tile with or without the MMAs running beside it, but the GPU
 // settles near 1.5 GHz with them and at its full 1.96 GHz without.  The polynomial costs 5.5 issue
 // slots per logit against 2 for the special-function path, so a larger share on the FMA pipe
-// (PE of every 16 column pairs) saves cycles and spends energy; measured at the cap, shares from 2
-// to 5 of 16 come out within the noise of the power controller, and below the cap the larger
-// share is faster.
+// (PE of every 16 column pairs) saves cycles and spends energy.  Measured with 3 against 5 of 16: at the cap (4 x 32
+// layers of 32K) 3,980 against 3,999 us a call, below it (one to four layers of 16K, 4 to 32 layers of 4K to 8K) 0 to 2 %
+// faster, with 16-token units alone 1 % slower.
 #pragma once
 #include "score_fast.cuh"
 

@@ -59,7 +59,7 @@ struct TraceRange {
 struct shotkv_ctx {
     int device = 0;
     char err[512] = {0};
-    // pinned staging ring for the small host tables (offsets, piece lists) that go to the device
+    // pinned staging ring for the small host tables (shot boundaries) that go to the device
     unsigned char* stage = nullptr;
     cudaEvent_t stage_done[kStageSlots] = {};
     int stage_next = 0;
@@ -436,7 +436,7 @@ int launch_score_tc_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorMap
 // power cap for as long as it runs (5, 4, 3, 2, 1, 0 pairs: 4 x 32 layers of 32K 3,570, 3,550, 3,530, 3,580,
 // 3,630, 3,705 us a call), with 128 it waits for memory as much as for power (32 layers of 16K 395, -, 397,
 // 398, 399, 402).
-constexpr int kPolyEvery = 5, kPolyEveryStream = 3;
+constexpr int kPolyPairs = 5, kPolyPairsStream = 3;
 constexpr int kShortUnit = 64;        // mean length below which the streaming kernel takes its form for short units
 
 template <int D>
@@ -445,7 +445,7 @@ int launch_score_fast_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorM
     constexpr int smem = ScoreFastCfg<D>::kSmemBytes;
     int grid = sp.total_items < ctx->sm_count ? sp.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    return launch(ctx, score_fast_kernel<D, kPolyEvery>, dim3(grid), ScoreFastCfg<D>::kThreads, smem, stream, 1, kEarly, tmQ, tmK, qbox, kbox, sp, tab);
+    return launch(ctx, score_fast_kernel<D, kPolyPairs>, dim3(grid), ScoreFastCfg<D>::kThreads, smem, stream, 1, kEarly, tmQ, tmK, qbox, kbox, sp, tab);
 }
 
 template <int D>
@@ -455,7 +455,7 @@ int launch_score_stream_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtenso
     int grid = sp.total_items < ctx->sm_count ? sp.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
     const bool few_tokens = sp.S > 0 && (long long)sp.N < (long long)kShortUnit * sp.S;
-    return launch(ctx, few_tokens ? score_stream_kernel<D, kPolyEveryStream, true> : score_stream_kernel<D, kPolyEveryStream, false>, dim3(grid),
+    return launch(ctx, few_tokens ? score_stream_kernel<D, kPolyPairsStream, true> : score_stream_kernel<D, kPolyPairsStream, false>, dim3(grid),
                   Cfg::kThreads, Cfg::kSmemBytes, stream, 1, kEarly, tmQ, tmK, qbox, kbox, sp, tab);
 }
 
@@ -515,7 +515,7 @@ int launch_colsum_tc_f(shotkv_ctx* ctx, const TcSetup& t, const ColsumTcParams& 
     constexpr int smem = ColsumTcCfg<D, MB>::kSmemBytes;
     int grid = cp.base.total_items < ctx->sm_count ? cp.base.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    return launch(ctx, colsum_tc_kernel<D, MB, kPolyEvery, FULL>, dim3(grid), ColsumTcCfg<D, MB>::kThreads, smem, stream, 1, kEarly, t.tmQ, t.tmK, t.qbox, t.kbox, cp);
+    return launch(ctx, colsum_tc_kernel<D, MB, kPolyPairs, FULL>, dim3(grid), ColsumTcCfg<D, MB>::kThreads, smem, stream, 1, kEarly, t.tmQ, t.tmK, t.qbox, t.kbox, cp);
 }
 template <int D, int MB>
 int launch_colsum_tc_t(shotkv_ctx* ctx, const TcSetup& t, const ColsumTcParams& cp, cudaStream_t stream) {
@@ -537,7 +537,7 @@ int launch_colsum_tc(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q
     return big ? launch_colsum_tc_t<64, 2>(ctx, t, cp, stream) : launch_colsum_tc_t<64, 1>(ctx, t, cp, stream);
 }
 
-// The scoring pass; S = -1: chunk ends alone cut the keys (`tab` is not read).
+// The scoring pass; S = -1: chunk ends alone cut the keys (`tab` then holds the three closing entries of empty_table).
 int launch_score_tc(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q, const shotkv_bf16* K, const PrefillWs& w,
                     int S, const ShotTable& tab, const ChunkPlan& plan, cudaStream_t stream) {
     TcSetup t;
@@ -737,15 +737,15 @@ cudaError_t set_tc_attributes() {
     cudaError_t e = cudaFuncSetAttribute(score_tc_kernel<D, MB>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreTcCfg<D, MB>::kSmemBytes);
     // the first scoring launch: one 128-row block of Q -> score_fast_kernel, two -> score_stream_kernel
     if (e == cudaSuccess && MB == 1)
-        e = cudaFuncSetAttribute(score_fast_kernel<D, kPolyEvery>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreFastCfg<D>::kSmemBytes);
+        e = cudaFuncSetAttribute(score_fast_kernel<D, kPolyPairs>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreFastCfg<D>::kSmemBytes);
     if (e == cudaSuccess && MB == 2)
-        e = cudaFuncSetAttribute(score_stream_kernel<D, kPolyEveryStream, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreStreamCfg<D>::kSmemBytes);
+        e = cudaFuncSetAttribute(score_stream_kernel<D, kPolyPairsStream, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreStreamCfg<D>::kSmemBytes);
     if (e == cudaSuccess && MB == 2)
-        e = cudaFuncSetAttribute(score_stream_kernel<D, kPolyEveryStream, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreStreamCfg<D>::kSmemBytes);
+        e = cudaFuncSetAttribute(score_stream_kernel<D, kPolyPairsStream, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreStreamCfg<D>::kSmemBytes);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(colsum_tc_kernel<D, MB, kPolyEvery, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColsumTcCfg<D, MB>::kSmemBytes);
+        e = cudaFuncSetAttribute(colsum_tc_kernel<D, MB, kPolyPairs, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColsumTcCfg<D, MB>::kSmemBytes);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(colsum_tc_kernel<D, MB, kPolyEvery, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColsumTcCfg<D, MB>::kSmemBytes);
+        e = cudaFuncSetAttribute(colsum_tc_kernel<D, MB, kPolyPairs, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColsumTcCfg<D, MB>::kSmemBytes);
     return e;
 }
 cudaError_t set_kernel_attributes() {
@@ -1247,6 +1247,7 @@ int shotkv_prefill_compress_host(shotkv_ctx* ctx, const shotkv_dims* dims, const
 size_t shotkv_decode_workspace_bytes(const shotkv_dims* dims, int32_t Dcap) {
     if (!dims || Dcap < 1 || dims->B < 1 || dims->L < 1 || dims->Hkv < 1) return 0;
     const size_t BL = (size_t)dims->B * dims->L;
+    // the heads' partial sums; the second part is not used any more, but programs size their buffers by this figure
     return align_up(BL * dims->Hkv * (size_t)Dcap * 4) + align_up(BL * (size_t)Dcap * 4);
 }
 

@@ -46,7 +46,7 @@ def test_prefill_between_other_work(ctx, how, path, W):
     side = torch.cuda.Stream()
     for _ in range(5):
         Kin.zero_(); Vin.zero_()
-        for n in ("shot_scores", "Kc", "Vc", "token_importance"):
+        for n in ("shot_scores", "keep", "kept_idx", "kept_count", "Kc", "Vc", "token_importance"):
             out[n].zero_()
         if how == "copy":
             torch.cuda._sleep(SLEEP)
@@ -64,7 +64,8 @@ def test_prefill_between_other_work(ctx, how, path, W):
         Kin.zero_(); Vin.zero_()                       # right behind the call
         kept = out["Kc"].clone()
         torch.cuda.synchronize()
-        assert torch.equal(out["shot_scores"], ref["shot_scores"]) and torch.equal(out["kept_idx"], ref["kept_idx"])
+        for n in ("shot_scores", "keep", "kept_idx", "kept_count"):
+            assert torch.equal(out[n], ref[n]), n
         assert torch.equal(kept, ref["Kc"]) and torch.equal(out["Vc"], ref["Vc"])
         if flags:
             assert torch.equal(out["token_importance"], ref["token_importance"])

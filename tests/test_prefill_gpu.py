@@ -325,7 +325,7 @@ def test_full_size_results_repeat_bit_exactly(ctx, cid):
     """Every reduction on the prefill path has a fixed order (per-piece sums inside one thread, pieces
     and rows merged in index order, no atomics on floating point), so repeated runs over the same
     bytes must agree bit for bit.  At the benchmark's sizes, where 148 persistent CTAs, their
-    producer, MMA and epilogue roles and (config 3) the repair launch all run concurrently, a run
+    producer, MMA and epilogue roles and (config 3) the repair at its end all run concurrently, a run
     that differs from the first one is a race: 24 runs of the single-pass form and 6 of the
     per-token form, all outputs compared with the first run's."""
     cfg = wl.CONFIGS[cid]
