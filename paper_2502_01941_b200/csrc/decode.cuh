@@ -20,32 +20,107 @@ struct DecodeParams {
     float scale_log2;
     const __nv_bfloat16* Vc;      // [U][Mcap][d]   (attention-output variant only)
     float* out;                   // [B][L][H][d]   (attention-output variant only)
+    int* err;                     // error word (host-visible); set to 1 when a bounded wait gave up
 };
 
 // ---- a unit's keys shared by a cluster -------------------------------------------------------
 // A unit (sequence, layer, kv head) whose batch is too small to fill the GPU is shared by a cluster of
 // p.nsplit CTAs: blocks of 16 keys go round the warps of all of them.  Every CTA sends its (m, z) per
 // query row to all others and each then knows the whole row's maximum and sum.
-constexpr int kMaxSplit = 8;
+constexpr int kMaxSplit = 16;
 
-// Every CTA's (m, z) of the 8 query rows (`own`, [8][2], in shared memory behind a barrier) to all
-// CTAs' `table` [nsplit][8][2]; returns when all have arrived.  Preceded by a cluster_arrive at the
-// start of the kernel (a CTA's memory may be written once it has begun).  What the CTA wrote to its own
-// shared memory before may be read by the others afterwards; they must be done before it ends.
-__device__ __forceinline__ void exchange_stats(const float* own, float* table, int rank, int nsplit) {
-    cluster_wait();
-#pragma unroll 1
-    for (int i = threadIdx.x; i < 16 * nsplit; i += blockDim.x) cluster_store(table + rank * 16 + (i & 15), i >> 4, own[i & 15]);
-    cluster_arrive();
-    cluster_wait();
+// What CTAs tell one another goes as messages: a store counts its bytes on the receiver's barrier, which is complete when
+// as many as the receiver expects are there.  That is one way across the cluster, where a barrier of all its threads is two
+// (1.7 us of a step of 4 sequences x 1 layer).  expect_messages: by one thread, ahead of the cluster_arrive at the start;
+// nobody sends before a cluster_wait (a CTA's memory may be written once it has begun), and a CTA that has been sent
+// everything may end.
+constexpr long long kMessageCycles = 4000000000LL;     // limit of the wait for them: about two seconds
+__device__ __forceinline__ void expect_messages(unsigned long long* bar, int bytes) {
+    const uint32_t b = smem_u32(bar);
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
 }
-// The row's maximum and 1 / sum over the whole cluster.
-__device__ __forceinline__ void merge_stats(const float* table, int nsplit, int row, float& m, float& iz) {
+__device__ __forceinline__ void send(float2* to, int rank, unsigned long long* bar, float2 v) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(cluster_addr(to, rank)),
+                 "f"(v.x), "f"(v.y), "r"(cluster_addr(bar, rank))
+                 : "memory");
+}
+__device__ __forceinline__ void send(float4* to, int rank, unsigned long long* bar, float4 v) {
+    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(cluster_addr(to, rank)),
+                 "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(cluster_addr(bar, rank))
+                 : "memory");
+}
+// Waits until all bytes expected are there; a wait that runs into its limit sets the error word.
+__device__ __forceinline__ void await_messages(unsigned long long* bar, int* err) {
+    const uint32_t b = smem_u32(bar);
+    const long long t0 = clock64();
+    for (;;) {
+        uint32_t done;
+        asm volatile(
+            "{\n\t.reg .pred q;\n\t"
+            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], 0;\n\t"
+            "selp.u32 %0, 1, 0, q;\n\t}"
+            : "=r"(done)
+            : "r"(b)
+            : "memory");
+        if (done) return;
+        if (clock64() - t0 > kMessageCycles) {
+            atomicExch(err, 1);
+            return;
+        }
+    }
+}
+// (m, z) of row r over the NW warps' sums in `sred`, [NW][8 rows], and the warps' factors (negative: nothing to add).
+template <int NW>
+__device__ __forceinline__ float2 row_of_cta(const float2* sred, int r, float (&f)[NW]) {
+    float2 w[NW];
+#pragma unroll
+    for (int i = 0; i < NW; ++i) w[i] = sred[i * 8 + r];
+    float m = SHOTKV_NEG_INF, z = 0.f;
+#pragma unroll
+    for (int i = 0; i < NW; ++i) m = fmaxf(m, w[i].x);
+    const float mu = m == SHOTKV_NEG_INF ? 0.f : m;        // a CTA of a cluster may have had no keys
+#pragma unroll
+    for (int i = 0; i < NW; ++i) {
+        const float e = ex2f(w[i].x - mu);
+        z += w[i].y * e;
+        f[i] = w[i].x == SHOTKV_NEG_INF ? -1.f : e;
+    }
+    return make_float2(m, z);
+}
+// Row lane / 4 over `parts` sums (those of the warps, or of the cluster's CTAs) in `table`, [parts][8 rows]: its maximum m and
+// 1 / its sum, the same in the four lanes of the row, of which each takes every fourth.
+__device__ __forceinline__ void row_of_unit(const float2* table, int parts, float& m, float& iz) {
+    const int lane = threadIdx.x & 31;
+    float2 part[kMaxSplit / 4];
     m = SHOTKV_NEG_INF;
-    for (int c = 0; c < nsplit; ++c) m = fmaxf(m, table[c * 16 + row * 2]);
+#pragma unroll
+    for (int i = 0; i < kMaxSplit / 4; ++i) {
+        const int c = (lane & 3) + 4 * i;
+        part[i] = c < parts ? table[c * 8 + (lane >> 2)] : make_float2(SHOTKV_NEG_INF, 0.f);
+        m = fmaxf(m, part[i].x);
+    }
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+    const float mu = m == SHOTKV_NEG_INF ? 0.f : m;        // a row without a finite logit has no weight anywhere
     float z = 0.f;
-    for (int c = 0; c < nsplit; ++c) z += table[c * 16 + row * 2 + 1] * ex2f(table[c * 16 + row * 2] - m);
+#pragma unroll
+    for (int i = 0; i < kMaxSplit / 4; ++i) z += part[i].y * ex2f(part[i].x - mu);
+    z += __shfl_xor_sync(0xffffffffu, z, 1);
+    z += __shfl_xor_sync(0xffffffffu, z, 2);
     iz = z > 0.f ? 1.f / z : 0.f;
+}
+// Weight of decode entry j summed over the G query rows, from its logits in `sdec`, [G or 8][Dcap]; (m, iz) from row_of_unit.
+// All lanes call; `valid`: this lane has an entry.
+__device__ __forceinline__ float entry_weight(const float* sdec, int Dcap, int G, int j, bool valid, float m, float iz) {
+    float s = 0.f;
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        const float mr = __shfl_sync(0xffffffffu, m, r * 4), izr = __shfl_sync(0xffffffffu, iz, r * 4);
+        if (valid && r < G) s += ex2f(sdec[r * Dcap + j] - mr) * izr;
+    }
+    return s;
 }
 
 // One CTA, or a cluster of p.nsplit, per (sequence, layer, kv head).  Each warp takes 16 keys at a
@@ -55,40 +130,38 @@ __device__ __forceinline__ void merge_stats(const float* table, int nsplit, int 
 // of the decode entries are parked in shared memory until the softmax statistics over all keys
 // (kept prefill keys + decode keys) are known.
 // A shared unit leaves few warps to an SM, so each asks for its next block before it computes this one.
-// SPLIT = false is the same for whole units, nsplit = 1: with the stride of the loop a constant the
-// compiler unrolls it and keeps more loads in flight (8 sequences x 32 layers: 245 us a step against 273).
+// SPLIT = false is the same for whole units, nsplit = 1: with the stride of the loop a constant it is
+// unrolled and more loads are in flight, to the depth that is written down here (left to itself the compiler
+// chose 1 to 4 by what stood around the loop: 8 sequences x 32 layers 301 to 259 us a step, 1 sequence 56 to 43; four
+// deep 255 and 39.5).
 template <int D, bool SPLIT>
 __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p) {
     constexpr int NB = D / 32;     // 32-dim blocks
     constexpr int VPR = D / 8;     // 16-byte vectors per row
     extern __shared__ __align__(16) unsigned char dsm[];
     float* sdec = reinterpret_cast<float*>(dsm);             // [8][Dcap]
-    float* sred = sdec + 8 * p.Dcap;                         // [8 warps][8 rows][2]
-    float* sfin = sred + 8 * 8 * 2;                          // [8 rows][2]  (m, z) of this CTA, then (m, 1/Z)
-    float* stab = sfin + 16;                                 // [nsplit][8 rows][2]  (m, z) of the cluster's CTAs
+    float2* sred = reinterpret_cast<float2*>(sdec + 8 * p.Dcap);   // [8 warps][8 rows]  (m, z)
+    float2* stab = sred + 8 * 8;                             // [kMaxSplit][8 rows]  (m, z) of the cluster's CTAs
+    unsigned long long* arrived = reinterpret_cast<unsigned long long*>(stab + kMaxSplit * 8);   // of a cluster: barrier of what they send here
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, t4 = lane & 3;
     const int nsplit = SPLIT ? p.nsplit : 1;
     const int u = blockIdx.x / nsplit, rank = blockIdx.x - u * nsplit;
-    if (SPLIT) cluster_arrive();
+    if (SPLIT) {
+        if (tid == 0) expect_messages(arrived, nsplit * 8 * (int)sizeof(float2));
+        cluster_arrive();
+    }
     grid_wait();
     grid_release();
     const int bl = u / p.Hkv, hk = u - bl * p.Hkv;
-    const int M = min(p.kept_count[bl], p.Mcap);
-    const int n = p.n_old + 1;
-    const int Ktot = M + n;
     const uint4* Kc_u = reinterpret_cast<const uint4*>(p.Kc + (size_t)u * p.Mcap * D);
     uint4* Kd_u = reinterpret_cast<uint4*>(p.Kd + (size_t)u * p.Dcap * D);
     uint4* Vd_u = reinterpret_cast<uint4*>(p.Vd + (size_t)u * p.Dcap * D);
     const uint4* knew_u = reinterpret_cast<const uint4*>(p.k_new + (size_t)u * D);
     const uint4* vnew_u = reinterpret_cast<const uint4*>(p.v_new + (size_t)u * D);
-
-    // append the new token's key and value as decode entry n_old
-    if (rank != 0) {
-    } else if (tid < VPR) Kd_u[(size_t)p.n_old * VPR + tid] = knew_u[tid];
-    else if (tid < 2 * VPR) Vd_u[(size_t)p.n_old * VPR + (tid - VPR)] = vnew_u[tid - VPR];
-
+    // the kept count, the queries and the new token's rows are asked for at once
+    const int kept = p.kept_count[bl];
     // query rows of this group as B fragments (row g of the fragment = query head hk*G+g)
     uint4 qf[NB];
     {
@@ -96,6 +169,14 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p)
 #pragma unroll
         for (int kb = 0; kb < NB; ++kb) qf[kb] = g < p.G ? qrow[kb * 4 + t4] : make_uint4(0, 0, 0, 0);
     }
+    const bool appends = rank == 0 && tid < 2 * VPR;         // the CTA that appends the new token's rows
+    uint4 fresh_row = make_uint4(0, 0, 0, 0);
+    if (appends) fresh_row = (tid < VPR ? knew_u + tid : vnew_u + (tid - VPR))[0];
+    const int M = min(kept, p.Mcap);
+    const int n = p.n_old + 1;
+    const int Ktot = M + n;
+    if (SPLIT) cluster_wait();                               // all CTAs of the cluster have begun: their memory may be written to
+    if (appends) (tid < VPR ? Kd_u + (size_t)p.n_old * VPR + tid : Vd_u + (size_t)p.n_old * VPR + (tid - VPR))[0] = fresh_row;   // decode entry n_old
 
     auto row_ptr = [&](int i, bool valid) -> const uint4* {
         if (!valid) return knew_u;                         // any readable row; the result is masked
@@ -123,6 +204,7 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p)
     float m0 = SHOTKV_NEG_INF, m1 = SHOTKV_NEG_INF, z0 = 0.f, z1 = 0.f;   // query rows 2*t4, 2*t4+1
     const int first = (rank * 8 + warp) * 16;
     if (SPLIT && first < Ktot) load(first, n_lo, n_hi);
+#pragma unroll 4
     for (int base = first; base < Ktot; base += nsplit * 8 * 16) {
         const int ia = base + g, ib = base + g + 8;
         const bool va = ia < Ktot, vb = ib < Ktot;
@@ -186,40 +268,32 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p)
         }
     }
     if (g == 0) {
-        sred[(warp * 8 + 2 * t4) * 2 + 0] = m0;
-        sred[(warp * 8 + 2 * t4) * 2 + 1] = z0;
-        sred[(warp * 8 + 2 * t4 + 1) * 2 + 0] = m1;
-        sred[(warp * 8 + 2 * t4 + 1) * 2 + 1] = z1;
-    }
-    __syncthreads();
-    if (tid < 8) {
-        float m = SHOTKV_NEG_INF;
-        for (int w = 0; w < 8; ++w) m = fmaxf(m, sred[(w * 8 + tid) * 2]);
-        const float mu = m == SHOTKV_NEG_INF ? 0.f : m;      // a CTA of a cluster may have had no keys
-        float z = 0.f;
-        for (int w = 0; w < 8; ++w) z += sred[(w * 8 + tid) * 2 + 1] * ex2f(sred[(w * 8 + tid) * 2] - mu);
-        sfin[tid * 2] = m;
-        sfin[tid * 2 + 1] = SPLIT ? z : (z > 0.f ? 1.f / z : 0.f);
+        sred[warp * 8 + 2 * t4] = make_float2(m0, z0);
+        sred[warp * 8 + 2 * t4 + 1] = make_float2(m1, z1);
     }
     __syncthreads();
     if (SPLIT) {
-        exchange_stats(sfin, stab, rank, nsplit);
-        if (tid < 8) merge_stats(stab, nsplit, tid, sfin[tid * 2], sfin[tid * 2 + 1]);
-        __syncthreads();
+        if (tid < 8 * nsplit) {                            // every CTA's rows to every CTA
+            float f[8];
+            send(stab + rank * 8 + (tid & 7), tid >> 3, arrived, row_of_cta(sred, tid & 7, f));
+        }
+        await_messages(arrived, p.err);
     }
-    auto weight = [&](int j) {
-        float s = 0.f;
-        for (int r = 0; r < p.G; ++r) s += ex2f(sdec[r * p.Dcap + j] - sfin[r * 2]) * sfin[r * 2 + 1];
-        p.partial[(size_t)u * p.Dcap + j] = s;
-    };
+    float rm, riz;                                         // of row lane / 4, over all keys of the unit
+    row_of_unit(SPLIT ? stab : sred, SPLIT ? nsplit : 8, rm, riz);
     if (SPLIT) {                                           // the decode entries among this warp's blocks
         const int stride = nsplit * 8 * 16;
         for (int base = first + max(0, (M - 15 - first + stride - 1) / stride) * stride; base < Ktot; base += stride) {
             const int j = base + lane - M;
-            if (lane < 16 && j >= 0 && j < n) weight(j);
+            const bool entry = lane < 16 && j >= 0 && j < n;
+            const float s = entry_weight(sdec, p.Dcap, p.G, j, entry, rm, riz);
+            if (entry) p.partial[(size_t)u * p.Dcap + j] = s;
         }
     } else {
-        for (int j = tid; j < n; j += 256) weight(j);
+        for (int j0 = warp * 32; j0 < n; j0 += 256) {
+            const float s = entry_weight(sdec, p.Dcap, p.G, j0 + lane, j0 + lane < n, rm, riz);
+            if (j0 + lane < n) p.partial[(size_t)u * p.Dcap + j0 + lane] = s;
+        }
     }
 }
 
@@ -260,8 +334,7 @@ struct AttendCfg {
     static constexpr int kTileBytes = 16 * kRowBytes;             // 16 rows of keys (or of values)
     static constexpr int kStageBytes = 2 * kTileBytes;
     static constexpr int kRingBytes = kWarps * kStages * kStageBytes;
-    static constexpr int kOBytes = kWarps * 8 * D * 4;            // the warps' outputs for the final merge (reuses the ring)
-    static_assert(kOBytes <= kRingBytes, "the merge area must fit into the ring");
+    static_assert(8 * D * 4 <= kStages * kStageBytes, "a warp's outputs take the place of its ring");
 };
 
 // The same step with the attention output fused in: o_h = sum_t alpha_{t,h} v_t over the kept
@@ -273,6 +346,9 @@ struct AttendCfg {
 // accumulators of the output leave too few registers for enough such warps.  So nothing is loaded
 // into registers from global memory here: key and value rows go global -> shared by cp.async one
 // block ahead of their use, into a per-warp ring (measured: two stages with three CTAs on an SM beat three stages with two).
+// The ring comes first in shared memory: its rows lie on 128-byte boundaries as they do in global memory, or a warp's copy
+// of 512 bytes takes five lines of it and part of its sectors from L2 twice (40 % more of them with the ring 16 bytes off a boundary;
+// 8 sequences x 32 layers 580 us a step there, 511 at 64 bytes, 495 at 128).
 //
 // Both products run on the tensor cores, transposed so that the few query rows of a group are the
 // narrow N = 8 side.  Per block of 16 keys a warp computes S^T[rows x keys] = Q . K^T with the
@@ -289,8 +365,10 @@ struct AttendCfg {
 // masks and parked logits are left to the blocks that need them, and the first product runs as four chains
 // of MMAs.  32 steps of 8 sequences x 32 layers 16.25 -> 15.93 ms, a step of 4 sequences x 1 layer 17.0 -> 15.9 us,
 // one unit of 8,000 keys 20.0 -> 15.5 us.
-// What follows the blocks runs once and its loops are not unrolled: code that runs once is fetched cold (32 steps
-// of one layer 439.2 -> 435.8 us).
+// Of a step of few units (13 us: 4 sequences x 1 layer, 3,276 keys) less than half was blocks of keys.  The rest is a chain of
+// latencies: everything the first two blocks need is now asked for in one go, each warp's outputs take the place of its own
+// ring (no barrier before they are written), every thread merges the rows it needs for itself, and the CTAs of a cluster
+// send each other their rows and the quads of output each adds up (12.9 -> 11.1 us; 2 sequences 12.2 -> 9.2).
 template <int D>
 __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_kernel(const DecodeParams p) {
     using Cfg = AttendCfg<D>;
@@ -299,21 +377,43 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     constexpr int MT = D / 16;     // 16-dim tiles of the output
     constexpr int NW = Cfg::kWarps, NS = Cfg::kStages, NT = NW * 32;
     extern __shared__ __align__(16) unsigned char dsm[];
-    float* sdec = reinterpret_cast<float*>(dsm);             // [8][Dcap]
-    float* sred = sdec + 8 * p.Dcap;                         // [NW warps][8 rows][2]
-    float* sfin = sred + NW * 8 * 2;                         // [8 rows][2]  (m, z) of this CTA, then (m, 1/Z)
-    float* stab = sfin + 16;                                 // [kMaxSplit][8 rows][2]  (m, z) of the cluster's CTAs
-    unsigned char* ring = reinterpret_cast<unsigned char*>(stab + kMaxSplit * 16);   // [NW][NS][keys | values][16 rows][D bf16]; later [NW][8 rows][D] floats
-    float* sO = reinterpret_cast<float*>(ring);
+    unsigned char* ring = dsm;                               // [NW][NS][keys | values][16 rows][D bf16]; later each warp's outputs [8 rows][PITCH]
+    float2* sred = reinterpret_cast<float2*>(ring + Cfg::kRingBytes + 16);   // [NW warps][8 rows]  (m, z)
+    float* sdec = reinterpret_cast<float*>(sred + NW * 8);   // [G][Dcap]  logits of the decode entries
+    float2* stab = reinterpret_cast<float2*>(sdec + ((p.G * p.Dcap + 3) & ~3));   // of a cluster: [nsplit][8 rows]  (m, z) of its CTAs,
+    float4* sin = reinterpret_cast<float4*>(stab + p.nsplit * 8);   // [nsplit][share]  and their outputs: this CTA's share of the quads
+    unsigned long long* arrived = reinterpret_cast<unsigned long long*>(sred) - 1;   // barrier of what they send here
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, t4 = lane & 3;
     const int u = blockIdx.x / p.nsplit, rank = blockIdx.x - u * p.nsplit;
-    if (p.nsplit > 1) cluster_arrive();
+    // The group's output rows are handed round in quads of four elements: quad q is added up by CTA q % nsplit, as its
+    // quad number q / nsplit (256 quads and 16 CTAs at most: the product is exact).
+    const int quads = p.G * (D / 4), over = 65536 / p.nsplit + 1;
+    const int share = (quads * over) >> 16, owned = share + (rank < quads - share * p.nsplit);
+    if (p.nsplit > 1) {
+        if (tid == 0) expect_messages(arrived, p.nsplit * (8 * (int)sizeof(float2) + owned * (int)sizeof(float4)));
+        cluster_arrive();
+    }
     grid_wait();
     grid_release();
     const int bl = u / p.Hkv, hk = u - bl * p.Hkv;
+    uint4* Kd_u = reinterpret_cast<uint4*>(p.Kd + (size_t)u * p.Dcap * D);
+    uint4* Vd_u = reinterpret_cast<uint4*>(p.Vd + (size_t)u * p.Dcap * D);
+    const uint4* knew_u = reinterpret_cast<const uint4*>(p.k_new + (size_t)u * D);
+    const uint4* vnew_u = reinterpret_cast<const uint4*>(p.v_new + (size_t)u * D);
+    // what the first block needs is asked for at once: the kept count, the queries, the new token's rows and the block itself
     const int kept = p.kept_count[bl];
+    // query row g of the group as A fragments (rows 8..15 of the 16-row operand are zero)
+    uint4 qf[NB];
+    {
+        const uint4* qrow = reinterpret_cast<const uint4*>(p.q + ((size_t)bl * p.H + (size_t)hk * p.G + g) * D);
+#pragma unroll
+        for (int kb = 0; kb < NB; ++kb) qf[kb] = g < p.G ? qrow[kb * 4 + t4] : make_uint4(0, 0, 0, 0);
+    }
+    const bool appends = rank == 0 && tid < 2 * VPR;         // the CTA that appends the new token's rows
+    uint4 fresh_row = make_uint4(0, 0, 0, 0);
+    if (appends) fresh_row = (tid < VPR ? knew_u + tid : vnew_u + (tid - VPR))[0];
     const uint4* Kc_u = reinterpret_cast<const uint4*>(p.Kc + (size_t)u * p.Mcap * D);
     const uint4* Vc_u = reinterpret_cast<const uint4*>(p.Vc + (size_t)u * p.Mcap * D);
     // this warp's ring.  A lane copies chunk (lane % VPR) of rows lane / VPR + k * (32 / VPR) of a block;
@@ -334,31 +434,19 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
         }
         cp_async_commit();
     };
-    // the first block is asked for before the kept count is there: rows below Mcap can be read, and where the
+    // the first blocks are asked for before the kept count is there: rows below Mcap can be read, and where the
     // count turns out to end before them they are fetched again
-    const int first = (rank * NW + warp) * 16;
-    const bool ahead = first + 16 <= p.Mcap;
-    if (ahead) fetch_prefill(first, 0);
+    const int first = (rank * NW + warp) * 16, STRIDE = p.nsplit * NW * 16;
+#pragma unroll
+    for (int k = 0; k < NS; ++k) {
+        if (first + k * STRIDE + 16 <= p.Mcap) fetch_prefill(first + k * STRIDE, k);
+        else cp_async_commit();
+    }
     const int M = min(kept, p.Mcap);
     const int n = p.n_old + 1;
     const int Ktot = M + n;
-    uint4* Kd_u = reinterpret_cast<uint4*>(p.Kd + (size_t)u * p.Dcap * D);
-    uint4* Vd_u = reinterpret_cast<uint4*>(p.Vd + (size_t)u * p.Dcap * D);
-    const uint4* knew_u = reinterpret_cast<const uint4*>(p.k_new + (size_t)u * D);
-    const uint4* vnew_u = reinterpret_cast<const uint4*>(p.v_new + (size_t)u * D);
-
-    // append the new token's key and value as decode entry n_old
-    if (rank != 0) {
-    } else if (tid < VPR) Kd_u[(size_t)p.n_old * VPR + tid] = knew_u[tid];
-    else if (tid < 2 * VPR) Vd_u[(size_t)p.n_old * VPR + (tid - VPR)] = vnew_u[tid - VPR];
-
-    // query row g of the group as A fragments (rows 8..15 of the 16-row operand are zero)
-    uint4 qf[NB];
-    {
-        const uint4* qrow = reinterpret_cast<const uint4*>(p.q + ((size_t)bl * p.H + (size_t)hk * p.G + g) * D);
-#pragma unroll
-        for (int kb = 0; kb < NB; ++kb) qf[kb] = g < p.G ? qrow[kb * 4 + t4] : make_uint4(0, 0, 0, 0);
-    }
+    if (p.nsplit > 1) cluster_wait();                        // all CTAs of the cluster have begun: their memory may be written to
+    if (appends) (tid < VPR ? Kd_u + (size_t)p.n_old * VPR + tid : Vd_u + (size_t)p.n_old * VPR + (tid - VPR))[0] = fresh_row;   // decode entry n_old
 
     // a block with decode entries in it, or past the end: rows past the end are filled with zeros (a weight of
     // zero must not meet a stray NaN)
@@ -393,30 +481,24 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     // running maximum of query row g over this warp's keys (the same in the 4 lanes that share g);
     // z: this lane's part of the row sum relative to it
     float m = SHOTKV_NEG_INF, z = 0.f;
-    // blocks are requested NS - 1 ahead; one copy group per block, empty past the end, so that
-    // "at most NS - 1 groups pending" always means this block's rows have landed
-    const int STRIDE = p.nsplit * NW * 16;
-    int stage = 0;
-    if (ahead && first + 16 > M) {                          // not all prefill rows after all
-        cp_async_wait<0>();
-        __syncwarp();
-    }
-    if (!ahead || first + 16 > M) {
-        if (first < Ktot) fetch_block(first, 0);
-        else cp_async_commit();
-    }
+    // One copy group per block, empty past the end, so that "at most NS - 1 groups pending" always means this
+    // block's rows have landed.  Of the blocks asked for above, those that are not all prefill rows are fetched now.
+    bool landed = false;
 #pragma unroll
-    for (int k = 1; k < NS - 1; ++k) {
-        if (first + k * STRIDE < Ktot) fetch_block(first + k * STRIDE, k);
-        else cp_async_commit();
-    }
-    for (int base = first; base < Ktot; base += STRIDE) {
-        __syncwarp();                                       // every lane has read the stage the next copy overwrites
-        {
-            const int nb = base + (NS - 1) * STRIDE;
-            if (nb < Ktot) fetch_block(nb, stage == 0 ? NS - 1 : stage - 1);
+    for (int k = 0; k < NS; ++k) {
+        const int base = first + k * STRIDE;
+        if (base + 16 > M) {
+            if (!landed) {
+                cp_async_wait<0>();
+                __syncwarp();
+                landed = true;
+            }
+            if (base < Ktot) fetch_block(base, k);
             else cp_async_commit();
         }
+    }
+    int stage = 0;
+    for (int base = first; base < Ktot; base += STRIDE) {
         cp_async_wait<NS - 1>();                            // this block's rows have landed (later blocks' may be in flight)
         __syncwarp();
         const uint32_t st = wring + (uint32_t)(stage * Cfg::kStageBytes);
@@ -480,76 +562,95 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
             mma_bf16_16816(O[mt], a, h0, h1);
             mma_bf16_16816(O[mt], a, l0, l1);
         }
+        __syncwarp();                                       // every lane has read the stage the next copy overwrites
+        if (base + NS * STRIDE < Ktot) fetch_block(base + NS * STRIDE, stage);
+        else cp_async_commit();
         stage = stage + 1 == NS ? 0 : stage + 1;
     }
     cp_async_wait<0>();
     // row sums over the 4 lanes that share g
     z += __shfl_xor_sync(0xffffffffu, z, 1);
     z += __shfl_xor_sync(0xffffffffu, z, 2);
-    if (t4 == 0) {
-        sred[(warp * 8 + g) * 2 + 0] = m;
-        sred[(warp * 8 + g) * 2 + 1] = z;
-    }
-    __syncthreads();                                        // all warps are done with their rings
+    if (t4 == 0) sred[warp * 8 + g] = make_float2(m, z);
+    __syncwarp();                                           // all lanes are done with the warp's ring: its outputs take its place
+    constexpr int PITCH = D + 4, kWarpRing = NS * Cfg::kStageBytes / 4;    // floats
+    float* sO = reinterpret_cast<float*>(ring);
 #pragma unroll
     for (int mt = 0; mt < MT; ++mt) {
-        sO[(warp * 8 + 2 * t4) * D + mt * 16 + g] = O[mt][0];
-        sO[(warp * 8 + 2 * t4 + 1) * D + mt * 16 + g] = O[mt][1];
-        sO[(warp * 8 + 2 * t4) * D + mt * 16 + 8 + g] = O[mt][2];
-        sO[(warp * 8 + 2 * t4 + 1) * D + mt * 16 + 8 + g] = O[mt][3];
-    }
-    if (tid < 8) {
-        float mm = SHOTKV_NEG_INF;
-        for (int w = 0; w < NW; ++w) mm = fmaxf(mm, sred[(w * 8 + tid) * 2]);
-        const float mu = mm == SHOTKV_NEG_INF ? 0.f : mm;    // a CTA of a cluster may have had no keys
-        float zz = 0.f;
-        for (int w = 0; w < NW; ++w) zz += sred[(w * 8 + tid) * 2 + 1] * ex2f(sred[(w * 8 + tid) * 2] - mu);
-        sfin[tid * 2] = mm;
-        sfin[tid * 2 + 1] = p.nsplit > 1 ? zz : (zz > 0.f ? 1.f / zz : 0.f);
+        float* o = sO + warp * kWarpRing + 2 * t4 * PITCH + mt * 16 + g;
+        o[0] = O[mt][0];
+        o[PITCH] = O[mt][1];
+        o[8] = O[mt][2];
+        o[PITCH + 8] = O[mt][3];
     }
     __syncthreads();
     float* out = p.out + ((size_t)bl * p.H + (size_t)hk * p.G) * D;
-    // the warps' outputs, relative to the CTA's maximum; alone, the CTA has the rows' whole sums already
-#pragma unroll 1
-    for (int idx = tid; idx < p.G * D; idx += NT) {
-        const int r = idx / D;
-        const float mm = sfin[r * 2];
-        float o = 0.f;
-        for (int w = 0; w < NW; ++w) {
-            const float mw = sred[(w * 8 + r) * 2];
-            if (mw != SHOTKV_NEG_INF) o += sO[w * 8 * D + idx] * ex2f(mw - mm);
-        }
-        if (p.nsplit > 1) sO[idx] = o;                       // read above by this thread alone
-        else out[idx] = o * sfin[r * 2 + 1];
+    if (p.nsplit > 1 && tid < 8 * p.nsplit) {                // every CTA's rows to every CTA
+        float f[NW];
+        send(stab + rank * 8 + (tid & 7), tid >> 3, arrived, row_of_cta(sred, tid & 7, f));
     }
-    if (p.nsplit > 1) {
-        __syncthreads();
-        exchange_stats(sfin, stab, rank, p.nsplit);          // and all CTAs' outputs may be read
-        if (tid < 8) merge_stats(stab, p.nsplit, tid, sfin[tid * 2], sfin[tid * 2 + 1]);
-        __syncthreads();
-        // each CTA adds up its share of the output elements
+    // the warps' outputs relative to the CTA's maximum: alone, the CTA has the rows' whole sums
 #pragma unroll 1
-        for (int idx = rank * NT + tid; idx < p.G * D; idx += p.nsplit * NT) {
-            const int r = idx / D;
-            const float mm = sfin[r * 2];
-            const float mu = mm == SHOTKV_NEG_INF ? 0.f : mm;    // a row without a finite logit has no weight anywhere
-            float o = 0.f;
-            for (int c = 0; c < p.nsplit; ++c) o += cluster_load(sO + idx, c) * ex2f(stab[c * 16 + r * 2] - mu);
-            out[idx] = o * sfin[r * 2 + 1];
+    for (int q = tid; q < quads; q += NT) {
+        const int r = q / (D / 4), c = q % (D / 4) * 4;
+        float f[NW];
+        const float2 row = row_of_cta(sred, r, f);
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            const float4 v = *reinterpret_cast<const float4*>(sO + w * kWarpRing + r * PITCH + c);
+            if (f[w] >= 0.f) o.x += v.x * f[w], o.y += v.y * f[w], o.z += v.z * f[w], o.w += v.w * f[w];
         }
-        cluster_arrive();                                    // done with the others' memory
+        if (p.nsplit > 1) {
+            const int slot = (q * over) >> 16, to = q - slot * p.nsplit;
+            send(sin + rank * (share + 1) + slot, to, arrived, o);
+        } else {
+            const float iz = row.y > 0.f ? 1.f / row.y : 0.f;
+            float* d = out + 4 * q;
+            d[0] = o.x * iz;
+            d[1] = o.y * iz;
+            d[2] = o.z * iz;
+            d[3] = o.w * iz;
+        }
+    }
+    if (p.nsplit > 1) await_messages(arrived, p.err);
+    float rm, riz;                                           // of row lane / 4, over all keys of the unit
+    row_of_unit(p.nsplit > 1 ? stab : sred, p.nsplit > 1 ? p.nsplit : NW, rm, riz);
+    const float rmu = rm == SHOTKV_NEG_INF ? 0.f : rm;
+    // the CTA's own quads, four lanes each of which adds up every fourth CTA's
+    if (p.nsplit > 1) {
+#pragma unroll 1
+        for (int x = tid; x < (owned * 4 + 31) / 32 * 32; x += NT) {
+            const int slot = x >> 2, q = slot * p.nsplit + rank;
+            const int r = slot < owned ? q / (D / 4) : 0;
+            const float mu = __shfl_sync(0xffffffffu, rmu, r * 4), iz = __shfl_sync(0xffffffffu, riz, r * 4);
+            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < kMaxSplit / 4; ++i) {
+                const int c = t4 + 4 * i;
+                if (slot < owned && c < p.nsplit) {
+                    const float4 v = sin[c * (share + 1) + slot];
+                    const float f = ex2f(stab[c * 8 + r].x - mu);
+                    o.x += v.x * f, o.y += v.y * f, o.z += v.z * f, o.w += v.w * f;
+                }
+            }
+#pragma unroll
+            for (int d = 1; d <= 2; d <<= 1) {
+                o.x += __shfl_xor_sync(0xffffffffu, o.x, d);
+                o.y += __shfl_xor_sync(0xffffffffu, o.y, d);
+                o.z += __shfl_xor_sync(0xffffffffu, o.z, d);
+                o.w += __shfl_xor_sync(0xffffffffu, o.w, d);
+            }
+            if (slot < owned) out[4 * q + t4] = (t4 == 0 ? o.x : t4 == 1 ? o.y : t4 == 2 ? o.z : o.w) * iz;
+        }
     }
     // the decode entries among this warp's blocks: their weights summed over the query rows
     for (int base = first + max(0, (M - 15 - first + STRIDE - 1) / STRIDE) * STRIDE; base < Ktot; base += STRIDE) {
         const int j = base + lane - M;
-        if (lane < 16 && j >= 0 && j < n) {
-            float s = 0.f;
-#pragma unroll 1
-            for (int r = 0; r < p.G; ++r) s += ex2f(sdec[r * p.Dcap + j] - sfin[r * 2]) * sfin[r * 2 + 1];
-            p.partial[(size_t)u * p.Dcap + j] = s;
-        }
+        const bool entry = lane < 16 && j >= 0 && j < n;
+        const float s = entry_weight(sdec, p.Dcap, p.G, j, entry, rm, riz);
+        if (entry) p.partial[(size_t)u * p.Dcap + j] = s;
     }
-    if (p.nsplit > 1) cluster_wait();                        // the others are done with this CTA's
 }
 
 // The rest of a step for one (b, l): acc[j] += sum over kv heads of the entries' weights (fixed order,

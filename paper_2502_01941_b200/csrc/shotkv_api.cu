@@ -724,10 +724,11 @@ int run_compact(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* K, con
 
 // Dynamic shared memory of the decode kernels for decode regions of Dcap rows.
 template <int D>
-size_t attend_smem(int Dcap) {
-    return ((size_t)8 * Dcap + AttendCfg<D>::kWarps * 8 * 2 + 16 + kMaxSplit * 16) * 4 + AttendCfg<D>::kRingBytes;
+size_t attend_smem(int G, int Dcap, int nsplit) {
+    const size_t shares = nsplit > 1 ? (size_t)nsplit * (16 + (G * D / 4 / nsplit + 1) * 4) : 0;   // (m, z) of 8 rows, and a share of the quads
+    return AttendCfg<D>::kRingBytes + 16 + ((size_t)AttendCfg<D>::kWarps * 16 + ((size_t)G * Dcap + 3) / 4 * 4 + shares) * 4;
 }
-size_t score_smem(int Dcap) { return ((size_t)8 * Dcap + 8 * 8 * 2 + 16 + kMaxSplit * 16) * 4; }
+size_t score_smem(int Dcap) { return ((size_t)8 * Dcap + 8 * 8 * 2 + kMaxSplit * 16 + 2) * 4; }
 
 // Dynamic shared-memory limits of every kernel that may need more than the 48 KB default.  A
 // function attribute belongs to the device's context, so it is set once when a shotkv_ctx is
@@ -761,6 +762,11 @@ cudaError_t set_kernel_attributes() {
                            (const void*)decode_evict_kernel<128>, (const void*)decode_evict_kernel<64>};
     for (const void* f : small)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kBigSmem);
+    // a decode unit may be shared by more CTAs than the eight that every device's clusters allow
+    const void* split[] = {(const void*)decode_attend_kernel<128>, (const void*)decode_attend_kernel<64>,
+                           (const void*)decode_score_kernel<128, true>, (const void*)decode_score_kernel<64, true>};
+    for (const void* f : split)
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     // the fused decode step wants three CTAs of ~74 KB each on an SM: ask for the largest shared-memory carve-out
     const void* wide[] = {(const void*)decode_attend_kernel<128>, (const void*)decode_attend_kernel<64>};
     for (const void* f : wide)
@@ -770,7 +776,7 @@ cudaError_t set_kernel_attributes() {
 
 // How many clusters of n decode CTAs the device runs at the same time, with decode regions of kRoomRows rows
 // (larger ones take more shared memory; the figure then is an estimate that costs a second wave at worst).
-constexpr int kRoomRows = 320;
+constexpr int kRoomRows = 320, kRoomGroup = 4;
 template <class K>
 cudaError_t ask_room(K* kernel, int threads, size_t smem, int* room) {
     for (int n = 2; n <= kMaxSplit; ++n) {
@@ -790,8 +796,8 @@ cudaError_t ask_room(K* kernel, int threads, size_t smem, int* room) {
     return cudaSuccess;
 }
 cudaError_t ask_decode_room(shotkv_ctx* ctx) {
-    cudaError_t e = ask_room(decode_attend_kernel<64>, AttendCfg<64>::kWarps * 32, attend_smem<64>(kRoomRows), ctx->room_attend[0]);
-    if (e == cudaSuccess) e = ask_room(decode_attend_kernel<128>, AttendCfg<128>::kWarps * 32, attend_smem<128>(kRoomRows), ctx->room_attend[1]);
+    cudaError_t e = ask_room(decode_attend_kernel<64>, AttendCfg<64>::kWarps * 32, attend_smem<64>(kRoomGroup, kRoomRows, kMaxSplit), ctx->room_attend[0]);
+    if (e == cudaSuccess) e = ask_room(decode_attend_kernel<128>, AttendCfg<128>::kWarps * 32, attend_smem<128>(kRoomGroup, kRoomRows, kMaxSplit), ctx->room_attend[1]);
     if (e == cudaSuccess) e = ask_room(decode_score_kernel<64, true>, 256, score_smem(kRoomRows), ctx->room_score[0]);
     if (e == cudaSuccess) e = ask_room(decode_score_kernel<128, true>, 256, score_smem(kRoomRows), ctx->room_score[1]);
     return e;
@@ -1304,16 +1310,19 @@ namespace {
 
 // CTAs that share a unit's keys: as many as still run at the same time for all units (`room[n]` clusters of
 // n CTAs do: a cluster stays within a group of SMs, so it is fewer than the SMs' slots / n) and leave every
-// warp at least kMinSplitBlocks blocks of 16 keys.
-constexpr int kMinSplitBlocks = 2;
-int decode_split(const int* room, long long U, long long keys, int warps) {
+// warp at least `least` sixths of a block of 16 keys.  The fused step gains from more CTAs down to little more than a block a
+// warp, whose chain is long (2 heads of 333 keys 6.5 -> 5.4 us a step with 4/3 of a block instead of 2, 185 keys 8.5 -> 7.1; 1 block:
+// 8 heads of 1,150 keys 7.0 -> 7.3).  Scores alone take less per block than a larger cluster costs (8 heads of 3,400 keys 5.3 us with 2.5
+// blocks, 6.1 with 2, 5.7 with 3).
+constexpr int kLeastAttend = 8, kLeastScore = 15;
+int decode_split(const int* room, long long U, long long keys, int warps, int least) {
     int n = kMaxSplit;
-    while (n > 1 && (U > room[n] || keys < (long long)n * warps * 16 * kMinSplitBlocks)) --n;
+    while (n > 1 && (U > room[n] || keys * 6 < (long long)n * warps * 16 * least)) --n;
     return n;
 }
 
-// Whole units of the fused step, more of them than SMs and at most two to an SM, are one uneven wave: its time is that of
-// the SMs with most CTAs.  Begun early, it was placed while CTAs of the kernel before still held 32 SMs or so that
+// Whole units of the fused step, at most two to an SM, are one uneven wave: its time is that of the SMs with most CTAs.
+// Begun early, it was placed while CTAs of the kernel before still held 32 SMs or so that
 // had another split of shared memory, and put three on others: 256 units of 3,276 keys 78 us a step, of 16,000 keys 350.
 // The kernels that end a step therefore ask for this kernel's split here, and this one for so much shared memory that
 // no third CTA fits: 71 and 310 us (288 units 88 -> 81 and 382 -> 365).
@@ -1325,16 +1334,16 @@ bool two_to_an_sm(const shotkv_ctx* ctx, const DecodeParams& p, int U) {
 template <int D>
 int launch_decode_attend(shotkv_ctx* ctx, DecodeParams& p, int U, cudaStream_t stream) {
     using Cfg = AttendCfg<D>;
-    size_t smem = attend_smem<D>(p.Dcap);
+    p.nsplit = decode_split(ctx->room_attend[D == 128], U, (long long)p.Mcap + p.n_old + 1, Cfg::kWarps, kLeastAttend);
+    size_t smem = attend_smem<D>(p.G, p.Dcap, p.nsplit);
     if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "Dcap too large for the attention-output step");
-    p.nsplit = decode_split(ctx->room_attend[D == 128], U, (long long)p.Mcap + p.n_old + 1, Cfg::kWarps);
     if (two_to_an_sm(ctx, p, U) && smem < kNoThirdCta) smem = kNoThirdCta;
     return launch(ctx, decode_attend_kernel<D>, dim3(U * p.nsplit), Cfg::kWarps * 32, smem, stream, p.nsplit, kEarly, p);
 }
 template <int D>
 int launch_decode_score(shotkv_ctx* ctx, DecodeParams& p, int U, cudaStream_t stream) {
+    p.nsplit = decode_split(ctx->room_score[D == 128], U, (long long)p.Mcap + p.n_old + 1, 8, kLeastScore);
     const size_t smem = score_smem(p.Dcap);
-    p.nsplit = decode_split(ctx->room_score[D == 128], U, (long long)p.Mcap + p.n_old + 1, 8);
     return p.nsplit > 1 ? launch(ctx, decode_score_kernel<D, true>, dim3(U * p.nsplit), 256, smem, stream, p.nsplit, kEarly, p)
                         : launch(ctx, decode_score_kernel<D, false>, dim3(U), 256, smem, stream, 1, kEarly, p);
 }
@@ -1362,6 +1371,7 @@ int decode_step_impl(shotkv_ctx* ctx, shotkv_decode_state* st, const shotkv_bf16
     p.H = d.H; p.Hkv = d.Hkv; p.G = d.H / d.Hkv; p.Mcap = st->Mcap; p.Dcap = st->Dcap; p.n_old = st->n_dec;
     p.scale_log2 = kLog2e / sqrtf((float)d.d);
     p.Vc = (const __nv_bfloat16*)Vc; p.out = attn_out;
+    p.err = ctx->err_dev;
     prof_begin(ctx);
     prof_mark(ctx, stream);
     if (attn_out) rc = d.d == 128 ? launch_decode_attend<128>(ctx, p, U, stream) : launch_decode_attend<64>(ctx, p, U, stream);

@@ -1,5 +1,5 @@
 """Units shared by a cluster of CTAs and the fused end of an eviction cycle, against the oracle: one to
-eight CTAs to a unit, CTAs without a single key, heads that do not divide by the cluster, regions on
+sixteen CTAs to a unit, CTAs without a single key, heads that do not divide by the cluster, regions on
 both sides of the ranking by counting (256 entries) and by sorting."""
 import numpy as np
 import pytest
@@ -25,6 +25,15 @@ def ctx():
 def test_unit_shared_by_a_cluster(ctx, Hkv, G, d, M, count, attend):
     cfg = wl.DecodeConfig("split", B=1, L=1, H=Hkv * G, Hkv=Hkv, d=d, steps=14, r_d=0.5, recompress_every=4, cfg_id=71)
     assert lockstep(ctx, cfg, M, [(0, 0)], np.full((1, 1), count, np.int32), attend=attend) <= 1
+
+
+@pytest.mark.parametrize("Hkv,G,d,M,count", [(1, 1, 64, 4096, 4000), (1, 7, 128, 4100, 4100), (1, 5, 64, 3000, 2999), (2, 8, 128, 5000, 4999),
+                                             (3, 3, 128, 1700, 1690), (7, 2, 64, 6000, 5900)])
+def test_unit_shared_by_more_than_eight(ctx, Hkv, G, d, M, count):
+    """Clusters of nine to sixteen, output elements that do and do not divide by them, for both steps."""
+    cfg = wl.DecodeConfig("split", B=1, L=1, H=Hkv * G, Hkv=Hkv, d=d, steps=6, r_d=0.5, recompress_every=4, cfg_id=76)
+    for attend in (False, True):
+        assert lockstep(ctx, cfg, M, [(0, 0)], np.full((1, 1), count, np.int32), attend=attend) <= 1
 
 
 @pytest.mark.parametrize("every", [255, 256, 257, 300, 530])
