@@ -118,9 +118,8 @@ __global__ void __launch_bounds__(ColsumTcCfg<D, MB>::kThreads, 1)
     float* slots = reinterpret_cast<float*>(plim_s + 8 * RG);                      // [4][2][32]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long total = p.total_items;
-    const int item_begin = (int)(total * blockIdx.x / gridDim.x);
-    const int item_end = (int)(total * (blockIdx.x + 1) / gridDim.x);
+    int item_begin, item_end;
+    tc::item_range(p, item_begin, item_end);
 
     // Every window row is a column of the accumulator and all columns are summed by one thread, so
     // the rows of the Q area that no copy ever writes (fewer than 128 query rows in all) must hold

@@ -29,48 +29,6 @@ struct DecodeParams {
 // query row to all others and each then knows the whole row's maximum and sum.
 constexpr int kMaxSplit = 16;
 
-// What CTAs tell one another goes as messages: a store counts its bytes on the receiver's barrier, which is complete when
-// as many as the receiver expects are there.  That is one way across the cluster, where a barrier of all its threads is two
-// (1.7 us of a step of 4 sequences x 1 layer).  expect_messages: by one thread, ahead of the cluster_arrive at the start;
-// nobody sends before a cluster_wait (a CTA's memory may be written once it has begun), and a CTA that has been sent
-// everything may end.
-constexpr long long kMessageCycles = 4000000000LL;     // limit of the wait for them: about two seconds
-__device__ __forceinline__ void expect_messages(unsigned long long* bar, int bytes) {
-    const uint32_t b = smem_u32(bar);
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void send(float2* to, int rank, unsigned long long* bar, float2 v) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v2.f32 [%0], {%1, %2}, [%3];" ::"r"(cluster_addr(to, rank)),
-                 "f"(v.x), "f"(v.y), "r"(cluster_addr(bar, rank))
-                 : "memory");
-}
-__device__ __forceinline__ void send(float4* to, int rank, unsigned long long* bar, float4 v) {
-    asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(cluster_addr(to, rank)),
-                 "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(cluster_addr(bar, rank))
-                 : "memory");
-}
-// Waits until all bytes expected are there; a wait that runs into its limit sets the error word.
-__device__ __forceinline__ void await_messages(unsigned long long* bar, int* err) {
-    const uint32_t b = smem_u32(bar);
-    const long long t0 = clock64();
-    for (;;) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred q;\n\t"
-            "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], 0;\n\t"
-            "selp.u32 %0, 1, 0, q;\n\t}"
-            : "=r"(done)
-            : "r"(b)
-            : "memory");
-        if (done) return;
-        if (clock64() - t0 > kMessageCycles) {
-            atomicExch(err, 1);
-            return;
-        }
-    }
-}
 // (m, z) of row r over the NW warps' sums in `sred`, [NW][8 rows], and the warps' factors (negative: nothing to add).
 template <int NW>
 __device__ __forceinline__ float2 row_of_cta(const float2* sred, int r, float (&f)[NW]) {

@@ -107,34 +107,34 @@ __global__ void row_stats_kernel(const PartialView v, int R, float* __restrict__
 // 4 x 32 layers of 32K, where reading the partials (115 MB) is 18 us of memory time.
 //
 // Per head: (1) a thread (two, with 128 rows) per row merges the item statistics into the row's
-// (m, 1/Z): the maximum first, then the sum, so that the items' loads are all in flight at once.
-// (2) Every warp takes a run of consecutive pieces, its lanes the rows four at a time; the weight
-// exp2(m_item[r] - m[r]) / Z[r] is the same for all pieces of an item and is formed when the run
-// enters the item (an exact item's pieces carry their own references and pay one exp2 per row); one
-// shuffle reduction gives the piece's mass.  (3) The pieces of each shot are added in index order.
+// (m, 1/Z): the maximum first, then the sum, so that the items' loads are all in flight at once; the weight
+// exp2(m_item[r] - m[r]) / Z[r], the same for all pieces of an item, goes to a table of items and rows.
+// (2) Every warp takes a run of consecutive pieces, its lanes the rows four at a time, and weights them from that
+// table (an exact item's pieces carry their own references and pay one exp2 per row); the sums over the lanes of the
+// pieces in flight go side by side.  (3) The pieces of each shot are added in index order.
 // All sums have a fixed order.
 constexpr int kReduceThreads = kSelectThreads;
 constexpr int kReduceCluster = 8;                  // most CTAs that share the kv heads of a (b, l)
 
 // Shared memory: boundaries; masses of the shots, one row per CTA of the cluster (the leader's copy is
-// read); row statistics, piece masses and piece -> item (reused by the selection).
-__host__ __device__ constexpr size_t reduce_smem_bytes(int Rpad, int P, int S, int ranks) {
+// read); row statistics, the items' weights, piece masses and piece -> item (reused by the selection).
+__host__ __device__ constexpr size_t reduce_smem_bytes(int Rpad, int P, int S, int nchunk, int ranks) {
     const size_t pieces = (size_t)(P + 3) / 4 * 4 * 4 + (size_t)(P + 15) / 16 * 16;
-    const size_t work = (size_t)Rpad * 16 + pieces, select = select_smem_bytes(S);
+    const size_t work = (size_t)(4 + nchunk) * Rpad * 4 + pieces, select = select_smem_bytes(S);
     return bounds_smem_bytes(S) + ranks * ((size_t)(S + 3) / 4 * 4 * 4) + (work > select ? work : select);
 }
 
 template <int ROWS>
 __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const PartialView v, const __grid_constant__ ShotTable tab,
                                                                       int R, int Hkv, int ranks,
-                                                                      float* __restrict__ shot_scores, const SelectArgs a) {
+                                                                      float* __restrict__ shot_scores, const SelectArgs a, int* err) {
     constexpr int NW = kReduceThreads / 32, NH = ROWS / 128, PARTS = kReduceThreads / ROWS;
     constexpr int AHEAD = 4 / NH, FIRST = 4;       // pieces whose z a warp has in flight; items whose statistics a thread has
     constexpr unsigned char kNoItem = 255;
     static_assert(ROWS == 128 || ROWS == 256, "padded window rows");
     extern __shared__ __align__(16) unsigned char sm[];
-    __shared__ int2 range[64];                     // first and last piece of every item
     __shared__ int exact[64];
+    __shared__ unsigned long long arrived;         // leader: barrier of the other CTAs' masses
     const int S = v.S, np = v.P;
     const int s4 = (S + 3) / 4 * 4;
     int* o = reinterpret_cast<int*>(sm);
@@ -142,30 +142,38 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
     unsigned char* work = reinterpret_cast<unsigned char*>(masses + (size_t)ranks * s4);
     float* row_m = reinterpret_cast<float*>(work); // [2][ROWS] maxima of the parts, then [ROWS]
     float* row_w = row_m + 2 * ROWS;               // [2][ROWS] sums of the parts, then [ROWS] 1/Z (0 for rows without weight)
-    float* piece_mass = row_w + 2 * ROWS;          // [P]
+    float* weight = row_w + 2 * ROWS;              // [nchunk][ROWS] 2^(m_item - row's m) / Z
+    float* piece_mass = weight + (size_t)v.nchunk * ROWS;   // [P]
     unsigned char* item_of = reinterpret_cast<unsigned char*>(piece_mass + (np + 3) / 4 * 4);   // [P]
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int bl = blockIdx.x / ranks, rank = blockIdx.x - bl * ranks;   // a cluster is the `ranks` CTAs of one (b, l)
     float* mass = masses + rank * s4;              // of this CTA's heads
 
     grid_release();
+    if (ranks > 1) {
+        if (rank == 0 && tid == 0) expect_messages(&arrived, (ranks - 1) * S * (int)sizeof(float));
+        cluster_arrive();
+    }
     if (tab.ptr) grid_wait();                      // boundaries among the launch parameters are there already
-    copy_bounds(o, tab, bl / a.L, S);
-    if (ranks > 1) cluster_arrive();               // (1) this CTA has begun: its shared memory may be written to
-    __syncthreads();
+    {   // a segment's pieces are one an item it reaches into; the index after them belongs to none where it ends with an item
+        const int* t = table_row(tab, bl / a.L);
 #pragma unroll 1
-    for (int j = tid; j < v.nchunk; j += kReduceThreads) range[j] = make_int2(first_piece(v, o, j), last_piece(v, o, j));
+        for (int s = tid; s <= S + 1; s += kReduceThreads) {
+            const int lo = s > 0 ? t[s - 1] : 0, hi = s <= S ? t[s] : v.N;
+            if (s <= S) o[s] = hi;
+            if (lo == hi) continue;                // no token before the first shot
+            int j = lo / v.chunk_keys, end = j * v.chunk_keys;
 #pragma unroll 1
-    for (int i = tid; i < S; i += kReduceThreads) mass[i] = 0.f;
-#pragma unroll 1
-    for (int q = tid; q < np; q += kReduceThreads) item_of[q] = kNoItem;   // an index no piece has (a boundary on a chunk end)
-    __syncthreads();
-#pragma unroll 1
-    for (int j = warp; j < v.nchunk; j += NW)
-#pragma unroll 1
-        for (int q = range[j].x + lane; q <= range[j].y; q += 32) item_of[q] = (unsigned char)j;
+            do {
+                item_of[s + j] = (unsigned char)j;
+                ++j;
+                end += v.chunk_keys;
+            } while (end < hi);
+            if (end == hi && s <= S) item_of[s + j] = kNoItem;
+        }
+    }
     grid_wait();
-    const int q_first = range[0].x, q_count = range[v.nchunk - 1].y + 1 - q_first;
+    const int q_first = table_row(tab, bl / a.L)[0] == 0, q_count = S + v.nchunk + 1 - q_first;
 
     for (int h = rank; h < Hkv; h += ranks) {
         const int u = bl * Hkv + h;
@@ -200,81 +208,91 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
             exact[j] = e;
             any |= e;
         }
-        any = __syncthreads_or(any);
-        {   // row statistics
-            float m = SHOTKV_NEG_INF, z = 0.f;
-            if (!any) {
+        // (m, z) of this thread's items, relative to their own maximum
+        float m = SHOTKV_NEG_INF, z = 0.f;
 #pragma unroll
-                for (int n = 0; n < FIRST; ++n) m = fmaxf(m, m_first[n]);
+        for (int n = 0; n < FIRST; ++n) m = fmaxf(m, m_first[n]);
 #pragma unroll 4
-                for (int j = part + FIRST * PARTS; j < v.nchunk; j += PARTS) m = fmaxf(m, im[(size_t)j * v.Rpad]);
-            } else if (part == 0) {
-                row_stats_of(v, o, u, r, m, z);
-            }
-            if (PARTS > 1) {
-                row_m[part * ROWS + r] = m;
-                __syncthreads();
-                m = fmaxf(row_m[r], row_m[ROWS + r]);
-            }
+        for (int j = part + FIRST * PARTS; j < v.nchunk; j += PARTS) m = fmaxf(m, im[(size_t)j * v.Rpad]);
+        {
             const float mu = m == SHOTKV_NEG_INF ? 0.f : m;
-            if (!any) {
 #pragma unroll
-                for (int n = 0; n < FIRST; ++n) z += z_first[n] * ex2f(m_first[n] - mu);
+            for (int n = 0; n < FIRST; ++n) z += z_first[n] * ex2f(m_first[n] - mu);
 #pragma unroll 4
-                for (int j = part + FIRST * PARTS; j < v.nchunk; j += PARTS) z += iz[(size_t)j * v.Rpad] * ex2f(im[(size_t)j * v.Rpad] - mu);
-            }
-            if (PARTS > 1) {
-                row_w[part * ROWS + r] = z;
-                __syncthreads();
-                z = row_w[r] + row_w[ROWS + r];
-                __syncthreads();
-            }
+            for (int j = part + FIRST * PARTS; j < v.nchunk; j += PARTS) z += iz[(size_t)j * v.Rpad] * ex2f(im[(size_t)j * v.Rpad] - mu);
+        }
+        if (PARTS > 1) {
+            row_m[part * ROWS + r] = m;
+            row_w[part * ROWS + r] = z;
+        }
+        any = __syncthreads_or(any);
+        if (any) {                                 // an item's statistics are those of its pieces
+            m = SHOTKV_NEG_INF, z = 0.f;
+            if (part == 0) row_stats_of(v, o, u, r, m, z);
+            __syncthreads();
+            row_m[part * ROWS + r] = m;
+            row_w[part * ROWS + r] = z;
+            __syncthreads();
+        }
+        if (PARTS > 1) {
+            m = row_m[r];
+            z = row_w[r];
+            merge_mz(m, z, row_m[ROWS + r], row_w[ROWS + r]);
+        }
+        const float rm = m == SHOTKV_NEG_INF ? 0.f : m;
+        const float rw = (r < R && z > 0.f) ? 1.f / z : 0.f;   // padding rows carry no weight
+        // 2^(m_item - row's m) / Z of this row; a row without weight (padding, or nothing but underflow) gets
+        // factor 0 whatever its reference
+        auto factor = [](float ref, float m, float w) { return w > 0.f ? ex2f(ref - m) * w : 0.f; };
+#pragma unroll
+        for (int n = 0; n < FIRST; ++n) {
+            const int j = part + n * PARTS;
+            if (j < v.nchunk) weight[j * ROWS + r] = factor(m_first[n], rm, rw);
+        }
+#pragma unroll 4
+        for (int j = part + FIRST * PARTS; j < v.nchunk; j += PARTS) weight[j * ROWS + r] = factor(im[(size_t)j * v.Rpad], rm, rw);
+        if (any) {                                 // for the pieces of exact items (the rows' statistics have been read)
+            __syncthreads();
             if (part == 0) {
-                row_m[r] = mu;
-                row_w[r] = (r < R && z > 0.f) ? 1.f / z : 0.f;   // padding rows carry no weight
+                row_m[r] = rm;
+                row_w[r] = rw;
             }
         }
         __syncthreads();
         // rows 4*lane .. 4*lane+3 (and the same 128 further on when there are 256 rows)
-        float4 rm[NH], rw[NH], f[NH];
-#pragma unroll
-        for (int k = 0; k < NH; ++k) {
-            rm[k] = reinterpret_cast<const float4*>(row_m)[k * 32 + lane];
-            rw[k] = reinterpret_cast<const float4*>(row_w)[k * 32 + lane];
-        }
-        // 2^(m - row's m) / Z of this lane's rows; a row without weight (padding, or nothing but
-        // underflow) gets factor 0 whatever its reference
-        auto weights = [&](const float* ref) {
-#pragma unroll
-            for (int k = 0; k < NH; ++k) {
-                const float4 mi = reinterpret_cast<const float4*>(ref)[k * 32 + lane];
-                f[k].x = rw[k].x > 0.f ? ex2f(mi.x - rm[k].x) * rw[k].x : 0.f;
-                f[k].y = rw[k].y > 0.f ? ex2f(mi.y - rm[k].y) * rw[k].y : 0.f;
-                f[k].z = rw[k].z > 0.f ? ex2f(mi.z - rm[k].z) * rw[k].z : 0.f;
-                f[k].w = rw[k].w > 0.f ? ex2f(mi.w - rm[k].w) * rw[k].w : 0.f;
-            }
-        };
-        int item = kNoItem;
         for (int q = q0; q < q1; q += AHEAD) {
             if (q != q0) load_pieces(q);
+            float s[AHEAD];
 #pragma unroll
             for (int n = 0; n < AHEAD; ++n) {
+                s[n] = 0.f;
                 const int j = q + n < q1 ? item_of[q + n] : kNoItem;
                 if (j == kNoItem) continue;
-                const bool e = exact[j] != 0;
-                if (e || j != item) weights(e ? pm + (size_t)(q + n) * v.Rpad : v.item_m + ((size_t)u * v.nchunk + j) * v.Rpad);
-                item = e ? kNoItem : j;
-                float s = 0.f;
+                const bool e = any && exact[j] != 0;
 #pragma unroll
                 for (int k = 0; k < NH; ++k) {
-                    s = fmaf(z4[n][k].x, f[k].x, s);
-                    s = fmaf(z4[n][k].y, f[k].y, s);
-                    s = fmaf(z4[n][k].z, f[k].z, s);
-                    s = fmaf(z4[n][k].w, f[k].w, s);
+                    float4 f;
+                    if (e) {
+                        const float4 ref = reinterpret_cast<const float4*>(pm + (size_t)(q + n) * v.Rpad)[k * 32 + lane];
+                        const float4 m4 = reinterpret_cast<const float4*>(row_m)[k * 32 + lane];
+                        const float4 w4 = reinterpret_cast<const float4*>(row_w)[k * 32 + lane];
+                        f = make_float4(factor(ref.x, m4.x, w4.x), factor(ref.y, m4.y, w4.y), factor(ref.z, m4.z, w4.z), factor(ref.w, m4.w, w4.w));
+                    } else {
+                        f = reinterpret_cast<const float4*>(weight + j * ROWS)[k * 32 + lane];
+                    }
+                    s[n] = fmaf(z4[n][k].x, f.x, s[n]);
+                    s[n] = fmaf(z4[n][k].y, f.y, s[n]);
+                    s[n] = fmaf(z4[n][k].z, f.z, s[n]);
+                    s[n] = fmaf(z4[n][k].w, f.w, s[n]);
                 }
-                s = warp_sum(s);
-                if (lane == 0) piece_mass[q + n] = s;
             }
+#pragma unroll
+            for (int d = 16; d > 0; d >>= 1)
+#pragma unroll
+                for (int n = 0; n < AHEAD; ++n) s[n] += __shfl_xor_sync(0xffffffffu, s[n], d);
+#pragma unroll
+            for (int n = 0; n < AHEAD; ++n)
+                if (lane == n && q + n < q1) piece_mass[q + n] = s[n];
         }
         __syncthreads();
 #pragma unroll 1
@@ -282,29 +300,30 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
             float s = 0.f;
 #pragma unroll 1
             for (int j = o[i] / v.chunk_keys, last = (o[i + 1] - 1) / v.chunk_keys; j <= last; ++j) s += piece_mass[i + 1 + j];
-            mass[i] += s;
+            mass[i] = h == rank ? s : mass[i] + s;
         }
-        __syncthreads();
+        if (h + ranks < Hkv) __syncthreads();
     }
     if (ranks > 1) {
-        cluster_wait();                            // (1) the leader has begun
-        if (rank != 0)
+        cluster_wait();                            // all CTAs have begun
+        if (rank != 0) {
 #pragma unroll 1
-            for (int i = tid; i < S; i += kReduceThreads) cluster_store(mass + i, 0, mass[i]);
-        cluster_arrive();                          // (2) this CTA's masses are with the leader
+            for (int i = tid; i < S; i += kReduceThreads) send(mass + i, 0, &arrived, mass[i]);
+            return;
+        }
+        await_messages(&arrived, err);
     }
-    if (rank == 0) {
-        if (ranks > 1) cluster_wait();             // (2)
-        float* scores = shot_scores + (size_t)bl * S;
-        select_body<kReduceThreads>(a, bl, o, work, [&](int i) {
-            float s = 0.f;
-#pragma unroll 1
-            for (int c = 0; c < ranks; ++c) s += masses[c * s4 + i];
-            s /= (float)(o[i + 1] - o[i]);
-            scores[i] = s;
-            return s;
-        });
-    }
+    float* scores = shot_scores + (size_t)bl * S;
+    __syncthreads();                               // the selection takes the place of the work area
+    select_body<kReduceThreads>(a, bl, o, work, [&](int i) {
+        float s = 0.f;
+#pragma unroll
+        for (int c = 0; c < kReduceCluster; ++c)
+            if (c < ranks) s += masses[c * s4 + i];
+        s /= (float)(o[i + 1] - o[i]);
+        scores[i] = s;
+        return s;
+    });
 }
 
 // Score(s_i) from per-token importance.  Latency-bound while the importances come from L2, so what counts is how

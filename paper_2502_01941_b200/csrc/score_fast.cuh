@@ -218,9 +218,8 @@ __global__ void __launch_bounds__(ScoreFastCfg<D>::kThreads, 1)
     tc::stamp(p.clk, 0);
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long total = p.total_items;
-    const int item_begin = (int)(total * blockIdx.x / gridDim.x);
-    const int item_end = (int)(total * (blockIdx.x + 1) / gridDim.x);
+    int item_begin, item_end;
+    tc::item_range(p, item_begin, item_end);
 
     if (warp == 0) {
         if (lane == 0) tc::producer_role<D, MB, false, false>(pp, &tmQ, &tmK, q_box_rows, k_box_rows, p, item_begin, item_end);

@@ -43,6 +43,7 @@ struct ScoreTcParams {
     int nchunk, chunk_keys;   // chunks per unit; keys per chunk (a multiple of 128)
     int L, Hkv, N, W, R, Rpad;
     int total_items;          // U * nchunk
+    int items_each, items_more;   // items of a CTA: items_each, and one more for the first items_more CTAs
     float scale_log2;     // log2(e)/sqrt(d)
     float* part_m;        // [U][P][Rpad]  per-piece reference: written by the exact kernel only
     float* part_z;        // [U][P][Rpad]
@@ -73,6 +74,13 @@ struct ScoreTcCfg {
 };
 
 namespace tc {
+
+// The run of consecutive items of this CTA.
+__device__ __forceinline__ void item_range(const ScoreTcParams& p, int& begin, int& end) {
+    const int b = blockIdx.x;
+    begin = b * p.items_each + min(b, p.items_more);
+    end = begin + p.items_each + (b < p.items_more);
+}
 
 constexpr int kTileKeys = 128;
 constexpr long long kWaitCycles = 4000000000LL;   // default limit of a bounded wait: about two seconds
@@ -688,9 +696,8 @@ template <int D, int MB, int EW, class Cfg>
 __device__ __noinline__ void repair_items(unsigned char* smem_raw, const CUtensorMap* tmQ, const CUtensorMap* tmK, int q_box_rows,
                                           int k_box_rows, const ScoreTcParams& p, const ShotTable& tab) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long total = p.total_items;
-    const int item_begin = (int)(total * blockIdx.x / gridDim.x);
-    const int item_end = (int)(total * (blockIdx.x + 1) / gridDim.x);
+    int item_begin, item_end;
+    item_range(p, item_begin, item_end);
     Pipe<Cfg> pp;
     pp.tmem_base = *pipe_map(pp, smem_raw);
     float* comb = pipe_scratch(pp, smem_raw);
@@ -718,9 +725,8 @@ __global__ void __launch_bounds__(ScoreTcCfg<D, MB>::kThreads, 1)
                     const int k_box_rows, const ScoreTcParams p, const __grid_constant__ ShotTable tab) {
     using Cfg = ScoreTcCfg<D, MB>;
     extern __shared__ unsigned char smem_raw[];
-    const long long total = p.total_items;
-    const int item_begin = (int)(total * blockIdx.x / gridDim.x);
-    const int item_end = (int)(total * (blockIdx.x + 1) / gridDim.x);
+    int item_begin, item_end;
+    tc::item_range(p, item_begin, item_end);
     grid_release();
     grid_wait();
     tc::stamp(p.clk, 0);

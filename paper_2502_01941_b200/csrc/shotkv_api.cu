@@ -501,6 +501,9 @@ int tc_setup(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* Q, const 
     sp.L = d->L; sp.Hkv = d->Hkv; sp.N = d->N; sp.W = d->W; sp.R = R; sp.Rpad = rpad_of(d);
     if (U * plan.nchunk > 0x7fffffffLL) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "too many work items");
     sp.total_items = (int)(U * plan.nchunk);
+    const int ctas = sp.total_items < ctx->sm_count ? sp.total_items : ctx->sm_count;      // as the launches do
+    sp.items_each = sp.total_items / ctas;
+    sp.items_more = sp.total_items % ctas;
     sp.scale_log2 = kLog2e / sqrtf((float)d->d);
     sp.part_m = w.part_m; sp.part_z = w.part_z;
     sp.item_m = w.item_m; sp.item_z = w.item_z;
@@ -694,11 +697,11 @@ int run_reduce_select_t(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView
     // a row of masses per CTA of the cluster: with thousands of shots fewer CTAs share the heads, so
     // that two still fit an SM (one from about 4,000 shots on)
     int ranks = d->Hkv < kReduceCluster ? d->Hkv : kReduceCluster;
-    while (ranks > 1 && reduce_smem_bytes(ROWS, pv.P, d->S, ranks) > kBigSmem / 2) ranks = (ranks + 1) / 2;
-    const size_t smem = reduce_smem_bytes(ROWS, pv.P, d->S, ranks);
+    while (ranks > 1 && reduce_smem_bytes(ROWS, pv.P, d->S, pv.nchunk, ranks) > kBigSmem / 2) ranks = (ranks + 1) / 2;
+    const size_t smem = reduce_smem_bytes(ROWS, pv.P, d->S, pv.nchunk, ranks);
     if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "too many shots for the single-pass path (S = %d)", d->S);
     return launch(ctx, reduce_select_kernel<ROWS>, dim3(d->B * d->L * ranks), kReduceThreads, smem, stream, ranks, kEarly, pv, tab,
-                  (d->H / d->Hkv) * d->W, (int)d->Hkv, ranks, shot_scores, sa);
+                  (d->H / d->Hkv) * d->W, (int)d->Hkv, ranks, shot_scores, sa, ctx->err_dev);
 }
 int run_reduce_select(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView& pv, const ShotTable& tab, float* shot_scores,
                       const SelectArgs& sa, cudaStream_t stream) {
