@@ -187,12 +187,15 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
         const int q0 = q_first + q_count * warp / NW, q1 = q_first + q_count * (warp + 1) / NW;
         float m_first[FIRST], z_first[FIRST];
         float4 z4[AHEAD][NH];
+        auto load_items = [&](int j0) {
 #pragma unroll
-        for (int n = 0; n < FIRST; ++n) {
-            const int j = part + n * PARTS;
-            m_first[n] = j < v.nchunk ? im[(size_t)j * v.Rpad] : SHOTKV_NEG_INF;
-            z_first[n] = j < v.nchunk ? iz[(size_t)j * v.Rpad] : 0.f;
-        }
+            for (int n = 0; n < FIRST; ++n) {
+                const int j = j0 + n * PARTS;
+                m_first[n] = j < v.nchunk ? im[(size_t)j * v.Rpad] : SHOTKV_NEG_INF;
+                z_first[n] = j < v.nchunk ? iz[(size_t)j * v.Rpad] : 0.f;
+            }
+        };
+        load_items(part);
         auto load_pieces = [&](int q) {
 #pragma unroll
             for (int n = 0; n < AHEAD; ++n)
@@ -208,18 +211,20 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
             exact[j] = e;
             any |= e;
         }
-        // (m, z) of this thread's items, relative to their own maximum
+        // (m, z) of this thread's items, as many at a time as its loads ahead
         float m = SHOTKV_NEG_INF, z = 0.f;
+#pragma unroll 1
+        for (int j0 = part;; ) {
+            float bm = SHOTKV_NEG_INF, bz = 0.f;
 #pragma unroll
-        for (int n = 0; n < FIRST; ++n) m = fmaxf(m, m_first[n]);
-#pragma unroll 4
-        for (int j = part + FIRST * PARTS; j < v.nchunk; j += PARTS) m = fmaxf(m, im[(size_t)j * v.Rpad]);
-        {
-            const float mu = m == SHOTKV_NEG_INF ? 0.f : m;
+            for (int n = 0; n < FIRST; ++n) bm = fmaxf(bm, m_first[n]);
+            const float mu = bm == SHOTKV_NEG_INF ? 0.f : bm;
 #pragma unroll
-            for (int n = 0; n < FIRST; ++n) z += z_first[n] * ex2f(m_first[n] - mu);
-#pragma unroll 4
-            for (int j = part + FIRST * PARTS; j < v.nchunk; j += PARTS) z += iz[(size_t)j * v.Rpad] * ex2f(im[(size_t)j * v.Rpad] - mu);
+            for (int n = 0; n < FIRST; ++n) bz += z_first[n] * ex2f(m_first[n] - mu);
+            merge_mz(m, z, bm, bz);
+            j0 += FIRST * PARTS;
+            if (j0 >= v.nchunk) break;
+            load_items(j0);
         }
         if (PARTS > 1) {
             row_m[part * ROWS + r] = m;
@@ -244,13 +249,8 @@ __global__ void __launch_bounds__(kReduceThreads, 4) reduce_select_kernel(const 
         // 2^(m_item - row's m) / Z of this row; a row without weight (padding, or nothing but underflow) gets
         // factor 0 whatever its reference
         auto factor = [](float ref, float m, float w) { return w > 0.f ? ex2f(ref - m) * w : 0.f; };
-#pragma unroll
-        for (int n = 0; n < FIRST; ++n) {
-            const int j = part + n * PARTS;
-            if (j < v.nchunk) weight[j * ROWS + r] = factor(m_first[n], rm, rw);
-        }
 #pragma unroll 4
-        for (int j = part + FIRST * PARTS; j < v.nchunk; j += PARTS) weight[j * ROWS + r] = factor(im[(size_t)j * v.Rpad], rm, rw);
+        for (int j = part; j < v.nchunk; j += PARTS) weight[j * ROWS + r] = factor(im[(size_t)j * v.Rpad], rm, rw);
         if (any) {                                 // for the pieces of exact items (the rows' statistics have been read)
             __syncthreads();
             if (part == 0) {
