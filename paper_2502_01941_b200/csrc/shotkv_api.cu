@@ -436,7 +436,9 @@ int launch_score_tc_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorMap
 // power cap for as long as it runs (5, 4, 3, 2, 1, 0 pairs: 4 x 32 layers of 32K 3,570, 3,550, 3,530, 3,580,
 // 3,630, 3,705 us a call), with 128 it waits for memory as much as for power (32 layers of 16K 395, -, 397,
 // 398, 399, 402).
-constexpr int kPolyPairs = 5, kPolyPairsStream = 3;
+// The second pass of the per-token form takes 4, 5 and 3 in the same time (16 layers of 8K with 256 rows 238 us a call each),
+// and its error grows with the share: 2.8e-6 to 4.8e-6 against 64 bits with 4, 3.2e-6 to 5.4e-6 with 5.
+constexpr int kPolyPairs = 5, kPolyPairsStream = 3, kPolyPairsTokens = 4;
 constexpr int kShortUnit = 64;        // mean length below which the streaming kernel takes its form for short units
 
 template <int D>
@@ -518,7 +520,7 @@ int launch_colsum_tc_f(shotkv_ctx* ctx, const TcSetup& t, const ColsumTcParams& 
     constexpr int smem = ColsumTcCfg<D, MB>::kSmemBytes;
     int grid = cp.base.total_items < ctx->sm_count ? cp.base.total_items : ctx->sm_count;
     if (grid < 1) grid = 1;
-    return launch(ctx, colsum_tc_kernel<D, MB, kPolyPairs, FULL>, dim3(grid), ColsumTcCfg<D, MB>::kThreads, smem, stream, 1, kEarly, t.tmQ, t.tmK, t.qbox, t.kbox, cp);
+    return launch(ctx, colsum_tc_kernel<D, MB, kPolyPairsTokens, FULL>, dim3(grid), ColsumTcCfg<D, MB>::kThreads, smem, stream, 1, kEarly, t.tmQ, t.tmK, t.qbox, t.kbox, cp);
 }
 template <int D, int MB>
 int launch_colsum_tc_t(shotkv_ctx* ctx, const TcSetup& t, const ColsumTcParams& cp, cudaStream_t stream) {
@@ -747,9 +749,9 @@ cudaError_t set_tc_attributes() {
     if (e == cudaSuccess && MB == 2)
         e = cudaFuncSetAttribute(score_stream_kernel<D, kPolyPairsStream, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ScoreStreamCfg<D>::kSmemBytes);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(colsum_tc_kernel<D, MB, kPolyPairs, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColsumTcCfg<D, MB>::kSmemBytes);
+        e = cudaFuncSetAttribute(colsum_tc_kernel<D, MB, kPolyPairsTokens, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColsumTcCfg<D, MB>::kSmemBytes);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(colsum_tc_kernel<D, MB, kPolyPairs, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColsumTcCfg<D, MB>::kSmemBytes);
+        e = cudaFuncSetAttribute(colsum_tc_kernel<D, MB, kPolyPairsTokens, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, ColsumTcCfg<D, MB>::kSmemBytes);
     return e;
 }
 cudaError_t set_kernel_attributes() {
