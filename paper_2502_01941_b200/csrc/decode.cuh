@@ -23,6 +23,132 @@ struct DecodeParams {
     int* err;                     // error word (host-visible); set to 1 when a bounded wait gave up
 };
 
+// The rest of a step for one (b, l): acc[j] += sum over kv heads of the entries' weights (fixed order,
+// a new entry starts from 0), and, every so many steps, the eviction: the k entries greatest in (acc
+// descending, index ascending) are kept, acc, born and the K and V rows moved up in place.  Entries
+// born at or after `protect_from` rank before all others (an option beyond the paper's rule; a value
+// above every step number protects nothing).
+struct DecodeFinishParams {
+    const float* partial;         // [U][Dcap]
+    float* acc;                   // [B*L][Dcap]
+    int* born;                    // [B*L][Dcap]
+    __nv_bfloat16* Kd;            // [U][Dcap][d]
+    __nv_bfloat16* Vd;            // [U][Dcap][d]
+    int Hkv, Dcap, n, T_old;      // n entries, the new one included
+    int k, protect_from;          // entries to keep
+    int ranks;                    // CTAs (a cluster) per (b, l), heads rank, rank + ranks, ... each
+};
+__device__ __forceinline__ float accumulated(const DecodeFinishParams& p, int bl, int j) {
+    const float* part = p.partial + (size_t)bl * p.Hkv * p.Dcap + j;
+    float s = 0.f;
+#pragma unroll 8
+    for (int h = 0; h < p.Hkv; ++h) s += part[(size_t)h * p.Dcap];
+    return (j == p.n - 1 ? 0.f : p.acc[(size_t)bl * p.Dcap + j]) + s;
+}
+
+// A step without eviction.
+constexpr int kAccumulateThreads = 128;         // one entry a thread
+__global__ void __launch_bounds__(kAccumulateThreads) decode_accumulate_kernel(const DecodeFinishParams p) {
+    const int bl = blockIdx.x, j = blockIdx.y * kAccumulateThreads + threadIdx.x;
+    grid_wait();
+    grid_release();
+    if (j < p.n) {
+        p.acc[(size_t)bl * p.Dcap + j] = accumulated(p, bl, j);
+        if (j == p.n - 1) p.born[(size_t)bl * p.Dcap + j] = p.T_old;
+    }
+}
+
+// A step with eviction.  Every CTA of the cluster adds up and ranks all entries for itself (a few
+// hundred: cheaper than handing the ranking round), so one barrier is all the cluster needs: nobody
+// writes acc and born before all have read them.  Then each moves the rows of its heads, as many at a
+// time as a thread keeps 16-byte vectors in flight; the source of row j is at or after j, so a pass
+// that first loads its rows and then, after a barrier, stores them never overwrites a later source.
+// Latency-bound: as three kernels (sum, ranking, rows) the end of a cycle took 2.5 + 4.8 + 2.4 us on one
+// small layer and 5 + 6.4 + 39 us on 8 sequences x 32 layers.
+// Shared memory: decode_evict_smem_bytes(n).  `value(j)`: entry j's accumulated score.  CTA `rank` of the `ranks` that share the
+// (b, l)'s heads; clustered: they are a cluster.  At most NT entries, or more than kRankByCount.
+__host__ __device__ constexpr size_t decode_evict_smem_bytes(int n) {
+    return rank_smem_bytes(n) + 5 * ((size_t)(n + 3) / 4 * 4 * 4) + 128;
+}
+template <int D, int NT, class Value>
+__device__ __forceinline__ void evict_entries(const DecodeFinishParams& p, int bl, int rank, int ranks, bool clustered, unsigned char* sm,
+                                              Value&& value) {
+    constexpr int VPR = D / 8, RPP = NT / VPR, Q = 4;   // 16-byte vectors a row, rows a pass per vector in flight
+    const int n = p.n, n4 = (n + 3) / 4 * 4;
+    float* a = reinterpret_cast<float*>(sm + rank_smem_bytes(n));   // accumulated scores
+    int* bs = reinterpret_cast<int*>(a + n4);      // born
+    int* kf = bs + n4;                             // kept?
+    int* ds = kf + n4;                             // its exclusive scan = destination
+    int* kp = ds + n4;                             // destination -> source
+    int* tmp = kp + n4;
+    int* first_gone = tmp + 31;
+    const int tid = threadIdx.x;
+    if (tid == 0) *first_gone = n;
+#pragma unroll 1
+    for (int j = tid; j < n; j += NT) {
+        const float v = value(j);
+        a[j] = v == v ? v : SHOTKV_NEG_INF;        // keep the order total even if a score is NaN
+        bs[j] = j < n - 1 ? p.born[(size_t)bl * p.Dcap + j] : p.T_old;
+    }
+    if (clustered) cluster_arrive();
+    __syncthreads();
+    const float top = __int_as_float(0x7f800000);
+    rank_all<NT>(n, sm, [&](int j) { return bs[j] >= p.protect_from ? top : a[j]; },
+                 [&](int r, int j) {
+                     kf[j] = ds[j] = r < p.k;
+                     if (r >= p.k) atomicMin(first_gone, j);
+                 });
+    __syncthreads();
+    block_exclusive_scan<NT>(ds, n, tmp);
+#pragma unroll 1
+    for (int j = tid; j < n; j += NT)
+        if (kf[j]) kp[ds[j]] = j;
+    if (clustered) cluster_wait();                 // all CTAs have read acc and born
+    __syncthreads();
+    if (rank == 0)
+#pragma unroll 1
+        for (int j = tid; j < p.k; j += NT) {
+            p.acc[(size_t)bl * p.Dcap + j] = a[kp[j]];
+            p.born[(size_t)bl * p.Dcap + j] = bs[kp[j]];
+        }
+    const int row_in = tid / VPR, vec = tid % VPR;
+    for (int h = rank; h < p.Hkv; h += ranks) {
+        uint4* Ku = reinterpret_cast<uint4*>(p.Kd + ((size_t)bl * p.Hkv + h) * p.Dcap * D);
+        uint4* Vu = reinterpret_cast<uint4*>(p.Vd + ((size_t)bl * p.Hkv + h) * p.Dcap * D);
+        for (int c = *first_gone; c < p.k; c += RPP * Q) {      // the rows before the first evicted entry stay
+            uint4 kk[Q], vv[Q];
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int j = c + q * RPP + row_in;
+                kk[q] = vv[q] = make_uint4(0, 0, 0, 0);
+                if (j < p.k) {
+                    const size_t at = (size_t)kp[j] * VPR + vec;
+                    kk[q] = Ku[at];
+                    vv[q] = Vu[at];
+                }
+            }
+            __syncthreads();
+#pragma unroll
+            for (int q = 0; q < Q; ++q) {
+                const int j = c + q * RPP + row_in;
+                if (j < p.k) {
+                    Ku[(size_t)j * VPR + vec] = kk[q];
+                    Vu[(size_t)j * VPR + vec] = vv[q];
+                }
+            }
+            __syncthreads();
+        }
+    }
+}
+template <int D>
+__global__ void __launch_bounds__(kSelectThreads) decode_evict_kernel(const DecodeFinishParams p) {
+    extern __shared__ __align__(16) unsigned char sm[];
+    const int bl = blockIdx.x / p.ranks, rank = blockIdx.x - bl * p.ranks;
+    grid_wait();
+    grid_release();
+    evict_entries<D, kSelectThreads>(p, bl, rank, p.ranks, p.ranks > 1, sm, [&](int j) { return accumulated(p, bl, j); });
+}
+
 // ---- a unit's keys shared by a cluster -------------------------------------------------------
 // A unit (sequence, layer, kv head) whose batch is too small to fill the GPU is shared by a cluster of
 // p.nsplit CTAs: blocks of 16 keys go round the warps of all of them.  Every CTA sends its (m, z) per
@@ -81,6 +207,59 @@ __device__ __forceinline__ float entry_weight(const float* sdec, int Dcap, int G
     return s;
 }
 
+// ---- a step that ends in the kernel it begins in -----------------------------------------------
+// Where all CTAs of a (sequence, layer) fit one cluster, its heads' and their shares', the end of the step needs no kernel of
+// its own: every CTA sends the weights of its decode entries to the CTA that adds them up, or to all where the step
+// evicts, and goes on as the kernels above do, in the same order of additions.  (One kernel boundary and one launch less: see
+// decode_step_impl.)
+constexpr int kFusedWeights = 4096;                // most weights, heads x entries, that a CTA is sent
+struct FusedEnd {
+    float* weights;               // [Hkv][n]  in shared memory
+    unsigned long long* arrived;
+    unsigned char* scratch;       // decode_evict_smem_bytes(n), where the step evicts
+};
+__host__ __device__ constexpr size_t fused_end_smem_bytes(int Hkv, int n, bool evicts) {
+    return 16 + ((size_t)Hkv * n + 3) / 4 * 16 + (evicts ? decode_evict_smem_bytes(n) : 0);
+}
+// By one thread, ahead of the cluster_arrive at the start; `c`: this CTA's number in the cluster.
+__device__ __forceinline__ FusedEnd fused_end_at(unsigned char* sm, const DecodeFinishParams& f) {
+    float* w = reinterpret_cast<float*>(sm + 16);
+    return FusedEnd{w, reinterpret_cast<unsigned long long*>(sm), reinterpret_cast<unsigned char*>(w + (f.Hkv * f.n + 3) / 4 * 4)};
+}
+__device__ __forceinline__ void fused_expect(const FusedEnd& e, const DecodeFinishParams& f, int c) {
+    if (f.k < f.n || c == 0) expect_messages(e.arrived, f.Hkv * f.n * (int)sizeof(float));
+}
+__device__ __forceinline__ void fused_send(const FusedEnd& e, const DecodeFinishParams& f, int hk, int j, float w, int ctas) {
+    float* to = e.weights + hk * f.n + j;
+    const int receivers = f.k < f.n ? ctas : 1;
+#pragma unroll 1
+    for (int c = 0; c < receivers; ++c) send(to, c, e.arrived, w);
+}
+// All threads of all CTAs, once a CTA has sent its weights and made its other outputs.
+template <int D, int NT>
+__device__ __forceinline__ void fused_finish(const FusedEnd& e, const DecodeFinishParams& f, int bl, int c, int ctas, int* err) {
+    const bool evicts = f.k < f.n;
+    if (!evicts && c != 0) return;
+    await_messages(e.arrived, err);
+    const auto value = [&](int j) {
+        float s = 0.f;
+#pragma unroll 1
+        for (int h = 0; h < f.Hkv; ++h) s += e.weights[h * f.n + j];
+        return (j == f.n - 1 ? 0.f : f.acc[(size_t)bl * f.Dcap + j]) + s;
+    };
+    if (evicts) {
+        evict_entries<D, NT>(f, bl, c, ctas, true, e.scratch, value);
+    } else {
+#pragma unroll 1
+        for (int j = threadIdx.x; j < f.n; j += NT) {
+            f.acc[(size_t)bl * f.Dcap + j] = value(j);
+            if (j == f.n - 1) f.born[(size_t)bl * f.Dcap + j] = f.T_old;
+        }
+    }
+}
+
+__host__ __device__ constexpr size_t score_smem_bytes(int Dcap) { return ((size_t)8 * Dcap + 8 * 8 * 2 + kMaxSplit * 16 + 4) * 4; }
+
 // One CTA, or a cluster of p.nsplit, per (sequence, layer, kv head).  Each warp takes 16 keys at a
 // time straight from global memory: thread (g, t) of a warp reads 16 contiguous bytes of key rows g
 // and g+8 per 32-dim block, which serve as the A fragments of two m16n8k16 MMAs whose B operand is
@@ -92,8 +271,9 @@ __device__ __forceinline__ float entry_weight(const float* sdec, int Dcap, int G
 // unrolled and more loads are in flight, to the depth that is written down here (left to itself the compiler
 // chose 1 to 4 by what stood around the loop: 8 sequences x 32 layers 301 to 259 us a step, 1 sequence 56 to 43; four
 // deep 255 and 39.5).
-template <int D, bool SPLIT>
-__global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p) {
+// FUSED (with SPLIT): the cluster is all CTAs of a (sequence, layer), and the step ends here.
+template <int D, bool SPLIT, bool FUSED>
+__global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p, const DecodeFinishParams f) {
     constexpr int NB = D / 32;     // 32-dim blocks
     constexpr int VPR = D / 8;     // 16-byte vectors per row
     extern __shared__ __align__(16) unsigned char dsm[];
@@ -106,13 +286,19 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p)
     const int g = lane >> 2, t4 = lane & 3;
     const int nsplit = SPLIT ? p.nsplit : 1;
     const int u = blockIdx.x / nsplit, rank = blockIdx.x - u * nsplit;
+    const int bl = u / p.Hkv, hk = u - bl * p.Hkv;
+    const int first_cta = FUSED ? hk * nsplit : 0, ctas = p.Hkv * nsplit;    // in the cluster: the unit's first; FUSED: all
+    FusedEnd end{};
+    if (FUSED) end = fused_end_at(dsm + score_smem_bytes(p.Dcap), f);
     if (SPLIT) {
-        if (tid == 0) expect_messages(arrived, nsplit * 8 * (int)sizeof(float2));
+        if (tid == 0) {
+            expect_messages(arrived, nsplit * 8 * (int)sizeof(float2));
+            if (FUSED) fused_expect(end, f, first_cta + rank);
+        }
         cluster_arrive();
     }
     grid_wait();
     grid_release();
-    const int bl = u / p.Hkv, hk = u - bl * p.Hkv;
     const uint4* Kc_u = reinterpret_cast<const uint4*>(p.Kc + (size_t)u * p.Mcap * D);
     uint4* Kd_u = reinterpret_cast<uint4*>(p.Kd + (size_t)u * p.Dcap * D);
     uint4* Vd_u = reinterpret_cast<uint4*>(p.Vd + (size_t)u * p.Dcap * D);
@@ -232,8 +418,8 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p)
     __syncthreads();
     if (SPLIT) {
         if (tid < 8 * nsplit) {                            // every CTA's rows to every CTA
-            float f[8];
-            send(stab + rank * 8 + (tid & 7), tid >> 3, arrived, row_of_cta(sred, tid & 7, f));
+            float fac[8];
+            send(stab + rank * 8 + (tid & 7), first_cta + (tid >> 3), arrived, row_of_cta(sred, tid & 7, fac));
         }
         await_messages(arrived, p.err);
     }
@@ -245,8 +431,10 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p)
             const int j = base + lane - M;
             const bool entry = lane < 16 && j >= 0 && j < n;
             const float s = entry_weight(sdec, p.Dcap, p.G, j, entry, rm, riz);
-            if (entry) p.partial[(size_t)u * p.Dcap + j] = s;
+            if (FUSED && entry) fused_send(end, f, hk, j, s, ctas);
+            else if (entry) p.partial[(size_t)u * p.Dcap + j] = s;
         }
+        if (FUSED) fused_finish<D, 256>(end, f, bl, first_cta + rank, ctas, p.err);
     } else {
         for (int j0 = warp * 32; j0 < n; j0 += 256) {
             const float s = entry_weight(sdec, p.Dcap, p.G, j0 + lane, j0 + lane < n, rm, riz);
@@ -295,6 +483,13 @@ struct AttendCfg {
     static_assert(8 * D * 4 <= kStages * kStageBytes, "a warp's outputs take the place of its ring");
 };
 
+// Dynamic shared memory of the decode kernels for decode regions of Dcap rows, multiples of 16 bytes.
+template <int D>
+__host__ __device__ constexpr size_t attend_smem_bytes(int G, int Dcap, int nsplit) {
+    const size_t shares = nsplit > 1 ? (size_t)nsplit * (16 + (G * D / 4 / nsplit + 1) * 4) : 0;   // (m, z) of 8 rows, and a share of the quads
+    return AttendCfg<D>::kRingBytes + 16 + ((size_t)AttendCfg<D>::kWarps * 16 + ((size_t)G * Dcap + 3) / 4 * 4 + shares) * 4;
+}
+
 // The same step with the attention output fused in: o_h = sum_t alpha_{t,h} v_t over the kept
 // prefill entries and the decode entries, with the very weights the decoding score sums, so that
 // scoring adds no pass over K to a decode step that has to read K and V anyway.
@@ -327,8 +522,9 @@ struct AttendCfg {
 // latencies: everything the first two blocks need is now asked for in one go, each warp's outputs take the place of its own
 // ring (no barrier before they are written), every thread merges the rows it needs for itself, and the CTAs of a cluster
 // send each other their rows and the quads of output each adds up (12.9 -> 11.1 us; 2 sequences 12.2 -> 9.2).
-template <int D>
-__global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_kernel(const DecodeParams p) {
+// FUSED: the cluster is all CTAs of a (sequence, layer), and the step ends here.
+template <int D, bool FUSED>
+__global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_kernel(const DecodeParams p, const DecodeFinishParams f) {
     using Cfg = AttendCfg<D>;
     constexpr int NB = D / 32;     // 32-dim blocks
     constexpr int VPR = D / 8;     // 16-byte chunks per row
@@ -349,13 +545,19 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     // quad number q / nsplit (256 quads and 16 CTAs at most: the product is exact).
     const int quads = p.G * (D / 4), over = 65536 / p.nsplit + 1;
     const int share = (quads * over) >> 16, owned = share + (rank < quads - share * p.nsplit);
-    if (p.nsplit > 1) {
-        if (tid == 0) expect_messages(arrived, p.nsplit * (8 * (int)sizeof(float2) + owned * (int)sizeof(float4)));
+    const int bl = u / p.Hkv, hk = u - bl * p.Hkv;
+    const int first_cta = FUSED ? hk * p.nsplit : 0, ctas = p.Hkv * p.nsplit;   // in the cluster: the unit's first; FUSED: all
+    FusedEnd end{};
+    if (FUSED) end = fused_end_at(dsm + attend_smem_bytes<D>(p.G, p.Dcap, p.nsplit), f);
+    if (FUSED || p.nsplit > 1) {
+        if (tid == 0) {
+            if (p.nsplit > 1) expect_messages(arrived, p.nsplit * (8 * (int)sizeof(float2) + owned * (int)sizeof(float4)));
+            if (FUSED) fused_expect(end, f, first_cta + rank);
+        }
         cluster_arrive();
     }
     grid_wait();
     grid_release();
-    const int bl = u / p.Hkv, hk = u - bl * p.Hkv;
     uint4* Kd_u = reinterpret_cast<uint4*>(p.Kd + (size_t)u * p.Dcap * D);
     uint4* Vd_u = reinterpret_cast<uint4*>(p.Vd + (size_t)u * p.Dcap * D);
     const uint4* knew_u = reinterpret_cast<const uint4*>(p.k_new + (size_t)u * D);
@@ -403,7 +605,7 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     const int M = min(kept, p.Mcap);
     const int n = p.n_old + 1;
     const int Ktot = M + n;
-    if (p.nsplit > 1) cluster_wait();                        // all CTAs of the cluster have begun: their memory may be written to
+    if (FUSED || p.nsplit > 1) cluster_wait();               // all CTAs of the cluster have begun: their memory may be written to
     if (appends) (tid < VPR ? Kd_u + (size_t)p.n_old * VPR + tid : Vd_u + (size_t)p.n_old * VPR + (tid - VPR))[0] = fresh_row;   // decode entry n_old
 
     // a block with decode entries in it, or past the end: rows past the end are filled with zeros (a weight of
@@ -544,24 +746,24 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     __syncthreads();
     float* out = p.out + ((size_t)bl * p.H + (size_t)hk * p.G) * D;
     if (p.nsplit > 1 && tid < 8 * p.nsplit) {                // every CTA's rows to every CTA
-        float f[NW];
-        send(stab + rank * 8 + (tid & 7), tid >> 3, arrived, row_of_cta(sred, tid & 7, f));
+        float fac[NW];
+        send(stab + rank * 8 + (tid & 7), first_cta + (tid >> 3), arrived, row_of_cta(sred, tid & 7, fac));
     }
     // the warps' outputs relative to the CTA's maximum: alone, the CTA has the rows' whole sums
 #pragma unroll 1
     for (int q = tid; q < quads; q += NT) {
         const int r = q / (D / 4), c = q % (D / 4) * 4;
-        float f[NW];
-        const float2 row = row_of_cta(sred, r, f);
+        float fac[NW];
+        const float2 row = row_of_cta(sred, r, fac);
         float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
 #pragma unroll
         for (int w = 0; w < NW; ++w) {
             const float4 v = *reinterpret_cast<const float4*>(sO + w * kWarpRing + r * PITCH + c);
-            if (f[w] >= 0.f) o.x += v.x * f[w], o.y += v.y * f[w], o.z += v.z * f[w], o.w += v.w * f[w];
+            if (fac[w] >= 0.f) o.x += v.x * fac[w], o.y += v.y * fac[w], o.z += v.z * fac[w], o.w += v.w * fac[w];
         }
         if (p.nsplit > 1) {
             const int slot = (q * over) >> 16, to = q - slot * p.nsplit;
-            send(sin + rank * (share + 1) + slot, to, arrived, o);
+            send(sin + rank * (share + 1) + slot, first_cta + to, arrived, o);
         } else {
             const float iz = row.y > 0.f ? 1.f / row.y : 0.f;
             float* d = out + 4 * q;
@@ -588,8 +790,8 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
                 const int c = t4 + 4 * i;
                 if (slot < owned && c < p.nsplit) {
                     const float4 v = sin[c * (share + 1) + slot];
-                    const float f = ex2f(stab[c * 8 + r].x - mu);
-                    o.x += v.x * f, o.y += v.y * f, o.z += v.z * f, o.w += v.w * f;
+                    const float e = ex2f(stab[c * 8 + r].x - mu);
+                    o.x += v.x * e, o.y += v.y * e, o.z += v.z * e, o.w += v.w * e;
                 }
             }
 #pragma unroll
@@ -607,128 +809,10 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
         const int j = base + lane - M;
         const bool entry = lane < 16 && j >= 0 && j < n;
         const float s = entry_weight(sdec, p.Dcap, p.G, j, entry, rm, riz);
-        if (entry) p.partial[(size_t)u * p.Dcap + j] = s;
+        if (FUSED && entry) fused_send(end, f, hk, j, s, ctas);
+        else if (entry) p.partial[(size_t)u * p.Dcap + j] = s;
     }
-}
-
-// The rest of a step for one (b, l): acc[j] += sum over kv heads of the entries' weights (fixed order,
-// a new entry starts from 0), and, every so many steps, the eviction: the k entries greatest in (acc
-// descending, index ascending) are kept, acc, born and the K and V rows moved up in place.  Entries
-// born at or after `protect_from` rank before all others (an option beyond the paper's rule; a value
-// above every step number protects nothing).
-struct DecodeFinishParams {
-    const float* partial;         // [U][Dcap]
-    float* acc;                   // [B*L][Dcap]
-    int* born;                    // [B*L][Dcap]
-    __nv_bfloat16* Kd;            // [U][Dcap][d]
-    __nv_bfloat16* Vd;            // [U][Dcap][d]
-    int Hkv, Dcap, n, T_old;      // n entries, the new one included
-    int k, protect_from;          // entries to keep
-    int ranks;                    // CTAs (a cluster) per (b, l), heads rank, rank + ranks, ... each
-};
-__device__ __forceinline__ float accumulated(const DecodeFinishParams& p, int bl, int j) {
-    const float* part = p.partial + (size_t)bl * p.Hkv * p.Dcap + j;
-    float s = 0.f;
-#pragma unroll 8
-    for (int h = 0; h < p.Hkv; ++h) s += part[(size_t)h * p.Dcap];
-    return (j == p.n - 1 ? 0.f : p.acc[(size_t)bl * p.Dcap + j]) + s;
-}
-
-// A step without eviction.
-constexpr int kAccumulateThreads = 128;         // one entry a thread
-__global__ void __launch_bounds__(kAccumulateThreads) decode_accumulate_kernel(const DecodeFinishParams p) {
-    const int bl = blockIdx.x, j = blockIdx.y * kAccumulateThreads + threadIdx.x;
-    grid_wait();
-    grid_release();
-    if (j < p.n) {
-        p.acc[(size_t)bl * p.Dcap + j] = accumulated(p, bl, j);
-        if (j == p.n - 1) p.born[(size_t)bl * p.Dcap + j] = p.T_old;
-    }
-}
-
-// A step with eviction.  Every CTA of the cluster adds up and ranks all entries for itself (a few
-// hundred: cheaper than handing the ranking round), so one barrier is all the cluster needs: nobody
-// writes acc and born before all have read them.  Then each moves the rows of its heads, as many at a
-// time as a thread keeps 16-byte vectors in flight; the source of row j is at or after j, so a pass
-// that first loads its rows and then, after a barrier, stores them never overwrites a later source.
-// Latency-bound: as three kernels (sum, ranking, rows) the end of a cycle took 2.5 + 4.8 + 2.4 us on one
-// small layer and 5 + 6.4 + 39 us on 8 sequences x 32 layers.
-// Shared memory: decode_evict_smem_bytes(n).
-__host__ __device__ constexpr size_t decode_evict_smem_bytes(int n) {
-    return rank_smem_bytes(n) + 5 * ((size_t)(n + 3) / 4 * 4 * 4) + 128;
-}
-template <int D>
-__global__ void __launch_bounds__(kSelectThreads) decode_evict_kernel(const DecodeFinishParams p) {
-    constexpr int NT = kSelectThreads, VPR = D / 8, RPP = NT / VPR, Q = 4;   // 16-byte vectors a row, rows a pass per vector in flight
-    extern __shared__ __align__(16) unsigned char sm[];
-    __shared__ int first_gone;
-    const int n = p.n, n4 = (n + 3) / 4 * 4;
-    float* a = reinterpret_cast<float*>(sm + rank_smem_bytes(n));   // accumulated scores
-    int* bs = reinterpret_cast<int*>(a + n4);      // born
-    int* kf = bs + n4;                             // kept?
-    int* ds = kf + n4;                             // its exclusive scan = destination
-    int* kp = ds + n4;                             // destination -> source
-    int* tmp = kp + n4;
-    const int tid = threadIdx.x;
-    const int bl = blockIdx.x / p.ranks, rank = blockIdx.x - bl * p.ranks;
-    if (tid == 0) first_gone = n;
-    grid_wait();
-    grid_release();
-#pragma unroll 1
-    for (int j = tid; j < n; j += NT) {
-        const float v = accumulated(p, bl, j);
-        a[j] = v == v ? v : SHOTKV_NEG_INF;        // keep the order total even if a score is NaN
-        bs[j] = j < n - 1 ? p.born[(size_t)bl * p.Dcap + j] : p.T_old;
-    }
-    if (p.ranks > 1) cluster_arrive();
-    __syncthreads();
-    const float top = __int_as_float(0x7f800000);
-    rank_all<NT>(n, sm, [&](int j) { return bs[j] >= p.protect_from ? top : a[j]; },
-                 [&](int r, int j) {
-                     kf[j] = ds[j] = r < p.k;
-                     if (r >= p.k) atomicMin(&first_gone, j);
-                 });
-    __syncthreads();
-    block_exclusive_scan<NT>(ds, n, tmp);
-#pragma unroll 1
-    for (int j = tid; j < n; j += NT)
-        if (kf[j]) kp[ds[j]] = j;
-    if (p.ranks > 1) cluster_wait();               // all CTAs have read acc and born
-    __syncthreads();
-    if (rank == 0)
-#pragma unroll 1
-        for (int j = tid; j < p.k; j += NT) {
-            p.acc[(size_t)bl * p.Dcap + j] = a[kp[j]];
-            p.born[(size_t)bl * p.Dcap + j] = bs[kp[j]];
-        }
-    const int row_in = tid / VPR, vec = tid % VPR;
-    for (int h = rank; h < p.Hkv; h += p.ranks) {
-        uint4* Ku = reinterpret_cast<uint4*>(p.Kd + ((size_t)bl * p.Hkv + h) * p.Dcap * D);
-        uint4* Vu = reinterpret_cast<uint4*>(p.Vd + ((size_t)bl * p.Hkv + h) * p.Dcap * D);
-        for (int c = first_gone; c < p.k; c += RPP * Q) {      // the rows before the first evicted entry stay
-            uint4 kk[Q], vv[Q];
-#pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                const int j = c + q * RPP + row_in;
-                kk[q] = vv[q] = make_uint4(0, 0, 0, 0);
-                if (j < p.k) {
-                    const size_t at = (size_t)kp[j] * VPR + vec;
-                    kk[q] = Ku[at];
-                    vv[q] = Vu[at];
-                }
-            }
-            __syncthreads();
-#pragma unroll
-            for (int q = 0; q < Q; ++q) {
-                const int j = c + q * RPP + row_in;
-                if (j < p.k) {
-                    Ku[(size_t)j * VPR + vec] = kk[q];
-                    Vu[(size_t)j * VPR + vec] = vv[q];
-                }
-            }
-            __syncthreads();
-        }
-    }
+    if (FUSED) fused_finish<D, NT>(end, f, bl, first_cta + rank, ctas, p.err);
 }
 
 }  // namespace shotkv

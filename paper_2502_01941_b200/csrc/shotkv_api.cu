@@ -727,14 +727,6 @@ int run_compact(shotkv_ctx* ctx, const shotkv_dims* d, const shotkv_bf16* K, con
                   kept_idx, kept_count, (int)d->Hkv, (int)d->N, (int)Mcap, (uint4*)Kc, (uint4*)Vc);
 }
 
-// Dynamic shared memory of the decode kernels for decode regions of Dcap rows.
-template <int D>
-size_t attend_smem(int G, int Dcap, int nsplit) {
-    const size_t shares = nsplit > 1 ? (size_t)nsplit * (16 + (G * D / 4 / nsplit + 1) * 4) : 0;   // (m, z) of 8 rows, and a share of the quads
-    return AttendCfg<D>::kRingBytes + 16 + ((size_t)AttendCfg<D>::kWarps * 16 + ((size_t)G * Dcap + 3) / 4 * 4 + shares) * 4;
-}
-size_t score_smem(int Dcap) { return ((size_t)8 * Dcap + 8 * 8 * 2 + kMaxSplit * 16 + 2) * 4; }
-
 // Dynamic shared-memory limits of every kernel that may need more than the 48 KB default.  A
 // function attribute belongs to the device's context, so it is set once when a shotkv_ctx is
 // created on that device, never on a launch path.
@@ -761,19 +753,19 @@ cudaError_t set_kernel_attributes() {
     if (e == cudaSuccess) e = set_tc_attributes<64, 2>();
     const void* small[] = {(const void*)select_shots_kernel<kSelectThreads>, (const void*)select_shots_kernel<kSortThreads>,
                            (const void*)reduce_select_kernel<128>, (const void*)reduce_select_kernel<256>,
-                           (const void*)decode_score_kernel<128, true>, (const void*)decode_score_kernel<64, true>,
-                           (const void*)decode_score_kernel<128, false>, (const void*)decode_score_kernel<64, false>,
-                           (const void*)decode_attend_kernel<128>, (const void*)decode_attend_kernel<64>,
+                           (const void*)decode_score_kernel<128, true, false>, (const void*)decode_score_kernel<128, true, true>, (const void*)decode_score_kernel<64, true, false>, (const void*)decode_score_kernel<64, true, true>,
+                           (const void*)decode_score_kernel<128, false, false>, (const void*)decode_score_kernel<64, false, false>,
+                           (const void*)decode_attend_kernel<128, false>, (const void*)decode_attend_kernel<128, true>, (const void*)decode_attend_kernel<64, false>, (const void*)decode_attend_kernel<64, true>,
                            (const void*)decode_evict_kernel<128>, (const void*)decode_evict_kernel<64>};
     for (const void* f : small)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kBigSmem);
     // a decode unit may be shared by more CTAs than the eight that every device's clusters allow
-    const void* split[] = {(const void*)decode_attend_kernel<128>, (const void*)decode_attend_kernel<64>,
-                           (const void*)decode_score_kernel<128, true>, (const void*)decode_score_kernel<64, true>};
+    const void* split[] = {(const void*)decode_attend_kernel<128, false>, (const void*)decode_attend_kernel<128, true>, (const void*)decode_attend_kernel<64, false>, (const void*)decode_attend_kernel<64, true>,
+                           (const void*)decode_score_kernel<128, true, false>, (const void*)decode_score_kernel<128, true, true>, (const void*)decode_score_kernel<64, true, false>, (const void*)decode_score_kernel<64, true, true>};
     for (const void* f : split)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     // the fused decode step wants three CTAs of ~74 KB each on an SM: ask for the largest shared-memory carve-out
-    const void* wide[] = {(const void*)decode_attend_kernel<128>, (const void*)decode_attend_kernel<64>};
+    const void* wide[] = {(const void*)decode_attend_kernel<128, false>, (const void*)decode_attend_kernel<128, true>, (const void*)decode_attend_kernel<64, false>, (const void*)decode_attend_kernel<64, true>};
     for (const void* f : wide)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     return e;
@@ -801,10 +793,10 @@ cudaError_t ask_room(K* kernel, int threads, size_t smem, int* room) {
     return cudaSuccess;
 }
 cudaError_t ask_decode_room(shotkv_ctx* ctx) {
-    cudaError_t e = ask_room(decode_attend_kernel<64>, AttendCfg<64>::kWarps * 32, attend_smem<64>(kRoomGroup, kRoomRows, kMaxSplit), ctx->room_attend[0]);
-    if (e == cudaSuccess) e = ask_room(decode_attend_kernel<128>, AttendCfg<128>::kWarps * 32, attend_smem<128>(kRoomGroup, kRoomRows, kMaxSplit), ctx->room_attend[1]);
-    if (e == cudaSuccess) e = ask_room(decode_score_kernel<64, true>, 256, score_smem(kRoomRows), ctx->room_score[0]);
-    if (e == cudaSuccess) e = ask_room(decode_score_kernel<128, true>, 256, score_smem(kRoomRows), ctx->room_score[1]);
+    cudaError_t e = ask_room(decode_attend_kernel<64, false>, AttendCfg<64>::kWarps * 32, attend_smem_bytes<64>(kRoomGroup, kRoomRows, kMaxSplit), ctx->room_attend[0]);
+    if (e == cudaSuccess) e = ask_room(decode_attend_kernel<128, false>, AttendCfg<128>::kWarps * 32, attend_smem_bytes<128>(kRoomGroup, kRoomRows, kMaxSplit), ctx->room_attend[1]);
+    if (e == cudaSuccess) e = ask_room(decode_score_kernel<64, true, false>, 256, score_smem_bytes(kRoomRows), ctx->room_score[0]);
+    if (e == cudaSuccess) e = ask_room(decode_score_kernel<128, true, false>, 256, score_smem_bytes(kRoomRows), ctx->room_score[1]);
     return e;
 }
 
@@ -1336,21 +1328,43 @@ bool two_to_an_sm(const shotkv_ctx* ctx, const DecodeParams& p, int U) {
     return p.nsplit == 1 && U > ctx->sm_count && U <= 2 * ctx->sm_count;
 }
 
+// Does the step end in its first kernel (decode.cuh)?  Where the CTAs that share the units of a (sequence, layer) are one cluster,
+// one CTA to an SM does all of the step, and what is sent round stays small.  It saves a launch and a kernel boundary: one small
+// layer (2 heads of 333 keys) 5.1 -> 4.3 us a step with the attention output, 5.3 -> 4.4 without, 15.2 -> 13.1 us a call that evicts; 3 x 1 head
+// of 5,000 keys 5.0 -> 4.1; 4 x 8 heads of 185 keys 7.0 -> 6.7.  With more CTAs than SMs the clusters are placed worse
+// than single CTAs (32 layers x 8 heads 40 -> 46 us a step, with the attention output 70.5 -> 74.6).  An eviction, which all CTAs rank for
+// themselves, is for clusters of eight (16 CTAs, 8 layers: 9.4 -> 10.0), and ranks by counting, a thread an entry.
+constexpr int kFusedEvictCtas = 8;
+bool ends_fused(const shotkv_ctx* ctx, const int* room, const DecodeParams& p, const DecodeFinishParams& f, int U, int threads) {
+    const int ctas = p.Hkv * p.nsplit;
+    const bool evicts = f.k < f.n;
+    return ctas > 1 && ctas <= (evicts ? kFusedEvictCtas : kMaxSplit) && U * p.nsplit <= ctx->sm_count && U / p.Hkv <= room[ctas] &&
+           f.Hkv * f.n <= kFusedWeights && (!evicts || f.n <= threads);
+}
+
 template <int D>
-int launch_decode_attend(shotkv_ctx* ctx, DecodeParams& p, int U, cudaStream_t stream) {
+int launch_decode_attend(shotkv_ctx* ctx, DecodeParams& p, const DecodeFinishParams& f, int U, bool& ended, cudaStream_t stream) {
     using Cfg = AttendCfg<D>;
-    p.nsplit = decode_split(ctx->room_attend[D == 128], U, (long long)p.Mcap + p.n_old + 1, Cfg::kWarps, kLeastAttend);
-    size_t smem = attend_smem<D>(p.G, p.Dcap, p.nsplit);
+    const int* room = ctx->room_attend[D == 128];
+    p.nsplit = decode_split(room, U, (long long)p.Mcap + p.n_old + 1, Cfg::kWarps, kLeastAttend);
+    size_t smem = attend_smem_bytes<D>(p.G, p.Dcap, p.nsplit);
+    const size_t end = fused_end_smem_bytes(p.Hkv, f.n, f.k < f.n);
+    ended = ends_fused(ctx, room, p, f, U, Cfg::kWarps * 32) && smem + end <= kBigSmem;
+    if (ended)
+        return launch(ctx, decode_attend_kernel<D, true>, dim3(U * p.nsplit), Cfg::kWarps * 32, smem + end, stream, p.Hkv * p.nsplit, kEarly, p, f);
     if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "Dcap too large for the attention-output step");
     if (two_to_an_sm(ctx, p, U) && smem < kNoThirdCta) smem = kNoThirdCta;
-    return launch(ctx, decode_attend_kernel<D>, dim3(U * p.nsplit), Cfg::kWarps * 32, smem, stream, p.nsplit, kEarly, p);
+    return launch(ctx, decode_attend_kernel<D, false>, dim3(U * p.nsplit), Cfg::kWarps * 32, smem, stream, p.nsplit, kEarly, p, f);
 }
 template <int D>
-int launch_decode_score(shotkv_ctx* ctx, DecodeParams& p, int U, cudaStream_t stream) {
-    p.nsplit = decode_split(ctx->room_score[D == 128], U, (long long)p.Mcap + p.n_old + 1, 8, kLeastScore);
-    const size_t smem = score_smem(p.Dcap);
-    return p.nsplit > 1 ? launch(ctx, decode_score_kernel<D, true>, dim3(U * p.nsplit), 256, smem, stream, p.nsplit, kEarly, p)
-                        : launch(ctx, decode_score_kernel<D, false>, dim3(U), 256, smem, stream, 1, kEarly, p);
+int launch_decode_score(shotkv_ctx* ctx, DecodeParams& p, const DecodeFinishParams& f, int U, bool& ended, cudaStream_t stream) {
+    const int* room = ctx->room_score[D == 128];
+    p.nsplit = decode_split(room, U, (long long)p.Mcap + p.n_old + 1, 8, kLeastScore);
+    const size_t smem = score_smem_bytes(p.Dcap), end = fused_end_smem_bytes(p.Hkv, f.n, f.k < f.n);
+    ended = ends_fused(ctx, room, p, f, U, 256) && smem + end <= kBigSmem;
+    if (ended) return launch(ctx, decode_score_kernel<D, true, true>, dim3(U * p.nsplit), 256, smem + end, stream, p.Hkv * p.nsplit, kEarly, p, f);
+    return p.nsplit > 1 ? launch(ctx, decode_score_kernel<D, true, false>, dim3(U * p.nsplit), 256, smem, stream, p.nsplit, kEarly, p, f)
+                        : launch(ctx, decode_score_kernel<D, false, false>, dim3(U), 256, smem, stream, 1, kEarly, p, f);
 }
 
 // One decode step; with `attn_out` the score kernel is the variant that also writes the attention output.
@@ -1377,13 +1391,6 @@ int decode_step_impl(shotkv_ctx* ctx, shotkv_decode_state* st, const shotkv_bf16
     p.scale_log2 = kLog2e / sqrtf((float)d.d);
     p.Vc = (const __nv_bfloat16*)Vc; p.out = attn_out;
     p.err = ctx->err_dev;
-    prof_begin(ctx);
-    prof_mark(ctx, stream);
-    if (attn_out) rc = d.d == 128 ? launch_decode_attend<128>(ctx, p, U, stream) : launch_decode_attend<64>(ctx, p, U, stream);
-    else rc = d.d == 128 ? launch_decode_score<128>(ctx, p, U, stream) : launch_decode_score<64>(ctx, p, U, stream);
-    if (rc) return rc;
-    prof_mark(ctx, stream);
-
     DecodeFinishParams f{};
     f.partial = p.partial; f.acc = st->acc; f.born = st->born; f.Kd = p.Kd; f.Vd = p.Vd;
     f.Hkv = d.Hkv; f.Dcap = st->Dcap; f.n = st->n_dec + 1; f.T_old = st->T;
@@ -1398,8 +1405,17 @@ int decode_step_impl(shotkv_ctx* ctx, shotkv_decode_state* st, const shotkv_bf16
         if (f.k > f.n) f.k = f.n;
         f.protect_from = prot > 0 ? T - prot : 0x7fffffff;
     }
+    bool ended = false;                                   // the step ends in this kernel
+    prof_begin(ctx);
+    prof_mark(ctx, stream);
+    if (attn_out) rc = d.d == 128 ? launch_decode_attend<128>(ctx, p, f, U, ended, stream) : launch_decode_attend<64>(ctx, p, f, U, ended, stream);
+    else rc = d.d == 128 ? launch_decode_score<128>(ctx, p, f, U, ended, stream) : launch_decode_score<64>(ctx, p, f, U, ended, stream);
+    if (rc) return rc;
+    prof_mark(ctx, stream);
+
     const int how = kEarly | (attn_out && two_to_an_sm(ctx, p, U) ? kWideShared : 0);
-    if (f.k < f.n) {
+    if (ended) {
+    } else if (f.k < f.n) {
         f.ranks = d.Hkv < kReduceCluster ? d.Hkv : kReduceCluster;
         rc = d.d == 128 ? launch(ctx, decode_evict_kernel<128>, dim3(BL * f.ranks), kSelectThreads, decode_evict_smem_bytes(f.n), stream, f.ranks, how, f)
                         : launch(ctx, decode_evict_kernel<64>, dim3(BL * f.ranks), kSelectThreads, decode_evict_smem_bytes(f.n), stream, f.ranks, how, f);

@@ -42,6 +42,17 @@ def test_eviction_of_a_large_region(ctx, every):
     assert lockstep(ctx, cfg, 40, [(0, 0)]) <= 2
 
 
+@pytest.mark.parametrize("attend", [False, True], ids=["plain", "attend"])
+@pytest.mark.parametrize("Hkv,G,d,M,every,steps", [(1, 8, 128, 3000, 1, 6), (2, 4, 64, 30, 1, 6), (5, 3, 128, 64, 3, 8), (8, 2, 128, 100, 4, 9),
+                                                   (16, 1, 64, 30, 2, 6), (17, 1, 64, 30, 2, 6), (2, 2, 64, 20, 127, 130), (2, 2, 64, 20, 128, 131),
+                                                   (2, 2, 128, 20, 129, 132), (16, 1, 64, 20, 400, 259)])
+def test_step_of_one_cluster(ctx, Hkv, G, d, M, every, steps, attend):
+    """A (sequence, layer) whose CTAs are one cluster ends its step in the first kernel; on both sides of where that
+    stops: 16 CTAs, 4,096 weights, evictions of 128 entries (with the attention output)."""
+    cfg = wl.DecodeConfig("one", B=2, L=1, H=Hkv * G, Hkv=Hkv, d=d, steps=steps, r_d=0.5, recompress_every=every, cfg_id=77)
+    assert lockstep(ctx, cfg, M, [(0, 0), (1, 0)], np.array([[M], [M - 7]], np.int32), attend=attend) <= 2
+
+
 @pytest.mark.parametrize("M", [40, 2048], ids=["whole_unit", "shared_unit"])
 def test_query_that_is_not_a_number_gives_no_output(ctx, M):
     """The same output, zero, whether one CTA has the unit or a cluster shares it; other heads are as without it."""
