@@ -116,8 +116,8 @@ __device__ __forceinline__ float cluster_load(const float* p, int rank) {
     return v;
 }
 
-// What the CTAs of a cluster tell one another goes as messages: a store counts its bytes on the receiver's barrier, which is complete when
-// as many as the receiver expects are there.  That is one way across the cluster, where a barrier of all its threads is two
+// What the CTAs of a cluster tell one another goes as messages: a store counts its bytes on the receiver's
+// barrier, which is complete when as many as the receiver expects are there.  That is one way across the cluster, where a barrier of all its threads is two
 // (1.7 us of a step of 4 sequences x 1 layer).  expect_messages: by one thread, ahead of the cluster_arrive at the start;
 // nobody sends before a cluster_wait (a CTA's memory may be written once it has begun), and a CTA that has been sent
 // everything may end.
