@@ -310,7 +310,8 @@ SHOTKV_API uint64_t shotkv_repaired_items(const shotkv_ctx* ctx);
  * memory is released and the kernel returns.  The next call on the context then returns
  * SHOTKV_ERR_TIMEOUT once (the outputs of the call that gave up are invalid); the call after
  * that proceeds normally.  shotkv_set_wait_limit changes the limit for later launches of this
- * context (0 restores the default).  */
+ * context (0 restores the default).  The CTAs of a cluster in the reduction and the decode steps wait for
+ * one another's messages within a fixed limit of about two seconds, and report in the same way.  */
 SHOTKV_API int shotkv_set_wait_limit(shotkv_ctx* ctx, int64_t cycles);
 /* Runs the bounded-wait helpers on purpose into their limit, so that the give-up path can be
  * checked on any installation without disturbing a real kernel: one CTA, two barriers nobody

@@ -107,14 +107,6 @@ __device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
     return a;
 }
-__device__ __forceinline__ void cluster_store(float* p, int rank, float v) {
-    asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(cluster_addr(p, rank)), "f"(v) : "memory");
-}
-__device__ __forceinline__ float cluster_load(const float* p, int rank) {
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr(p, rank)) : "memory");
-    return v;
-}
 
 // What the CTAs of a cluster tell one another goes as messages: a store counts its bytes on the receiver's
 // barrier, which is complete when as many as the receiver expects are there.  That is one way across the cluster, where a barrier of all its threads is two
