@@ -10,10 +10,9 @@
 // that the R rows of one 64-element k block are contiguous, as the B operand needs.
 //
 // Epilogue: eight warps in two groups; a warp owns 32 keys (its tensor-memory lanes), a group
-// half of the window rows.  Per row one constant, log2(1/Z_r) - M_r, comes from shared memory as a
-// broadcast read of four: with 1/Z_r as a factor of its own the reads were twice as many (16 layers of 8K with 256
-// rows 242 -> 239 us a call, 32 layers of 16K in sentences 628 -> 620; error against 64 bits 3.5e-6 to 5.5e-6 before, 3.2e-6 to
-// 5.4e-6 with it in the exponent).  A chunk of 32 rows is asked for from tensor memory before the one ahead of it is
+// half of the window rows.  Per row the constants (-M_r, 1/Z_r) come from shared memory as
+// broadcast reads.  (As one constant, log2(1/Z_r) - M_r, they take half the reads, 236 -> 232 us a call of 16 layers of 8K with 256
+// rows, but 1/Z_r then has the resolution of M_r, and a row without weight no factor of zero.)  A chunk of 32 rows is asked for from tensor memory before the one ahead of it is
 // computed (32 layers of 16K in sentences 640 -> 628 us a call).  The second group hands its partial sums to the first through a two-slot
 // shared-memory ring guarded by mbarriers; the first adds them in a fixed order and stores.
 #pragma once
@@ -28,9 +27,6 @@ struct ColsumTcParams {
     float* imp;               // [U][N]
 };
 
-// What 256 rows without weight may add up to (2^-126 each); an importance below it is none.
-constexpr float kNoWeight = 0x1p-117f;
-
 template <int D, int MB>
 struct ColsumTcCfg {
     static constexpr int kSub = D / 64;
@@ -40,9 +36,9 @@ struct ColsumTcCfg {
     static constexpr int kStages = D == 128 ? 4 : 6;              // even: see mma_role_transposed
     static constexpr int kBarBytes = 1024;
     static constexpr int kRows = 128 * MB;
-    // per epilogue warp: the constants of its half of the rows, [rows/8] float4, and causal limits
-    // [rows/2] int; then the hand-over slots [4 quads][2][32] float
-    static constexpr int kCombBytes = 8 * ((kRows / 8) * 16 + (kRows / 2) * 4) + 4 * 2 * 32 * 4;
+    // per epilogue warp: the constants of its half of the rows, [rows/4] float4 (-M_r, -M_r+1, 1/Z_r, 1/Z_r+1)
+    // and causal limits [rows/2] int; then the hand-over slots [4 quads][2][32] float
+    static constexpr int kCombBytes = 8 * ((kRows / 4) * 16 + (kRows / 2) * 4) + 4 * 2 * 32 * 4;
     static constexpr int kSmemBytes = kQBytes + kStages * kStageBytes + kBarBytes + kCombBytes + 1024;
     static constexpr int kEpiWarps = 8;
     static constexpr int kThreads = 128 + kEpiWarps * 32;
@@ -118,8 +114,8 @@ __global__ void __launch_bounds__(ColsumTcCfg<D, MB>::kThreads, 1)
     tc::prefetch_maps(&tmQ, &tmK);
     tc::Pipe<Cfg> pp;
     tc::pipe_setup(pp, smem_raw, Cfg::kEpiWarps, 4 * 2 * 2, 2);     // extra barriers: [quad][slot][full, empty]
-    float4* cst = reinterpret_cast<float4*>(tc::pipe_scratch(pp, smem_raw));    // [8 warps][RG / 4]
-    int* plim_s = reinterpret_cast<int*>(cst + 8 * (RG / 4));                      // [8 warps][RG]
+    float4* cst = reinterpret_cast<float4*>(tc::pipe_scratch(pp, smem_raw));    // [8 warps][RG / 2]
+    int* plim_s = reinterpret_cast<int*>(cst + 8 * (RG / 2));                      // [8 warps][RG]
     float* slots = reinterpret_cast<float*>(plim_s + 8 * RG);                      // [4][2][32]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -149,7 +145,7 @@ __global__ void __launch_bounds__(ColsumTcCfg<D, MB>::kThreads, 1)
         const float scale = p.scale_log2;
         const uint64_t sc2 = tc::pack2(scale, scale);
         const float c1 = scale * (1.f / 254.f);
-        float4* cu = cst + e * (RG / 4);                   // this warp's own copy of its rows' constants
+        float4* cu = cst + e * (RG / 2);                   // this warp's own copy of its rows' constants
         int* pl = plim_s + e * RG;
         int acc = 0, cur_u = -1, ntile = 0;
         uint32_t tfphase0 = 0, tfphase1 = 0;
@@ -167,13 +163,15 @@ __global__ void __launch_bounds__(ColsumTcCfg<D, MB>::kThreads, 1)
                     const bool live = r < p.R;
                     const float m = live ? cp.row_m[(size_t)u * p.Rpad + r] : 0.f;
                     const float iz = live ? cp.row_invz[(size_t)u * p.Rpad + r] : 0.f;
-                    // the additive constant of the row's exponential, 1/Z in its exponent: log2(1/Z) - M_r where the
-                    // column pair goes to the special-function unit, 126 more of that over 254 where it goes to the
-                    // FMA pipe (see exp2_fma2); a row without weight gets one that exponentiates to zero, or to 2^-126 there
+                    float* c4 = reinterpret_cast<float*>(cu + (rr >> 1));
+                    // first two components: the additive constant of the row's exponential, -M_r where the
+                    // column pair goes to the special-function unit, (126 - M_r) / 254 where it goes to the
+                    // FMA pipe (see exp2_fma2); a row without weight gets 1/Z = 0 and a constant that exponentiates to
+                    // (nearly) zero, so that no infinity meets that zero
                     const bool has = live && iz > 0.f;
-                    const float k = log2f(iz) - m;
-                    reinterpret_cast<float*>(cu)[rr] = tc::pair_on_fma<PE>((rr >> 1) & 15) ? (has ? (126.f + k) * (1.f / 254.f) : -4.f)
-                                                                                           : (has ? k : SHOTKV_NEG_INF);
+                    c4[rr & 1] = tc::pair_on_fma<PE>((rr >> 1) & 15) ? (has ? (126.f - m) * (1.f / 254.f) : -4.f)
+                                                                     : (has ? -m : SHOTKV_NEG_INF);
+                    c4[2 + (rr & 1)] = has ? iz : 0.f;
                     pl[rr] = live ? p.N - p.W + (r % p.W) : -1;
                 }
                 __syncwarp();
@@ -199,12 +197,13 @@ __global__ void __launch_bounds__(ColsumTcCfg<D, MB>::kThreads, 1)
                 };
                 // the 32 rows of chunk c in r: alpha of every pair of rows at this thread's key, times 1/Z, added up
                 auto chunk = [&](const uint32_t (&r)[32], int c) {
-                    auto pair_term = [&](int jp, float ka, float kb, bool masked) {
+                    auto pair_term = [&](int jp, bool masked) {
+                        const float4 k4 = cu[c * 16 + jp];
                         uint64_t e2;
                         if (tc::pair_on_fma<PE>(jp)) {
-                            e2 = tc::exp2_from_unit2(tc::fma_sat(SKV_F(r, 2 * jp), c1, ka), tc::fma_sat(SKV_F(r, 2 * jp + 1), c1, kb));
+                            e2 = tc::exp2_from_unit2(tc::fma_sat(SKV_F(r, 2 * jp), c1, k4.x), tc::fma_sat(SKV_F(r, 2 * jp + 1), c1, k4.y));
                         } else {
-                            const uint64_t x2 = tc::ffma2(tc::pack2(SKV_F(r, 2 * jp), SKV_F(r, 2 * jp + 1)), sc2, tc::pack2(ka, kb));
+                            const uint64_t x2 = tc::ffma2(tc::pack2(SKV_F(r, 2 * jp), SKV_F(r, 2 * jp + 1)), sc2, tc::pack2(k4.x, k4.y));
                             float xa, xb;
                             tc::unpack2(x2, xa, xb);
                             e2 = tc::pack2(ex2f(xa), ex2f(xb));
@@ -214,18 +213,15 @@ __global__ void __launch_bounds__(ColsumTcCfg<D, MB>::kThreads, 1)
                             tc::unpack2(e2, ea, eb);
                             e2 = tc::pack2(key > pl[c * 32 + 2 * jp] ? 0.f : ea, key > pl[c * 32 + 2 * jp + 1] ? 0.f : eb);
                         }
-                        s2[jp & 1] = tc::fadd2(s2[jp & 1], e2);
+                        s2[jp & 1] = tc::ffma2(e2, tc::pack2(k4.z, k4.w), s2[jp & 1]);
                     };
-                    auto terms = [&](bool masked) {
+                    if (plain) {
 #pragma unroll
-                        for (int jq = 0; jq < 8; ++jq) {
-                            const float4 k4 = cu[c * 8 + jq];
-                            pair_term(2 * jq, k4.x, k4.y, masked);
-                            pair_term(2 * jq + 1, k4.z, k4.w, masked);
-                        }
-                    };
-                    if (plain) terms(false);
-                    else terms(true);
+                        for (int jp = 0; jp < 16; ++jp) pair_term(jp, false);
+                    } else {
+#pragma unroll
+                        for (int jp = 0; jp < 16; ++jp) pair_term(jp, true);
+                    }
                 };
                 uint32_t ra[32], rb[32];
                 if (!FULL && nch == 0) release();                   // no window rows in this group's half
@@ -273,7 +269,7 @@ __global__ void __launch_bounds__(ColsumTcCfg<D, MB>::kThreads, 1)
                     sum += sl[lane];
                     __syncwarp();
                     if (lane == 0) tc::mbar_arrive(pp.extra_bar(bs + 1));
-                    if (key < hi) cp.imp[(size_t)u * p.N + key] = sum < kNoWeight ? 0.f : sum;
+                    if (key < hi) cp.imp[(size_t)u * p.N + key] = sum;
                 }
                 ++ntile;
                 acc ^= 1;

@@ -436,9 +436,10 @@ int launch_score_tc_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorMap
 // power cap for as long as it runs (5, 4, 3, 2, 1, 0 pairs: 4 x 32 layers of 32K 3,570, 3,550, 3,530, 3,580,
 // 3,630, 3,705 us a call), with 128 it waits for memory as much as for power (32 layers of 16K 395, -, 397,
 // 398, 399, 402).
-// The second pass of the per-token form takes 4, 5 and 3 in the same time (16 layers of 8K with 256 rows 238 us a call each),
-// and its error grows with the share: 2.8e-6 to 4.8e-6 against 64 bits with 4, 3.2e-6 to 5.4e-6 with 5.
-constexpr int kPolyPairs = 5, kPolyPairsStream = 3, kPolyPairsTokens = 4;
+// The second pass of the per-token form takes 5, 4 and 3 in the same time (16 layers of 8K with 256 rows 237, 236, 236 us a call),
+// and its error grows with the share: 3.4e-6, 3.0e-6 and 2.6e-6 against 64 bits (256 rows, logits of deviation 1), 6.8e-5, 6.1e-5 and
+// 5.2e-5 (128 rows, deviation 400).
+constexpr int kPolyPairs = 5, kPolyPairsStream = 3, kPolyPairsTokens = 3;
 constexpr int kShortUnit = 64;        // mean length below which the streaming kernel takes its form for short units
 
 template <int D>

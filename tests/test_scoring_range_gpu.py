@@ -3,6 +3,7 @@ FMA pipe (column pairs 3 and 5 of a 32-column chunk) and on the special-function
 must be recomputed and the result must match."""
 import numpy as np
 import pytest
+import torch
 
 import paper_2502_01941_b200 as skv
 from paper_2502_01941_b200 import workloads as wl
@@ -80,4 +81,26 @@ def test_out_of_range_among_short_units(mean, d):
     gpu = P.gpu_prefill(ctx, P.dims_of(cfg), Q, K, V, off, cfg.r_p, 0, "fused")
     assert skv.shotkv_repaired_items(ctx) == cfg.Hkv
     P.check_all_units(gpu, Q, K, V, off, cfg.r_p, check_tokens=False)
+    ctx.close()
+
+
+@pytest.mark.parametrize("d,G,W", [(64, 3, 33), (128, 3, 33), (128, 5, 45), (64, 7, 9)], ids=["99_rows", "99_rows_d128", "225_rows", "63_rows"])
+def test_token_importance_of_wide_logits(d, G, W):
+    """Logits of a standard deviation of 400 beside rows that fill the operand up (the next unit's queries, so their logits are as
+    wide): those carry no weight.  In units of log2 a logit stays below 4,000, where fp32 resolves 2.4e-4; a few such
+    roundings in the dot product and in its reference make 1e-3 of a weight."""
+    ctx = skv.Context(0)
+    L, Hkv, N = 2, 2, 3000
+    g = torch.Generator(device="cuda").manual_seed(1)
+    Q = (20 * torch.randn(1, L, G * Hkv, W, d, generator=g, device="cuda")).bfloat16()
+    K = (20 * torch.randn(1, L, Hkv, N, d, generator=g, device="cuda")).bfloat16()
+    dims = skv.make_dims(1, L, G * Hkv, Hkv, d, N, W, 0)
+    imp = torch.zeros(1, L, Hkv, N, device="cuda")
+    ws = torch.empty(skv.shotkv_workspace_bytes(dims), dtype=torch.uint8, device="cuda")
+    skv.shotkv_prefill_score(ctx, dims, Q, K, imp, ws)
+    x = torch.einsum("blhgwd,blhnd->blhgwn", Q.double().view(1, L, Hkv, G, W, d), K.double()) / d ** 0.5
+    own = N - W + torch.arange(W, device="cuda")
+    want = x.masked_fill_(torch.arange(N, device="cuda") > own[:, None], float("-inf")).softmax(-1).sum((3, 4))
+    assert torch.isfinite(imp).all()
+    assert (imp.double() - want).norm() <= 1e-3 * want.norm()
     ctx.close()
