@@ -304,21 +304,23 @@ SHOTKV_API uint64_t shotkv_repaired_items(const shotkv_ctx* ctx);
 
 /* Failure detection.  The tensor-core kernels of this library (the scoring pass of Section 5.1's
  * prefill score equation and the per-token second pass) hand tiles between warps through shared-
- * memory barriers.  Every such wait is bounded: after `cycles` SM clock cycles (default 4e9, about
+ * memory barriers; the CTAs of a cluster in the reduction and the decode steps wait for one another's
+ * messages.  Every such wait is bounded: after `cycles` SM clock cycles (default 4e9, about
  * two seconds) the waiting warp gives up, raises its CTA's abort flag and a host-visible error
- * word, all roles leave their loops, copies in flight are waited for (bounded again), tensor
- * memory is released and the kernel returns.  The next call on the context then returns
+ * word, all roles leave their loops, copies and messages in flight are waited for (bounded again),
+ * tensor memory is released and the kernel returns.  The next call on the context then returns
  * SHOTKV_ERR_TIMEOUT once (the outputs of the call that gave up are invalid); the call after
- * that proceeds normally.  shotkv_set_wait_limit changes the limit for later launches of this
- * context (0 restores the default).  The CTAs of a cluster in the reduction and the decode steps wait for
- * one another's messages within a fixed limit of about two seconds, and report in the same way.  */
+ * that proceeds normally.  A decode state whose step gave up is invalid as a whole: initialise it again.
+ * shotkv_set_wait_limit changes the limit for later launches of this context (0 restores the default).  */
 SHOTKV_API int shotkv_set_wait_limit(shotkv_ctx* ctx, int64_t cycles);
 /* Runs the bounded-wait helpers on purpose into their limit, so that the give-up path can be
  * checked on any installation without disturbing a real kernel: one CTA, two barriers nobody
  * arrives on.  Warp 0 waits as the epilogue warps do, with `limit_cycles` (1e3..1e9); one thread
  * of warp 1 waits as the producer and MMA threads do, with four times that, and must leave early
  * because warp 0 raised the abort flag.  Tensor memory is allocated and released around it as in
- * the kernels' exit path.  Nothing faults and nothing spins past its limit.
+ * the kernels' exit path.  Then a cluster of two CTAs: one waits for two messages, the second of which comes
+ * after its limit, and must give up and still be there when that message lands; otherwise this call fails.
+ * Nothing faults and nothing spins past its limit.
  *   report host [4] = {warp 0's wait succeeded (0 expected), warp 1's wait succeeded (0 expected),
  *                      abort flag at exit (1 expected), cycles warp 1 waited (< 4*limit_cycles)}
  * This call SYNCHRONISES `stream`.  It leaves the error word raised exactly as a real give-up

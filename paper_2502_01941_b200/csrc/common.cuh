@@ -113,7 +113,6 @@ __device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {
 // (1.7 us of a step of 4 sequences x 1 layer).  expect_messages: by one thread, ahead of the cluster_arrive at the start;
 // nobody sends before a cluster_wait (a CTA's memory may be written once it has begun), and a CTA that has been sent
 // everything may end.
-constexpr long long kMessageCycles = 4000000000LL;     // limit of the wait for them: about two seconds
 __device__ __forceinline__ void expect_messages(unsigned long long* bar, int bytes) {
     const uint32_t b = smem_u32(bar);
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b) : "memory");
@@ -135,8 +134,9 @@ __device__ __forceinline__ void send(float4* to, int rank, unsigned long long* b
                  "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w), "r"(cluster_addr(bar, rank))
                  : "memory");
 }
-// Waits until all bytes expected are there; a wait that runs into its limit sets the error word.
-__device__ __forceinline__ void await_messages(unsigned long long* bar, int* err) {
+// Waits, `limit` cycles at most, until all bytes expected are there.  False: it gave up and has set the error word; what it
+// waited for may still come, so the thread passes outlive_messages before it ends.
+__device__ __forceinline__ bool await_messages(unsigned long long* bar, int* err, long long limit) {
     const uint32_t b = smem_u32(bar);
     const long long t0 = clock64();
     for (;;) {
@@ -148,12 +148,47 @@ __device__ __forceinline__ void await_messages(unsigned long long* bar, int* err
             : "=r"(done)
             : "r"(b)
             : "memory");
-        if (done) return;
-        if (clock64() - t0 > kMessageCycles) {
+        if (done) return true;
+        if (clock64() - t0 > limit) {
             atomicExch(err, 1);
-            return;
+            return false;
         }
     }
+}
+// For single threads whose wait gave up, at their end: keeps their CTA, whose memory the others write to, until all other threads of
+// the cluster have ended or are here too (every wait of theirs ends), and until what they sent has landed, if it does within the
+// limit.  `bar`, `more`: the barriers waited for in vain, or NULL.
+__device__ __forceinline__ void outlive_messages(unsigned long long* bar, unsigned long long* more, int* err, long long limit) {
+    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    if (bar) await_messages(bar, err, limit);
+    if (more) await_messages(more, err, limit);
+}
+
+// Self-test of that, for the host to run on demand: a cluster of two CTAs of one warp.  The first expects two words; the
+// second sends one at once and the other well after the limit, when the first has given up.  Lane 0 of the first waits on
+// behalf of its warp, as a thread of a cluster's CTA does.  report[0..1] = {that wait succeeded, the late word was there before the CTA ended}.
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(32) message_wait_selftest_kernel(long long limit, int* err, int* report) {
+    __shared__ __align__(8) unsigned long long arrived;
+    __shared__ float words[2];
+    const int lane = threadIdx.x;
+    if (lane == 0) {
+        words[0] = words[1] = 0.f;
+        if (blockIdx.x == 0) expect_messages(&arrived, 2 * (int)sizeof(float));
+    }
+    cluster_arrive();
+    cluster_wait();
+    if (lane != 0) return;
+    if (blockIdx.x != 0) {
+        send(words, 0, &arrived, 1.f);
+        for (const long long t0 = clock64(); clock64() - t0 < 4 * limit + 1000000;) __nanosleep(100);
+        send(words + 1, 0, &arrived, 2.f);
+        return;
+    }
+    const bool ok = await_messages(&arrived, err, limit);
+    report[0] = ok;
+    if (!ok) outlive_messages(&arrived, nullptr, err, limit);
+    report[1] = *(volatile float*)&words[0] == 1.f && *(volatile float*)&words[1] == 2.f;
 }
 
 __device__ __forceinline__ float warp_sum(float v) {

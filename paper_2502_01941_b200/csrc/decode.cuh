@@ -21,6 +21,7 @@ struct DecodeParams {
     const __nv_bfloat16* Vc;      // [U][Mcap][d]   (attention-output variant only)
     float* out;                   // [B][L][H][d]   (attention-output variant only)
     int* err;                     // error word (host-visible); set to 1 when a bounded wait gave up
+    long long wait_cycles;        // its limit
 };
 
 // The rest of a step for one (b, l): acc[j] += sum over kv heads of the entries' weights (fixed order,
@@ -235,12 +236,13 @@ __device__ __forceinline__ void fused_send(const FusedEnd& e, const DecodeFinish
 #pragma unroll 1
     for (int c = 0; c < receivers; ++c) send(to, c, e.arrived, w);
 }
-// All threads of all CTAs, once a CTA has sent its weights and made its other outputs.
+// All threads of all CTAs, once a CTA has sent its weights and made its other outputs.  False: the wait gave up,
+// and the end was made with whatever weights are there; every index stays in range, and the state is no longer a valid one anyhow.
 template <int D, int NT>
-__device__ __forceinline__ void fused_finish(const FusedEnd& e, const DecodeFinishParams& f, int bl, int c, int ctas, int* err) {
+__device__ __forceinline__ bool fused_finish(const FusedEnd& e, const DecodeFinishParams& f, int bl, int c, int ctas, const DecodeParams& p) {
     const bool evicts = f.k < f.n;
-    if (!evicts && c != 0) return;
-    await_messages(e.arrived, err);
+    if (!evicts && c != 0) return true;
+    const bool ok = await_messages(e.arrived, p.err, p.wait_cycles);
     const auto value = [&](int j) {
         float s = 0.f;
 #pragma unroll 1
@@ -256,6 +258,7 @@ __device__ __forceinline__ void fused_finish(const FusedEnd& e, const DecodeFini
             if (j == f.n - 1) f.born[(size_t)bl * f.Dcap + j] = f.T_old;
         }
     }
+    return ok;
 }
 
 __host__ __device__ constexpr size_t score_smem_bytes(int Dcap) { return ((size_t)8 * Dcap + 8 * 8 * 2 + kMaxSplit * 16 + 4) * 4; }
@@ -416,12 +419,13 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p,
         sred[warp * 8 + 2 * t4 + 1] = make_float2(m1, z1);
     }
     __syncthreads();
+    bool ok = true;
     if (SPLIT) {
         if (tid < 8 * nsplit) {                            // every CTA's rows to every CTA
             float fac[8];
             send(stab + rank * 8 + (tid & 7), first_cta + (tid >> 3), arrived, row_of_cta(sred, tid & 7, fac));
         }
-        await_messages(arrived, p.err);
+        ok = await_messages(arrived, p.err, p.wait_cycles);
     }
     float rm, riz;                                         // of row lane / 4, over all keys of the unit
     row_of_unit(SPLIT ? stab : sred, SPLIT ? nsplit : 8, rm, riz);
@@ -434,7 +438,8 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p,
             if (FUSED && entry) fused_send(end, f, hk, j, s, ctas);
             else if (entry) p.partial[(size_t)u * p.Dcap + j] = s;
         }
-        if (FUSED) fused_finish<D, 256>(end, f, bl, first_cta + rank, ctas, p.err);
+        const bool all = !FUSED || fused_finish<D, 256>(end, f, bl, first_cta + rank, ctas, p);
+        if (!(ok && all)) outlive_messages(ok ? nullptr : arrived, all ? nullptr : end.arrived, p.err, p.wait_cycles);
     } else {
         for (int j0 = warp * 32; j0 < n; j0 += 256) {
             const float s = entry_weight(sdec, p.Dcap, p.G, j0 + lane, j0 + lane < n, rm, riz);
@@ -773,7 +778,7 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
             d[3] = o.w * iz;
         }
     }
-    if (p.nsplit > 1) await_messages(arrived, p.err);
+    const bool ok = p.nsplit <= 1 || await_messages(arrived, p.err, p.wait_cycles);
     float rm, riz;                                           // of row lane / 4, over all keys of the unit
     row_of_unit(p.nsplit > 1 ? stab : sred, p.nsplit > 1 ? p.nsplit : NW, rm, riz);
     const float rmu = rm == SHOTKV_NEG_INF ? 0.f : rm;
@@ -812,7 +817,8 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
         if (FUSED && entry) fused_send(end, f, hk, j, s, ctas);
         else if (entry) p.partial[(size_t)u * p.Dcap + j] = s;
     }
-    if (FUSED) fused_finish<D, NT>(end, f, bl, first_cta + rank, ctas, p.err);
+    const bool all = !FUSED || fused_finish<D, NT>(end, f, bl, first_cta + rank, ctas, p);
+    if (!(ok && all)) outlive_messages(ok ? nullptr : arrived, all ? nullptr : end.arrived, p.err, p.wait_cycles);
 }
 
 }  // namespace shotkv

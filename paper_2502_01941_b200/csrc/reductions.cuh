@@ -129,7 +129,8 @@ __host__ __device__ constexpr size_t reduce_smem_bytes(int Rpad, int P, int S, i
 template <int ROWS>
 __global__ void __launch_bounds__(kReduceThreads, ROWS == 128 ? 4 : 3) reduce_select_kernel(const PartialView v, const __grid_constant__ ShotTable tab,
                                                                       int R, int Hkv, int ranks,
-                                                                      float* __restrict__ shot_scores, const SelectArgs a, int* err) {
+                                                                      float* __restrict__ shot_scores, const SelectArgs a, int* err,
+                                                                      long long wait_cycles) {
     constexpr int NW = kReduceThreads / 32, NH = ROWS / 128, PARTS = kReduceThreads / ROWS;
     constexpr int AHEAD = 4, FIRST = 4;       // pieces whose z a warp has in flight; items whose statistics a thread has
     constexpr unsigned char kNoItem = 255;
@@ -306,6 +307,7 @@ __global__ void __launch_bounds__(kReduceThreads, ROWS == 128 ? 4 : 3) reduce_se
         }
         if (h + ranks < Hkv) __syncthreads();
     }
+    bool ok = true;
     if (ranks > 1) {
         cluster_wait();                            // all CTAs have begun
         if (rank != 0) {
@@ -313,7 +315,7 @@ __global__ void __launch_bounds__(kReduceThreads, ROWS == 128 ? 4 : 3) reduce_se
             for (int i = tid; i < S; i += kReduceThreads) send(mass + i, 0, &arrived, mass[i]);
             return;
         }
-        await_messages(&arrived, err);
+        ok = await_messages(&arrived, err, wait_cycles);   // if not, the selection is one of whatever masses are there
     }
     float* scores = shot_scores + (size_t)bl * S;
     __syncthreads();                               // the selection takes the place of the work area
@@ -326,6 +328,7 @@ __global__ void __launch_bounds__(kReduceThreads, ROWS == 128 ? 4 : 3) reduce_se
         scores[i] = s;
         return s;
     });
+    if (!ok) outlive_messages(&arrived, nullptr, err, wait_cycles);
 }
 
 // Score(s_i) from per-token importance.  Latency-bound while the importances come from L2, so what counts is how

@@ -402,7 +402,7 @@ int set_device(shotkv_ctx* ctx) {
     CUDA_TRY(ctx, cudaSetDevice(ctx->device));
     if (ctx->err_host && *(volatile int*)ctx->err_host) {
         *(volatile int*)ctx->err_host = 0;
-        return fail(ctx, SHOTKV_ERR_TIMEOUT, "an earlier scoring kernel gave up a bounded wait; its outputs are invalid");
+        return fail(ctx, SHOTKV_ERR_TIMEOUT, "an earlier kernel gave up a bounded wait; its outputs are invalid");
     }
     return SHOTKV_OK;
 }
@@ -704,7 +704,7 @@ int run_reduce_select_t(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView
     const size_t smem = reduce_smem_bytes(ROWS, pv.P, d->S, pv.nchunk, ranks);
     if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "too many shots for the single-pass path (S = %d)", d->S);
     return launch(ctx, reduce_select_kernel<ROWS>, dim3(d->B * d->L * ranks), kReduceThreads, smem, stream, ranks, kEarly, pv, tab,
-                  (d->H / d->Hkv) * d->W, (int)d->Hkv, ranks, shot_scores, sa, ctx->err_dev);
+                  (d->H / d->Hkv) * d->W, (int)d->Hkv, ranks, shot_scores, sa, ctx->err_dev, ctx->wait_cycles);
 }
 int run_reduce_select(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView& pv, const ShotTable& tab, float* shot_scores,
                       const SelectArgs& sa, cudaStream_t stream) {
@@ -844,7 +844,7 @@ int shotkv_create(shotkv_ctx** out, int device) {
         return SHOTKV_ERR_CUDA;
     }
     for (int i = 0; i < kErrWords; ++i) ctx->err_host[i] = 0;   // word 0: a bounded wait gave up; word 1: work items
-                                                                 // recomputed with a running maximum; words 2-5: self-test report
+                                                                 // recomputed with a running maximum; words 2-7: self-test reports
     ctx->sm_count = prop.multiProcessorCount;
     ctx->encode_tiled = resolve_encode_tiled();
     if (set_kernel_attributes() != cudaSuccess || ask_decode_room(ctx) != cudaSuccess) {
@@ -1392,6 +1392,7 @@ int decode_step_impl(shotkv_ctx* ctx, shotkv_decode_state* st, const shotkv_bf16
     p.scale_log2 = kLog2e / sqrtf((float)d.d);
     p.Vc = (const __nv_bfloat16*)Vc; p.out = attn_out;
     p.err = ctx->err_dev;
+    p.wait_cycles = ctx->wait_cycles;
     DecodeFinishParams f{};
     f.partial = p.partial; f.acc = st->acc; f.born = st->born; f.Kd = p.Kd; f.Vd = p.Vd;
     f.Hkv = d.Hkv; f.Dcap = st->Dcap; f.n = st->n_dec + 1; f.T_old = st->T;
@@ -1498,11 +1499,16 @@ int shotkv_selftest_bounded_wait(shotkv_ctx* ctx, int64_t limit_cycles, int32_t*
     if (limit_cycles < 1000 || limit_cycles > 1000000000LL)
         return fail(ctx, SHOTKV_ERR_INVALID_ARG, "self-test limit must be between 1e3 and 1e9 cycles");
     cudaStream_t stream = (cudaStream_t)stream_;
-    for (int i = 0; i < 4; ++i) ((volatile int*)ctx->err_host)[2 + i] = -1;
+    volatile int* words = ctx->err_host + 2;
+    for (int i = 0; i < 6; ++i) words[i] = -1;
     bounded_wait_selftest_kernel<<<1, 64, 0, stream>>>((long long)limit_cycles, ctx->err_dev, ctx->err_dev + 2);
     LAUNCH_CHECK(ctx);
+    message_wait_selftest_kernel<<<2, 32, 0, stream>>>((long long)limit_cycles, ctx->err_dev, ctx->err_dev + 6);
+    LAUNCH_CHECK(ctx);
     CUDA_TRY(ctx, cudaStreamSynchronize(stream));
-    for (int i = 0; i < 4; ++i) report[i] = ((volatile int*)ctx->err_host)[2 + i];
+    for (int i = 0; i < 4; ++i) report[i] = words[i];
+    if (words[4] != 0 || words[5] != 1)
+        return fail(ctx, SHOTKV_ERR_CUDA, "the wait for messages did not give up as it should (succeeded %d, outlived its sender %d)", words[4], words[5]);
     return SHOTKV_OK;
 }
 

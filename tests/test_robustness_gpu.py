@@ -12,6 +12,7 @@ import paper_2502_01941_b200 as skv
 from oracle import shotkv_oracle as O
 from paper_2502_01941_b200 import workloads as wl
 import parity as P
+from test_decode_gpu import lockstep
 
 pytestmark = pytest.mark.gpu
 
@@ -62,6 +63,25 @@ def test_bounded_wait_gives_up_and_the_context_recovers(ctx):
     with pytest.raises(skv.ShotKVError):
         skv.shotkv_profile_enable(ctx, False)
     assert _prefill_ok(ctx) == 0
+
+
+def test_message_wait_gives_up_and_outlives_its_sender(ctx):
+    """The self-test's second kernel: a cluster whose first CTA waits for a message that comes after the limit.  The call
+    fails unless that wait gave up and the CTA was still there when the message landed."""
+    before = skv.shotkv_launch_count(ctx)
+    t0 = torch.cuda.Event(enable_timing=True); t1 = torch.cuda.Event(enable_timing=True)
+    for limit in (1_000, 200_000, 5_000_000):
+        t0.record()
+        skv.shotkv_selftest_bounded_wait(ctx, limit)
+        t1.record(); torch.cuda.synchronize()
+        assert t0.elapsed_time(t1) < 100.0, "the self-test took far longer than its limit"
+        with pytest.raises(skv.ShotKVError) as e:
+            skv.shotkv_profile_enable(ctx, False)
+        assert e.value.code == skv.ERR_TIMEOUT
+    assert skv.shotkv_launch_count(ctx) - before == 6          # both kernels, three times
+    cfg = wl.DecodeConfig("after", B=1, L=1, H=8, Hkv=2, d=128, steps=6, r_d=0.5, recompress_every=4, cfg_id=78)
+    for attend in (False, True):                              # clusters that wait for messages work on
+        assert lockstep(ctx, cfg, 2048, [(0, 0)], attend=attend) <= 1
 
 
 def test_selftest_rejects_limits_outside_its_range(ctx):
