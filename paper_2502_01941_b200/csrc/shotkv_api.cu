@@ -54,6 +54,24 @@ struct TraceRange {
     TraceRange& operator=(const TraceRange&) = delete;
 };
 
+// Clusters of n decode CTAs that the device runs at a time, by what a CTA takes of shared memory: four, three, two and one of them
+// fit an SM.  (As one figure, for three, 16 units of 3,276 keys with the attention output and room for 750 decode entries took 13.1 us a step,
+// 32 units 16.0: one figure put more CTAs to a unit than run at the same time.)
+constexpr int kRoomClasses = 4;
+constexpr size_t kRoomSmem[kRoomClasses] = {56 * 1024, 75 * 1024, 113 * 1024, kBigSmem};
+struct DecodeRoom {
+    int clusters[kRoomClasses][kMaxSplit + 1];
+    DecodeRoom() {
+        for (auto& of_class : clusters)
+            for (int& n : of_class) n = 0x7fffffff;
+    }
+    const int* with(size_t smem) const {
+        int c = 0;
+        while (c < kRoomClasses - 1 && smem > kRoomSmem[c]) ++c;
+        return clusters[c];
+    }
+};
+
 }  // namespace
 
 struct shotkv_ctx {
@@ -89,8 +107,7 @@ struct shotkv_ctx {
     long long wait_cycles = tc::kWaitCycles;   // limit of every bounded device-side wait
     int32_t* static_offsets = nullptr;         // device address of the built-in boundary table (looked up on first use)
     void* encode_tiled = nullptr;              // cuTensorMapEncodeTiled, resolved at creation
-    int room_attend[2][kMaxSplit + 1] = {};    // clusters of n CTAs the device runs at a time, d = 64 and 128 (asked at creation)
-    int room_score[2][kMaxSplit + 1] = {};
+    DecodeRoom room_attend[2], room_score[2];  // d = 64 and 128 (asked at creation)
 };
 
 namespace {
@@ -772,33 +789,46 @@ cudaError_t set_kernel_attributes() {
     return e;
 }
 
-// How many clusters of n decode CTAs the device runs at the same time, with decode regions of kRoomRows rows
-// (larger ones take more shared memory; the figure then is an estimate that costs a second wave at worst).
-constexpr int kRoomRows = 320, kRoomGroup = 4;
+// How many clusters of n decode CTAs the device runs at the same time: for every class of shared memory the smaller of the
+// figures of the kernel that ends a step and of the one that does not.  More than eight CTAs are not every device's, nor every
+// part of one: where it has no room for such a cluster, or does not know it, the figure is 0 and none is launched.
 template <class K>
-cudaError_t ask_room(K* kernel, int threads, size_t smem, int* room) {
-    for (int n = 2; n <= kMaxSplit; ++n) {
-        cudaLaunchAttribute at[1] = {};
-        at[0].id = cudaLaunchAttributeClusterDimension;
-        at[0].val.clusterDim.x = n;
-        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-        cudaLaunchConfig_t lc{};
-        lc.gridDim = dim3(n * 1024);
-        lc.blockDim = dim3(threads);
-        lc.dynamicSmemBytes = smem;
-        lc.attrs = at;
-        lc.numAttrs = 1;
-        const cudaError_t e = cudaOccupancyMaxActiveClusters(&room[n], kernel, &lc);
-        if (e != cudaSuccess) return e;
-    }
+cudaError_t ask_room(K* kernel, int threads, DecodeRoom& room) {
+    for (int c = 0; c < kRoomClasses; ++c)
+        for (int n = 2; n <= kMaxSplit; ++n) {
+            cudaLaunchAttribute at[1] = {};
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = n;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            cudaLaunchConfig_t lc{};
+            lc.gridDim = dim3(n * 1024);
+            lc.blockDim = dim3(threads);
+            lc.dynamicSmemBytes = kRoomSmem[c];
+            lc.attrs = at;
+            lc.numAttrs = 1;
+            int clusters = 0;
+            const cudaError_t e = cudaOccupancyMaxActiveClusters(&clusters, kernel, &lc);
+            if (e != cudaSuccess) {
+                if (n <= 8) return e;
+                cudaGetLastError();
+                clusters = 0;
+            }
+            if (clusters < room.clusters[c][n]) room.clusters[c][n] = clusters;
+        }
     return cudaSuccess;
 }
-cudaError_t ask_decode_room(shotkv_ctx* ctx) {
-    cudaError_t e = ask_room(decode_attend_kernel<64, false>, AttendCfg<64>::kWarps * 32, attend_smem_bytes<64>(kRoomGroup, kRoomRows, kMaxSplit), ctx->room_attend[0]);
-    if (e == cudaSuccess) e = ask_room(decode_attend_kernel<128, false>, AttendCfg<128>::kWarps * 32, attend_smem_bytes<128>(kRoomGroup, kRoomRows, kMaxSplit), ctx->room_attend[1]);
-    if (e == cudaSuccess) e = ask_room(decode_score_kernel<64, true, false>, 256, score_smem_bytes(kRoomRows), ctx->room_score[0]);
-    if (e == cudaSuccess) e = ask_room(decode_score_kernel<128, true, false>, 256, score_smem_bytes(kRoomRows), ctx->room_score[1]);
+template <int D>
+cudaError_t ask_decode_room_t(shotkv_ctx* ctx) {
+    DecodeRoom &attend = ctx->room_attend[D == 128], &score = ctx->room_score[D == 128];
+    cudaError_t e = ask_room(decode_attend_kernel<D, false>, AttendCfg<D>::kWarps * 32, attend);
+    if (e == cudaSuccess) e = ask_room(decode_attend_kernel<D, true>, AttendCfg<D>::kWarps * 32, attend);
+    if (e == cudaSuccess) e = ask_room(decode_score_kernel<D, true, false>, 256, score);
+    if (e == cudaSuccess) e = ask_room(decode_score_kernel<D, true, true>, 256, score);
     return e;
+}
+cudaError_t ask_decode_room(shotkv_ctx* ctx) {
+    const cudaError_t e = ask_decode_room_t<64>(ctx);
+    return e == cudaSuccess ? ask_decode_room_t<128>(ctx) : e;
 }
 
 }  // namespace
@@ -1306,16 +1336,17 @@ int shotkv_decode_init(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv_po
 
 namespace {
 
-// CTAs that share a unit's keys: as many as still run at the same time for all units (`room[n]` clusters of
-// n CTAs do: a cluster stays within a group of SMs, so it is fewer than the SMs' slots / n) and leave every
+// CTAs that share a unit's keys: as many as still run at the same time for all units (as clusters of n CTAs with
+// `smem(n)` bytes each: a cluster stays within a group of SMs, so it is fewer than the SMs' slots / n) and leave every
 // warp at least `least` sixths of a block of 16 keys.  The fused step gains from more CTAs down to little more than a block a
 // warp, whose chain is long (2 heads of 333 keys 6.5 -> 5.4 us a step with 4/3 of a block instead of 2, 185 keys 8.5 -> 7.1; 1 block:
 // 8 heads of 1,150 keys 7.0 -> 7.3).  Scores alone take less per block than a larger cluster costs (8 heads of 3,400 keys 5.3 us with 2.5
 // blocks, 6.1 with 2, 5.7 with 3).
 constexpr int kLeastAttend = 8, kLeastScore = 15;
-int decode_split(const int* room, long long U, long long keys, int warps, int least) {
+template <class Smem>
+int decode_split(const DecodeRoom& room, Smem&& smem, long long U, long long keys, int warps, int least) {
     int n = kMaxSplit;
-    while (n > 1 && (U > room[n] || keys * 6 < (long long)n * warps * 16 * least)) --n;
+    while (n > 1 && (U > room.with(smem(n))[n] || keys * 6 < (long long)n * warps * 16 * least)) --n;
     return n;
 }
 
@@ -1346,11 +1377,12 @@ bool ends_fused(const shotkv_ctx* ctx, const int* room, const DecodeParams& p, c
 template <int D>
 int launch_decode_attend(shotkv_ctx* ctx, DecodeParams& p, const DecodeFinishParams& f, int U, bool& ended, cudaStream_t stream) {
     using Cfg = AttendCfg<D>;
-    const int* room = ctx->room_attend[D == 128];
-    p.nsplit = decode_split(room, U, (long long)p.Mcap + p.n_old + 1, Cfg::kWarps, kLeastAttend);
-    size_t smem = attend_smem_bytes<D>(p.G, p.Dcap, p.nsplit);
+    const DecodeRoom& room = ctx->room_attend[D == 128];
+    const auto smem_of = [&](int n) { return attend_smem_bytes<D>(p.G, p.Dcap, n); };
+    p.nsplit = decode_split(room, smem_of, U, (long long)p.Mcap + p.n_old + 1, Cfg::kWarps, kLeastAttend);
+    size_t smem = smem_of(p.nsplit);
     const size_t end = fused_end_smem_bytes(p.Hkv, f.n, f.k < f.n);
-    ended = ends_fused(ctx, room, p, f, U, Cfg::kWarps * 32) && smem + end <= kBigSmem;
+    ended = smem + end <= kBigSmem && ends_fused(ctx, room.with(smem + end), p, f, U, Cfg::kWarps * 32);
     if (ended)
         return launch(ctx, decode_attend_kernel<D, true>, dim3(U * p.nsplit), Cfg::kWarps * 32, smem + end, stream, p.Hkv * p.nsplit, kEarly, p, f);
     if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "Dcap too large for the attention-output step");
@@ -1359,10 +1391,10 @@ int launch_decode_attend(shotkv_ctx* ctx, DecodeParams& p, const DecodeFinishPar
 }
 template <int D>
 int launch_decode_score(shotkv_ctx* ctx, DecodeParams& p, const DecodeFinishParams& f, int U, bool& ended, cudaStream_t stream) {
-    const int* room = ctx->room_score[D == 128];
-    p.nsplit = decode_split(room, U, (long long)p.Mcap + p.n_old + 1, 8, kLeastScore);
+    const DecodeRoom& room = ctx->room_score[D == 128];
     const size_t smem = score_smem_bytes(p.Dcap), end = fused_end_smem_bytes(p.Hkv, f.n, f.k < f.n);
-    ended = ends_fused(ctx, room, p, f, U, 256) && smem + end <= kBigSmem;
+    p.nsplit = decode_split(room, [&](int) { return smem; }, U, (long long)p.Mcap + p.n_old + 1, 8, kLeastScore);
+    ended = smem + end <= kBigSmem && ends_fused(ctx, room.with(smem + end), p, f, U, 256);
     if (ended) return launch(ctx, decode_score_kernel<D, true, true>, dim3(U * p.nsplit), 256, smem + end, stream, p.Hkv * p.nsplit, kEarly, p, f);
     return p.nsplit > 1 ? launch(ctx, decode_score_kernel<D, true, false>, dim3(U * p.nsplit), 256, smem, stream, p.nsplit, kEarly, p, f)
                         : launch(ctx, decode_score_kernel<D, false, false>, dim3(U), 256, smem, stream, 1, kEarly, p, f);

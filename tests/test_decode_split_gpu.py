@@ -78,3 +78,14 @@ def test_whole_units_two_to_an_sm(ctx, L):
     """More units than SMs and at most two to an SM, an eviction among the steps."""
     cfg = wl.DecodeConfig("pairs", B=1, L=L, H=32, Hkv=8, d=128, steps=9, r_d=0.5, recompress_every=4, cfg_id=75)
     assert lockstep(ctx, cfg, 300, [(0, 0), (0, L - 1)], attend=True) <= 1
+
+
+@pytest.mark.parametrize("L,Hkv,G,d,M,Dcap", [(1, 1, 8, 128, 6000, 4096), (1, 2, 8, 128, 3000, 1500), (2, 8, 4, 128, 3276, 750), (1, 16, 1, 64, 60, 4096),
+                                              (1, 16, 8, 128, 40, 2100)])
+def test_clusters_of_ctas_that_take_much_memory(ctx, L, Hkv, G, d, M, Dcap):
+    """Decode regions of which two or one fit an SM: units shared by up to sixteen CTAs, and steps of sixteen heads that end in
+    their first kernel."""
+    cfg = wl.DecodeConfig("room", B=1, L=L, H=Hkv * G, Hkv=Hkv, d=d, steps=2 * (Dcap - 4), r_d=0.5, recompress_every=4, cfg_id=79)
+    assert cfg.Dcap == Dcap
+    for attend in (False, True):
+        assert lockstep(ctx, cfg, M, [(0, 0)], np.full((1, L), M, np.int32), steps=5, attend=attend) <= 1
