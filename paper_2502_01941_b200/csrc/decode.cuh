@@ -261,7 +261,7 @@ __device__ __forceinline__ bool fused_finish(const FusedEnd& e, const DecodeFini
     return ok;
 }
 
-__host__ __device__ constexpr size_t score_smem_bytes(int Dcap) { return ((size_t)8 * Dcap + 8 * 8 * 2 + kMaxSplit * 16 + 4) * 4; }
+__host__ __device__ constexpr size_t score_smem_bytes(int Dcap, bool split) { return ((size_t)8 * Dcap + 8 * 8 * 2 + (split ? kMaxSplit * 16 + 4 : 0)) * 4; }
 
 // One CTA, or a cluster of p.nsplit, per (sequence, layer, kv head).  Each warp takes 16 keys at a
 // time straight from global memory: thread (g, t) of a warp reads 16 contiguous bytes of key rows g
@@ -271,11 +271,12 @@ __host__ __device__ constexpr size_t score_smem_bytes(int Dcap) { return ((size_
 // (kept prefill keys + decode keys) are known.
 // A shared unit leaves few warps to an SM, so each asks for its next block before it computes this one.
 // SPLIT = false is the same for whole units, nsplit = 1: with the stride of the loop a constant it is
-// unrolled and more loads are in flight, to the depth that is written down here (left to itself the compiler
-// chose 1 to 4 by what stood around the loop: 8 sequences x 32 layers 301 to 259 us a step, 1 sequence 56 to 43; four
-// deep 255 and 39.5).
+// unrolled DEPTH times and more loads are in flight (left to itself the compiler chose 1 to 4 by what stood around the
+// loop: 8 sequences x 32 layers 301 to 259 us a step, 1 sequence 56 to 43; two or four deep 255 and 39.5).  Four deep takes
+// the registers of a CTA on the SM: three there instead of four with d = 128, four instead of five with d = 64.
 // FUSED (with SPLIT): the cluster is all CTAs of a (sequence, layer), and the step ends here.
-template <int D, bool SPLIT, bool FUSED>
+constexpr int kDeep = 4, kShallow = 2;
+template <int D, bool SPLIT, bool FUSED, int DEPTH>
 __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p, const DecodeFinishParams f) {
     constexpr int NB = D / 32;     // 32-dim blocks
     constexpr int VPR = D / 8;     // 16-byte vectors per row
@@ -292,7 +293,7 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p,
     const int bl = u / p.Hkv, hk = u - bl * p.Hkv;
     const int first_cta = FUSED ? hk * nsplit : 0, ctas = p.Hkv * nsplit;    // in the cluster: the unit's first; FUSED: all
     FusedEnd end{};
-    if (FUSED) end = fused_end_at(dsm + score_smem_bytes(p.Dcap), f);
+    if (FUSED) end = fused_end_at(dsm + score_smem_bytes(p.Dcap, true), f);
     if (SPLIT) {
         if (tid == 0) {
             expect_messages(arrived, nsplit * 8 * (int)sizeof(float2));
@@ -351,7 +352,7 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p,
     float m0 = SHOTKV_NEG_INF, m1 = SHOTKV_NEG_INF, z0 = 0.f, z1 = 0.f;   // query rows 2*t4, 2*t4+1
     const int first = (rank * 8 + warp) * 16;
     if (SPLIT && first < Ktot) load(first, n_lo, n_hi);
-#pragma unroll 4
+#pragma unroll DEPTH
     for (int base = first; base < Ktot; base += nsplit * 8 * 16) {
         const int ia = base + g, ib = base + g + 8;
         const bool va = ia < Ktot, vb = ib < Ktot;

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -60,11 +61,7 @@ struct TraceRange {
 constexpr int kRoomClasses = 4;
 constexpr size_t kRoomSmem[kRoomClasses] = {56 * 1024, 75 * 1024, 113 * 1024, kBigSmem};
 struct DecodeRoom {
-    int clusters[kRoomClasses][kMaxSplit + 1];
-    DecodeRoom() {
-        for (auto& of_class : clusters)
-            for (int& n : of_class) n = 0x7fffffff;
-    }
+    int clusters[kRoomClasses][kMaxSplit + 1] = {};
     const int* with(size_t smem) const {
         int c = 0;
         while (c < kRoomClasses - 1 && smem > kRoomSmem[c]) ++c;
@@ -107,7 +104,9 @@ struct shotkv_ctx {
     long long wait_cycles = tc::kWaitCycles;   // limit of every bounded device-side wait
     int32_t* static_offsets = nullptr;         // device address of the built-in boundary table (looked up on first use)
     void* encode_tiled = nullptr;              // cuTensorMapEncodeTiled, resolved at creation
-    DecodeRoom room_attend[2], room_score[2];  // d = 64 and 128 (asked at creation)
+    // [d = 128][the step ends in its first kernel], and [0][2] of shared units scored two blocks of keys deep (asked at creation)
+    DecodeRoom room_attend[2][2], room_score[2][3];
+    int whole_score[2][2] = {};                // CTAs that have a unit each and fit an SM, two and four blocks of keys deep
 };
 
 namespace {
@@ -771,26 +770,30 @@ cudaError_t set_kernel_attributes() {
     if (e == cudaSuccess) e = set_tc_attributes<64, 2>();
     const void* small[] = {(const void*)select_shots_kernel<kSelectThreads>, (const void*)select_shots_kernel<kSortThreads>,
                            (const void*)reduce_select_kernel<128>, (const void*)reduce_select_kernel<256>,
-                           (const void*)decode_score_kernel<128, true, false>, (const void*)decode_score_kernel<128, true, true>, (const void*)decode_score_kernel<64, true, false>, (const void*)decode_score_kernel<64, true, true>,
-                           (const void*)decode_score_kernel<128, false, false>, (const void*)decode_score_kernel<64, false, false>,
-                           (const void*)decode_attend_kernel<128, false>, (const void*)decode_attend_kernel<128, true>, (const void*)decode_attend_kernel<64, false>, (const void*)decode_attend_kernel<64, true>,
+                           (const void*)decode_score_kernel<128, false, false, kDeep>, (const void*)decode_score_kernel<64, false, false, kDeep>,
+                           (const void*)decode_score_kernel<128, false, false, kShallow>, (const void*)decode_score_kernel<64, false, false, kShallow>,
                            (const void*)decode_evict_kernel<128>, (const void*)decode_evict_kernel<64>};
     for (const void* f : small)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kBigSmem);
     // a decode unit may be shared by more CTAs than the eight that every device's clusters allow
-    const void* split[] = {(const void*)decode_attend_kernel<128, false>, (const void*)decode_attend_kernel<128, true>, (const void*)decode_attend_kernel<64, false>, (const void*)decode_attend_kernel<64, true>,
-                           (const void*)decode_score_kernel<128, true, false>, (const void*)decode_score_kernel<128, true, true>, (const void*)decode_score_kernel<64, true, false>, (const void*)decode_score_kernel<64, true, true>};
-    for (const void* f : split)
+    const void* attend[] = {(const void*)decode_attend_kernel<128, false>, (const void*)decode_attend_kernel<128, true>,
+                            (const void*)decode_attend_kernel<64, false>, (const void*)decode_attend_kernel<64, true>};
+    const void* score[] = {(const void*)decode_score_kernel<128, true, false, kDeep>, (const void*)decode_score_kernel<128, true, true, kDeep>,
+                           (const void*)decode_score_kernel<64, true, false, kDeep>, (const void*)decode_score_kernel<64, true, true, kDeep>,
+                           (const void*)decode_score_kernel<64, true, false, kShallow>};
+    const auto in_clusters = [&](const void* f) {
+        if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kBigSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    };
+    for (const void* f : attend) in_clusters(f);
+    for (const void* f : score) in_clusters(f);
     // the fused decode step wants three CTAs of ~74 KB each on an SM: ask for the largest shared-memory carve-out
-    const void* wide[] = {(const void*)decode_attend_kernel<128, false>, (const void*)decode_attend_kernel<128, true>, (const void*)decode_attend_kernel<64, false>, (const void*)decode_attend_kernel<64, true>};
-    for (const void* f : wide)
+    for (const void* f : attend)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
     return e;
 }
 
-// How many clusters of n decode CTAs the device runs at the same time: for every class of shared memory the smaller of the
-// figures of the kernel that ends a step and of the one that does not.  More than eight CTAs are not every device's, nor every
+// How many clusters of n decode CTAs the device runs at the same time: for every class of shared memory.  More than eight CTAs are not every device's, nor every
 // part of one: where it has no room for such a cluster, or does not know it, the figure is 0 and none is launched.
 template <class K>
 cudaError_t ask_room(K* kernel, int threads, DecodeRoom& room) {
@@ -813,17 +816,21 @@ cudaError_t ask_room(K* kernel, int threads, DecodeRoom& room) {
                 cudaGetLastError();
                 clusters = 0;
             }
-            if (clusters < room.clusters[c][n]) room.clusters[c][n] = clusters;
+            room.clusters[c][n] = clusters;
         }
     return cudaSuccess;
 }
 template <int D>
 cudaError_t ask_decode_room_t(shotkv_ctx* ctx) {
-    DecodeRoom &attend = ctx->room_attend[D == 128], &score = ctx->room_score[D == 128];
-    cudaError_t e = ask_room(decode_attend_kernel<D, false>, AttendCfg<D>::kWarps * 32, attend);
-    if (e == cudaSuccess) e = ask_room(decode_attend_kernel<D, true>, AttendCfg<D>::kWarps * 32, attend);
-    if (e == cudaSuccess) e = ask_room(decode_score_kernel<D, true, false>, 256, score);
-    if (e == cudaSuccess) e = ask_room(decode_score_kernel<D, true, true>, 256, score);
+    DecodeRoom *attend = ctx->room_attend[D == 128], *score = ctx->room_score[D == 128];
+    cudaError_t e = ask_room(decode_attend_kernel<D, false>, AttendCfg<D>::kWarps * 32, attend[0]);
+    if (e == cudaSuccess) e = ask_room(decode_attend_kernel<D, true>, AttendCfg<D>::kWarps * 32, attend[1]);
+    if (e == cudaSuccess) e = ask_room(decode_score_kernel<D, true, false, kDeep>, 256, score[0]);
+    if (e == cudaSuccess) e = ask_room(decode_score_kernel<D, true, true, kDeep>, 256, score[1]);
+    if (e == cudaSuccess && D == 64) e = ask_room(decode_score_kernel<64, true, false, kShallow>, 256, score[2]);
+    int* whole = ctx->whole_score[D == 128];
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&whole[0], decode_score_kernel<D, false, false, kShallow>, 256, 0);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&whole[1], decode_score_kernel<D, false, false, kDeep>, 256, 0);
     return e;
 }
 cudaError_t ask_decode_room(shotkv_ctx* ctx) {
@@ -1341,7 +1348,9 @@ namespace {
 // warp at least `least` sixths of a block of 16 keys.  The fused step gains from more CTAs down to little more than a block a
 // warp, whose chain is long (2 heads of 333 keys 6.5 -> 5.4 us a step with 4/3 of a block instead of 2, 185 keys 8.5 -> 7.1; 1 block:
 // 8 heads of 1,150 keys 7.0 -> 7.3).  Scores alone take less per block than a larger cluster costs (8 heads of 3,400 keys 5.3 us with 2.5
-// blocks, 6.1 with 2, 5.7 with 3).
+// blocks, 6.1 with 2, 5.7 with 3).  Shared units are scored four blocks deep, the better by 1 to 15 % where both forms fit; with d = 64
+// that takes registers of a fourth CTA on the SM, and long units it leaves whole, but two deep does not, go two deep (256 units of 3,400 keys
+// 28.9 -> 20.7 us; of 1,150 keys whole 19.1, two deep 19.7).
 constexpr int kLeastAttend = 8, kLeastScore = 15;
 template <class Smem>
 int decode_split(const DecodeRoom& room, Smem&& smem, long long U, long long keys, int warps, int least) {
@@ -1377,27 +1386,43 @@ bool ends_fused(const shotkv_ctx* ctx, const int* room, const DecodeParams& p, c
 template <int D>
 int launch_decode_attend(shotkv_ctx* ctx, DecodeParams& p, const DecodeFinishParams& f, int U, bool& ended, cudaStream_t stream) {
     using Cfg = AttendCfg<D>;
-    const DecodeRoom& room = ctx->room_attend[D == 128];
+    const DecodeRoom* room = ctx->room_attend[D == 128];
     const auto smem_of = [&](int n) { return attend_smem_bytes<D>(p.G, p.Dcap, n); };
-    p.nsplit = decode_split(room, smem_of, U, (long long)p.Mcap + p.n_old + 1, Cfg::kWarps, kLeastAttend);
+    p.nsplit = decode_split(room[0], smem_of, U, (long long)p.Mcap + p.n_old + 1, Cfg::kWarps, kLeastAttend);
     size_t smem = smem_of(p.nsplit);
     const size_t end = fused_end_smem_bytes(p.Hkv, f.n, f.k < f.n);
-    ended = smem + end <= kBigSmem && ends_fused(ctx, room.with(smem + end), p, f, U, Cfg::kWarps * 32);
+    ended = smem + end <= kBigSmem && ends_fused(ctx, room[1].with(smem + end), p, f, U, Cfg::kWarps * 32);
     if (ended)
         return launch(ctx, decode_attend_kernel<D, true>, dim3(U * p.nsplit), Cfg::kWarps * 32, smem + end, stream, p.Hkv * p.nsplit, kEarly, p, f);
     if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "Dcap too large for the attention-output step");
     if (two_to_an_sm(ctx, p, U) && smem < kNoThirdCta) smem = kNoThirdCta;
     return launch(ctx, decode_attend_kernel<D, false>, dim3(U * p.nsplit), Cfg::kWarps * 32, smem, stream, p.nsplit, kEarly, p, f);
 }
+// Are whole units scored two blocks of keys deep, which leaves an SM one CTA more than four deep does?  Where four deep they would
+// take a wave more, less than half full.  Two | four deep, us a step of units of 3,276 keys, d = 128: 256 units 39.4 | 39.7, 448 61.6 |
+// 81.0, 592 82.0 | 89.0, 640 104 | 91, 896 118 | 134, 1,024 130 | 141, 1,184 157 | 152, 2,048 255 | 256; of 300 keys, 64 units
+// 8.1 | 7.8; d = 64: 736 units 52 | 67, 744 70 | 67, 1,024 79 | 75.
+// Each CTA takes 1 KB of shared memory beside its own, of the 196 KB that an SM is split for where nothing asks for more.
+bool shallow_score(const shotkv_ctx* ctx, int d, int U, size_t smem) {
+    const int fit = (int)(196 * 1024 / (smem + 1024));
+    const auto wave = [&](int deep) { return ctx->sm_count * std::max(1, std::min(ctx->whole_score[d == 128][deep], fit)); };
+    const int two = wave(0), four = wave(1);
+    return (U + two - 1) / two < (U + four - 1) / four && ((U - 1) % four + 1) * 2 < four;
+}
 template <int D>
 int launch_decode_score(shotkv_ctx* ctx, DecodeParams& p, const DecodeFinishParams& f, int U, bool& ended, cudaStream_t stream) {
-    const DecodeRoom& room = ctx->room_score[D == 128];
-    const size_t smem = score_smem_bytes(p.Dcap), end = fused_end_smem_bytes(p.Hkv, f.n, f.k < f.n);
-    p.nsplit = decode_split(room, [&](int) { return smem; }, U, (long long)p.Mcap + p.n_old + 1, 8, kLeastScore);
-    ended = smem + end <= kBigSmem && ends_fused(ctx, room.with(smem + end), p, f, U, 256);
-    if (ended) return launch(ctx, decode_score_kernel<D, true, true>, dim3(U * p.nsplit), 256, smem + end, stream, p.Hkv * p.nsplit, kEarly, p, f);
-    return p.nsplit > 1 ? launch(ctx, decode_score_kernel<D, true, false>, dim3(U * p.nsplit), 256, smem, stream, p.nsplit, kEarly, p, f)
-                        : launch(ctx, decode_score_kernel<D, false, false>, dim3(U), 256, smem, stream, 1, kEarly, p, f);
+    const DecodeRoom* room = ctx->room_score[D == 128];
+    const size_t smem = score_smem_bytes(p.Dcap, true), end = fused_end_smem_bytes(p.Hkv, f.n, f.k < f.n);
+    const auto split = [&](const DecodeRoom& r, int least) { return decode_split(r, [&](int) { return smem; }, U, (long long)p.Mcap + p.n_old + 1, 8, least); };
+    p.nsplit = split(room[0], kLeastScore);
+    if (D == 64 && p.nsplit == 1 && (p.nsplit = split(room[2], 2 * kLeastScore)) > 1)
+        return launch(ctx, decode_score_kernel<64, true, false, kShallow>, dim3(U * p.nsplit), 256, smem, stream, p.nsplit, kEarly, p, f);
+    ended = smem + end <= kBigSmem && ends_fused(ctx, room[1].with(smem + end), p, f, U, 256);
+    if (ended) return launch(ctx, decode_score_kernel<D, true, true, kDeep>, dim3(U * p.nsplit), 256, smem + end, stream, p.Hkv * p.nsplit, kEarly, p, f);
+    if (p.nsplit > 1) return launch(ctx, decode_score_kernel<D, true, false, kDeep>, dim3(U * p.nsplit), 256, smem, stream, p.nsplit, kEarly, p, f);
+    const size_t whole = score_smem_bytes(p.Dcap, false);
+    return launch(ctx, shallow_score(ctx, D, U, whole) ? decode_score_kernel<D, false, false, kShallow> : decode_score_kernel<D, false, false, kDeep>,
+                  dim3(U), 256, whole, stream, 1, kEarly, p, f);
 }
 
 // One decode step; with `attn_out` the score kernel is the variant that also writes the attention output.

@@ -89,3 +89,10 @@ def test_clusters_of_ctas_that_take_much_memory(ctx, L, Hkv, G, d, M, Dcap):
     assert cfg.Dcap == Dcap
     for attend in (False, True):
         assert lockstep(ctx, cfg, M, [(0, 0)], np.full((1, L), M, np.int32), steps=5, attend=attend) <= 1
+
+
+@pytest.mark.parametrize("d,L", [(128, 55), (128, 56), (128, 74), (128, 75), (64, 28), (64, 32), (64, 37), (64, 92), (64, 93), (64, 127)])
+def test_whole_units_on_both_sides_of_a_wave(ctx, d, L):
+    """Units that are scored two and four blocks of keys deep, shared and whole, one wave of them and more."""
+    cfg = wl.DecodeConfig("waves", B=1, L=L, H=16, Hkv=8, d=d, steps=5, r_d=0.5, recompress_every=4, cfg_id=80)
+    assert lockstep(ctx, cfg, 1400, [(0, 0), (0, L - 1)], np.full((1, L), 1311, np.int32)) <= 1
