@@ -713,10 +713,12 @@ int run_token_scores(shotkv_ctx* ctx, const shotkv_dims* d, const float* imp, co
 template <int ROWS>
 int run_reduce_select_t(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView& pv, const ShotTable& tab, float* shot_scores,
                         const SelectArgs& sa, cudaStream_t stream) {
-    // a row of masses per CTA of the cluster: with thousands of shots fewer CTAs share the heads, so
-    // that two still fit an SM (one from about 4,000 shots on)
+    // A row of masses per CTA of the cluster, and the items' weights: with thousands of shots fewer CTAs share the heads, so
+    // that two still fit an SM, unless all of them run at once with one to an SM (clusters of eight fill 7/8 of the SMs).  32K
+    // tokens, 256 rows, 1,800 shots, half the CTAs with two to an SM | all with one: 1 layer 267 | 204 us a call, 4 layers 477 | 387.
+    const auto limit = [&](int ranks) { return (long long)d->B * d->L * ranks * 8 <= 7LL * ctx->sm_count ? kBigSmem : kBigSmem / 2; };
     int ranks = d->Hkv < kReduceCluster ? d->Hkv : kReduceCluster;
-    while (ranks > 1 && reduce_smem_bytes(ROWS, pv.P, d->S, pv.nchunk, ranks) > kBigSmem / 2) ranks = (ranks + 1) / 2;
+    while (ranks > 1 && reduce_smem_bytes(ROWS, pv.P, d->S, pv.nchunk, ranks) > (size_t)limit(ranks)) ranks = (ranks + 1) / 2;
     const size_t smem = reduce_smem_bytes(ROWS, pv.P, d->S, pv.nchunk, ranks);
     if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "too many shots for the single-pass path (S = %d)", d->S);
     return launch(ctx, reduce_select_kernel<ROWS>, dim3(d->B * d->L * ranks), kReduceThreads, smem, stream, ranks, kEarly, pv, tab,

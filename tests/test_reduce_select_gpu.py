@@ -112,3 +112,13 @@ def test_scores_from_token_importances(ctx, B, L, S, mean, Hkv):
         o = torch.from_numpy(off[b]).long().cuda()
         want = (total[b][:, o[1:]] - total[b][:, o[:-1]]) / (o[1:] - o[:-1])
         assert torch.allclose(out["shot_scores"][b].double(), want, rtol=1e-5, atol=0)
+
+
+@pytest.mark.parametrize("S,L", [(1440, 1), (1475, 1), (1475, 2)])
+def test_clusters_of_ctas_that_fill_an_sm(ctx, S, L):
+    """256 window rows, more shots than leave two CTAs of the reduction room on an SM."""
+    cfg = wl.PrefillConfig("many", B=1, L=L, H=32, Hkv=8, d=64, N=23680, W=64, S=S, shot_dist="uniform", shot_lo=10,
+                           shot_hi=24, question_len=200, r_p=0.3, cfg_id=63)
+    Q, K, V, off = wl.prefill_batch(cfg, "cuda")
+    gpu = P.gpu_prefill(ctx, P.dims_of(cfg), Q, K, V, off, cfg.r_p, 0, "fused")
+    P.check_all_units(gpu, Q, K, V, off, cfg.r_p, units=[(0, L - 1)], check_tokens=False)
