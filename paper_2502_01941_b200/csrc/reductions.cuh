@@ -112,9 +112,11 @@ __global__ void row_stats_kernel(const PartialView v, int R, float* __restrict__
 // (2) Every warp takes a run of consecutive pieces, its lanes the rows four at a time, and weights them from that
 // table (an exact item's pieces carry their own references and pay one exp2 per row); the sums over the lanes of the
 // pieces in flight go side by side.  (3) The pieces of each shot are added in index order.
-// All sums have a fixed order.  What a warp does is wait for its pieces, so it has four in flight, with 256 rows too, where that
-// takes registers of a fourth CTA on the SM: two there made 12 layers x 2 heads of 193 shots 113.9 us a call, four 108.5; 4 layers
-// x 8 heads of 400 shots 151.8 and 140.5.  The weights of an item kept in registers from piece to piece: 112.7 and 156.4.
+// All sums have a fixed order.  What a warp does is wait for its pieces, so it has four in flight.  With 256 rows that
+// takes registers of a fourth CTA on the SM: three in flight and four CTAs made 12 layers x 2 heads of 193 shots 114.6 us a call, four
+// in flight 109.1; 4 layers x 8 heads of 400 shots 155.6 and 140.8.  Where three CTAs to an SM are more than one wave, three in flight
+// are the better (this kernel with 256 shots and 8 heads: 48 layers 49.4 | 49.4 us, 56 layers 55.5 | 63.6, 64 layers 55.6 | 61.8, 128
+// layers 90 | 94.6).  The weights of an item kept in registers from piece to piece: 112.7 and 156.4.
 constexpr int kReduceThreads = kSelectThreads;
 constexpr int kReduceCluster = 8;                  // most CTAs that share the kv heads of a (b, l)
 
@@ -126,13 +128,13 @@ __host__ __device__ constexpr size_t reduce_smem_bytes(int Rpad, int P, int S, i
     return bounds_smem_bytes(S) + ranks * ((size_t)(S + 3) / 4 * 4 * 4) + (work > select ? work : select);
 }
 
-template <int ROWS>
-__global__ void __launch_bounds__(kReduceThreads, ROWS == 128 ? 4 : 3) reduce_select_kernel(const PartialView v, const __grid_constant__ ShotTable tab,
+template <int ROWS, int AHEAD>
+__global__ void __launch_bounds__(kReduceThreads, ROWS == 128 || AHEAD < 4 ? 4 : 3) reduce_select_kernel(const PartialView v, const __grid_constant__ ShotTable tab,
                                                                       int R, int Hkv, int ranks,
                                                                       float* __restrict__ shot_scores, const SelectArgs a, int* err,
                                                                       long long wait_cycles) {
     constexpr int NW = kReduceThreads / 32, NH = ROWS / 128, PARTS = kReduceThreads / ROWS;
-    constexpr int AHEAD = 4, FIRST = 4;       // pieces whose z a warp has in flight; items whose statistics a thread has
+    constexpr int FIRST = 4;                       // items whose statistics a thread has in flight (AHEAD: pieces whose z a warp has)
     constexpr unsigned char kNoItem = 255;
     static_assert(ROWS == 128 || ROWS == 256, "padded window rows");
     extern __shared__ __align__(16) unsigned char sm[];

@@ -721,7 +721,9 @@ int run_reduce_select_t(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView
     while (ranks > 1 && reduce_smem_bytes(ROWS, pv.P, d->S, pv.nchunk, ranks) > (size_t)limit(ranks)) ranks = (ranks + 1) / 2;
     const size_t smem = reduce_smem_bytes(ROWS, pv.P, d->S, pv.nchunk, ranks);
     if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "too many shots for the single-pass path (S = %d)", d->S);
-    return launch(ctx, reduce_select_kernel<ROWS>, dim3(d->B * d->L * ranks), kReduceThreads, smem, stream, ranks, kEarly, pv, tab,
+    const int ctas = d->B * d->L * ranks;
+    const auto kernel = ROWS == 256 && ctas > 3 * ctx->sm_count ? reduce_select_kernel<ROWS, ROWS == 256 ? 3 : 4> : reduce_select_kernel<ROWS, 4>;
+    return launch(ctx, kernel, dim3(ctas), kReduceThreads, smem, stream, ranks, kEarly, pv, tab,
                   (d->H / d->Hkv) * d->W, (int)d->Hkv, ranks, shot_scores, sa, ctx->err_dev, ctx->wait_cycles);
 }
 int run_reduce_select(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView& pv, const ShotTable& tab, float* shot_scores,
@@ -771,7 +773,7 @@ cudaError_t set_kernel_attributes() {
     if (e == cudaSuccess) e = set_tc_attributes<64, 1>();
     if (e == cudaSuccess) e = set_tc_attributes<64, 2>();
     const void* small[] = {(const void*)select_shots_kernel<kSelectThreads>, (const void*)select_shots_kernel<kSortThreads>,
-                           (const void*)reduce_select_kernel<128>, (const void*)reduce_select_kernel<256>,
+                           (const void*)reduce_select_kernel<128, 4>, (const void*)reduce_select_kernel<256, 4>, (const void*)reduce_select_kernel<256, 3>,
                            (const void*)decode_score_kernel<128, false, false, kDeep>, (const void*)decode_score_kernel<64, false, false, kDeep>,
                            (const void*)decode_score_kernel<128, false, false, kShallow>, (const void*)decode_score_kernel<64, false, false, kShallow>,
                            (const void*)decode_evict_kernel<128>, (const void*)decode_evict_kernel<64>};

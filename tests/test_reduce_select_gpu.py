@@ -122,3 +122,13 @@ def test_clusters_of_ctas_that_fill_an_sm(ctx, S, L):
     Q, K, V, off = wl.prefill_batch(cfg, "cuda")
     gpu = P.gpu_prefill(ctx, P.dims_of(cfg), Q, K, V, off, cfg.r_p, 0, "fused")
     P.check_all_units(gpu, Q, K, V, off, cfg.r_p, units=[(0, L - 1)], check_tokens=False)
+
+
+@pytest.mark.parametrize("L", [27, 28])
+def test_more_clusters_than_one_wave(ctx, L):
+    """256 window rows on both sides of three CTAs to an SM (444): four and three pieces in flight a warp."""
+    cfg = wl.PrefillConfig("waves", B=2, L=L, H=32, Hkv=8, d=64, N=1700, W=64, S=61, shot_dist="uniform", shot_lo=17,
+                           shot_hi=31, question_len=150, r_p=0.4, cfg_id=64)
+    Q, K, V, off = wl.prefill_batch(cfg, "cuda")
+    gpu = P.gpu_prefill(ctx, P.dims_of(cfg), Q, K, V, off, cfg.r_p, 0, "fused")
+    P.check_all_units(gpu, Q, K, V, off, cfg.r_p, units=[(0, 0), (0, L - 1), (1, L - 1)], check_tokens=False)
