@@ -280,7 +280,7 @@ template <int D, bool SPLIT, bool FUSED, int DEPTH>
 __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p, const DecodeFinishParams f) {
     constexpr int NB = D / 32;     // 32-dim blocks
     constexpr int VPR = D / 8;     // 16-byte vectors per row
-    extern __shared__ __align__(16) unsigned char dsm[];
+    extern __shared__ __align__(128) unsigned char dsm[];
     float* sdec = reinterpret_cast<float*>(dsm);             // [8][Dcap]
     float2* sred = reinterpret_cast<float2*>(sdec + 8 * p.Dcap);   // [8 warps][8 rows]  (m, z)
     float2* stab = sred + 8 * 8;                             // [kMaxSplit][8 rows]  (m, z) of the cluster's CTAs
@@ -486,7 +486,8 @@ struct AttendCfg {
     static constexpr int kTileBytes = 16 * kRowBytes;             // 16 rows of keys (or of values)
     static constexpr int kStageBytes = 2 * kTileBytes;
     static constexpr int kRingBytes = kWarps * kStages * kStageBytes;
-    static_assert(8 * D * 4 <= kStages * kStageBytes, "a warp's outputs take the place of its ring");
+    static constexpr int kOutPitch = D + 4;                       // floats a row of a warp's outputs
+    static_assert(8 * kOutPitch * 4 <= kStages * kStageBytes, "a warp's outputs take the place of its ring");
 };
 
 // Dynamic shared memory of the decode kernels for decode regions of Dcap rows, multiples of 16 bytes.
@@ -505,7 +506,7 @@ __host__ __device__ constexpr size_t attend_smem_bytes(int G, int Dcap, int nspl
 // accumulators of the output leave too few registers for enough such warps.  So nothing is loaded
 // into registers from global memory here: key and value rows go global -> shared by cp.async one
 // block ahead of their use, into a per-warp ring (measured: two stages with three CTAs on an SM beat three stages with two).
-// The ring comes first in shared memory: its rows lie on 128-byte boundaries as they do in global memory, or a warp's copy
+// The ring comes first in shared memory, which is declared so: its rows lie on 128-byte boundaries as they do in global memory, or a warp's copy
 // of 512 bytes takes five lines of it and part of its sectors from L2 twice (40 % more of them with the ring 16 bytes off a boundary;
 // 8 sequences x 32 layers 580 us a step there, 511 at 64 bytes, 495 at 128).
 //
@@ -536,7 +537,7 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     constexpr int VPR = D / 8;     // 16-byte chunks per row
     constexpr int MT = D / 16;     // 16-dim tiles of the output
     constexpr int NW = Cfg::kWarps, NS = Cfg::kStages, NT = NW * 32;
-    extern __shared__ __align__(16) unsigned char dsm[];
+    extern __shared__ __align__(128) unsigned char dsm[];
     unsigned char* ring = dsm;                               // [NW][NS][keys | values][16 rows][D bf16]; later each warp's outputs [8 rows][PITCH]
     float2* sred = reinterpret_cast<float2*>(ring + Cfg::kRingBytes + 16);   // [NW warps][8 rows]  (m, z)
     float* sdec = reinterpret_cast<float*>(sred + NW * 8);   // [G][Dcap]  logits of the decode entries
@@ -739,7 +740,7 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     z += __shfl_xor_sync(0xffffffffu, z, 2);
     if (t4 == 0) sred[warp * 8 + g] = make_float2(m, z);
     __syncwarp();                                           // all lanes are done with the warp's ring: its outputs take its place
-    constexpr int PITCH = D + 4, kWarpRing = NS * Cfg::kStageBytes / 4;    // floats
+    constexpr int PITCH = Cfg::kOutPitch, kWarpRing = NS * Cfg::kStageBytes / 4;    // floats
     float* sO = reinterpret_cast<float*>(ring);
 #pragma unroll
     for (int mt = 0; mt < MT; ++mt) {

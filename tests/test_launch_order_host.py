@@ -30,3 +30,10 @@ def test_nothing_is_read_through_the_read_only_path():
     for name, params, body in early:
         assert not re.search(r"const\s+\w+\s*\*\s*__restrict__", params), f"{name}: read-only pointer among the parameters"
         assert "__ldg" not in body, f"{name}: read-only load"
+
+
+def test_the_ring_of_the_attention_step_is_declared_on_a_line():
+    """A warp's 512-byte copies reach one line of shared memory more where the ring does not begin on one."""
+    body = {name: body for name, _, body in _kernels()}["decode_attend_kernel"]
+    assert re.search(r"extern\s+__shared__\s+__align__\(128\)", body)
+    assert re.search(r"ring\s*=\s*dsm;", body), "the ring comes first"
