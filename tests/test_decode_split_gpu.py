@@ -28,7 +28,7 @@ def test_unit_shared_by_a_cluster(ctx, Hkv, G, d, M, count, attend):
 
 
 @pytest.mark.parametrize("Hkv,G,d,M,count", [(1, 1, 64, 4096, 4000), (1, 7, 128, 4100, 4100), (1, 5, 64, 3000, 2999), (2, 8, 128, 5000, 4999),
-                                             (3, 3, 128, 1700, 1690), (7, 2, 64, 6000, 5900)])
+                                             (3, 3, 128, 3000, 2990), (7, 2, 64, 6000, 5900)])
 def test_unit_shared_by_more_than_eight(ctx, Hkv, G, d, M, count):
     """Clusters of nine to sixteen, output elements that do and do not divide by them, for both steps."""
     cfg = wl.DecodeConfig("split", B=1, L=1, H=Hkv * G, Hkv=Hkv, d=d, steps=6, r_d=0.5, recompress_every=4, cfg_id=76)
@@ -43,14 +43,22 @@ def test_eviction_of_a_large_region(ctx, every):
 
 
 @pytest.mark.parametrize("attend", [False, True], ids=["plain", "attend"])
-@pytest.mark.parametrize("Hkv,G,d,M,every,steps", [(1, 8, 128, 3000, 1, 6), (2, 4, 64, 30, 1, 6), (5, 3, 128, 64, 3, 8), (8, 2, 128, 100, 4, 9),
-                                                   (16, 1, 64, 30, 2, 6), (17, 1, 64, 30, 2, 6), (2, 2, 64, 20, 127, 130), (2, 2, 64, 20, 128, 131),
-                                                   (2, 2, 128, 20, 129, 132), (16, 1, 64, 20, 400, 259)])
-def test_step_of_one_cluster(ctx, Hkv, G, d, M, every, steps, attend):
-    """A (sequence, layer) whose CTAs are one cluster ends its step in the first kernel; on both sides of where that
-    stops: 16 CTAs, 4,096 weights, evictions of 128 entries (with the attention output)."""
+@pytest.mark.parametrize("Hkv,G,d,M,every,steps,one", [
+    (1, 8, 128, 3000, 1, 6, (3, 3)),            # nine and sixteen CTAs to the unit: no eviction in the first kernel, every second step
+    (1, 8, 128, 2000, 1, 6, (6, 3)),            # six and sixteen
+    (1, 8, 128, 600, 1, 6, (0, 6)),             # one, which is no cluster, and seven
+    (2, 4, 64, 30, 1, 6, (6, 6)), (5, 3, 128, 64, 3, 8, (8, 8)), (8, 2, 128, 100, 4, 9, (9, 9)),
+    (16, 1, 64, 30, 2, 6, (3, 3)), (17, 1, 64, 30, 2, 6, (0, 0)),                          # heads
+    (2, 2, 64, 20, 127, 130, (130, 130)), (2, 2, 64, 20, 128, 131, (131, 131)),            # entries when it evicts
+    (2, 2, 128, 20, 129, 132, (132, 131)), (16, 1, 64, 20, 400, 259, (256, 150))])         # weights; from 171 keys on two CTAs a unit
+def test_step_of_one_cluster(ctx, Hkv, G, d, M, every, steps, one, attend):
+    """A (sequence, layer) whose CTAs are one cluster ends its step in the first kernel: `one` of the steps do, scores only and
+    with the attention output, on both sides of where that stops: 16 CTAs (8 when it evicts), 4,096 weights, evictions of 128
+    entries (with the attention output)."""
     cfg = wl.DecodeConfig("one", B=2, L=1, H=Hkv * G, Hkv=Hkv, d=d, steps=steps, r_d=0.5, recompress_every=every, cfg_id=77)
+    before = skv.shotkv_launch_count(ctx)
     assert lockstep(ctx, cfg, M, [(0, 0), (1, 0)], np.array([[M], [M - 7]], np.int32), attend=attend) <= 2
+    assert skv.shotkv_launch_count(ctx) - before == 2 * steps - one[attend]
 
 
 @pytest.mark.parametrize("M", [40, 2048], ids=["whole_unit", "shared_unit"])
