@@ -348,9 +348,10 @@ SHOTKV_API int shotkv_set_pipeline_groups(shotkv_ctx* ctx, int groups);
 SHOTKV_API int shotkv_profile_enable(shotkv_ctx* ctx, int enable);
 /* Stage durations in milliseconds of the profiled call made `calls_back` calls ago (0 = latest);
  * waits for that call to finish.  Prefill: {scoring kernel, per-shot reduce, select, compact} (reduce
- * and select are one kernel in the single-pass form: its time is the reduce's, select is about 0), each summed over the groups of a pipelined call (stages of different groups overlap, so the
- * sum can exceed the call's duration); decode: {score kernel, accumulate+evict (about 0 where the step ends in its first kernel), -1, -1}.  Returns the number of stages or a negative
- * error. */
+ * and select are one kernel in the single-pass form: its time is the reduce's, select is about 0), each
+ * summed over the groups of a pipelined call (stages of different groups overlap, so the sum can exceed
+ * the call's duration); decode: {score kernel, accumulate+evict (about 0 where the step ends in its first
+ * kernel), -1, -1}.  Returns the number of stages or a negative error. */
 SHOTKV_API int shotkv_profile_read(shotkv_ctx* ctx, int calls_back, float* stage_ms /* [4] */);
 /* Kernels launched through this context since it was created. */
 SHOTKV_API uint64_t shotkv_launch_count(const shotkv_ctx* ctx);

@@ -1,20 +1,20 @@
 // Second pass of per-token importance on the 5th-generation tensor cores.
 //
-// With every window row's final maximum M_r and 1/Z_r known (row_stats_kernel), the logits are
-// recomputed, normalised and summed over the rows: token_importance[t] = sum_r alpha[r][t].
-// The product is taken transposed, S^T = K_tile . Q^T (A = a tile of 128 keys, B = all R window
-// rows of the unit, N = 128 or 256 in one instruction), so that a key is a tensor-memory lane and
-// the window rows run along the columns: the sum over rows is then a sum inside one thread, with
-// no exchange between lanes.  Same persistent structure, work items, TMA producer and barrier
-// protocol as the scoring kernels (score_tc.cuh); Q is laid out in shared memory k-block major so
-// that the R rows of one 64-element k block are contiguous, as the B operand needs.
+// With every window row's final maximum M_r and 1/Z_r known (row_stats_kernel), the logits are recomputed, normalised
+// and summed over the rows: token_importance[t] = sum_r alpha[r][t].
+// The product is taken transposed, S^T = K_tile . Q^T (A = a tile of 128 keys, B = all R window rows of the unit, N =
+// 128 or 256 in one instruction), so that a key is a tensor-memory lane and the window rows run along the columns:
+// the sum over rows is then a sum inside one thread, with no exchange between lanes.  Same persistent structure, work
+// items, TMA producer and barrier protocol as the scoring kernels (score_tc.cuh); Q is laid out in shared memory
+// k-block major so that the R rows of one 64-element k block are contiguous, as the B operand needs.
 //
-// Epilogue: eight warps in two groups; a warp owns 32 keys (its tensor-memory lanes), a group
-// half of the window rows.  Per row the constants (-M_r, 1/Z_r) come from shared memory as
-// broadcast reads.  (As one constant, log2(1/Z_r) - M_r, they take half the reads, 236 -> 232 us a call of 16 layers of 8K with 256
-// rows, but 1/Z_r then has the resolution of M_r, and a row without weight no factor of zero.)  A chunk of 32 rows is asked for from tensor memory before the one ahead of it is
-// computed (32 layers of 16K in sentences 640 -> 628 us a call).  The second group hands its partial sums to the first through a two-slot
-// shared-memory ring guarded by mbarriers; the first adds them in a fixed order and stores.
+// Epilogue: eight warps in two groups; a warp owns 32 keys (its tensor-memory lanes), a group half of the window
+// rows.  Per row the constants (-M_r, 1/Z_r) come from shared memory as broadcast reads.  (As one constant,
+// log2(1/Z_r) - M_r, they take half the reads, 236 -> 232 us a call of 16 layers of 8K with 256 rows, but 1/Z_r then
+// has the resolution of M_r, and a row without weight no factor of zero.)  A chunk of 32 rows is asked for from
+// tensor memory before the one ahead of it is computed (32 layers of 16K in sentences 640 -> 628 us a call).  The
+// second group hands its partial sums to the first through a two-slot shared-memory ring guarded by mbarriers; the
+// first adds them in a fixed order and stores.
 #pragma once
 #include "score_stream.cuh"
 

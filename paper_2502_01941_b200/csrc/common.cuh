@@ -108,11 +108,11 @@ __device__ __forceinline__ uint32_t cluster_addr(const void* p, int rank) {
     return a;
 }
 
-// What the CTAs of a cluster tell one another goes as messages: a store counts its bytes on the receiver's
-// barrier, which is complete when as many as the receiver expects are there.  That is one way across the cluster, where a barrier of all its threads is two
-// (1.7 us of a step of 4 sequences x 1 layer).  expect_messages: by one thread, ahead of the cluster_arrive at the start;
-// nobody sends before a cluster_wait (a CTA's memory may be written once it has begun), and a CTA that has been sent
-// everything may end.
+// What the CTAs of a cluster tell one another goes as messages: a store counts its bytes on the receiver's barrier,
+// which is complete when as many as the receiver expects are there.  That is one way across the cluster, where a
+// barrier of all its threads is two (1.7 us of a step of 4 sequences x 1 layer).  expect_messages: by one thread,
+// ahead of the cluster_arrive at the start; nobody sends before a cluster_wait (a CTA's memory may be written once it
+// has begun), and a CTA that has been sent everything may end.
 __device__ __forceinline__ void expect_messages(unsigned long long* bar, int bytes) {
     const uint32_t b = smem_u32(bar);
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(b) : "memory");
@@ -155,9 +155,9 @@ __device__ __forceinline__ bool await_messages(unsigned long long* bar, int* err
         }
     }
 }
-// For single threads whose wait gave up, at their end: keeps their CTA, whose memory the others write to, until all other threads of
-// the cluster have ended or are here too (every wait of theirs ends), and until what they sent has landed, if it does within the
-// limit.  `bar`, `more`: the barriers waited for in vain, or NULL.
+// For single threads whose wait gave up, at their end: keeps their CTA, whose memory the others write to, until all
+// other threads of the cluster have ended or are here too (every wait of theirs ends), and until what they sent has
+// landed, if it does within the limit.  `bar`, `more`: the barriers waited for in vain, or NULL.
 __device__ __forceinline__ void outlive_messages(unsigned long long* bar, unsigned long long* more, int* err, long long limit) {
     asm volatile("barrier.cluster.arrive.release;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
@@ -165,9 +165,10 @@ __device__ __forceinline__ void outlive_messages(unsigned long long* bar, unsign
     if (more) await_messages(more, err, limit);
 }
 
-// Self-test of that, for the host to run on demand: a cluster of two CTAs of one warp.  The first expects two words; the
-// second sends one at once and the other well after the limit, when the first has given up.  Lane 0 of the first waits on
-// behalf of its warp, as a thread of a cluster's CTA does.  report[0..1] = {that wait succeeded, the late word was there before the CTA ended}.
+// Self-test of that, for the host to run on demand: a cluster of two CTAs of one warp.  The first expects two words;
+// the second sends one at once and the other well after the limit, when the first has given up.  Lane 0 of the first
+// waits on behalf of its warp, as a thread of a cluster's CTA does.  report[0..1] = {that wait succeeded, the late
+// word was there before the CTA ended}.
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(32) message_wait_selftest_kernel(long long limit, int* err, int* report) {
     __shared__ __align__(8) unsigned long long arrived;
     __shared__ float words[2];

@@ -72,8 +72,8 @@ __host__ __device__ constexpr size_t decode_evict_smem_bytes(int n) {
     return rank_smem_bytes(n) + 5 * ((size_t)(n + 3) / 4 * 4 * 4) + 128;
 }
 template <int D, int NT, class Value>
-__device__ __forceinline__ void evict_entries(const DecodeFinishParams& p, int bl, int rank, int ranks, bool clustered, unsigned char* sm,
-                                              Value&& value) {
+__device__ __forceinline__ void evict_entries(const DecodeFinishParams& p, int bl, int rank, int ranks, bool clustered,
+                                              unsigned char* sm, Value&& value) {
     constexpr int VPR = D / 8, RPP = NT / VPR, Q = 4;   // 16-byte vectors a row, rows a pass per vector in flight
     const int n = p.n, n4 = (n + 3) / 4 * 4;
     float* a = reinterpret_cast<float*>(sm + rank_smem_bytes(n));   // accumulated scores
@@ -239,7 +239,8 @@ __device__ __forceinline__ void fused_send(const FusedEnd& e, const DecodeFinish
 // All threads of all CTAs, once a CTA has sent its weights and made its other outputs.  False: the wait gave up,
 // and the end was made with whatever weights are there; every index stays in range, and the state is no longer a valid one anyhow.
 template <int D, int NT>
-__device__ __forceinline__ bool fused_finish(const FusedEnd& e, const DecodeFinishParams& f, int bl, int c, int ctas, const DecodeParams& p) {
+__device__ __forceinline__ bool fused_finish(const FusedEnd& e, const DecodeFinishParams& f, int bl, int c, int ctas,
+                                             const DecodeParams& p) {
     const bool evicts = f.k < f.n;
     if (!evicts && c != 0) return true;
     const bool ok = await_messages(e.arrived, p.err, p.wait_cycles);
@@ -261,7 +262,9 @@ __device__ __forceinline__ bool fused_finish(const FusedEnd& e, const DecodeFini
     return ok;
 }
 
-__host__ __device__ constexpr size_t score_smem_bytes(int Dcap, bool split) { return ((size_t)8 * Dcap + 8 * 8 * 2 + (split ? kMaxSplit * 16 + 4 : 0)) * 4; }
+__host__ __device__ constexpr size_t score_smem_bytes(int Dcap, bool split) {
+    return ((size_t)8 * Dcap + 8 * 8 * 2 + (split ? kMaxSplit * 16 + 4 : 0)) * 4;
+}
 
 // One CTA, or a cluster of p.nsplit, per (sequence, layer, kv head).  Each warp takes 16 keys at a
 // time straight from global memory: thread (g, t) of a warp reads 16 contiguous bytes of key rows g
@@ -284,7 +287,8 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p,
     float* sdec = reinterpret_cast<float*>(dsm);             // [8][Dcap]
     float2* sred = reinterpret_cast<float2*>(sdec + 8 * p.Dcap);   // [8 warps][8 rows]  (m, z)
     float2* stab = sred + 8 * 8;                             // [kMaxSplit][8 rows]  (m, z) of the cluster's CTAs
-    unsigned long long* arrived = reinterpret_cast<unsigned long long*>(stab + kMaxSplit * 8);   // of a cluster: barrier of what they send here
+    // of a cluster: barrier of what they send here
+    unsigned long long* arrived = reinterpret_cast<unsigned long long*>(stab + kMaxSplit * 8);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, t4 = lane & 3;
@@ -324,7 +328,8 @@ __global__ void __launch_bounds__(256) decode_score_kernel(const DecodeParams p,
     const int n = p.n_old + 1;
     const int Ktot = M + n;
     if (SPLIT) cluster_wait();                               // all CTAs of the cluster have begun: their memory may be written to
-    if (appends) (tid < VPR ? Kd_u + (size_t)p.n_old * VPR + tid : Vd_u + (size_t)p.n_old * VPR + (tid - VPR))[0] = fresh_row;   // decode entry n_old
+    if (appends)                                             // decode entry n_old
+        (tid < VPR ? Kd_u + (size_t)p.n_old * VPR + tid : Vd_u + (size_t)p.n_old * VPR + (tid - VPR))[0] = fresh_row;
 
     auto row_ptr = [&](int i, bool valid) -> const uint4* {
         if (!valid) return knew_u;                         // any readable row; the result is masked
@@ -497,39 +502,38 @@ __host__ __device__ constexpr size_t attend_smem_bytes(int G, int Dcap, int nspl
     return AttendCfg<D>::kRingBytes + 16 + ((size_t)AttendCfg<D>::kWarps * 16 + ((size_t)G * Dcap + 3) / 4 * 4 + shares) * 4;
 }
 
-// The same step with the attention output fused in: o_h = sum_t alpha_{t,h} v_t over the kept
-// prefill entries and the decode entries, with the very weights the decoding score sums, so that
-// scoring adds no pass over K to a decode step that has to read K and V anyway.
+// The same step with the attention output fused in: o_h = sum_t alpha_{t,h} v_t over the kept prefill entries and the
+// decode entries, with the very weights the decoding score sums, so that scoring adds no pass over K to a decode step
+// that has to read K and V anyway.
 //
-// HBM-bound, and what it takes to stay there is bytes in flight: a warp that loads a block's keys
-// into registers and then waits for them is idle for the whole (loaded) memory latency, and the
-// accumulators of the output leave too few registers for enough such warps.  So nothing is loaded
-// into registers from global memory here: key and value rows go global -> shared by cp.async one
-// block ahead of their use, into a per-warp ring (measured: two stages with three CTAs on an SM beat three stages with two).
-// The ring comes first in shared memory, which is declared so: its rows lie on 128-byte boundaries as they do in global memory, or a warp's copy
-// of 512 bytes takes five lines of it and part of its sectors from L2 twice (40 % more of them with the ring 16 bytes off a boundary;
-// 8 sequences x 32 layers 580 us a step there, 511 at 64 bytes, 495 at 128).
+// HBM-bound, and what it takes to stay there is bytes in flight: a warp that loads a block's keys into registers and
+// then waits for them is idle for the whole (loaded) memory latency, and the accumulators of the output leave too few
+// registers for enough such warps.  So nothing is loaded into registers from global memory here: key and value rows
+// go global -> shared by cp.async one block ahead of their use, into a per-warp ring (measured: two stages with three
+// CTAs on an SM beat three stages with two). The ring comes first in shared memory, which is declared so: its rows
+// lie on 128-byte boundaries as they do in global memory, or a warp's copy of 512 bytes takes five lines of it and
+// part of its sectors from L2 twice (40 % more of them with the ring 16 bytes off a boundary; 8 sequences x 32 layers
+// 580 us a step there, 511 at 64 bytes, 495 at 128).
 //
-// Both products run on the tensor cores, transposed so that the few query rows of a group are the
-// narrow N = 8 side.  Per block of 16 keys a warp computes S^T[rows x keys] = Q . K^T with the
-// group's query rows as the A operand (held in registers) and the key rows as B fragments (16
-// contiguous bytes per lane and 32-dim block; the same k-index permutation on both operands).
-// The accumulator fragment of that product -- lane (g, t4) holds row g, keys 2*t4, 2*t4+1,
-// 8+2*t4, 9+2*t4 -- is, after the exponential, exactly the B fragment of O^T[dims x rows] =
-// V^T . P^T, so the weights never leave their registers; they enter as a bf16 pair (high part plus
-// remainder: relative error 2^-17) in two MMAs per 16 dimensions, and ldmatrix.trans turns the
-// value rows into the A fragments of V^T.  Online softmax per warp with a running maximum per
-// query row (lanes that share g); the warps' (m, z, O) are merged at the end in warp order.
-// With few CTAs on an SM what bounds it is the chain of one block in one warp (0.7 us before, 0.5 now): the
-// copies of a block that is all prefill rows take their addresses from one pointer and immediate offsets,
-// masks and parked logits are left to the blocks that need them, and the first product runs as four chains
-// of MMAs.  32 steps of 8 sequences x 32 layers 16.25 -> 15.93 ms, a step of 4 sequences x 1 layer 17.0 -> 15.9 us,
-// one unit of 8,000 keys 20.0 -> 15.5 us.
-// Of a step of few units (13 us: 4 sequences x 1 layer, 3,276 keys) less than half was blocks of keys.  The rest is a chain of
-// latencies: everything the first two blocks need is now asked for in one go, each warp's outputs take the place of its own
-// ring (no barrier before they are written), every thread merges the rows it needs for itself, and the CTAs of a cluster
-// send each other their rows and the quads of output each adds up (12.9 -> 11.1 us; 2 sequences 12.2 -> 9.2).
-// FUSED: the cluster is all CTAs of a (sequence, layer), and the step ends here.
+// Both products run on the tensor cores, transposed so that the few query rows of a group are the narrow N = 8 side.
+// Per block of 16 keys a warp computes S^T[rows x keys] = Q . K^T with the group's query rows as the A operand (held
+// in registers) and the key rows as B fragments (16 contiguous bytes per lane and 32-dim block; the same k-index
+// permutation on both operands).
+// The accumulator fragment of that product -- lane (g, t4) holds row g, keys 2*t4, 2*t4+1, 8+2*t4, 9+2*t4 -- is,
+// after the exponential, exactly the B fragment of O^T[dims x rows] = V^T . P^T, so the weights never leave their
+// registers; they enter as a bf16 pair (high part plus remainder: relative error 2^-17) in two MMAs per 16
+// dimensions, and ldmatrix.trans turns the value rows into the A fragments of V^T.  Online softmax per warp with a
+// running maximum per query row (lanes that share g); the warps' (m, z, O) are merged at the end in warp order.
+// With few CTAs on an SM what bounds it is the chain of one block in one warp (0.7 us before, 0.5 now): the copies of
+// a block that is all prefill rows take their addresses from one pointer and immediate offsets, masks and parked
+// logits are left to the blocks that need them, and the first product runs as four chains of MMAs.  32 steps of 8
+// sequences x 32 layers 16.25 -> 15.93 ms, a step of 4 sequences x 1 layer 17.0 -> 15.9 us, one unit of 8,000 keys
+// 20.0 -> 15.5 us.
+// Of a step of few units (13 us: 4 sequences x 1 layer, 3,276 keys) less than half was blocks of keys.  The rest is a
+// chain of latencies: everything the first two blocks need is now asked for in one go, each warp's outputs take the
+// place of its own ring (no barrier before they are written), every thread merges the rows it needs for itself, and
+// the CTAs of a cluster send each other their rows and the quads of output each adds up (12.9 -> 11.1 us; 2 sequences
+// 12.2 -> 9.2). FUSED: the cluster is all CTAs of a (sequence, layer), and the step ends here.
 template <int D, bool FUSED>
 __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_kernel(const DecodeParams p, const DecodeFinishParams f) {
     using Cfg = AttendCfg<D>;
@@ -538,12 +542,15 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     constexpr int MT = D / 16;     // 16-dim tiles of the output
     constexpr int NW = Cfg::kWarps, NS = Cfg::kStages, NT = NW * 32;
     extern __shared__ __align__(128) unsigned char dsm[];
-    unsigned char* ring = dsm;                               // [NW][NS][keys | values][16 rows][D bf16]; later each warp's outputs [8 rows][PITCH]
+    // [NW][NS][keys | values][16 rows][D bf16]; later each warp's outputs [8 rows][PITCH]
+    unsigned char* ring = dsm;
     float2* sred = reinterpret_cast<float2*>(ring + Cfg::kRingBytes + 16);   // [NW warps][8 rows]  (m, z)
     float* sdec = reinterpret_cast<float*>(sred + NW * 8);   // [G][Dcap]  logits of the decode entries
-    float2* stab = reinterpret_cast<float2*>(sdec + ((p.G * p.Dcap + 3) & ~3));   // of a cluster: [nsplit][8 rows]  (m, z) of its CTAs,
-    float4* sin = reinterpret_cast<float4*>(stab + p.nsplit * 8);   // [nsplit][share]  and their outputs: this CTA's share of the quads
-    unsigned long long* arrived = reinterpret_cast<unsigned long long*>(sred) - 1;   // barrier of what they send here
+    // of a cluster: [nsplit][8 rows] (m, z) of its CTAs, [nsplit][share] their outputs, of which this CTA has its share of the
+    // quads, and the barrier of what they send here
+    float2* stab = reinterpret_cast<float2*>(sdec + ((p.G * p.Dcap + 3) & ~3));
+    float4* sin = reinterpret_cast<float4*>(stab + p.nsplit * 8);
+    unsigned long long* arrived = reinterpret_cast<unsigned long long*>(sred) - 1;
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int g = lane >> 2, t4 = lane & 3;
@@ -613,7 +620,8 @@ __global__ void __launch_bounds__(AttendCfg<D>::kWarps * 32, 3) decode_attend_ke
     const int n = p.n_old + 1;
     const int Ktot = M + n;
     if (FUSED || p.nsplit > 1) cluster_wait();               // all CTAs of the cluster have begun: their memory may be written to
-    if (appends) (tid < VPR ? Kd_u + (size_t)p.n_old * VPR + tid : Vd_u + (size_t)p.n_old * VPR + (tid - VPR))[0] = fresh_row;   // decode entry n_old
+    if (appends)                                             // decode entry n_old
+        (tid < VPR ? Kd_u + (size_t)p.n_old * VPR + tid : Vd_u + (size_t)p.n_old * VPR + (tid - VPR))[0] = fresh_row;
 
     // a block with decode entries in it, or past the end: rows past the end are filled with zeros (a weight of
     // zero must not meet a stray NaN)

@@ -95,28 +95,28 @@ __global__ void row_stats_kernel(const PartialView v, int R, float* __restrict__
     row_invz[(size_t)u * v.Rpad + r] = (r < R && z > 0.f) ? 1.f / z : 0.f;
 }
 
-// One (b, l): the mass every window row puts on every shot, normalised and summed over the rows and
-// the kv heads,
+// One (b, l): the mass every window row puts on every shot, normalised and summed over the rows and the kv heads,
 //   mass[h][i] = sum_r ( sum_{pieces q of shot i} z_q[r] * exp2(m_q[r] - m[r]) ) / Z[r]
 //   Score(s_i) = (1/k_i) * sum_h mass[h][i]                             (prefill score equation)
-// then the selection.  A cluster of CTAs shares the kv heads of a (b, l), CTA c taking heads c,
-// c + cluster size, ...; each leaves its masses in the leader's shared memory and ends, and the leader
-// adds them in a fixed order and selects.  In one kernel because the three steps are latency, not work:
-// separate kernels for the masses (one CTA a unit, items and pieces one after the other), the sum
-// over heads and the selection took 20 + 2.3 + 5.5 us on one layer of 4K and 38 + 2.6 + 8.4 us on
-// 4 x 32 layers of 32K, where reading the partials (115 MB) is 18 us of memory time.
+// then the selection.  A cluster of CTAs shares the kv heads of a (b, l), CTA c taking heads c, c + cluster size,
+// ...; each leaves its masses in the leader's shared memory and ends, and the leader adds them in a fixed order and
+// selects.  In one kernel because the three steps are latency, not work: separate kernels for the masses (one CTA a
+// unit, items and pieces one after the other), the sum over heads and the selection took 20 + 2.3 + 5.5 us on one
+// layer of 4K and 38 + 2.6 + 8.4 us on 4 x 32 layers of 32K, where reading the partials (115 MB) is 18 us of memory
+// time.
 //
-// Per head: (1) a thread (two, with 128 rows) per row merges the item statistics into the row's
-// (m, 1/Z): the maximum first, then the sum, so that the items' loads are all in flight at once; the weight
-// exp2(m_item[r] - m[r]) / Z[r], the same for all pieces of an item, goes to a table of items and rows.
-// (2) Every warp takes a run of consecutive pieces, its lanes the rows four at a time, and weights them from that
-// table (an exact item's pieces carry their own references and pay one exp2 per row); the sums over the lanes of the
-// pieces in flight go side by side.  (3) The pieces of each shot are added in index order.
-// All sums have a fixed order.  What a warp does is wait for its pieces, so it has four in flight.  With 256 rows that
-// takes registers of a fourth CTA on the SM: three in flight and four CTAs made 12 layers x 2 heads of 193 shots 114.6 us a call, four
-// in flight 109.1; 4 layers x 8 heads of 400 shots 155.6 and 140.8.  Where three CTAs to an SM are more than one wave, three in flight
-// are the better (this kernel with 256 shots and 8 heads: 48 layers 49.4 | 49.4 us, 56 layers 55.5 | 63.6, 64 layers 55.6 | 61.8, 128
-// layers 90 | 94.6).  The weights of an item kept in registers from piece to piece: 112.7 and 156.4.
+// Per head: (1) a thread (two, with 128 rows) per row merges the item statistics into the row's (m, 1/Z), four items
+// at a time, whose loads are in flight together; the weight exp2(m_item[r] - m[r]) / Z[r], the same for all pieces of
+// an item, goes to a table of items and rows. (2) Every warp takes a run of consecutive pieces, its lanes the rows
+// four at a time, and weights them from that table (an exact item's pieces carry their own references and pay one
+// exp2 per row); the sums over the lanes of the pieces in flight go side by side.  (3) The pieces of each shot are
+// added in index order.
+// All sums have a fixed order.  What a warp does is wait for its pieces, so it has four in flight.  With 256 rows
+// that takes registers of a fourth CTA on the SM: three in flight and four CTAs made 12 layers x 2 heads of 193 shots
+// 114.6 us a call, four in flight 109.1; 4 layers x 8 heads of 400 shots 155.6 and 140.8.  Where three CTAs to an SM
+// are more than one wave, three in flight are the better (this kernel with 256 shots and 8 heads: 48 layers 49.4 |
+// 49.4 us, 56 layers 55.5 | 63.6, 64 layers 55.6 | 61.8, 128 layers 90 | 94.6).  The weights of an item kept in
+// registers from piece to piece: 112.7 and 156.4.
 constexpr int kReduceThreads = kSelectThreads;
 constexpr int kReduceCluster = 8;                  // most CTAs that share the kv heads of a (b, l)
 
@@ -129,10 +129,9 @@ __host__ __device__ constexpr size_t reduce_smem_bytes(int Rpad, int P, int S, i
 }
 
 template <int ROWS, int AHEAD>
-__global__ void __launch_bounds__(kReduceThreads, ROWS == 128 || AHEAD < 4 ? 4 : 3) reduce_select_kernel(const PartialView v, const __grid_constant__ ShotTable tab,
-                                                                      int R, int Hkv, int ranks,
-                                                                      float* __restrict__ shot_scores, const SelectArgs a, int* err,
-                                                                      long long wait_cycles) {
+__global__ void __launch_bounds__(kReduceThreads, ROWS == 128 || AHEAD < 4 ? 4 : 3)
+    reduce_select_kernel(const PartialView v, const __grid_constant__ ShotTable tab, int R, int Hkv, int ranks, float* __restrict__ shot_scores,
+                         const SelectArgs a, int* err, long long wait_cycles) {
     constexpr int NW = kReduceThreads / 32, NH = ROWS / 128, PARTS = kReduceThreads / ROWS;
     constexpr int FIRST = 4;                       // items whose statistics a thread has in flight (AHEAD: pieces whose z a warp has)
     constexpr unsigned char kNoItem = 255;
@@ -145,8 +144,8 @@ __global__ void __launch_bounds__(kReduceThreads, ROWS == 128 || AHEAD < 4 ? 4 :
     int* o = reinterpret_cast<int*>(sm);
     float* masses = reinterpret_cast<float*>(sm + bounds_smem_bytes(S));   // [ranks][s4]
     unsigned char* work = reinterpret_cast<unsigned char*>(masses + (size_t)ranks * s4);
-    float* row_m = reinterpret_cast<float*>(work); // [2][ROWS] maxima of the parts, then [ROWS]
-    float* row_w = row_m + 2 * ROWS;               // [2][ROWS] sums of the parts, then [ROWS] 1/Z (0 for rows without weight)
+    float* row_m = reinterpret_cast<float*>(work); // [2][ROWS] maxima of the parts; where an item is exact, then [ROWS]
+    float* row_w = row_m + 2 * ROWS;               // [2][ROWS] sums of the parts; then [ROWS] 1/Z (0 for rows without weight)
     float* weight = row_w + 2 * ROWS;              // [nchunk][ROWS] 2^(m_item - row's m) / Z
     float* piece_mass = weight + (size_t)v.nchunk * ROWS;   // [P]
     unsigned char* item_of = reinterpret_cast<unsigned char*>(piece_mass + (np + 3) / 4 * 4);   // [P]

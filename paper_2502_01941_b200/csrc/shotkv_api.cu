@@ -55,9 +55,10 @@ struct TraceRange {
     TraceRange& operator=(const TraceRange&) = delete;
 };
 
-// Clusters of n decode CTAs that the device runs at a time, by what a CTA takes of shared memory: four, three, two and one of them
-// fit an SM.  (As one figure, for three, 16 units of 3,276 keys with the attention output and room for 750 decode entries took 13.1 us a step,
-// 32 units 16.0: one figure put more CTAs to a unit than run at the same time.)
+// Clusters of n decode CTAs that the device runs at a time, by what a CTA takes of shared memory: four, three, two
+// and one of them fit an SM.  (As one figure, for three, 16 units of 3,276 keys with the attention output and room
+// for 750 decode entries took 13.1 us a step, 32 units 16.0: one figure put more CTAs to a unit than run at the same
+// time.)
 constexpr int kRoomClasses = 4;
 constexpr size_t kRoomSmem[kRoomClasses] = {56 * 1024, 75 * 1024, 113 * 1024, kBigSmem};
 struct DecodeRoom {
@@ -447,14 +448,13 @@ int launch_score_tc_t(shotkv_ctx* ctx, const CUtensorMap& tmQ, const CUtensorMap
     return launch(ctx, score_tc_kernel<D, MB>, dim3(grid), ScoreTcCfg<D, MB>::kThreads, smem, stream, 1, kEarly, tmQ, tmK, qbox, kbox, sp, tab);
 }
 
-// Column pairs, of every 16, whose exponentials run on the FMA pipe instead of the special-function unit.
-// The larger share takes fewer cycles and more energy: with 256 window rows the scoring pass runs at the
-// power cap for as long as it runs (5, 4, 3, 2, 1, 0 pairs: 4 x 32 layers of 32K 3,570, 3,550, 3,530, 3,580,
-// 3,630, 3,705 us a call), with 128 it waits for memory as much as for power (32 layers of 16K 395, -, 397,
-// 398, 399, 402).
-// The second pass of the per-token form takes 5, 4 and 3 in the same time (16 layers of 8K with 256 rows 237, 236, 236 us a call),
-// and its error grows with the share: 3.4e-6, 3.0e-6 and 2.6e-6 against 64 bits (256 rows, logits of deviation 1), 6.8e-5, 6.1e-5 and
-// 5.2e-5 (128 rows, deviation 400).
+// Column pairs, of every 16, whose exponentials run on the FMA pipe instead of the special-function unit. The larger
+// share takes fewer cycles and more energy: with 256 window rows the scoring pass runs at the power cap for as long
+// as it runs (5, 4, 3, 2, 1, 0 pairs: 4 x 32 layers of 32K 3,570, 3,550, 3,530, 3,580, 3,630, 3,705 us a call), with
+// 128 it waits for memory as much as for power (32 layers of 16K 395, -, 397, 398, 399, 402).
+// The second pass of the per-token form takes 5, 4 and 3 in the same time (16 layers of 8K with 256 rows 237, 236,
+// 236 us a call), and its error grows with the share: 3.4e-6, 3.0e-6 and 2.6e-6 against 64 bits (256 rows, logits of
+// deviation 1), 6.8e-5, 6.1e-5 and 5.2e-5 (128 rows, deviation 400).
 constexpr int kPolyPairs = 5, kPolyPairsStream = 3, kPolyPairsTokens = 3;
 constexpr int kShortUnit = 64;        // mean length below which the streaming kernel takes its form for short units
 
@@ -713,9 +713,10 @@ int run_token_scores(shotkv_ctx* ctx, const shotkv_dims* d, const float* imp, co
 template <int ROWS>
 int run_reduce_select_t(shotkv_ctx* ctx, const shotkv_dims* d, const PartialView& pv, const ShotTable& tab, float* shot_scores,
                         const SelectArgs& sa, cudaStream_t stream) {
-    // A row of masses per CTA of the cluster, and the items' weights: with thousands of shots fewer CTAs share the heads, so
-    // that two still fit an SM, unless all of them run at once with one to an SM (clusters of eight fill 7/8 of the SMs).  32K
-    // tokens, 256 rows, 1,800 shots, half the CTAs with two to an SM | all with one: 1 layer 267 | 204 us a call, 4 layers 477 | 387.
+    // A row of masses per CTA of the cluster, and the items' weights: with thousands of shots fewer CTAs share the
+    // heads, so that two still fit an SM, unless all of them run at once with one to an SM (clusters of eight fill
+    // 7/8 of the SMs).  32K tokens, 256 rows, 1,800 shots, half the CTAs with two to an SM | all with one: 1 layer
+    // 267 | 204 us a call, 4 layers 477 | 387.
     const auto limit = [&](int ranks) { return (long long)d->B * d->L * ranks * 8 <= 7LL * ctx->sm_count ? kBigSmem : kBigSmem / 2; };
     int ranks = d->Hkv < kReduceCluster ? d->Hkv : kReduceCluster;
     while (ranks > 1 && reduce_smem_bytes(ROWS, pv.P, d->S, pv.nchunk, ranks) > (size_t)limit(ranks)) ranks = (ranks + 1) / 2;
@@ -772,18 +773,26 @@ cudaError_t set_kernel_attributes() {
     if (e == cudaSuccess) e = set_tc_attributes<128, 2>();
     if (e == cudaSuccess) e = set_tc_attributes<64, 1>();
     if (e == cudaSuccess) e = set_tc_attributes<64, 2>();
-    const void* small[] = {(const void*)select_shots_kernel<kSelectThreads>, (const void*)select_shots_kernel<kSortThreads>,
-                           (const void*)reduce_select_kernel<128, 4>, (const void*)reduce_select_kernel<256, 4>, (const void*)reduce_select_kernel<256, 3>,
-                           (const void*)decode_score_kernel<128, false, false, kDeep>, (const void*)decode_score_kernel<64, false, false, kDeep>,
-                           (const void*)decode_score_kernel<128, false, false, kShallow>, (const void*)decode_score_kernel<64, false, false, kShallow>,
-                           (const void*)decode_evict_kernel<128>, (const void*)decode_evict_kernel<64>};
+    const void* small[] = {(const void*)select_shots_kernel<kSelectThreads>,
+                           (const void*)select_shots_kernel<kSortThreads>,
+                           (const void*)reduce_select_kernel<128, 4>,
+                           (const void*)reduce_select_kernel<256, 4>,
+                           (const void*)reduce_select_kernel<256, 3>,
+                           (const void*)decode_score_kernel<128, false, false, kDeep>,
+                           (const void*)decode_score_kernel<64, false, false, kDeep>,
+                           (const void*)decode_score_kernel<128, false, false, kShallow>,
+                           (const void*)decode_score_kernel<64, false, false, kShallow>,
+                           (const void*)decode_evict_kernel<128>,
+                           (const void*)decode_evict_kernel<64>};
     for (const void* f : small)
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kBigSmem);
     // a decode unit may be shared by more CTAs than the eight that every device's clusters allow
     const void* attend[] = {(const void*)decode_attend_kernel<128, false>, (const void*)decode_attend_kernel<128, true>,
                             (const void*)decode_attend_kernel<64, false>, (const void*)decode_attend_kernel<64, true>};
-    const void* score[] = {(const void*)decode_score_kernel<128, true, false, kDeep>, (const void*)decode_score_kernel<128, true, true, kDeep>,
-                           (const void*)decode_score_kernel<64, true, false, kDeep>, (const void*)decode_score_kernel<64, true, true, kDeep>,
+    const void* score[] = {(const void*)decode_score_kernel<128, true, false, kDeep>,
+                           (const void*)decode_score_kernel<128, true, true, kDeep>,
+                           (const void*)decode_score_kernel<64, true, false, kDeep>,
+                           (const void*)decode_score_kernel<64, true, true, kDeep>,
                            (const void*)decode_score_kernel<64, true, false, kShallow>};
     const auto in_clusters = [&](const void* f) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kBigSmem);
@@ -797,8 +806,9 @@ cudaError_t set_kernel_attributes() {
     return e;
 }
 
-// How many clusters of n decode CTAs the device runs at the same time: for every class of shared memory.  More than eight CTAs are not every device's, nor every
-// part of one: where it has no room for such a cluster, or does not know it, the figure is 0 and none is launched.
+// How many clusters of n decode CTAs the device runs at the same time: for every class of shared memory.  More than
+// eight CTAs are not every device's, nor every part of one: where it has no room for such a cluster, or does not know
+// it, the figure is 0 and none is launched.
 template <class K>
 cudaError_t ask_room(K* kernel, int threads, DecodeRoom& room) {
     for (int c = 0; c < kRoomClasses; ++c)
@@ -833,8 +843,11 @@ cudaError_t ask_decode_room_t(shotkv_ctx* ctx) {
     if (e == cudaSuccess) e = ask_room(decode_score_kernel<D, true, true, kDeep>, 256, score[1]);
     if (e == cudaSuccess && D == 64) e = ask_room(decode_score_kernel<64, true, false, kShallow>, 256, score[2]);
     int* whole = ctx->whole_score[D == 128];
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&whole[0], decode_score_kernel<D, false, false, kShallow>, 256, 0);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&whole[1], decode_score_kernel<D, false, false, kDeep>, 256, 0);
+    const auto fit = [&](int& ctas, auto* kernel) {
+        if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel, 256, 0);
+    };
+    fit(whole[0], decode_score_kernel<D, false, false, kShallow>);
+    fit(whole[1], decode_score_kernel<D, false, false, kDeep>);
     return e;
 }
 cudaError_t ask_decode_room(shotkv_ctx* ctx) {
@@ -1348,13 +1361,15 @@ int shotkv_decode_init(shotkv_ctx* ctx, const shotkv_dims* dims, const shotkv_po
 namespace {
 
 // CTAs that share a unit's keys: as many as still run at the same time for all units (as clusters of n CTAs with
-// `smem(n)` bytes each: a cluster stays within a group of SMs, so it is fewer than the SMs' slots / n) and leave every
-// warp at least `least` sixths of a block of 16 keys.  The fused step gains from more CTAs down to little more than a block a
-// warp, whose chain is long (2 heads of 333 keys 6.5 -> 5.4 us a step with 4/3 of a block instead of 2, 185 keys 8.5 -> 7.1; 1 block:
-// 8 heads of 1,150 keys 7.0 -> 7.3).  Scores alone take less per block than a larger cluster costs (8 heads of 3,400 keys 5.3 us with 2.5
-// blocks, 6.1 with 2, 5.7 with 3).  Shared units are scored four blocks deep, the better by 1 to 15 % where both forms fit; with d = 64
-// that takes registers of a fourth CTA on the SM, and long units it leaves whole, but two deep does not, go two deep (256 units of 3,400 keys
-// 28.9 -> 20.7 us; of 1,150 keys whole 19.1, two deep 19.7).
+// `smem(n)` bytes each: a cluster stays within a group of SMs, so it is fewer than the SMs' slots / n) and leave
+// every warp at least `least` sixths of a block of 16 keys.  The fused step gains from more CTAs down to little more
+// than a block a warp, whose chain is long (2 heads of 333 keys 6.5 -> 5.4 us a step with 4/3 of a block instead of
+// 2, 185 keys 8.5 -> 7.1; 1 block: 8 heads of 1,150 keys 7.0 -> 7.3).  Scores alone take less per block than a larger
+// cluster costs (8 heads of 3,400 keys 5.3 us with 2.5 blocks, 6.1 with 2, 5.7 with 3; with 2.5, 1 to 148 units of 64
+// to 8,192 keys all take what they took with 2 and at most eight CTAs, within 2 %, or less).  Shared units are scored
+// four blocks deep, the better by 1 to 15 % where both forms fit; with d = 64 that takes registers of a fourth CTA on
+// the SM, and long units it leaves whole, but two deep does not, go two deep (256 units of 3,400 keys 28.9 -> 20.7
+// us; of 1,150 keys whole 19.1, two deep 19.7).
 constexpr int kLeastAttend = 8, kLeastScore = 15;
 template <class Smem>
 int decode_split(const DecodeRoom& room, Smem&& smem, long long U, long long keys, int warps, int least) {
@@ -1363,7 +1378,8 @@ int decode_split(const DecodeRoom& room, Smem&& smem, long long U, long long key
     return n;
 }
 
-// Whole units of the fused step, at most two to an SM, are one uneven wave: its time is that of the SMs with most CTAs.
+// Whole units of the fused step, more of them than SMs and at most two to an SM, are one uneven wave: its time is that of the
+// SMs with most CTAs.
 // Begun early, it was placed while CTAs of the kernel before still held 32 SMs or so that
 // had another split of shared memory, and put three on others: 256 units of 3,276 keys 78 us a step, of 16,000 keys 350.
 // The kernels that end a step therefore ask for this kernel's split here, and this one for so much shared memory that
@@ -1373,12 +1389,13 @@ bool two_to_an_sm(const shotkv_ctx* ctx, const DecodeParams& p, int U) {
     return p.nsplit == 1 && U > ctx->sm_count && U <= 2 * ctx->sm_count;
 }
 
-// Does the step end in its first kernel (decode.cuh)?  Where the CTAs that share the units of a (sequence, layer) are one cluster,
-// one CTA to an SM does all of the step, and what is sent round stays small.  It saves a launch and a kernel boundary: one small
-// layer (2 heads of 333 keys) 5.1 -> 4.3 us a step with the attention output, 5.3 -> 4.4 without, 15.2 -> 13.1 us a call that evicts; 3 x 1 head
-// of 5,000 keys 5.0 -> 4.1; 4 x 8 heads of 185 keys 7.0 -> 6.7.  With more CTAs than SMs the clusters are placed worse
-// than single CTAs (32 layers x 8 heads 40 -> 46 us a step, with the attention output 70.5 -> 74.6).  An eviction, which all CTAs rank for
-// themselves, is for clusters of eight (16 CTAs, 8 layers: 9.4 -> 10.0), and ranks by counting, a thread an entry.
+// Does the step end in its first kernel (decode.cuh)?  Where the CTAs that share the units of a (sequence, layer) are
+// one cluster, one CTA to an SM does all of the step, and what is sent round stays small.  It saves a launch and a
+// kernel boundary: one small layer (2 heads of 333 keys) 5.1 -> 4.3 us a step with the attention output, 5.3 -> 4.4
+// without, 15.2 -> 13.1 us a call that evicts; 3 x 1 head of 5,000 keys 5.0 -> 4.1; 4 x 8 heads of 185 keys 7.0 ->
+// 6.7.  With more CTAs than SMs the clusters are placed worse than single CTAs (32 layers x 8 heads 40 -> 46 us a
+// step, with the attention output 70.5 -> 74.6).  An eviction, which all CTAs rank for themselves, is for clusters of
+// eight (16 CTAs, 8 layers: 9.4 -> 10.0), and ranks by counting, a thread an entry.
 constexpr int kFusedEvictCtas = 8;
 bool ends_fused(const shotkv_ctx* ctx, const int* room, const DecodeParams& p, const DecodeFinishParams& f, int U, int threads) {
     const int ctas = p.Hkv * p.nsplit;
@@ -1396,17 +1413,20 @@ int launch_decode_attend(shotkv_ctx* ctx, DecodeParams& p, const DecodeFinishPar
     size_t smem = smem_of(p.nsplit);
     const size_t end = fused_end_smem_bytes(p.Hkv, f.n, f.k < f.n);
     ended = smem + end <= kBigSmem && ends_fused(ctx, room[1].with(smem + end), p, f, U, Cfg::kWarps * 32);
+    const dim3 grid(U * p.nsplit);
     if (ended)
-        return launch(ctx, decode_attend_kernel<D, true>, dim3(U * p.nsplit), Cfg::kWarps * 32, smem + end, stream, p.Hkv * p.nsplit, kEarly, p, f);
+        return launch(ctx, decode_attend_kernel<D, true>, grid, Cfg::kWarps * 32, smem + end, stream, p.Hkv * p.nsplit, kEarly, p, f);
     if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "Dcap too large for the attention-output step");
     if (two_to_an_sm(ctx, p, U) && smem < kNoThirdCta) smem = kNoThirdCta;
-    return launch(ctx, decode_attend_kernel<D, false>, dim3(U * p.nsplit), Cfg::kWarps * 32, smem, stream, p.nsplit, kEarly, p, f);
+    return launch(ctx, decode_attend_kernel<D, false>, grid, Cfg::kWarps * 32, smem, stream, p.nsplit, kEarly, p, f);
 }
-// Are whole units scored two blocks of keys deep, which leaves an SM one CTA more than four deep does?  Where four deep they would
-// take a wave more, less than half full.  Two | four deep, us a step of units of 3,276 keys, d = 128: 256 units 39.4 | 39.7, 448 61.6 |
-// 81.0, 592 82.0 | 89.0, 640 104 | 91, 896 118 | 134, 1,024 130 | 141, 1,184 157 | 152, 2,048 255 | 256; of 300 keys, 64 units
-// 8.1 | 7.8; d = 64: 736 units 52 | 67, 744 70 | 67, 1,024 79 | 75.
-// Each CTA takes 1 KB of shared memory beside its own, of the 196 KB that an SM is split for where nothing asks for more.
+
+// Are whole units scored two blocks of keys deep, which leaves an SM one CTA more than four deep does?  Where four
+// deep they would take a wave more, less than half full.  Two | four deep, us a step of units of 3,276 keys, d = 128:
+// 256 units 39.4 | 39.7, 448 61.6 | 81.0, 592 82.0 | 89.0, 640 104 | 91, 896 118 | 134, 1,024 130 | 141, 1,184 157 |
+// 152, 2,048 255 | 256; of 300 keys, 64 units 8.1 | 7.8; d = 64: 736 units 52 | 67, 744 70 | 67, 1,024 79 | 75.
+// Each CTA takes 1 KB of shared memory beside its own, of the 196 KB that an SM is split for where nothing asks for
+// more.
 bool shallow_score(const shotkv_ctx* ctx, int d, int U, size_t smem) {
     const int fit = (int)(196 * 1024 / (smem + 1024));
     const auto wave = [&](int deep) { return ctx->sm_count * std::max(1, std::min(ctx->whole_score[d == 128][deep], fit)); };
@@ -1417,16 +1437,23 @@ template <int D>
 int launch_decode_score(shotkv_ctx* ctx, DecodeParams& p, const DecodeFinishParams& f, int U, bool& ended, cudaStream_t stream) {
     const DecodeRoom* room = ctx->room_score[D == 128];
     const size_t smem = score_smem_bytes(p.Dcap, true), end = fused_end_smem_bytes(p.Hkv, f.n, f.k < f.n);
-    const auto split = [&](const DecodeRoom& r, int least) { return decode_split(r, [&](int) { return smem; }, U, (long long)p.Mcap + p.n_old + 1, 8, least); };
+    const auto split = [&](const DecodeRoom& r, int least) {
+        return decode_split(r, [&](int) { return smem; }, U, (long long)p.Mcap + p.n_old + 1, 8, least);
+    };
+    auto* shared = decode_score_kernel<D, true, false, kDeep>;
     p.nsplit = split(room[0], kLeastScore);
-    if (D == 64 && p.nsplit == 1 && (p.nsplit = split(room[2], 2 * kLeastScore)) > 1)
-        return launch(ctx, decode_score_kernel<64, true, false, kShallow>, dim3(U * p.nsplit), 256, smem, stream, p.nsplit, kEarly, p, f);
+    if (D == 64 && p.nsplit == 1) {
+        p.nsplit = split(room[2], 2 * kLeastScore);
+        if (p.nsplit > 1) shared = decode_score_kernel<D, true, false, D == 64 ? kShallow : kDeep>;
+    }
+    const dim3 grid(U * p.nsplit);
     ended = smem + end <= kBigSmem && ends_fused(ctx, room[1].with(smem + end), p, f, U, 256);
-    if (ended) return launch(ctx, decode_score_kernel<D, true, true, kDeep>, dim3(U * p.nsplit), 256, smem + end, stream, p.Hkv * p.nsplit, kEarly, p, f);
-    if (p.nsplit > 1) return launch(ctx, decode_score_kernel<D, true, false, kDeep>, dim3(U * p.nsplit), 256, smem, stream, p.nsplit, kEarly, p, f);
+    if (ended) return launch(ctx, decode_score_kernel<D, true, true, kDeep>, grid, 256, smem + end, stream, p.Hkv * p.nsplit, kEarly, p, f);
+    if (p.nsplit > 1) return launch(ctx, shared, grid, 256, smem, stream, p.nsplit, kEarly, p, f);
     const size_t whole = score_smem_bytes(p.Dcap, false);
-    return launch(ctx, shallow_score(ctx, D, U, whole) ? decode_score_kernel<D, false, false, kShallow> : decode_score_kernel<D, false, false, kDeep>,
-                  dim3(U), 256, whole, stream, 1, kEarly, p, f);
+    auto* kernel = decode_score_kernel<D, false, false, kDeep>;
+    if (shallow_score(ctx, D, U, whole)) kernel = decode_score_kernel<D, false, false, kShallow>;
+    return launch(ctx, kernel, grid, 256, whole, stream, 1, kEarly, p, f);
 }
 
 // One decode step; with `attn_out` the score kernel is the variant that also writes the attention output.
@@ -1471,19 +1498,19 @@ int decode_step_impl(shotkv_ctx* ctx, shotkv_decode_state* st, const shotkv_bf16
     bool ended = false;                                   // the step ends in this kernel
     prof_begin(ctx);
     prof_mark(ctx, stream);
-    if (attn_out) rc = d.d == 128 ? launch_decode_attend<128>(ctx, p, f, U, ended, stream) : launch_decode_attend<64>(ctx, p, f, U, ended, stream);
-    else rc = d.d == 128 ? launch_decode_score<128>(ctx, p, f, U, ended, stream) : launch_decode_score<64>(ctx, p, f, U, ended, stream);
-    if (rc) return rc;
+    const auto first = attn_out ? (d.d == 128 ? launch_decode_attend<128> : launch_decode_attend<64>)
+                                : (d.d == 128 ? launch_decode_score<128> : launch_decode_score<64>);
+    if ((rc = first(ctx, p, f, U, ended, stream))) return rc;
     prof_mark(ctx, stream);
 
     const int how = kEarly | (attn_out && two_to_an_sm(ctx, p, U) ? kWideShared : 0);
-    if (ended) {
-    } else if (f.k < f.n) {
+    if (!ended && f.k < f.n) {
         f.ranks = d.Hkv < kReduceCluster ? d.Hkv : kReduceCluster;
-        rc = d.d == 128 ? launch(ctx, decode_evict_kernel<128>, dim3(BL * f.ranks), kSelectThreads, decode_evict_smem_bytes(f.n), stream, f.ranks, how, f)
-                        : launch(ctx, decode_evict_kernel<64>, dim3(BL * f.ranks), kSelectThreads, decode_evict_smem_bytes(f.n), stream, f.ranks, how, f);
-    } else {
-        rc = launch(ctx, decode_accumulate_kernel, dim3(BL, (f.n + kAccumulateThreads - 1) / kAccumulateThreads), kAccumulateThreads, 0, stream, 1, how, f);
+        rc = launch(ctx, d.d == 128 ? decode_evict_kernel<128> : decode_evict_kernel<64>, dim3(BL * f.ranks), kSelectThreads,
+                    decode_evict_smem_bytes(f.n), stream, f.ranks, how, f);
+    } else if (!ended) {
+        rc = launch(ctx, decode_accumulate_kernel, dim3(BL, (f.n + kAccumulateThreads - 1) / kAccumulateThreads), kAccumulateThreads, 0,
+                    stream, 1, how, f);
     }
     if (rc) return rc;
     st->T = T;
@@ -1569,7 +1596,8 @@ int shotkv_selftest_bounded_wait(shotkv_ctx* ctx, int64_t limit_cycles, int32_t*
     CUDA_TRY(ctx, cudaStreamSynchronize(stream));
     for (int i = 0; i < 4; ++i) report[i] = words[i];
     if (words[4] != 0 || words[5] != 1)
-        return fail(ctx, SHOTKV_ERR_CUDA, "the wait for messages did not give up as it should (succeeded %d, outlived its sender %d)", words[4], words[5]);
+        return fail(ctx, SHOTKV_ERR_CUDA, "the wait for messages did not give up as it should (succeeded %d, outlived its sender %d)",
+                    words[4], words[5]);
     return SHOTKV_OK;
 }
 
