@@ -104,3 +104,9 @@ def test_whole_units_on_both_sides_of_a_wave(ctx, d, L):
     """Units that are scored two and four blocks of keys deep, shared and whole, one wave of them and more."""
     cfg = wl.DecodeConfig("waves", B=1, L=L, H=16, Hkv=8, d=d, steps=5, r_d=0.5, recompress_every=4, cfg_id=80)
     assert lockstep(ctx, cfg, 1400, [(0, 0), (0, L - 1)], np.full((1, L), 1311, np.int32)) <= 1
+
+
+def test_entries_of_whole_units(ctx):
+    """The attention-output step of units that no cluster shares, with more decode entries than a CTA has threads."""
+    cfg = wl.DecodeConfig("entries", B=1, L=20, H=24, Hkv=8, d=64, steps=133, r_d=0.5, recompress_every=131, cfg_id=81)
+    assert lockstep(ctx, cfg, 30, [(0, 7)], np.full((1, 20), 29, np.int32), attend=True) <= 1
