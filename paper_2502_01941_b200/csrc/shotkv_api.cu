@@ -105,8 +105,7 @@ struct shotkv_ctx {
     long long wait_cycles = tc::kWaitCycles;   // limit of every bounded device-side wait
     int32_t* static_offsets = nullptr;         // device address of the built-in boundary table (looked up on first use)
     void* encode_tiled = nullptr;              // cuTensorMapEncodeTiled, resolved at creation
-    // [d = 128][the step ends in its first kernel], and [0][2] of shared units scored two blocks of keys deep (asked at creation)
-    DecodeRoom room_attend[2][2], room_score[2][3];
+    DecodeRoom room_attend[2][2], room_score[2][2];   // [d = 128][the step ends in its first kernel] (asked at creation)
     int whole_score[2][2] = {};                // CTAs that have a unit each and fit an SM, two and four blocks of keys deep
 };
 
@@ -792,8 +791,7 @@ cudaError_t set_kernel_attributes() {
     const void* score[] = {(const void*)decode_score_kernel<128, true, false, kDeep>,
                            (const void*)decode_score_kernel<128, true, true, kDeep>,
                            (const void*)decode_score_kernel<64, true, false, kDeep>,
-                           (const void*)decode_score_kernel<64, true, true, kDeep>,
-                           (const void*)decode_score_kernel<64, true, false, kShallow>};
+                           (const void*)decode_score_kernel<64, true, true, kDeep>};
     const auto in_clusters = [&](const void* f) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, kBigSmem);
         if (e == cudaSuccess) e = cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -841,7 +839,6 @@ cudaError_t ask_decode_room_t(shotkv_ctx* ctx) {
     if (e == cudaSuccess) e = ask_room(decode_attend_kernel<D, true>, AttendCfg<D>::kWarps * 32, attend[1]);
     if (e == cudaSuccess) e = ask_room(decode_score_kernel<D, true, false, kDeep>, 256, score[0]);
     if (e == cudaSuccess) e = ask_room(decode_score_kernel<D, true, true, kDeep>, 256, score[1]);
-    if (e == cudaSuccess && D == 64) e = ask_room(decode_score_kernel<64, true, false, kShallow>, 256, score[2]);
     int* whole = ctx->whole_score[D == 128];
     const auto fit = [&](int& ctas, auto* kernel) {
         if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&ctas, kernel, 256, 0);
@@ -1366,10 +1363,7 @@ namespace {
 // than a block a warp, whose chain is long (2 heads of 333 keys 6.5 -> 5.4 us a step with 4/3 of a block instead of
 // 2, 185 keys 8.5 -> 7.1; 1 block: 8 heads of 1,150 keys 7.0 -> 7.3).  Scores alone take less per block than a larger
 // cluster costs (8 heads of 3,400 keys 5.3 us with 2.5 blocks, 6.1 with 2, 5.7 with 3; with 2.5, 1 to 148 units of 64
-// to 8,192 keys all take what they took with 2 and at most eight CTAs, within 2 %, or less).  Shared units are scored
-// four blocks deep, the better by 1 to 15 % where both forms fit; with d = 64 that takes registers of a fourth CTA on
-// the SM, and long units it leaves whole, but two deep does not, go two deep (256 units of 3,400 keys 28.9 -> 20.7
-// us; of 1,150 keys whole 19.1, two deep 19.7).
+// to 8,192 keys all take what they took with 2 and at most eight CTAs, within 2 %, or less).
 constexpr int kLeastAttend = 8, kLeastScore = 15;
 template <class Smem>
 int decode_split(const DecodeRoom& room, Smem&& smem, long long U, long long keys, int warps, int least) {
@@ -1378,9 +1372,8 @@ int decode_split(const DecodeRoom& room, Smem&& smem, long long U, long long key
     return n;
 }
 
-// Whole units of the fused step, more of them than SMs and at most two to an SM, are one uneven wave: its time is that of the
-// SMs with most CTAs.
-// Begun early, it was placed while CTAs of the kernel before still held 32 SMs or so that
+// Whole units of the fused step, more of them than SMs and at most two to an SM, are one uneven wave: its time is that
+// of the SMs with most CTAs.  Begun early, it was placed while CTAs of the kernel before still held 32 SMs or so that
 // had another split of shared memory, and put three on others: 256 units of 3,276 keys 78 us a step, of 16,000 keys 350.
 // The kernels that end a step therefore ask for this kernel's split here, and this one for so much shared memory that
 // no third CTA fits: 71 and 310 us (288 units 88 -> 81 and 382 -> 365).
@@ -1396,12 +1389,15 @@ bool two_to_an_sm(const shotkv_ctx* ctx, const DecodeParams& p, int U) {
 // 6.7.  With more CTAs than SMs the clusters are placed worse than single CTAs (32 layers x 8 heads 40 -> 46 us a
 // step, with the attention output 70.5 -> 74.6).  An eviction, which all CTAs rank for themselves, is for clusters of
 // eight (16 CTAs, 8 layers: 9.4 -> 10.0), and ranks by counting, a thread an entry.
-constexpr int kFusedEvictCtas = 8;
-bool ends_fused(const shotkv_ctx* ctx, const int* room, const DecodeParams& p, const DecodeFinishParams& f, int U, int threads) {
+// One CTA adds up the entries of a step that does not evict, so with many of them the kernel that spreads them is the better.  One head of
+// 600 keys, first kernel | two, us a step, scores: 700 entries 4.9 | 5.1, 1,000 5.4 | 5.2, 2,000 6.2 | 5.4; with the attention output: 310
+// 5.4 | 5.6, 500 6.1 | 5.6, 2,000 11.1 | 7.1.
+constexpr int kFusedEvictCtas = 8, kFusedEntriesScore = 1024, kFusedEntriesAttend = 400;
+bool ends_fused(const shotkv_ctx* ctx, const int* room, const DecodeParams& p, const DecodeFinishParams& f, int U, int threads, int entries) {
     const int ctas = p.Hkv * p.nsplit;
     const bool evicts = f.k < f.n;
     return ctas > 1 && ctas <= (evicts ? kFusedEvictCtas : kMaxSplit) && U * p.nsplit <= ctx->sm_count && U / p.Hkv <= room[ctas] &&
-           f.Hkv * f.n <= kFusedWeights && (!evicts || f.n <= threads);
+           f.Hkv * f.n <= kFusedWeights && f.n <= entries && (!evicts || f.n <= threads);
 }
 
 template <int D>
@@ -1412,7 +1408,7 @@ int launch_decode_attend(shotkv_ctx* ctx, DecodeParams& p, const DecodeFinishPar
     p.nsplit = decode_split(room[0], smem_of, U, (long long)p.Mcap + p.n_old + 1, Cfg::kWarps, kLeastAttend);
     size_t smem = smem_of(p.nsplit);
     const size_t end = fused_end_smem_bytes(p.Hkv, f.n, f.k < f.n);
-    ended = smem + end <= kBigSmem && ends_fused(ctx, room[1].with(smem + end), p, f, U, Cfg::kWarps * 32);
+    ended = smem + end <= kBigSmem && ends_fused(ctx, room[1].with(smem + end), p, f, U, Cfg::kWarps * 32, kFusedEntriesAttend);
     const dim3 grid(U * p.nsplit);
     if (ended)
         return launch(ctx, decode_attend_kernel<D, true>, grid, Cfg::kWarps * 32, smem + end, stream, p.Hkv * p.nsplit, kEarly, p, f);
@@ -1437,19 +1433,11 @@ template <int D>
 int launch_decode_score(shotkv_ctx* ctx, DecodeParams& p, const DecodeFinishParams& f, int U, bool& ended, cudaStream_t stream) {
     const DecodeRoom* room = ctx->room_score[D == 128];
     const size_t smem = score_smem_bytes(p.Dcap, true), end = fused_end_smem_bytes(p.Hkv, f.n, f.k < f.n);
-    const auto split = [&](const DecodeRoom& r, int least) {
-        return decode_split(r, [&](int) { return smem; }, U, (long long)p.Mcap + p.n_old + 1, 8, least);
-    };
-    auto* shared = decode_score_kernel<D, true, false, kDeep>;
-    p.nsplit = split(room[0], kLeastScore);
-    if (D == 64 && p.nsplit == 1) {
-        p.nsplit = split(room[2], 2 * kLeastScore);
-        if (p.nsplit > 1) shared = decode_score_kernel<D, true, false, D == 64 ? kShallow : kDeep>;
-    }
+    p.nsplit = decode_split(room[0], [&](int) { return smem; }, U, (long long)p.Mcap + p.n_old + 1, 8, kLeastScore);
     const dim3 grid(U * p.nsplit);
-    ended = smem + end <= kBigSmem && ends_fused(ctx, room[1].with(smem + end), p, f, U, 256);
+    ended = smem + end <= kBigSmem && ends_fused(ctx, room[1].with(smem + end), p, f, U, 256, kFusedEntriesScore);
     if (ended) return launch(ctx, decode_score_kernel<D, true, true, kDeep>, grid, 256, smem + end, stream, p.Hkv * p.nsplit, kEarly, p, f);
-    if (p.nsplit > 1) return launch(ctx, shared, grid, 256, smem, stream, p.nsplit, kEarly, p, f);
+    if (p.nsplit > 1) return launch(ctx, decode_score_kernel<D, true, false, kDeep>, grid, 256, smem, stream, p.nsplit, kEarly, p, f);
     const size_t whole = score_smem_bytes(p.Dcap, false);
     auto* kernel = decode_score_kernel<D, false, false, kDeep>;
     if (shallow_score(ctx, D, U, whole)) kernel = decode_score_kernel<D, false, false, kShallow>;

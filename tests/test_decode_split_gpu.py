@@ -7,6 +7,7 @@ import torch
 
 import paper_2502_01941_b200 as skv
 from paper_2502_01941_b200 import workloads as wl
+import parity as P
 from test_decode_gpu import GpuDecoder, OUT_ATOL, OUT_RTOL, lockstep
 
 pytestmark = pytest.mark.gpu
@@ -110,3 +111,30 @@ def test_entries_of_whole_units(ctx):
     """The attention-output step of units that no cluster shares, with more decode entries than a CTA has threads."""
     cfg = wl.DecodeConfig("entries", B=1, L=20, H=24, Hkv=8, d=64, steps=133, r_d=0.5, recompress_every=131, cfg_id=81)
     assert lockstep(ctx, cfg, 30, [(0, 7)], np.full((1, 20), 29, np.int32), attend=True) <= 1
+
+
+@pytest.mark.parametrize("G,d", [(1, 64), (3, 128), (5, 64), (8, 128)])
+@pytest.mark.parametrize("attend,most", [(False, 1024), (True, 400)], ids=["plain", "attend"])
+def test_many_entries(ctx, G, d, attend, most):
+    """Steps on both sides of the number of entries up to which they end in their first kernel, rows in two halves of four."""
+    cfg = wl.DecodeConfig("many", B=1, L=1, H=2 * G, Hkv=2, d=d, steps=most + 3, r_d=0.9, recompress_every=most + 3, cfg_id=82)
+    Kc, kept = wl.random_prefill_cache(cfg, 40, "cuda", np.full((1, 1), 37, np.int32))
+    gpu = GpuDecoder(ctx, cfg, Kc, kept, Vc=wl.random_prefill_values(cfg, 40, "cuda") if attend else None)
+    g = torch.Generator(device="cuda").manual_seed(5)
+    n = most - 2
+    for x in (gpu.Kd, gpu.Vd):
+        x.copy_(torch.randn(x.shape, generator=g, device="cuda"))
+    gpu.acc.copy_(torch.rand(gpu.acc.shape, generator=g, device="cuda"))
+    gpu.state.T = gpu.state.n_dec = n
+    for one in (True, True, False, False):
+        q, k, v = wl.decode_step_inputs(cfg, n, "cuda")
+        want = gpu.acc[0, 0, :n].double()
+        before = skv.shotkv_launch_count(ctx)
+        gpu.step(q, k, v)
+        torch.cuda.synchronize()
+        assert skv.shotkv_launch_count(ctx) - before == (1 if one else 2)
+        n += 1
+        keys = torch.cat([Kc[0, 0, :, :37], gpu.Kd[0, 0, :, :n]], 1).double()
+        w = ((q[0, 0].double().view(2, G, 1, d) * keys[:, None]).sum(-1) / d ** 0.5).softmax(-1)
+        want = torch.cat([want, want.new_zeros(1)]) + w[:, :, 37:].sum((0, 1))
+        np.testing.assert_allclose(gpu.acc[0, 0, :n].double().cpu().numpy(), want.cpu().numpy(), rtol=P.SCORE_RTOL, atol=P.SCORE_ATOL)
