@@ -1376,10 +1376,13 @@ int decode_split(const DecodeRoom& room, Smem&& smem, long long U, long long key
 // of the SMs with most CTAs.  Begun early, it was placed while CTAs of the kernel before still held 32 SMs or so that
 // had another split of shared memory, and put three on others: 256 units of 3,276 keys 78 us a step, of 16,000 keys 350.
 // The kernels that end a step therefore ask for this kernel's split here, and this one for so much shared memory that
-// no third CTA fits: 71 and 310 us (288 units 88 -> 81 and 382 -> 365).
+// no third CTA fits: 71 and 310 us (288 units 88 -> 81 and 382 -> 365).  So do 3 to 4 times as many units as SMs with d = 128, of
+// which three fit an SM: as two full waves of pairs they are the better than as one of three and a rest.  448, 512, 592 units of
+// 3,276 keys three | two to an SM 131, 148, 158 | 120, 132, 153 us; of 600 keys and 400 entries 49, 56, 58 | 46, 49, 55.
 constexpr size_t kNoThirdCta = 80 * 1024;
-bool two_to_an_sm(const shotkv_ctx* ctx, const DecodeParams& p, int U) {
-    return p.nsplit == 1 && U > ctx->sm_count && U <= 2 * ctx->sm_count;
+bool two_to_an_sm(const shotkv_ctx* ctx, const DecodeParams& p, int U, int d) {
+    const int sms = ctx->sm_count;
+    return p.nsplit == 1 && ((U > sms && U <= 2 * sms) || (d == 128 && U > 3 * sms && U <= 4 * sms));
 }
 
 // Does the step end in its first kernel (decode.cuh)?  Where the CTAs that share the units of a (sequence, layer) are
@@ -1413,7 +1416,7 @@ int launch_decode_attend(shotkv_ctx* ctx, DecodeParams& p, const DecodeFinishPar
     if (ended)
         return launch(ctx, decode_attend_kernel<D, true>, grid, Cfg::kWarps * 32, smem + end, stream, p.Hkv * p.nsplit, kEarly, p, f);
     if (smem > kBigSmem) return fail(ctx, SHOTKV_ERR_UNSUPPORTED_SHAPE, "Dcap too large for the attention-output step");
-    if (two_to_an_sm(ctx, p, U) && smem < kNoThirdCta) smem = kNoThirdCta;
+    if (two_to_an_sm(ctx, p, U, D) && smem < kNoThirdCta) smem = kNoThirdCta;
     return launch(ctx, decode_attend_kernel<D, false>, grid, Cfg::kWarps * 32, smem, stream, p.nsplit, kEarly, p, f);
 }
 
@@ -1491,7 +1494,7 @@ int decode_step_impl(shotkv_ctx* ctx, shotkv_decode_state* st, const shotkv_bf16
     if ((rc = first(ctx, p, f, U, ended, stream))) return rc;
     prof_mark(ctx, stream);
 
-    const int how = kEarly | (attn_out && two_to_an_sm(ctx, p, U) ? kWideShared : 0);
+    const int how = kEarly | (attn_out && two_to_an_sm(ctx, p, U, d.d) ? kWideShared : 0);
     if (!ended && f.k < f.n) {
         f.ranks = d.Hkv < kReduceCluster ? d.Hkv : kReduceCluster;
         rc = launch(ctx, d.d == 128 ? decode_evict_kernel<128> : decode_evict_kernel<64>, dim3(BL * f.ranks), kSelectThreads,

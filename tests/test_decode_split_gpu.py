@@ -82,9 +82,9 @@ def test_query_that_is_not_a_number_gives_no_output(ctx, M):
     assert (err <= OUT_RTOL * want[:, 0].abs().amax(1, keepdim=True) + OUT_ATOL).all(), err.amax(1)
 
 
-@pytest.mark.parametrize("L", [19, 32, 37])
+@pytest.mark.parametrize("L", [19, 32, 37, 55, 56, 74, 75])
 def test_whole_units_two_to_an_sm(ctx, L):
-    """More units than SMs and at most two to an SM, an eviction among the steps."""
+    """More units than SMs and at most two to an SM, and three to four times as many, an eviction among the steps."""
     cfg = wl.DecodeConfig("pairs", B=1, L=L, H=32, Hkv=8, d=128, steps=9, r_d=0.5, recompress_every=4, cfg_id=75)
     assert lockstep(ctx, cfg, 300, [(0, 0), (0, L - 1)], attend=True) <= 1
 
