@@ -224,8 +224,8 @@ __device__ __forceinline__ void entry_weights(const float* sdec, int Dcap, int G
             for (int r = 0; r < 4; ++r) x[r] = sdec[min(half + r, G - 1) * Dcap + j];
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
-                const float w = ex2f(x[r] - mr[half + r]) * izr[half + r];
-                s += half + r < G ? w : 0.f;
+                const float more = fmaf(ex2f(x[r] - mr[half + r]), izr[half + r], s);
+                s = half + r < G ? more : s;
             }
         }
         emit(j, s);
